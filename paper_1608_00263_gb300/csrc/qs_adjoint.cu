@@ -255,13 +255,20 @@ k_adj_group(typename V2T<R>::T *__restrict__ psi, typename V2T<R>::T *__restrict
     for (int k = tid; k < P.nparam; k += blockDim.x) part[(size_t)k * nparts + blockIdx.x] = acc_sh[k];
 }
 
+// One warp per parameter: lanes add the CTAs' partials lane, lane + 32, ...
+// (independent loads), then the warp in a fixed order.  A thread per
+// parameter adding 456 partials in turn took 66 us.
 __global__ void k_adj_sums(const double *__restrict__ part, int nparts, int nparam, const double *__restrict__ scale,
                            double *__restrict__ out)
 {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nparam; k += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, warps = (int)(gridDim.x * (blockDim.x >> 5));
+    for (int k = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); k < nparam; k += warps) {
         double s = 0;
-        for (int b = 0; b < nparts; ++b) s += part[(size_t)k * nparts + b];
-        out[k] = s * scale[k];
+#pragma unroll 8
+        for (int b = lane; b < nparts; b += 32) s += part[(size_t)k * nparts + b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[k] = s * scale[k];
     }
 }
 
@@ -396,7 +403,7 @@ static qs_status adjoint_t(qs_state *s, const qs_gate *g, size_t ng, const uint6
                 slot0 += groups[gi].nparam;
             }
             if (nparam)
-                k_adj_sums<<<grid_for(nparam, 128, s->num_sms, 1), 128, 0, s->stream>>>(
+                k_adj_sums<<<grid_for(nparam * 32, 128, s->num_sms, 4), 128, 0, s->stream>>>(
                     (const double *)(dev + o_part), ctas, (int)nparam, (const double *)(dev + o_scale),
                     (double *)(dev + o_out));
             if (e == cudaSuccess) e = cudaGetLastError();

@@ -21,17 +21,49 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Sums acc over the block's kStatThreads threads (warp shuffles, then the
-// warps' sums in warp order) and stores the K sums at dst (threads < K).
+// Sums acc[k] over the warp for every k < K <= 16 by recursive halving: at
+// each step a lane hands half of its sums to its partner and keeps the other
+// half, so a warp spends K (rounded up to 16) additions in all instead of
+// 5 K.  FP64 additions are what bounds this tail (two lanes per clock and
+// SM).  Lane l returns the total of accumulator (l & 15) (K <= l: 0).
+template <int K>
+__device__ __forceinline__ double warp_sum_many(const double (&acc)[K])
+{
+    static_assert(K <= 16, "at most 16 accumulators");
+    const int lane = threadIdx.x & 31;
+    double v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = k < K ? acc[k < K ? k : 0] : 0.0;
+    // bit o of the lane selects the upper half of the sums left
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < o; ++k) {
+            const double give = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
+}
+
+// Sums acc over the block's kStatThreads threads (recursive halving inside a
+// warp, then the warps' sums in warp order) and stores the K sums at dst
+// (threads < K).
 template <int K>
 __device__ __forceinline__ void block_sum_store(double (&acc)[K], double *dst)
 {
-    __shared__ double red[kStatThreads / 32][K];
+    __shared__ double red[kStatThreads / 32][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (K >= 4) {
+        const double v = warp_sum_many<K>(acc);
+        if (lane < 16) red[warp][lane] = v;
+    } else {
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double v = warp_sum(acc[k]);
-        if (lane == 0) red[warp][k] = v;
+        for (int k = 0; k < K; ++k) {
+            const double v = warp_sum(acc[k]);
+            if (lane == 0) red[warp][k] = v;
+        }
     }
     __syncthreads();
     if (threadIdx.x < K) {
