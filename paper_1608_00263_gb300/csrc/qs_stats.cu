@@ -318,21 +318,37 @@ void stats_from_sums(const double *h, int n, int kmax, double *norm, double *ent
 // exactly this arithmetic, so chunk sums and in-chunk prefixes agree (the
 // chunk offsets themselves are FP64 scans of the chunk sums).
 template <typename R>
+__device__ __forceinline__ R amp_prob(typename V2T<R>::T v)
+{
+    if constexpr (sizeof(R) == 4) return prob32(v);
+    else return v.x * v.x + v.y * v.y;
+}
+
+// The 8 probabilities from amplitude `first` on (16-byte loads; elements at
+// N or above, in a state's one partial chunk, count as 0).
+template <typename R>
+__device__ __forceinline__ void probs8(const typename V2T<R>::T *a, uint64_t first, uint64_t N, R (&p)[8])
+{
+    using V = typename V2T<R>::T;
+    constexpr int E = 16 / (int)sizeof(V);
+    if (first + 8 <= N) {
+        V v[8];
+        const float4 *src = reinterpret_cast<const float4 *>(a + first);
+#pragma unroll
+        for (int i = 0; i < 8 / E; ++i) reinterpret_cast<float4 *>(v)[i] = src[i];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p[i] = amp_prob<R>(v[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p[i] = first + i < N ? amp_prob<R>(a[first + i]) : (R)0;
+    }
+}
+
+template <typename R>
 __device__ __forceinline__ void lane_probs(const typename V2T<R>::T *a, uint64_t chunk, int lane,
                                            uint64_t N, R (&p)[8])
 {
-    const uint64_t base = chunk * kChunk + (uint64_t)lane * 8;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        uint64_t idx = base + i;
-        if (idx < N) {
-            auto v = a[idx];
-            if constexpr (sizeof(R) == 4) p[i] = prob32(v);
-            else p[i] = v.x * v.x + v.y * v.y;
-        } else {
-            p[i] = (R)0;
-        }
-    }
+    probs8<R>(a, chunk * kChunk + (uint64_t)lane * 8, N, p);
 }
 
 template <typename R>
@@ -475,8 +491,75 @@ __device__ __forceinline__ uint64_t splitmix_out(uint64_t seed, uint64_t j)
     return z ^ (z >> 31);
 }
 
+// a > b for doubles that are never negative: the order of their bit patterns
+// (this GPU's FP64 pipe does two lanes per clock and SM, comparisons included)
+__device__ __forceinline__ bool gt_nonneg(double a, double b)
+{
+    return __double_as_longlong(a) > __double_as_longlong(b);
+}
+
+// Inclusive in-chunk prefix of the lanes, in the state's precision.
+__device__ __forceinline__ float chunk_incl(float lt) { return warp_incl_scan_f(lt); }
+__device__ __forceinline__ double chunk_incl(double lt) { return warp_incl_scan(lt); }
+// x > t for an in-chunk prefix x and the threshold of a sample: FP32 prefixes
+// are compared with the threshold rounded down to FP32 (x > t exactly when
+// x > round_down(t), x being an FP32 value).
+__device__ __forceinline__ float chunk_threshold(double t, float) { return __double2float_rd(t); }
+__device__ __forceinline__ double chunk_threshold(double t, double) { return t; }
+__device__ __forceinline__ bool prefix_above(float x, float t) { return x > t; }
+__device__ __forceinline__ bool prefix_above(double x, double t) { return gt_nonneg(x, t); }
+__device__ __forceinline__ double widen(float x) { return widen_f32(x); }
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// The lane (eight amplitudes) of chunk c that holds the sample whose
+// in-chunk threshold is th, and the prefix before that lane: the whole warp
+// rescans the chunk with the arithmetic that formed its sum.  Rounding edge
+// (no prefix above th): the last lane with a nonzero sum; none: -1.
+template <typename R>
+__device__ __forceinline__ int chunk_lane(const R (&p)[8], R th, R *excl)
+{
+    const R lt = lane_total<R>(p);
+    const R incl = chunk_incl(lt);
+    const unsigned hit = __ballot_sync(0xffffffffu, prefix_above(incl, th));
+    const unsigned nz = __ballot_sync(0xffffffffu, lt > (R)0);
+    const int L = hit ? __ffs(hit) - 1 : 31 - __clz(nz);
+    R before;
+    if constexpr (sizeof(R) == 4) {
+        before = __shfl_sync(0xffffffffu, incl, L > 0 ? L - 1 : 0);
+        if (L <= 0) before = (R)0;
+    } else {
+        before = __shfl_sync(0xffffffffu, incl - lt, L > 0 ? L : 0);
+    }
+    *excl = before;
+    return L;
+}
+
+// Which of the eight amplitudes p of a lane the sample falls on: the first
+// nonzero one whose prefix (excl + their running sum) exceeds t, else the
+// last nonzero one, else -1.
+template <typename R>
+__device__ __forceinline__ int pick8(const R (&p)[8], R excl, double t)
+{
+    const double ex = widen(excl);
+    R acc = (R)0;
+    int pick = -1, last_nz = -1;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        acc += p[i];
+        if (p[i] > (R)0) last_nz = i;
+        if (pick < 0 && p[i] > (R)0 && gt_nonneg(ex + widen(acc), t)) pick = i;
+    }
+    return pick < 0 ? last_nz : pick;
+}
+
 // One warp handles 32 samples: each lane binary-searches the chunk of its
-// own sample, then the warp rescans each of the 32 chunks in turn.
+// own sample; the warp rescans the 32 chunks in turn (coalesced 16-byte
+// loads), which leaves each lane the eight-amplitude group of its own sample;
+// then every lane resolves its own group.  What bounds it is the m random
+// 2 KB chunk reads; the FP64 additions of the last step run once per 32
+// samples.  Resolving the group inside the rescan (one lane active) and
+// comparing prefixes in FP64 had made the FP64 pipe the bound: 1.69 ms for
+// 10^6 samples at 26 qubits.
 template <typename R>
 __global__ void k_sample_search(const typename V2T<R>::T *__restrict__ a, uint64_t N, uint64_t nchunks,
                                 const double *__restrict__ cincl, uint64_t k, uint64_t seed,
@@ -496,39 +579,35 @@ __global__ void k_sample_search(const typename V2T<R>::T *__restrict__ a, uint64
             uint64_t lo = 0, hi = nchunks - 1;   // cincl[hi] = total > target
             while (lo < hi) {
                 uint64_t mid = lo + (hi - lo) / 2;
-                if (cincl[mid] > target) hi = mid; else lo = mid + 1;
+                if (gt_nonneg(cincl[mid], target)) hi = mid; else lo = mid + 1;
             }
             chunk = lo;
             tloc = target - (lo ? cincl[lo - 1] : 0.0);
         }
+        const R th = chunk_threshold(tloc, (R)0);
         const int cnt = (int)((k - j0) < 32 ? (k - j0) : 32);
+        int L = 0;
+        R excl = (R)0;
+#pragma unroll 2
         for (int q = 0; q < cnt; ++q) {
             const uint64_t c = __shfl_sync(0xffffffffu, chunk, q);
-            const double tq = __shfl_sync(0xffffffffu, tloc, q);
-            R p[8];
+            const R tq = __shfl_sync(0xffffffffu, th, q);
+            R p[8], ex;
             lane_probs<R>(a, c, lane, N, p);
-            const R lt = lane_total<R>(p);
-            double incl, excl;
-            chunk_scan(lt, incl, excl);
-            unsigned hit = __ballot_sync(0xffffffffu, incl > tq);
-            unsigned nz = __ballot_sync(0xffffffffu, lt > (R)0);
-            int L = hit ? __ffs(hit) - 1 : 31 - __clz(nz);   // rounding edge: last non-empty lane
-            uint64_t res = 0;
-            if (lane == L) {
-                R acc = (R)0;
-                int pick = -1, last_nz = -1;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    acc += p[i];
-                    if (p[i] > (R)0) last_nz = i;
-                    if (pick < 0 && p[i] > (R)0 && excl + (double)acc > tq) pick = i;
-                }
-                if (pick < 0) pick = last_nz;
-                res = c * kChunk + (uint64_t)L * 8 + (uint64_t)pick;
+            const int lq = chunk_lane<R>(p, tq, &ex);
+            if (lane == q) {
+                L = lq;
+                excl = ex;
             }
-            res = __shfl_sync(0xffffffffu, res, L);
+        }
+        if (j < k) {
+            R p[8];
+            const uint64_t first = chunk * kChunk + (uint64_t)(L < 0 ? 0 : L) * 8;
+            probs8<R>(a, first, N, p);
+            const int pick = pick8<R>(p, excl, tloc);
+            const uint64_t res = first + (uint64_t)(pick < 0 ? 0 : pick);
             // the sample lies inside the state (checked build)
-            if (lane == q && QS_DCHECK(res < N && c < nchunks, 301)) out[j0 + q] = res;
+            if (QS_DCHECK(res < N && chunk < nchunks, 301)) out[j] = res;
         }
     }
 }
@@ -830,46 +909,39 @@ __global__ void k_batch_sample_search(const float2 *__restrict__ amps, const uin
             chunk = lo;
             tloc = target - (lo ? cincl[lo - 1] : 0.0);
         }
+        const float th = chunk_threshold(tloc, 0.f);
         const int cnt = (int)((m - j0) < 32 ? (m - j0) : 32);
+        int L = 0;
+        float excl = 0.f;
+#pragma unroll 2
         for (int q = 0; q < cnt; ++q) {
             const uint64_t c = __shfl_sync(0xffffffffu, chunk, q);
-            const double tq = __shfl_sync(0xffffffffu, tloc, q);
+            const float tq = __shfl_sync(0xffffffffu, th, q);
             const int iq = __shfl_sync(0xffffffffu, inst, q);
-            const uint64_t lc = c - cbase[iq];
-            float p[8];
-            lane_probs<float>(amps + off[iq], lc, lane, 1ULL << nq[iq], p);
-            const float lt = lane_total<float>(p);
-            double incl, excl;
-            chunk_scan(lt, incl, excl);
-            const unsigned hit = __ballot_sync(0xffffffffu, incl > tq);
-            const unsigned nz = __ballot_sync(0xffffffffu, lt > 0.f);
-            const int L = hit ? __ffs(hit) - 1 : (nz ? 31 - __clz(nz) : 0);
-            uint64_t res = 0;
-            if (lane == L) {
-                float acc = 0.f;
-                int pick = -1, last_nz = -1;
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    acc += p[t];
-                    if (p[t] > 0.f) last_nz = t;
-                    if (pick < 0 && p[t] > 0.f && excl + (double)acc > tq) pick = t;
-                }
-                if (pick < 0) pick = last_nz < 0 ? 0 : last_nz;
-                res = lc * kChunk + (uint64_t)L * 8 + (uint64_t)pick;
-            }
-            res = __shfl_sync(0xffffffffu, res, L);
+            float p[8], ex;
+            lane_probs<float>(amps + off[iq], c - cbase[iq], lane, 1ULL << nq[iq], p);
+            const int lq = chunk_lane<float>(p, tq, &ex);
             if (lane == q) {
-                if (ok) {
-                    for (int b = 0; b < nq[iq]; ++b) {
-                        const double v = (double)(splitmix_out(flip_seed, j * 64 + (uint64_t)b) >> 11) *
-                                         (1.0 / 9007199254740992.0);
-                        if (v < r_mes) res ^= 1ULL << b;
-                    }
-                } else {
-                    res = ~0ULL;      // instance with zero norm: no sample
-                }
-                out[j0 + q] = res;
+                L = lq;
+                excl = ex;
             }
+        }
+        if (j < m) {
+            uint64_t res = ~0ULL;      // instance with zero norm: no sample
+            if (ok) {
+                const uint64_t N = 1ULL << nq[inst];
+                const uint64_t first = (chunk - cbase[inst]) * kChunk + (uint64_t)(L < 0 ? 0 : L) * 8;
+                float p[8];
+                probs8<float>(amps + off[inst], first, N, p);
+                const int pick = pick8<float>(p, excl, tloc);
+                res = first + (uint64_t)(pick < 0 ? 0 : pick);
+                for (int b = 0; b < nq[inst]; ++b) {
+                    const double v = (double)(splitmix_out(flip_seed, j * 64 + (uint64_t)b) >> 11) *
+                                     (1.0 / 9007199254740992.0);
+                    if (v < r_mes) res ^= 1ULL << b;
+                }
+            }
+            out[j] = res;
         }
     }
 }
