@@ -11,6 +11,7 @@ on x86_64 and aarch64 hosts.
 """
 import concurrent.futures as cf
 import hashlib
+import importlib.util
 import os
 import shutil
 import subprocess
@@ -40,7 +41,7 @@ def _sources():
 
 
 def _headers():
-    hs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh", ".inc"))]
+    hs = [os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC)) if f.endswith((".h", ".cuh", ".inc", ".py"))]
     hs.append(os.path.join(ROOT, "include", "qs.h"))
     return hs
 
@@ -48,6 +49,15 @@ def _headers():
 def _flags(checked=False):
     common = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include")]
     return common + ["-gencode", GENCODE, "-lineinfo"] + (["-DQS_CHECKED"] if checked else [])
+
+
+def _generate(build_dir):
+    """Writes the generated op loop of the wide pass into the build directory."""
+    spec = importlib.util.spec_from_file_location("gen_op_loop", os.path.join(CSRC, "gen_op_loop.py"))
+    gen = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(gen)
+    with open(os.path.join(build_dir, "qs_op_loop.inc"), "w") as f:
+        f.write(gen.emit())
 
 
 def _digest(paths, extra):
@@ -82,6 +92,8 @@ def build(force=False, verbose=False, checked=False):
         with open(stamp) as f:
             if f.read().strip() == digest:
                 return lib
+    _generate(build_dir)
+    flags = flags + ["-I" + build_dir]
     with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
         results = list(ex.map(lambda s: _compile(nvcc, s, flags, verbose, build_dir), srcs))
     if verbose:

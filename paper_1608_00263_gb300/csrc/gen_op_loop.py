@@ -1,0 +1,392 @@
+"""Writes qs_op_loop.inc: the op loop of the wide fused pass (complex64, 64
+amplitudes, 6 register bits per thread) as inline PTX with one indexed branch
+per op.
+
+A thread's amplitudes are 32 units of two: the amplitudes that differ in
+register bit 0 (always tile bit 0, qubit 0).  A unit is two 64-bit registers,
+the two real parts and the two imaginary parts, so every gate on register
+bits 1..5 is packed FP32x2 arithmetic throughout -- with (re, im) in one
+register X^1/2 and T mix the halves and take twice the instructions.  Gates
+on register bit 0 work on the halves with scalar instructions.
+
+Every op is one byte code (the host lowers a plan to them, lower_wide in
+qs_host.cpp) and a 16-byte record: the selection outside the register set
+(8 bytes, tested as (idx & sel) == sel) and two FP32 parameters.
+
+    W_H  + j   H on register bit j (the 1/sqrt2 deferred to the pass end)
+    W_XH + j   X^1/2 on register bit j (deferred)
+    W_YH + j   Y^1/2 on register bit j (deferred)
+    W_T  + j   T phase on the amplitudes with bit j set
+    W_CZ + p   sign on the amplitudes with both bits of pair p set
+    W_CZO + j  sign on the amplitudes with bit j set where the selection holds
+               (an empty selection always holds: Z)
+  and, in the loop of passes with parameterised gates (FULL):
+    W_RY + j   R_Y on register bit j as three shears x += a y, y += b x,
+               x += a y with (a, b) = (-tan(phi/2), sin(phi)), phi = theta/2
+    W_RX + j   R_X on register bit j: the same shears between x and i y
+    W_PH + j   amplitudes with bit j set times a + i b where the selection holds
+    W_PP + p   amplitudes with both bits of pair p set times a + i b
+
+Every case ends with its own copy of the dispatch (threaded code): the next
+op's code, loaded while the case ran, picks the next case by one indexed
+branch, and the code after it is loaded in turn.
+
+The build writes the file into its object directory (build.py).
+"""
+RB = 6           # register bits
+NS = 1 << RB     # amplitudes per thread
+NU = NS // 2     # units: two amplitudes that differ in register bit 0
+NPAIR = RB * (RB - 1) // 2
+W_H, W_XH, W_YH, W_T = 0, RB, 2 * RB, 3 * RB
+W_CZ = 4 * RB
+W_CZO = W_CZ + NPAIR
+W_CT = W_CZO + RB            # codes of the Clifford+T loop
+W_RY = W_CT
+W_RX = W_RY + RB
+W_PH = W_RX + RB
+W_PP = W_PH + RB
+W_ALL = W_PP + NPAIR         # codes of the full loop
+
+F_C = "0f3F3504F3"       # 1/sqrt2 rounded to FP32
+F_2C = "0f3FB504F3"      # 2 * that (exact)
+F_NC = "0fBF3504F3"      # -(1/sqrt2)
+F_2 = "0f40000000"
+F_M1 = "0fBF800000"
+F_M2 = "0fC0000000"
+F_P1 = "0f3F800000"
+F_0 = "0f00000000"
+# operands: offset of the thread's unit 0 in the tile, shared address of the
+# tile, shared address of the staged pass, offset of the phase record in it,
+# begin and end op, index, factor (re, im), factor mode, then the offsets of
+# the codes and of the records (immediates)
+ADDR, TILE, BASE, PHASE, BEGIN, END, IDX, FR, FI, FMODE, O_CODES, O_RECS = ("%%%d" % k for k in range(12))
+
+
+def pair_index(j, k):
+    """Pairs (j, k), j < k < RB, numbered (0,1) (0,2) ... (1,2) (1,3) ..."""
+    return j * (RB - 1) - (j * (j - 1)) // 2 + (k - j - 1)
+
+
+def re(k):
+    return "u%d" % (2 * k)
+
+
+def im(k):
+    return "u%d" % (2 * k + 1)
+
+
+def units(j):
+    """Unit pairs (bit clear, bit set) of register bit j >= 1."""
+    b = 1 << (j - 1)
+    return [(k, k | b) for k in range(NU) if not k & b]
+
+
+def const(name, value):
+    return "mov.b64 %s, {%s, %s};" % (name, value, value)
+
+
+def unpack(k, both=True):
+    """The unit's components: element 0 (xr, xi), element 1 (yr, yi)."""
+    return ["mov.b64 {xr, yr}, %s;" % re(k), "mov.b64 {xi, yi}, %s;" % im(k)]
+
+
+def pack(k):
+    return ["mov.b64 %s, {xr, yr};" % re(k), "mov.b64 %s, {xi, yi};" % im(k)]
+
+
+def on_bit0(body):
+    out = []
+    for k in range(NU):
+        out += unpack(k) + body + pack(k)
+    return out
+
+
+def case_h(j):
+    if j == 0:
+        # x' = x + y; y' = x' - 2 y
+        return on_bit0(["add.rn.f32 xr, xr, yr;", "fma.rn.f32 yr, yr, %s, xr;" % F_M2,
+                        "add.rn.f32 xi, xi, yi;", "fma.rn.f32 yi, yi, %s, xi;" % F_M2])
+    out = [const("qS", F_M2)]
+    for x, y in units(j):
+        for c in (re, im):
+            out += ["add.rn.f32x2 %s, %s, %s;" % (c(x), c(x), c(y)),
+                    "fma.rn.f32x2 %s, %s, qS, %s;" % (c(y), c(y), c(x))]
+    return out
+
+
+def case_yh(j):
+    # x' = x - y; y' = x' + 2 y
+    if j == 0:
+        return on_bit0(["sub.rn.f32 xr, xr, yr;", "fma.rn.f32 yr, yr, %s, xr;" % F_2,
+                        "sub.rn.f32 xi, xi, yi;", "fma.rn.f32 yi, yi, %s, xi;" % F_2])
+    out = []
+    for x, y in units(j):
+        for c in (re, im):
+            out += ["fma.rn.f32x2 %s, %s, qM1, %s;" % (c(x), c(y), c(x)),
+                    "fma.rn.f32x2 %s, %s, qP2, %s;" % (c(y), c(y), c(x))]
+    return out
+
+
+def case_xh(j):
+    # x' = x - i y, y' = y - i x: y'.im = y.im - x.re, x'.re = y'.im + 2 x.re;
+    # x'.im = x.im - y.re, y'.re = x'.im + 2 y.re
+    if j == 0:
+        return on_bit0(["sub.rn.f32 yi, yi, xr;", "fma.rn.f32 xr, xr, %s, yi;" % F_2,
+                        "sub.rn.f32 xi, xi, yr;", "fma.rn.f32 yr, yr, %s, xi;" % F_2])
+    out = []
+    for x, y in units(j):
+        out += ["fma.rn.f32x2 %s, %s, qM1, %s;" % (im(y), re(x), im(y)),
+                "fma.rn.f32x2 %s, %s, qP2, %s;" % (re(x), re(x), im(y)),
+                "fma.rn.f32x2 %s, %s, qM1, %s;" % (im(x), re(y), im(x)),
+                "fma.rn.f32x2 %s, %s, qP2, %s;" % (re(y), re(y), im(x))]
+    return out
+
+
+def case_t(j):
+    # re' = c re - c im; im' = re' + 2 c im
+    if j == 0:
+        return on_bit0(["mul.rn.f32 yr, yr, %s;" % F_C, "fma.rn.f32 yr, yi, %s, yr;" % F_NC,
+                        "fma.rn.f32 yi, yi, %s, yr;" % F_2C])
+    out = [const("qS", F_C), const("qt", F_NC), const("qm", F_2C)]
+    for _, y in units(j):
+        out += ["mul.rn.f32x2 %s, %s, qS;" % (re(y), re(y)),
+                "fma.rn.f32x2 %s, %s, qt, %s;" % (re(y), im(y), re(y)),
+                "fma.rn.f32x2 %s, %s, qm, %s;" % (im(y), im(y), re(y))]
+    return out
+
+
+def element1(body, mask=0):
+    """`body` on element 1 (yr, yi) of the units whose bits include mask."""
+    out = []
+    for k in range(NU):
+        if (k & mask) == mask:
+            out += unpack(k) + body + pack(k)
+    return out
+
+
+def sign_units(mask, factor):
+    return ["mul.rn.f32x2 %s, %s, %s;" % (c(k), c(k), factor) for k in range(NU) if (k & mask) == mask
+            for c in (re, im)]
+
+
+def case_cz(j, k):
+    if j == 0:
+        return element1(["neg.f32 yr, yr;", "neg.f32 yi, yi;"], 1 << (k - 1))
+    return sign_units((1 << (j - 1)) | (1 << (k - 1)), "qM1")
+
+
+# The record of the op that runs is op qo - 1 (the dispatch has advanced qo).
+RECORD = ["mad.lo.u32 qa, qo, 16, %s;" % BASE]
+SELECTED = ["ld.shared.u64 qm, [qa+%s];" % O_RECS,
+            "and.b64 qt, %s, qm;" % IDX,
+            "setp.eq.u64 qp, qt, qm;"]
+PARAMS = ["add.u32 qa, qa, %s;" % O_RECS, "ld.shared.v2.f32 {pa, pb}, [qa+8];"]
+
+
+def case_czo(j):
+    out = RECORD + SELECTED + ["selp.f32 pa, %s, %s, qp;" % (F_M1, F_P1)]
+    if j == 0:
+        return out + element1(["mul.rn.f32 yr, yr, pa;", "mul.rn.f32 yi, yi, pa;"])
+    return out + ["mov.b64 qS, {pa, pa};"] + sign_units(1 << (j - 1), "qS")
+
+
+def case_ry(j):
+    # x += a y, y += b x, x += a y
+    if j == 0:
+        return RECORD + PARAMS + on_bit0([
+            "fma.rn.f32 xr, yr, pa, xr;", "fma.rn.f32 yr, xr, pb, yr;", "fma.rn.f32 xr, yr, pa, xr;",
+            "fma.rn.f32 xi, yi, pa, xi;", "fma.rn.f32 yi, xi, pb, yi;", "fma.rn.f32 xi, yi, pa, xi;"])
+    out = RECORD + PARAMS + ["mov.b64 qS, {pa, pa};", "mov.b64 qt, {pb, pb};"]
+    for x, y in units(j):
+        for c in (re, im):
+            out += ["fma.rn.f32x2 %s, %s, qS, %s;" % (c(x), c(y), c(x)),
+                    "fma.rn.f32x2 %s, %s, qt, %s;" % (c(y), c(x), c(y)),
+                    "fma.rn.f32x2 %s, %s, qS, %s;" % (c(x), c(y), c(x))]
+    return out
+
+
+def case_rx(j):
+    # with w = i y (w.re = -y.im, w.im = y.re): x += a w, w += b x, x += a w
+    out = RECORD + PARAMS + ["neg.f32 na, pa;", "neg.f32 nb, pb;"]
+    if j == 0:
+        return out + on_bit0([
+            "fma.rn.f32 xr, yi, na, xr;", "fma.rn.f32 xi, yr, pa, xi;",
+            "fma.rn.f32 yi, xr, nb, yi;", "fma.rn.f32 yr, xi, pb, yr;",
+            "fma.rn.f32 xr, yi, na, xr;", "fma.rn.f32 xi, yr, pa, xi;"])
+    out += ["mov.b64 qS, {pa, pa};", "mov.b64 qt, {na, na};", "mov.b64 qm, {pb, pb};", "mov.b64 qn, {nb, nb};"]
+    for x, y in units(j):
+        out += ["fma.rn.f32x2 %s, %s, qt, %s;" % (re(x), im(y), re(x)),
+                "fma.rn.f32x2 %s, %s, qS, %s;" % (im(x), re(y), im(x)),
+                "fma.rn.f32x2 %s, %s, qn, %s;" % (im(y), re(x), im(y)),
+                "fma.rn.f32x2 %s, %s, qm, %s;" % (re(y), im(x), re(y)),
+                "fma.rn.f32x2 %s, %s, qt, %s;" % (re(x), im(y), re(x)),
+                "fma.rn.f32x2 %s, %s, qS, %s;" % (im(x), re(y), im(x))]
+    return out
+
+
+def phase_units(mask):
+    # re' = re a - im b; im' = re b + im a
+    out = ["neg.f32 nb, pb;", "mov.b64 qS, {pa, pa};", "mov.b64 qt, {pb, pb};", "mov.b64 qm, {nb, nb};"]
+    for k in range(NU):
+        if (k & mask) == mask:
+            out += ["mul.rn.f32x2 qn, %s, qm;" % im(k),
+                    "mul.rn.f32x2 qu, %s, qt;" % re(k),
+                    "fma.rn.f32x2 %s, %s, qS, qn;" % (re(k), re(k)),
+                    "fma.rn.f32x2 %s, %s, qS, qu;" % (im(k), im(k))]
+    return out
+
+
+PHASE1 = ["neg.f32 nb, pb;"]
+PHASE1_BODY = ["mul.rn.f32 na, yi, nb;", "mul.rn.f32 xx, yr, pb;", "fma.rn.f32 yr, yr, pa, na;",
+               "fma.rn.f32 yi, yi, pa, xx;"]
+
+
+def case_ph(j):
+    out = RECORD + SELECTED + PARAMS + ["selp.f32 pa, pa, %s, qp;" % F_P1, "selp.f32 pb, pb, %s, qp;" % F_0]
+    return out + (PHASE1 + element1(PHASE1_BODY) if j == 0 else phase_units(1 << (j - 1)))
+
+
+def case_pp(j, k):
+    out = RECORD + PARAMS
+    return out + (PHASE1 + element1(PHASE1_BODY, 1 << (k - 1)) if j == 0
+                  else phase_units((1 << (j - 1)) | (1 << (k - 1))))
+
+
+def cases(full):
+    body = [None] * (W_ALL if full else W_CT)
+    for j in range(RB):
+        body[W_H + j] = case_h(j)
+        body[W_XH + j] = case_xh(j)
+        body[W_YH + j] = case_yh(j)
+        body[W_T + j] = case_t(j)
+        body[W_CZO + j] = case_czo(j)
+        if full:
+            body[W_RY + j] = case_ry(j)
+            body[W_RX + j] = case_rx(j)
+            body[W_PH + j] = case_ph(j)
+        for k in range(j + 1, RB):
+            body[W_CZ + pair_index(j, k)] = case_cz(j, k)
+            if full:
+                body[W_PP + pair_index(j, k)] = case_pp(j, k)
+    assert all(b is not None for b in body)
+    return body
+
+
+def dispatch(L, ncodes):
+    """Runs op qo (its code in qcn, loaded earlier): leaves when qo reaches
+    the end, loads op qo + 1's code (the staged codes run past the last op),
+    and branches to op qo's case; a code outside the table is clamped to the
+    extra entry, which only dispatches the next op (the lowering never makes
+    one)."""
+    return ["setp.ge.s32 qp, qo, %s;" % END,
+            "@qp bra.uni " + L("DONE") + ";",
+            "min.u32 qc, qcn, %d;" % ncodes,
+            "add.u32 qo, qo, 1;",
+            "add.u32 qa, %s, qo;" % BASE,
+            "ld.shared.u8 qcn, [qa+%s];" % O_CODES,
+            "brx.idx.uni qc, " + L("TBL") + ";"]
+
+
+def slots(store):
+    """All units from / to the tile, in Gray-code order (one XOR with a
+    register bit's offset per address), the two halves of the units as two
+    chains."""
+    out = ["ld.shared.v4.u32 {b0, b1, b2, b3}, [qh];", "ld.shared.v2.u32 {b4, b5}, [qh+16];",
+           "mov.u32 a0, %s;" % ADDR, "xor.b32 a1, %s, b%d;" % (ADDR, RB - 1)]
+    for i in range(NU // 2):
+        if i:
+            bit = (i & -i).bit_length()          # register bit 1 + trailing zeros
+            out += ["xor.b32 a0, a0, b%d;" % bit, "xor.b32 a1, a1, b%d;" % bit]
+        for a, k in (("a0", i ^ (i >> 1)), ("a1", (i ^ (i >> 1)) + NU // 2)):
+            # the XORs act on offsets in the tile (its address is not a
+            # multiple of its size)
+            out.append("add.u32 qa, %s, %s;" % (a, TILE))
+            out.append("st.shared.v2.b64 [qa], {%s, %s};" % (re(k), im(k)) if store
+                       else "ld.shared.v2.b64 {%s, %s}, [qa];" % (re(k), im(k)))
+    return out
+
+
+def factor(L):
+    """The thread's factor: mode 0 none, 1 real, 2 complex."""
+    out = ["setp.eq.u32 qp, %s, 0;" % FMODE,
+           "@qp bra.uni " + L("STORE") + ";",
+           "mov.b64 qS, {%s, %s};" % (FR, FR),
+           "setp.eq.u32 qp, %s, 1;" % FMODE,
+           "@qp bra.uni " + L("REAL") + ";",
+           "neg.f32 nb, %s;" % FI,
+           "mov.b64 qt, {%s, %s};" % (FI, FI),
+           "mov.b64 qm, {nb, nb};"]
+    for k in range(NU):
+        out += ["mul.rn.f32x2 qn, %s, qm;" % im(k),
+                "mul.rn.f32x2 qu, %s, qt;" % re(k),
+                "fma.rn.f32x2 %s, %s, qS, qn;" % (re(k), re(k)),
+                "fma.rn.f32x2 %s, %s, qS, qu;" % (im(k), im(k))]
+    out += ["bra.uni " + L("STORE") + ";", L("REAL") + ":"]
+    out += sign_units(0, "qS")
+    return out
+
+
+def asm_text(prefix, full):
+    """PTX of one phase: loads the thread's units, runs the ops [begin, end),
+    applies the factor, stores the units.  The units live in registers of the
+    block's own, so nothing has to be moved at its boundary."""
+    def L(name):
+        return "%s_%s" % (prefix, name)
+    body = cases(full)
+    n = len(body)
+    lines = ["{",
+             ".reg .pred qp;",
+             ".reg .u32 qo, qc, qcn, qa, qh, a0, a1, b<%d>;" % RB,
+             ".reg .b64 qm, qt, qS, qn, qu, qM1, qP2;",
+             ".reg .f32 xr, xi, yr, yi, xx, pa, pb, na, nb;",
+             ".reg .b64 u<%d>;" % NS,
+             "add.u32 qh, %s, %s;" % (BASE, PHASE)]
+    lines += slots(False)
+    lines += ["mov.b64 qM1, {%s, %s};" % (F_M1, F_M1),
+              "mov.b64 qP2, {%s, %s};" % (F_2, F_2),
+              "mov.u32 qo, %s;" % BEGIN,
+              "add.u32 qa, %s, qo;" % BASE,
+              "ld.shared.u8 qcn, [qa+%s];" % O_CODES,
+              L("TBL") + ": .branchtargets " + ", ".join([L("C%d" % c) for c in range(n)] + [L("NEXT")]) + ";",
+              L("NEXT") + ":"]
+    lines += dispatch(L, n)
+    for c, b in enumerate(body):
+        lines.append(L("C%d" % c) + ":")
+        lines += b
+        lines += dispatch(L, n)
+    lines.append(L("DONE") + ":")
+    lines += factor(L)
+    lines.append(L("STORE") + ":")
+    lines.append("add.u32 qh, %s, %s;" % (BASE, PHASE))
+    lines += slots(True)
+    lines.append("}")
+    return lines
+
+
+def emit():
+    out = ["// qs_op_loop.inc -- generated by gen_op_loop.py; do not edit.",
+           "//",
+           "// The op loop of the wide fused pass (complex64, %d slots, %d register" % (NS, RB),
+           "// bits) as inline PTX: one byte-code load and one indexed branch per op.",
+           "// OpLoop<false>: the Clifford+T gates; OpLoop<true>: also the",
+           "// parameterised gates.",
+           "",
+           "template <bool FULL> struct OpLoop;"]
+    for full, prefix in ((False, "QSWCT"), (True, "QSWFL")):
+        out.append("template <> struct OpLoop<%s> {" % ("true" if full else "false"))
+        out.append("    template <int O_CODES, int O_RECS>")
+        out.append("    static __device__ __forceinline__ void run(uint32_t addr, uint32_t tile, uint32_t base,")
+        out.append("                                               uint32_t phase, int ob, int ub,")
+        out.append("                                               unsigned long long idx, float fr, float fi,")
+        out.append("                                               uint32_t fmode)")
+        out.append("    {")
+        out.append("        asm volatile(")
+        for line in asm_text(prefix, full):
+            out.append('            "%s\\n"' % line)
+        out.append('            : : "r"(addr), "r"(tile), "r"(base), "r"(phase), "r"(ob), "r"(ub), "l"(idx), "f"(fr), "f"(fi), "r"(fmode),')
+        out.append('                "n"(O_CODES), "n"(O_RECS)')
+        out.append('            : "memory");')
+        out.append("    }")
+        out.append("};")
+    return "\n".join(out) + "\n"
+

@@ -235,7 +235,11 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
         const size_t b_phase = p.phases.size() * sizeof(DevPhase);
         const size_t b_ops = p.ops.size() * sizeof(DevOp);
         const size_t b_blk = p.tc_words.size() * sizeof(uint32_t);
-        const size_t total = b_pass + b_phase + b_ops + b_blk + 16;
+        // complex64 plans of six register bits go up lowered
+        WidePlan wide;
+        if (s->dt == QS_C64 && wide_plan(p.passes, p.phases)) lower_wide(p.passes, p.phases, p.ops, &wide);
+        const size_t w_pass = wide.passes.size() * sizeof(WidePass), w_ops = wide.ops.size() * sizeof(WideOp);
+        const size_t total = (w_pass ? w_pass + w_ops + wide.codes.size() : b_pass + b_phase + b_ops + b_blk) + 16;
         if (c->bytes < total) {
             if (c->dev) cudaFree(c->dev);
             if (c->staging) cudaFreeHost(c->staging);
@@ -255,16 +259,24 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
         }
         unsigned char *h = static_cast<unsigned char *>(c->staging);
         std::memset(h, 0, total);
-        std::memcpy(h, p.passes.data(), b_pass);
-        std::memcpy(h + b_pass, p.phases.data(), b_phase);
-        std::memcpy(h + b_pass + b_phase, p.ops.data(), b_ops);
-        if (b_blk) std::memcpy(h + b_pass + b_phase + b_ops, p.tc_words.data(), b_blk);
+        if (w_pass) {
+            std::memcpy(h, wide.passes.data(), w_pass);
+            std::memcpy(h + w_pass, wide.ops.data(), w_ops);
+            std::memcpy(h + w_pass + w_ops, wide.codes.data(), wide.codes.size());
+        } else {
+            std::memcpy(h, p.passes.data(), b_pass);
+            std::memcpy(h + b_pass, p.phases.data(), b_phase);
+            std::memcpy(h + b_pass + b_phase, p.ops.data(), b_ops);
+            if (b_blk) std::memcpy(h + b_pass + b_phase + b_ops, p.tc_words.data(), b_blk);
+        }
         QS_CUDA_TRY(cudaMemcpyAsync(c->dev, h, total, cudaMemcpyHostToDevice, s->stream));
         if (!c->done) QS_CUDA_TRY(cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming));
         QS_CUDA_TRY(cudaEventRecord(c->done, s->stream));
         c->key = key;
         c->ngates = ng;
         c->plan = std::move(p);
+        c->wide_ops = wide.ops.size();
+        c->wide = std::move(wide.passes);
         c->valid = true;
     }
     c->last_use = ++pc.clock;
@@ -438,7 +450,10 @@ static qs_status qs_apply_circuit_impl(qs_state *s, const qs_gate *gates, size_t
         if (uniform != 0.0) launch_init_uniform(s);
         return st;
     }
-    if (qs_status st = run_fused_plan(s, *plan, dev, uniform, fold.nfold > 0 ? &fold : nullptr)) return st;
+    const FoldArgs *folded = fold.nfold > 0 ? &fold : nullptr;
+    if (qs_status st = slot->wide.empty() ? run_fused_plan(s, *plan, dev, uniform, folded)
+                                          : run_wide_plan(s, slot->wide, slot->wide_ops, dev, uniform, folded))
+        return st;
     return slot_in_use(s, slot);
 }
 
@@ -810,7 +825,7 @@ qs_status check_poll_all()
 {
 #ifdef QS_CHECKED
     QS_CUDA_TRY(cudaDeviceSynchronize());
-    for (qs_status (*f)() : {check_poll_api, check_poll_plain, check_poll_fused, check_poll_stats,
+    for (qs_status (*f)() : {check_poll_api, check_poll_plain, check_poll_fused, check_poll_wide, check_poll_stats,
                              check_poll_batch, check_poll_adjoint})
         if (qs_status st = f()) return st;
 #endif

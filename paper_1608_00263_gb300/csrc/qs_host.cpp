@@ -881,6 +881,145 @@ static void pack_block(const std::vector<Cplx> &U, int precision, std::vector<ui
 
 }  // namespace
 
+bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases)
+{
+    if (passes.empty()) return false;
+    for (const DevPass &p : passes)
+        if (p.r != kWideRegBits || p.t < kWideMinTile || p.t > 13) return false;
+    for (const DevPhase &h : phases)
+        if (h.kind != 0 || h.R[0] != 0) return false;
+    return true;
+}
+
+// Lowers one phase's ops: gates on register bits to byte codes, the shears
+// of R_Y and R_X back to one op each, diagonal ops without a register bit to
+// the tail.
+static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<DevOp> &ops, WidePlan *out,
+                        std::vector<WideOp> *tail, std::vector<uint8_t> *tail_codes, bool *full)
+{
+    const size_t begin = out->codes.size();
+    auto selection = [&](uint64_t qmask, WideOp *w) {
+        for (int b = 0; b < P.t; ++b)
+            if ((qmask >> P.L[b]) & 1) w->sel_tile |= 1u << b;
+        for (int i = 0; i < P.n - P.t; ++i)
+            if ((qmask >> P.G[i]) & 1) w->sel_out |= 1u << i;
+    };
+    auto put = [&](int code, const WideOp &w) {
+        out->codes.push_back((uint8_t)code);
+        out->ops.push_back(w);
+    };
+    for (int o = H.op_begin; o < H.op_end; ++o) {
+        const DevOp &d = ops[o];
+        WideOp w{0, 0, 1.f, 0.f};
+        int bits = 0, lo = -1, hi = -1;
+        for (int b = 0; b < kWideRegBits; ++b)
+            if ((d.rmask >> b) & 1) {
+                if (lo < 0) lo = b;
+                hi = b;
+                ++bits;
+            }
+        switch (d.type) {
+        case OP_H: put(W_H + d.a, w); break;
+        case OP_XH: put(W_XH + d.a, w); break;
+        case OP_YH: put(W_YH + d.a, w); break;
+        case OP_SHX: {
+            // x += a y, y += b x, x += a y
+            const float a = (float)d.m[0], b = (float)ops[o + 1].m[0];
+            const bool pre = out->codes.size() > begin && out->codes.back() == W_PH + d.a &&
+                             out->ops.back().p0 == 0.f && out->ops.back().p1 == -1.f &&
+                             out->ops.back().sel_tile == 0 && out->ops.back().sel_out == 0;
+            const bool post = o + 3 < H.op_end && ops[o + 3].type == OP_PHASE && ops[o + 3].rmask == 1u << d.a &&
+                              ops[o + 3].qmask == 0 && ops[o + 3].m[0] == 0 && ops[o + 3].m[1] == 1;
+            *full = true;
+            if (pre && post) {
+                // S R_Y S^dagger: the shears between x and i y
+                out->codes.back() = (uint8_t)(W_RX + d.a);
+                out->ops.back().p0 = -a;
+                out->ops.back().p1 = -b;
+                o += 3;
+            } else {
+                w.p0 = a;
+                w.p1 = b;
+                put(W_RY + d.a, w);
+                o += 2;
+            }
+            break;
+        }
+        case OP_PHASE: case OP_NEG: {
+            const bool neg = d.type == OP_NEG;
+            const bool tphase = !neg && d.m[0] == d.m[1] && d.m[0] > 0.7071 && d.m[0] < 0.7072;
+            selection(d.qmask, &w);
+            if (bits == 0) {
+                if (!neg && !tphase) {
+                    w.p0 = (float)d.m[0];
+                    w.p1 = (float)d.m[1];
+                    *full = true;
+                }
+                tail->push_back(w);
+                tail_codes->push_back(neg ? 4 : tphase ? 1 : 0);
+            } else if (neg) {
+                put(bits == 2 ? W_CZ + wide_pair_index(lo, hi) : W_CZO + hi, w);
+            } else if (tphase && bits == 1 && d.qmask == 0) {
+                put(W_T + hi, w);
+            } else {
+                w.p0 = (float)d.m[0];
+                w.p1 = (float)d.m[1];
+                put(bits == 2 ? W_PP + wide_pair_index(lo, hi) : W_PH + hi, w);
+                *full = true;
+            }
+            break;
+        }
+        default: break;
+        }
+    }
+}
+
+void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
+                const std::vector<DevOp> &ops, WidePlan *out)
+{
+    *out = WidePlan();
+    for (const DevPass &P : passes) {
+        WidePass W;
+        std::memset(&W, 0, sizeof W);
+        // records and codes of a pass start at a multiple of 16; the code
+        // loads run one past the last op
+        out->ops.resize((out->ops.size() + 31) / 16 * 16);
+        out->codes.resize(out->ops.size(), 0);
+        W.op_begin = (uint32_t)out->ops.size();
+        W.t = P.t;
+        W.n = P.n;
+        W.nphases = P.nphases;
+        W.gs_re = (float)P.gscale_re;
+        W.gs_im = (float)P.gscale_im;
+        std::memcpy(W.L, P.L, sizeof W.L);
+        std::memcpy(W.G, P.G, sizeof W.G);
+        bool full = false;
+        for (int ph = 0; ph < P.nphases; ++ph) {
+            const DevPhase &H = phases[P.phase_begin + ph];
+            WidePhase &V = W.ph[ph];
+            for (int j = 0; j < kWideRegBits; ++j) V.pb[j] = tile_swizzle(1u << H.R[j], 2) * 8u;
+            std::memcpy(V.T, H.T, sizeof V.T);
+            V.op_begin = (int16_t)(out->ops.size() - W.op_begin);
+            std::vector<WideOp> tail;
+            std::vector<uint8_t> tail_codes;
+            lower_phase(P, H, ops, out, &tail, &tail_codes, &full);
+            V.tail_begin = (int16_t)(out->ops.size() - W.op_begin);
+            out->ops.insert(out->ops.end(), tail.begin(), tail.end());
+            out->codes.insert(out->codes.end(), tail_codes.begin(), tail_codes.end());
+            V.op_end = (int16_t)(out->ops.size() - W.op_begin);
+        }
+        W.nops = (int)(out->ops.size() - W.op_begin);
+        // between the passes of a plan units are kept as the kernel works on
+        // them; the first reads and the last writes canonical order
+        W.canon_in = &P == &passes.front();
+        W.canon_out = &P == &passes.back();
+        W.full = full;
+        out->passes.push_back(W);
+    }
+    out->ops.resize((out->ops.size() + 31) / 16 * 16);
+    out->codes.resize(out->ops.size(), 0);
+}
+
 // Persistent ensemble work list (declared with its order and dependency
 // rules in qs_internal.h).
 static uint64_t tiles_per_item(int t)
@@ -1002,6 +1141,14 @@ PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o)
         pp.look_steps = pp.look_top = 64;
     else if (n >= 28)
         pp.look_steps = pp.look_top = 8;
+    // complex64 register passes run the wide form (six register bits, one of
+    // them qubit 0) wherever a tile fills whole warps; measured against five
+    // register bits, evolve + read: 12 qubits 39.9 -> 37.2 us, 20 qubits 96.0
+    // -> 88.1 us, 23 qubits 400 -> 331 us, 30 qubits 66.6 -> 51.8 ms
+    if (dt == QS_C64 && pp.mode == QS_MODE_FUSED && pp.t >= kWideMinTile) {
+        pp.r = kWideRegBits;
+        pp.pack0 = 1;
+    }
     pp.r = std::min(pp.r, pp.t);
     return pp;
 }
@@ -1136,7 +1283,9 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
         int pass_ops = 0;
         int tc_in_pass = 0;
         while (prem && dp.nphases < kMaxPhasesPerPass && pass_ops < kMaxOpsPerPass) {
-            uint64_t reg = choose_local(g, pass_gates, pdone, n, 0, local, dp.r);
+            // (with pack0 qubit 0 is always a register qubit)
+            uint64_t reg = pp.pack0 ? choose_local(g, pass_gates, pdone, n, 1, local, dp.r - 1)
+                                    : choose_local(g, pass_gates, pdone, n, 0, local, dp.r);
             collect(g, pass_gates, pdone, reg, &phase_gates, &cnt);
             if (cnt == 0) return set_error(QS_ERR_INVALID_ARG, "planner made no phase progress");
             if (pp.tc_ok && tc_in_pass < kMaxTcPerPass && dp.t == 13) {

@@ -192,6 +192,7 @@ struct PlanParams {
     int precision = QS_PREC_FP16X3;   // TC operand precision (qs_precision, not DEFAULT)
     int look_steps = 2;   // tile choice: additions scored by greedy completion
     int look_top = 6;     // ... among this many best-scoring candidates
+    int pack0 = 0;        // qubit 0 in every register set (the wide pass)
     int hoist_diagonals = 1;   // move late diagonal ops to the last phase's uniform tail
 };
 
@@ -210,6 +211,69 @@ QS_HD inline uint32_t tile_swizzle(uint32_t e, uint32_t CE)
     const uint32_t f = ((u >> 3) ^ (u >> 6) ^ (u >> 9) ^ (u >> 12)) & 7u;
     return e ^ (f * CE);
 }
+
+// ---------------------------------------------------------------------------
+// Wide fused pass (complex64, 6 register bits): a plan lowered to byte codes
+// and 16-byte records, so the kernel's staging is a copy.
+// ---------------------------------------------------------------------------
+constexpr int kWideRegBits = 6;
+constexpr int kWideMinTile = 11;        // tiles of whole warps (2^(t - 6) threads)
+
+struct WideOp {             // 16 bytes
+    uint32_t sel_tile;      // selection outside the register set: tile bits ...
+    uint32_t sel_out;       // ... and bits of the tile number (out-of-tile qubits)
+    float p0, p1;           // parameters of the op (see gen_op_loop.py)
+};
+
+struct alignas(16) WidePhase {
+    uint32_t pb[kWideRegBits];   // swizzled tile byte offset of each register bit
+    uint8_t T[8];                // tile bit of thread-index bit k
+    int16_t op_begin;            // ops of the phase, from the pass's first
+    int16_t tail_begin;          // first op of the thread-uniform diagonal tail
+    int16_t op_end;
+    int16_t pad;
+};
+
+// Between the passes of one plan a 16-byte unit of the state (the amplitudes
+// 2u, 2u + 1) is stored as the kernel works on it: the two real parts, then
+// the two imaginary parts.
+struct WidePass {
+    int32_t t, n, nphases, nops;
+    uint32_t op_begin;           // first record and code (a multiple of 16)
+    int32_t full;                // some op needs the loop with parameterised gates
+    float gs_re, gs_im;          // pass-wide factor, applied in the last phase
+    int32_t canon_in, canon_out; // the pass reads / writes canonical units
+                                 // (re, im, re, im), else (re, re, im, im)
+    int32_t pad[2];
+    uint8_t L[kMaxTileBits];     // qubit of each tile bit (ascending)
+    uint8_t G[32];               // qubits outside the tile (ascending)
+    WidePhase ph[kMaxPhasesPerPass];
+};
+
+// Byte codes (gen_op_loop.py); codes of the tail: eighths of a turn the op
+// adds (T: 1, sign flip: 4, general phase: 0, its factor in p0 + i p1).
+constexpr int wide_pair_index(int j, int k)
+{
+    return j * (kWideRegBits - 1) - (j * (j - 1)) / 2 + (k - j - 1);
+}
+enum : uint8_t {
+    W_H = 0, W_XH = kWideRegBits, W_YH = 2 * kWideRegBits, W_T = 3 * kWideRegBits, W_CZ = 4 * kWideRegBits,
+    W_CZO = W_CZ + kWideRegBits * (kWideRegBits - 1) / 2,
+    W_CT = W_CZO + kWideRegBits,                 // codes of the Clifford+T loop
+    W_RY = W_CT, W_RX = W_RY + kWideRegBits, W_PH = W_RX + kWideRegBits, W_PP = W_PH + kWideRegBits
+};
+
+struct WidePlan {
+    std::vector<WidePass> passes;
+    std::vector<WideOp> ops;
+    std::vector<uint8_t> codes;
+};
+// Whether a plan's passes can run the wide form: six register bits, register
+// phases only, tiles of at least 2^kWideMinTile.
+bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases);
+// Lowers a pass list (phase and op indices into the given arrays).
+void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
+                const std::vector<DevOp> &ops, WidePlan *out);
 
 qs_status build_plan(const PlanParams &pp, const qs_gate *g, size_t ng, Plan *out);
 uint16_t f64_to_f16_bits(double x);
@@ -298,6 +362,8 @@ struct DevicePlanSlot {
     cudaEvent_t done = nullptr;   // after the slot's last upload or apply
     uint64_t last_use = 0;
     Plan plan;
+    std::vector<WidePass> wide;   // not empty: the plan runs the wide form
+    size_t wide_ops = 0;          // records (and codes) uploaded
 };
 
 struct DevicePlanCache {
@@ -372,6 +438,9 @@ qs_status launch_plain_gate(qs_state *s, const qs_gate &g);
 // (nfold > 0) those tiles also carry the folded diagonal prefix's phases.
 qs_status run_fused_plan(qs_state *s, const Plan &plan, const void *dev_plan, double uniform = 0.0,
                          const FoldArgs *fold = nullptr);
+// The same for a lowered plan; dev holds passes | records | codes.
+qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t nops, const void *dev,
+                        double uniform, const FoldArgs *fold);
 qs_status run_tc_plan(qs_state *s, const Plan &plan, const void *dev_plan,
                       int precision);
 qs_status launch_probabilities(const qs_state *s, void *out, int fp64,
@@ -394,6 +463,7 @@ size_t dtype_bytes(qs_dtype dt);
 qs_status check_poll_all();
 qs_status check_poll_plain();
 qs_status check_poll_fused();
+qs_status check_poll_wide();
 qs_status check_poll_stats();
 qs_status check_poll_api();
 qs_status check_poll_batch();

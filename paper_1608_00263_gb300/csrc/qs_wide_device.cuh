@@ -1,0 +1,290 @@
+// qs_wide_device.cuh -- body of the wide fused pass (complex64).
+//
+// The same tile pass as in qs_fused.cu -- a tile of 2^t amplitudes in shared
+// memory, register phases, one byte code per op -- with 64 amplitudes (6
+// register bits) per thread instead of 32, held as packed pairs of real and
+// of imaginary parts (gen_op_loop.py).  The pass is bound by instruction
+// issue and by the latency of its op dispatch, not by HBM, so what counts is
+// the work per issued instruction: every gate outside register bit 0 is
+// packed FP32x2 arithmetic (X^1/2 and T half the instructions of the
+// (re, im) layout), and twice the amplitudes per thread halve dispatch,
+// addressing and tables.  Register bit 0 is tile bit 0 in every phase, so all
+// slot accesses are 16 bytes.  128 threads hold a 13-qubit tile at 168
+// registers and 75 KB of shared memory, so three CTAs share an SM: while one
+// waits for its tile, two compute.
+#pragma once
+
+#include <cstddef>
+
+#include "qs_tile_device.cuh"
+
+namespace qs {
+
+#include "qs_op_loop.inc"
+
+constexpr int kWideThreads = 1 << (13 - kWideRegBits);   // threads of a 13-qubit tile
+constexpr int kWideSlots = 1 << kWideRegBits;
+constexpr int kWideUnits = kWideSlots / 2;               // 16-byte units per thread
+
+struct WideUnit {           // unit `it` of every thread
+    uint64_t goff;          // byte offset in the state
+    uint32_t soff;          // swizzled byte offset in the tile
+    uint32_t pad;
+};
+
+struct WideSmem {
+    WidePass P;
+    WideOp ops[kMaxOpsPerPass];
+    uint32_t codes[kMaxOpsPerPass / 4 + 4];
+    uint64_t toff[kWideThreads];                     // byte offset of the thread's unit 0 in the state
+    uint64_t gmask;                                  // out-of-tile qubits
+    uint16_t thr[kMaxPhasesPerPass][kWideThreads];   // tile element of the thread's slot 0
+    WideUnit unit[kWideUnits];
+    float2 w8[8];                                    // e^{i pi k / 4}
+};
+
+// Tables of the folded diagonal prefix (first pass of a circuit, see
+// FoldArgs): CZ partners as a qubit mask and as a mask of tile bits, T
+// counts, the unit table, and 2^(-n/2) e^{i pi k / 4}.
+struct WideFoldSmem {
+    uint64_t nb[kMaxQubits];
+    uint64_t m[3];
+    uint16_t g[kMaxQubits];
+    uint8_t u[kWideSlots];
+    float2 w[8];
+};
+
+// A unit between canonical order (re, im, re, im) and (re, re, im, im).
+__device__ __forceinline__ float4 swap_unit(float4 v) { return make_float4(v.x, v.z, v.y, v.w); }
+
+// Barrier of a tile's threads: the CTA, or its group of whole warps.
+template <bool GROUPED>
+__device__ __forceinline__ void wide_sync(int nthr, int gi)
+{
+    if constexpr (!GROUPED) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(gi + 1), "r"(nthr) : "memory");
+}
+
+// Runs tiles [t_begin, t_end) of one pass on `amps`.  blockDim.x threads; a
+// tile takes 2^(t - 6) of them: all (GROUPED = false), or a group of whole
+// warps (t >= 11) with its own tile buffer, group g running tiles t_begin +
+// g, + groups, ...  FOLD: the circuit's first pass, which writes its tiles
+// (the uniform state times the folded prefix's phases) instead of loading
+// them; F's nb and m are set by the caller (published by the first barrier).
+// The caller's CTA is converged; ends with a CTA barrier.
+template <bool FULL, bool FOLD, bool GROUPED>
+__device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g,
+                                               const WideOp *__restrict__ ops_g, const uint8_t *__restrict__ codes_g,
+                                               uint32_t t_begin, uint32_t t_end, WideSmem &S, WideFoldSmem *F,
+                                               unsigned char *smem_raw)
+{
+    constexpr int RB = kWideRegBits, NS = kWideSlots, NU = kWideUnits;
+    for (int i = threadIdx.x; i < (int)(sizeof(WidePass) / 4); i += blockDim.x)
+        reinterpret_cast<uint32_t *>(&S.P)[i] = reinterpret_cast<const uint32_t *>(pass_g)[i];
+    __syncthreads();
+    const int t = S.P.t, ng = S.P.n - t, nph = S.P.nphases, nops = S.P.nops;
+    const int nthr = GROUPED ? 1 << (t - RB) : (int)blockDim.x;
+    const int tid = GROUPED ? (int)(threadIdx.x & (unsigned)(nthr - 1)) : (int)threadIdx.x;
+    const int gi = GROUPED ? (int)(threadIdx.x >> (t - RB)) : 0;
+    const int ngr = GROUPED ? (int)(blockDim.x >> (t - RB)) : 1;
+    // ---- stage the ops and the per-thread tables (once per CTA and pass) ----
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(ops_g + S.P.op_begin);
+        for (int i = threadIdx.x; i < nops; i += blockDim.x) reinterpret_cast<uint4 *>(S.ops)[i] = src[i];
+        const uint32_t *cw = reinterpret_cast<const uint32_t *>(codes_g + S.P.op_begin);
+        for (int i = threadIdx.x; i < (nops + 7) / 4; i += blockDim.x) S.codes[i] = cw[i];
+    }
+    if (gi == 0)
+        for (int ph = 0; ph < nph; ++ph) {
+            uint32_t e = 0;
+            for (int k = 0; k < t - RB; ++k) e |= (((uint32_t)tid >> k) & 1u) << S.P.ph[ph].T[k];
+            S.thr[ph][tid] = (uint16_t)e;
+        }
+    for (int i = threadIdx.x; i < NU; i += blockDim.x) {
+        const uint32_t e = 2u * (uint32_t)nthr * (uint32_t)i;
+        S.unit[i].goff = deposit(e, S.P.L, t) * 8u;
+        S.unit[i].soff = swz<2>(e) * 8u;
+    }
+    if (threadIdx.x < 8) {
+        const float c = 0.70710678118654752440f;
+        const int k = (int)threadIdx.x;
+        const float re = (k & 3) == 2 ? 0.f : (k & 3) == 0 ? 1.f : ((k & 3) == 1 ? c : -c);
+        const float im = (k & 3) == 0 ? 0.f : (k & 3) == 2 ? 1.f : c;
+        S.w8[k] = k < 4 ? make_float2(re, im) : make_float2(-re, -im);
+    }
+    auto fcount = [&](int q) -> uint32_t {
+        return (uint32_t)((F->m[0] >> q) & 1) + 2u * (uint32_t)((F->m[1] >> q) & 1) + 4u * (uint32_t)((F->m[2] >> q) & 1);
+    };
+    if constexpr (FOLD) {
+        // each qubit's CZ partners as tile bits
+        for (int q = threadIdx.x; q < S.P.n; q += blockDim.x) {
+            uint32_t m = 0;
+            for (int b = 0; b < t; ++b) m |= (uint32_t)((F->nb[q] >> S.P.L[b]) & 1) << b;
+            F->g[q] = (uint16_t)m;
+        }
+        // unit u = (it, q) of every thread: tile element 2 nthr it + q;
+        // 4 (CZ pairs among its tile bits) + (its T counts), mod 8
+        for (int u = threadIdx.x; u < NS; u += blockDim.x) {
+            const uint32_t eu = 2u * (uint32_t)nthr * (uint32_t)(u / 2) + (uint32_t)(u & 1);
+            uint32_t pairs = 0, tcnt = 0;
+            for (uint32_t w = eu; w; w &= w - 1) {
+                const int qb = S.P.L[__ffs(w) - 1];
+                for (uint32_t v = w & (w - 1); v; v &= v - 1) pairs += (uint32_t)(F->nb[qb] >> S.P.L[__ffs(v) - 1]) & 1u;
+                tcnt += fcount(qb);
+            }
+            F->u[u] = (uint8_t)((4u * (pairs & 1u) + tcnt) & 7u);
+        }
+        // 2^(-n/2) e^{i pi k / 4}, formed in FP64 from n
+        if (threadIdx.x < 8) {
+            const int k = (int)threadIdx.x;
+            const double a = std::exp2(-0.5 * S.P.n), c = a * 0.70710678118654752440;
+            const double re = (k & 3) == 2 ? 0.0 : (k & 3) == 0 ? a : ((k & 3) == 1 ? c : -c);
+            const double im = (k & 3) == 0 ? 0.0 : (k & 3) == 2 ? a : c;
+            F->w[k] = k < 4 ? make_float2((float)re, (float)im) : make_float2((float)-re, (float)-im);
+        }
+    }
+    if (gi == 0) S.toff[tid] = deposit(2u * (uint32_t)tid, S.P.L, t) * 8u;
+    if (threadIdx.x == 0) {
+        uint64_t m = 0;
+        for (int i = 0; i < ng; ++i) m |= 1ULL << S.P.G[i];
+        S.gmask = m;
+    }
+    __syncthreads();
+    unsigned char *gsm = GROUPED ? smem_raw + (((size_t)gi << t) * sizeof(float2)) : smem_raw;
+    const uint32_t tile_sa = smem_addr(gsm);
+    const uint32_t sw_tid = swz<2>(2u * (uint32_t)tid) * 8u;
+    uint32_t tau = t_begin + (uint32_t)gi;
+    uint64_t base = deposit(tau, S.P.G, ng);
+    // the tile's highest element index must lie inside the state
+    auto inside = [&](uint64_t b) {
+        uint64_t lmask = 0;
+#ifdef QS_CHECKED
+        for (int i = 0; i < t; ++i) lmask |= 1ULL << S.P.L[i];
+#endif
+        (void)lmask;
+        (void)b;
+        return QS_DCHECK(((b | lmask) >> S.P.n) == 0, 202);
+    };
+    if constexpr (!FOLD) {
+        if (tau < t_end && inside(base)) {
+            const char *src = reinterpret_cast<const char *>(amps) + (base * 8u + S.toff[tid]);
+#pragma unroll 4
+            for (int it = 0; it < NU; ++it)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tile_sa + (sw_tid ^ S.unit[it].soff)),
+                             "l"(src + S.unit[it].goff)
+                             : "memory");
+        }
+    }
+    while (tau < t_end && inside(base)) {
+        if constexpr (FOLD) {
+            // element x gets 2^(-n/2) e^{i pi k(x) / 4}, k = 4 (CZ pairs within
+            // x) + (T counts of x), mod 8, summed over the out-of-tile bits,
+            // the thread's tile bits and the unit's, plus the pairs across
+            uint32_t pb = 0, nbm = 0;
+            for (uint64_t w = base; w; w &= w - 1) {
+                const int i = __ffsll((long long)w) - 1;
+                pb ^= (uint32_t)__popcll(base & F->nb[i] & (~0ULL << i << 1));
+                nbm ^= F->g[i];
+            }
+            const uint32_t lb = (uint32_t)(__popcll(base & F->m[0]) + 2 * __popcll(base & F->m[1]) +
+                                           4 * __popcll(base & F->m[2]));
+            const uint32_t et = 2u * (uint32_t)tid;
+            uint32_t pt = 0, nt = 0, lt = 0;
+            for (uint32_t w = et; w; w &= w - 1) {
+                const int b = __ffs(w) - 1;
+                const int q = S.P.L[b];
+                pt ^= (uint32_t)__popc(et & (uint32_t)F->g[q] & (~0u << b << 1));
+                nt ^= F->g[q];
+                lt += fcount(q);
+            }
+            const uint32_t k0 = 4u * ((pb ^ pt ^ (uint32_t)__popc(et & nbm)) & 1u) + lb + lt;
+            const uint32_t nu = nbm ^ nt;
+#pragma unroll 4
+            for (int it = 0; it < NU; ++it) {
+                float2 fill[2];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const uint32_t eu = 2u * (uint32_t)nthr * (uint32_t)it + (uint32_t)q;
+                    fill[q] = F->w[(k0 + F->u[it * 2 + q] + 4u * ((uint32_t)__popc(eu & nu) & 1u)) & 7u];
+                }
+                *reinterpret_cast<float4 *>(gsm + (sw_tid ^ S.unit[it].soff)) =
+                    make_float4(fill[0].x, fill[1].x, fill[0].y, fill[1].y);
+            }
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        if (!FOLD && S.P.canon_in) {
+            // the units this thread copied, to the order the phases work on
+#pragma unroll 4
+            for (int it = 0; it < NU; ++it) {
+                float4 *u = reinterpret_cast<float4 *>(gsm + (sw_tid ^ S.unit[it].soff));
+                *u = swap_unit(*u);
+            }
+        }
+        wide_sync<GROUPED>(nthr, gi);
+        for (int ph = 0; ph < nph; ++ph) {
+            const WidePhase &H = S.P.ph[ph];
+            const uint32_t te = S.thr[ph][tid], to = tau;
+            const int ub = H.tail_begin, oe = H.op_end;
+            // diagonal ops selected outside the register set scale the
+            // thread's slots by one factor: T and sign flips count eighths
+            // of a turn (their codes), general phases multiply; the last
+            // phase adds the pass-wide factor
+            const bool last = ph == nph - 1;
+            float fr = 1.f, fi = 0.f;
+            uint32_t mode = 0;
+            if (ub < oe || last) {
+                uint32_t k = 0;
+                for (int o = ub; o < oe; ++o) {
+                    const WideOp op = S.ops[o];
+                    if ((te & op.sel_tile) == op.sel_tile && (to & op.sel_out) == op.sel_out) {
+                        k += reinterpret_cast<const uint8_t *>(S.codes)[o];
+                        if constexpr (FULL) {
+                            const float x = fr * op.p0 - fi * op.p1;
+                            fi = fr * op.p1 + fi * op.p0;
+                            fr = x;
+                        }
+                    }
+                }
+                const float2 w = S.w8[k & 7u];
+                float x = fr * w.x - fi * w.y;
+                fi = fr * w.y + fi * w.x;
+                fr = x;
+                if (last) {
+                    const float gr = S.P.gs_re, gim = S.P.gs_im;
+                    x = fr * gr - fi * gim;
+                    fi = fr * gim + fi * gr;
+                    fr = x;
+                }
+                mode = __any_sync(0xffffffffu, fi != 0.f) ? 2u : 1u;
+            }
+            OpLoop<FULL>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16>(
+                swz<2>(te) * 8u, tile_sa, smem_addr(&S),
+                (uint32_t)(offsetof(WideSmem, P) + offsetof(WidePass, ph)) + (uint32_t)ph * (uint32_t)sizeof(WidePhase),
+                H.op_begin, ub, ((uint64_t)to << 32) | te, fr, fi, mode);
+            wide_sync<GROUPED>(nthr, gi);
+        }
+        // ---- store the tile; each unit's place takes the same unit of the
+        // next tile as soon as this thread has read it (no other thread
+        // touches it before the next barrier) ----
+        const uint64_t toff = S.toff[tid];
+        const bool canon_out = S.P.canon_out != 0;
+        char *dst = reinterpret_cast<char *>(amps) + (base * 8u + toff);
+        tau += (uint32_t)ngr;
+        base = GROUPED && ngr > 1 ? deposit(tau, S.P.G, ng) : (((base | ~S.gmask) + 1) & S.gmask);
+        const bool more = !FOLD && tau < t_end && inside(base);
+        const char *src = reinterpret_cast<const char *>(amps) + (base * 8u + toff);
+#pragma unroll 4
+        for (int it = 0; it < NU; ++it) {
+            const WideUnit u = S.unit[it];
+            const uint32_t so = sw_tid ^ u.soff;
+            const float4 v = *reinterpret_cast<const float4 *>(gsm + so);
+            *reinterpret_cast<float4 *>(dst + u.goff) = canon_out ? swap_unit(v) : v;
+            if (more)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tile_sa + so), "l"(src + u.goff)
+                             : "memory");
+        }
+    }
+    __syncthreads();
+}
+
+}  // namespace qs

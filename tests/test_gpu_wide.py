@@ -1,0 +1,77 @@
+"""The wide fused pass (complex64, tiles of 11 to 13 qubits) against the FP64
+oracle where it can go wrong: one tile and two, every tile size, the first
+pass reading a given state instead of generating it, one pass reading and
+writing canonical order, state memory the caller holds, and gate lists with
+every kind of gate.  Tolerance: the state bound of complex64, 1e-5 relative
+L2 (the deviation of an FP32 evolution of a few hundred gates is below 3e-6)."""
+import numpy as np
+import pytest
+
+import oracle as O
+import paper_1608_00263_gb300 as qs
+from paper_1608_00263_gb300 import build as qs_build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    qs_build.build()
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+
+
+def gate_list(rng, n, count, kinds):
+    g = np.zeros(count, dtype=qs.GATE_DTYPE)
+    g["kind"] = rng.choice(kinds, size=count)
+    for x in g:
+        a, b = rng.choice(n, size=2, replace=False)
+        x["q0"], x["q1"] = a, b
+    g["theta"] = rng.uniform(-7, 7, size=count)
+    return g
+
+
+CT = [qs.QS_H, qs.QS_X_HALF, qs.QS_Y_HALF, qs.QS_T, qs.QS_CZ]
+ALL = CT + [qs.QS_RX, qs.QS_RY, qs.QS_RZ, qs.QS_CPHASE]
+
+
+@pytest.mark.parametrize("kinds", [CT, ALL], ids=["clifford_t", "all"])
+@pytest.mark.parametrize("n,tile", [(11, 0), (12, 0), (13, 0), (14, 0), (14, 11), (15, 12), (17, 13), (18, 0)])
+def test_state(n, tile, kinds):
+    rng = np.random.default_rng(100 * n + tile + len(kinds))
+    start = rng.normal(size=1 << n) + 1j * rng.normal(size=1 << n)
+    start = (start / np.linalg.norm(start)).astype(np.complex64)
+    h = qs.qs_state_create(n, qs.QS_C64)
+    try:
+        for count in (1, 7, 300):
+            g = gate_list(rng, n, count, kinds)
+            qs.qs_state_copy_in(h, start)
+            qs.qs_apply_circuit(h, g, tile_log2=tile)
+            ref = start.astype(np.complex128)
+            O.apply_circuit(ref, g)
+            got = qs.qs_state_copy_out(h, n)
+            assert np.linalg.norm(got - ref) < 1e-5 * np.linalg.norm(ref), count
+    finally:
+        qs.qs_state_destroy(h)
+
+
+@pytest.mark.parametrize("n", [11, 16, 20])
+def test_generated_and_held_states_agree(n):
+    """A circuit on |0...0>: generated first pass (created state), and the
+    same list on memory the caller holds (every pass loads)."""
+    import torch
+    rows, cols = (1, n) if n < 12 else (4, -(-n // 4))
+    g = O.generate_circuit(rows, cols, 17, 3)
+    ref = O.simulate(n, g)
+    buf = torch.zeros(1 << n, dtype=torch.complex64, device="cuda")
+    buf[0] = 1
+    held = qs.qs_state_attach(n, qs.QS_C64, buf)
+    made = qs.qs_state_create(n, qs.QS_C64)
+    try:
+        for h in (held, made):
+            qs.qs_apply_circuit(h, g)
+            got = qs.qs_state_copy_out(h, n)
+            assert np.linalg.norm(got - ref) < 1e-5
+    finally:
+        qs.qs_state_destroy(held)
+        qs.qs_state_destroy(made)
