@@ -132,6 +132,8 @@ static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const u
                 o.mode = QS_MODE_FUSED;
                 o.tile_log2 = tbits[i];
                 PlanParams pp = default_plan_params(b->n[i], QS_C64, &o);
+                pp.r = std::min(5, pp.t);      // the batched passes hold five register bits
+                pp.pack0 = 0;
                 st[k] = build_plan(pp, gates + offsets[i] + hl[i], ng, &(*plans)[i]);
                 if (st[k]) msg[k] = last_error_cstr();
             }
