@@ -27,9 +27,9 @@ qs_host.cpp) and a 16-byte record: the selection outside the register set
     W_PH + j   amplitudes with bit j set times a + i b where the selection holds
     W_PP + p   amplitudes with both bits of pair p set times a + i b
 
-Every case ends with its own copy of the dispatch (threaded code): the next
-op's code, loaded while the case ran, picks the next case by one indexed
-branch, and the code after it is loaded in turn.
+Every case ends with its own indexed branch to the next op's case (threaded
+code); the code is known when the case starts, and the end of a phase is a
+code like any other.
 
 The build writes the file into its object directory (build.py).
 """
@@ -57,9 +57,14 @@ F_P1 = "0f3F800000"
 F_0 = "0f00000000"
 # operands: offset of the thread's unit 0 in the tile, shared address of the
 # tile, shared address of the staged pass, offset of the phase record in it,
-# begin and end op, index, factor (re, im), factor mode, then the offsets of
-# the codes and of the records (immediates)
-ADDR, TILE, BASE, PHASE, BEGIN, END, IDX, FR, FI, FMODE, O_CODES, O_RECS = ("%%%d" % k for k in range(12))
+# first op, index, factor (re, im), flags (bits 0..1 the factor's
+# mode, then the F_ bits below), swizzled offset of the thread's copies,
+# source of the next tile's copies, barrier and its threads, then immediate
+# offsets in the staged pass: codes, records (less one), unit table, state
+# offsets of the last phase's register bits, threads' state addresses
+(ADDR, TILE, BASE, PHASE, BEGIN, IDX, FR, FI, FLAGS, SWT, NSRC, BARID, NTHR,
+ O_CODES, O_RECS, O_UNIT, O_DREG, O_DST) = ("%%%d" % k for k in range(18))
+F_DIRECT, F_MORE, F_CANON = 4, 8, 16    # store to the state; copy the next tile in; canonical order
 
 
 def pair_index(j, k):
@@ -85,7 +90,10 @@ def const(name, value):
     return "mov.b64 %s, {%s, %s};" % (name, value, value)
 
 
-def unpack(k, both=True):
+TEMPS = 4      # units whose scalar instructions are interleaved
+
+
+def unpack(k):
     """The unit's components: element 0 (xr, xi), element 1 (yr, yi)."""
     return ["mov.b64 {xr, yr}, %s;" % re(k), "mov.b64 {xi, yi}, %s;" % im(k)]
 
@@ -94,11 +102,24 @@ def pack(k):
     return ["mov.b64 %s, {xr, yr};" % re(k), "mov.b64 %s, {xi, yi};" % im(k)]
 
 
-def on_bit0(body):
+def scalar_units(ks, body):
+    """`body` on the halves of the units ks, TEMPS units step by step (their
+    scalar registers are numbered apart)."""
     out = []
-    for k in range(NU):
-        out += unpack(k) + body + pack(k)
+    for g in range(0, len(ks), TEMPS):
+        chains = []
+        for n, k in enumerate(ks[g:g + TEMPS]):
+            c = unpack(k) + body + pack(k)
+            for t in ("xr", "xi", "yr", "yi", "na", "xx"):
+                c = [x.replace(t, t + str(n)) for x in c]
+            chains.append(c)
+        for step in range(len(chains[0])):
+            out += [c[step] for c in chains]
     return out
+
+
+def on_bit0(body):
+    return scalar_units(list(range(NU)), body)
 
 
 def case_h(j):
@@ -106,12 +127,9 @@ def case_h(j):
         # x' = x + y; y' = x' - 2 y
         return on_bit0(["add.rn.f32 xr, xr, yr;", "fma.rn.f32 yr, yr, %s, xr;" % F_M2,
                         "add.rn.f32 xi, xi, yi;", "fma.rn.f32 yi, yi, %s, xi;" % F_M2])
-    out = [const("qS", F_M2)]
-    for x, y in units(j):
-        for c in (re, im):
-            out += ["add.rn.f32x2 %s, %s, %s;" % (c(x), c(x), c(y)),
-                    "fma.rn.f32x2 %s, %s, qS, %s;" % (c(y), c(y), c(x))]
-    return out
+    return [const("qS", F_M2)] + interleave([["add.rn.f32x2 %s, %s, %s;" % (c(x), c(x), c(y)),
+                                              "fma.rn.f32x2 %s, %s, qS, %s;" % (c(y), c(y), c(x))]
+                                             for x, y in units(j) for c in (re, im)])
 
 
 def case_yh(j):
@@ -119,12 +137,9 @@ def case_yh(j):
     if j == 0:
         return on_bit0(["sub.rn.f32 xr, xr, yr;", "fma.rn.f32 yr, yr, %s, xr;" % F_2,
                         "sub.rn.f32 xi, xi, yi;", "fma.rn.f32 yi, yi, %s, xi;" % F_2])
-    out = []
-    for x, y in units(j):
-        for c in (re, im):
-            out += ["fma.rn.f32x2 %s, %s, qM1, %s;" % (c(x), c(y), c(x)),
-                    "fma.rn.f32x2 %s, %s, qP2, %s;" % (c(y), c(y), c(x))]
-    return out
+    return interleave([["fma.rn.f32x2 %s, %s, qM1, %s;" % (c(x), c(y), c(x)),
+                        "fma.rn.f32x2 %s, %s, qP2, %s;" % (c(y), c(y), c(x))]
+                       for x, y in units(j) for c in (re, im)])
 
 
 def case_xh(j):
@@ -133,13 +148,13 @@ def case_xh(j):
     if j == 0:
         return on_bit0(["sub.rn.f32 yi, yi, xr;", "fma.rn.f32 xr, xr, %s, yi;" % F_2,
                         "sub.rn.f32 xi, xi, yr;", "fma.rn.f32 yr, yr, %s, xi;" % F_2])
-    out = []
+    chains = []
     for x, y in units(j):
-        out += ["fma.rn.f32x2 %s, %s, qM1, %s;" % (im(y), re(x), im(y)),
-                "fma.rn.f32x2 %s, %s, qP2, %s;" % (re(x), re(x), im(y)),
-                "fma.rn.f32x2 %s, %s, qM1, %s;" % (im(x), re(y), im(x)),
-                "fma.rn.f32x2 %s, %s, qP2, %s;" % (re(y), re(y), im(x))]
-    return out
+        chains += [["fma.rn.f32x2 %s, %s, qM1, %s;" % (im(y), re(x), im(y)),
+                    "fma.rn.f32x2 %s, %s, qP2, %s;" % (re(x), re(x), im(y))],
+                   ["fma.rn.f32x2 %s, %s, qM1, %s;" % (im(x), re(y), im(x)),
+                    "fma.rn.f32x2 %s, %s, qP2, %s;" % (re(y), re(y), im(x))]]
+    return interleave(chains)
 
 
 def case_t(j):
@@ -147,21 +162,15 @@ def case_t(j):
     if j == 0:
         return on_bit0(["mul.rn.f32 yr, yr, %s;" % F_C, "fma.rn.f32 yr, yi, %s, yr;" % F_NC,
                         "fma.rn.f32 yi, yi, %s, yr;" % F_2C])
-    out = [const("qS", F_C), const("qt", F_NC), const("qm", F_2C)]
-    for _, y in units(j):
-        out += ["mul.rn.f32x2 %s, %s, qS;" % (re(y), re(y)),
-                "fma.rn.f32x2 %s, %s, qt, %s;" % (re(y), im(y), re(y)),
-                "fma.rn.f32x2 %s, %s, qm, %s;" % (im(y), im(y), re(y))]
-    return out
+    return [const("qS", F_C), const("qt", F_NC), const("qm", F_2C)] + interleave([
+        ["mul.rn.f32x2 %s, %s, qS;" % (re(y), re(y)),
+         "fma.rn.f32x2 %s, %s, qt, %s;" % (re(y), im(y), re(y)),
+         "fma.rn.f32x2 %s, %s, qm, %s;" % (im(y), im(y), re(y))] for _, y in units(j)])
 
 
 def element1(body, mask=0):
     """`body` on element 1 (yr, yi) of the units whose bits include mask."""
-    out = []
-    for k in range(NU):
-        if (k & mask) == mask:
-            out += unpack(k) + body + pack(k)
-    return out
+    return scalar_units([k for k in range(NU) if (k & mask) == mask], body)
 
 
 def sign_units(mask, factor):
@@ -175,7 +184,7 @@ def case_cz(j, k):
     return sign_units((1 << (j - 1)) | (1 << (k - 1)), "qM1")
 
 
-# The record of the op that runs is op qo - 1 (the dispatch has advanced qo).
+# The record of the op that runs is op qo - 1 (the head has advanced qo).
 RECORD = ["mad.lo.u32 qa, qo, 16, %s;" % BASE]
 SELECTED = ["ld.shared.u64 qm, [qa+%s];" % O_RECS,
             "and.b64 qt, %s, qm;" % IDX,
@@ -196,32 +205,30 @@ def case_ry(j):
         return RECORD + PARAMS + on_bit0([
             "fma.rn.f32 xr, yr, pa, xr;", "fma.rn.f32 yr, xr, pb, yr;", "fma.rn.f32 xr, yr, pa, xr;",
             "fma.rn.f32 xi, yi, pa, xi;", "fma.rn.f32 yi, xi, pb, yi;", "fma.rn.f32 xi, yi, pa, xi;"])
-    out = RECORD + PARAMS + ["mov.b64 qS, {pa, pa};", "mov.b64 qt, {pb, pb};"]
-    for x, y in units(j):
-        for c in (re, im):
-            out += ["fma.rn.f32x2 %s, %s, qS, %s;" % (c(x), c(y), c(x)),
-                    "fma.rn.f32x2 %s, %s, qt, %s;" % (c(y), c(x), c(y)),
-                    "fma.rn.f32x2 %s, %s, qS, %s;" % (c(x), c(y), c(x))]
-    return out
+    return RECORD + PARAMS + ["mov.b64 qS, {pa, pa};", "mov.b64 qt, {pb, pb};"] + interleave([
+        ["fma.rn.f32x2 %s, %s, qS, %s;" % (c(x), c(y), c(x)),
+         "fma.rn.f32x2 %s, %s, qt, %s;" % (c(y), c(x), c(y)),
+         "fma.rn.f32x2 %s, %s, qS, %s;" % (c(x), c(y), c(x))] for x, y in units(j) for c in (re, im)])
 
 
 def case_rx(j):
     # with w = i y (w.re = -y.im, w.im = y.re): x += a w, w += b x, x += a w
-    out = RECORD + PARAMS + ["neg.f32 na, pa;", "neg.f32 nb, pb;"]
+    out = RECORD + PARAMS + ["neg.f32 nc, pa;", "neg.f32 nb, pb;"]
     if j == 0:
         return out + on_bit0([
-            "fma.rn.f32 xr, yi, na, xr;", "fma.rn.f32 xi, yr, pa, xi;",
+            "fma.rn.f32 xr, yi, nc, xr;", "fma.rn.f32 xi, yr, pa, xi;",
             "fma.rn.f32 yi, xr, nb, yi;", "fma.rn.f32 yr, xi, pb, yr;",
-            "fma.rn.f32 xr, yi, na, xr;", "fma.rn.f32 xi, yr, pa, xi;"])
-    out += ["mov.b64 qS, {pa, pa};", "mov.b64 qt, {na, na};", "mov.b64 qm, {pb, pb};", "mov.b64 qn, {nb, nb};"]
+            "fma.rn.f32 xr, yi, nc, xr;", "fma.rn.f32 xi, yr, pa, xi;"])
+    out += ["mov.b64 qS, {pa, pa};", "mov.b64 qt, {nc, nc};", "mov.b64 qm, {pb, pb};", "mov.b64 qv, {nb, nb};"]
+    chains = []
     for x, y in units(j):
-        out += ["fma.rn.f32x2 %s, %s, qt, %s;" % (re(x), im(y), re(x)),
-                "fma.rn.f32x2 %s, %s, qS, %s;" % (im(x), re(y), im(x)),
-                "fma.rn.f32x2 %s, %s, qn, %s;" % (im(y), re(x), im(y)),
-                "fma.rn.f32x2 %s, %s, qm, %s;" % (re(y), im(x), re(y)),
-                "fma.rn.f32x2 %s, %s, qt, %s;" % (re(x), im(y), re(x)),
-                "fma.rn.f32x2 %s, %s, qS, %s;" % (im(x), re(y), im(x))]
-    return out
+        chains += [["fma.rn.f32x2 %s, %s, qt, %s;" % (re(x), im(y), re(x)),
+                    "fma.rn.f32x2 %s, %s, qv, %s;" % (im(y), re(x), im(y)),
+                    "fma.rn.f32x2 %s, %s, qt, %s;" % (re(x), im(y), re(x))],
+                   ["fma.rn.f32x2 %s, %s, qS, %s;" % (im(x), re(y), im(x)),
+                    "fma.rn.f32x2 %s, %s, qm, %s;" % (re(y), im(x), re(y)),
+                    "fma.rn.f32x2 %s, %s, qS, %s;" % (im(x), re(y), im(x))]]
+    return out + interleave(chains)
 
 
 def phase_units(mask):
@@ -229,9 +236,9 @@ def phase_units(mask):
     out = ["neg.f32 nb, pb;", "mov.b64 qS, {pa, pa};", "mov.b64 qt, {pb, pb};", "mov.b64 qm, {nb, nb};"]
     for k in range(NU):
         if (k & mask) == mask:
-            out += ["mul.rn.f32x2 qn, %s, qm;" % im(k),
+            out += ["mul.rn.f32x2 qv, %s, qm;" % im(k),
                     "mul.rn.f32x2 qu, %s, qt;" % re(k),
-                    "fma.rn.f32x2 %s, %s, qS, qn;" % (re(k), re(k)),
+                    "fma.rn.f32x2 %s, %s, qS, qv;" % (re(k), re(k)),
                     "fma.rn.f32x2 %s, %s, qS, qu;" % (im(k), im(k))]
     return out
 
@@ -250,6 +257,21 @@ def case_pp(j, k):
     out = RECORD + PARAMS
     return out + (PHASE1 + element1(PHASE1_BODY, 1 << (k - 1)) if j == 0
                   else phase_units((1 << (j - 1)) | (1 << (k - 1))))
+
+
+GROUP = 8     # independent chains interleaved
+
+
+def interleave(chains):
+    """The instructions of independent chains, GROUP chains at a time step by
+    step: a dependent instruction follows its source at a distance that covers
+    the FMA latency."""
+    out = []
+    for g in range(0, len(chains), GROUP):
+        grp = chains[g:g + GROUP]
+        for step in range(max(len(c) for c in grp)):
+            out += [c[step] for c in grp if step < len(c)]
+    return out
 
 
 def cases(full):
@@ -272,19 +294,21 @@ def cases(full):
     return body
 
 
-def dispatch(L, ncodes):
-    """Runs op qo (its code in qcn, loaded earlier): leaves when qo reaches
-    the end, loads op qo + 1's code (the staged codes run past the last op),
-    and branches to op qo's case; a code outside the table is clamped to the
-    extra entry, which only dispatches the next op (the lowering never makes
-    one)."""
-    return ["setp.ge.s32 qp, qo, %s;" % END,
-            "@qp bra.uni " + L("DONE") + ";",
-            "min.u32 qc, qcn, %d;" % ncodes,
+def head(ncodes):
+    """Start of every case (op qo, the next op's code in qn): advances qo, takes
+    the next op's code for the branch at the case's end and loads the one
+    after it.  No test separates the head from the branch -- a phase's codes
+    end with the end code -- so the table look-up of the branch target runs
+    under the case's arithmetic.  A code outside the table ends the phase (the
+    lowering never makes one)."""
+    return ["min.u32 qc, qn, %d;" % ncodes,
             "add.u32 qo, qo, 1;",
             "add.u32 qa, %s, qo;" % BASE,
-            "ld.shared.u8 qcn, [qa+%s];" % O_CODES,
-            "brx.idx.uni qc, " + L("TBL") + ";"]
+            "ld.shared.u8 qn, [qa+%s+1];" % O_CODES]
+
+
+def branch(L):
+    return ["brx.idx.uni qc, " + L("TBL") + ";"]
 
 
 def slots(store):
@@ -308,58 +332,112 @@ def slots(store):
 
 def factor(L):
     """The thread's factor: mode 0 none, 1 real, 2 complex."""
-    out = ["setp.eq.u32 qp, %s, 0;" % FMODE,
+    out = ["and.b32 qc, %s, 3;" % FLAGS,
+           "setp.eq.u32 qp, qc, 0;",
            "@qp bra.uni " + L("STORE") + ";",
            "mov.b64 qS, {%s, %s};" % (FR, FR),
-           "setp.eq.u32 qp, %s, 1;" % FMODE,
+           "setp.eq.u32 qp, qc, 1;",
            "@qp bra.uni " + L("REAL") + ";",
            "neg.f32 nb, %s;" % FI,
            "mov.b64 qt, {%s, %s};" % (FI, FI),
            "mov.b64 qm, {nb, nb};"]
     for k in range(NU):
-        out += ["mul.rn.f32x2 qn, %s, qm;" % im(k),
+        out += ["mul.rn.f32x2 qv, %s, qm;" % im(k),
                 "mul.rn.f32x2 qu, %s, qt;" % re(k),
-                "fma.rn.f32x2 %s, %s, qS, qn;" % (re(k), re(k)),
+                "fma.rn.f32x2 %s, %s, qS, qv;" % (re(k), re(k)),
                 "fma.rn.f32x2 %s, %s, qS, qu;" % (im(k), im(k))]
     out += ["bra.uni " + L("STORE") + ";", L("REAL") + ":"]
     out += sign_units(0, "qS")
     return out
 
 
+def flag(bit):
+    return ["and.b32 qc, %s, %d;" % (FLAGS, bit), "setp.eq.u32 qp, qc, 0;"]
+
+
+def next_tile(L):
+    """Last phase of a direct pass: once every thread has loaded its units the
+    tile's buffer is free, and the next tile is copied in while the ops run."""
+    out = flag(F_DIRECT) + ["@qp bra.uni " + L("OPS") + ";", "bar.sync %s, %s;" % (BARID, NTHR)]
+    out += flag(F_MORE) + ["@qp bra.uni " + L("OPS") + ";"]
+    for it in range(NU):
+        out += ["ld.shared.v2.u64 {qt, qm}, [%s+%s];" % (BASE, "%s+%d" % (O_UNIT, 16 * it)),
+                "cvt.u32.u64 qc, qm;",
+                "xor.b32 qc, qc, %s;" % SWT,
+                "add.u32 qc, qc, %s;" % TILE,
+                "add.u64 qt, qt, %s;" % NSRC,
+                "cp.async.cg.shared.global [qc], [qt], 16;"]
+    return out + [L("OPS") + ":"]
+
+
+def state_stores(canon):
+    """All units to the state, Gray-code order: from one unit to the next one
+    register bit's offset is added or subtracted."""
+    out, prev = [], 0
+    for i in range(NU):
+        k = i ^ (i >> 1)
+        if i:
+            bit = (k ^ prev).bit_length()       # register bit of the unit bit that changed
+            out.append("%s.s64 qt, qt, d%d;" % ("add" if k > prev else "sub", bit))
+        prev = k
+        if canon:
+            out += unpack(k) + ["st.global.v4.f32 [qt], {xr, xi, yr, yi};"]
+        else:
+            out.append("st.global.v2.b64 [qt], {%s, %s};" % (re(k), im(k)))
+    return out
+
+
+def direct_store(L):
+    out = flag(F_DIRECT) + ["@qp bra.uni " + L("TILE") + ";",
+                            "mov.u32 qa, %tid.x;",
+                            "mad.lo.u32 qa, qa, 8, %s;" % BASE,
+                            "ld.shared.u64 qt, [qa+%s];" % O_DST]
+    for j in range(1, RB):
+        out.append("ld.shared.u64 d%d, [%s+%s];" % (j, BASE, "%s+%d" % (O_DREG, 8 * j)))
+    out += flag(F_CANON) + ["@qp bra.uni " + L("RAW") + ";"]
+    out += state_stores(True) + ["bra.uni " + L("END") + ";", L("RAW") + ":"]
+    out += state_stores(False) + ["bra.uni " + L("END") + ";", L("TILE") + ":"]
+    return out
+
+
 def asm_text(prefix, full):
-    """PTX of one phase: loads the thread's units, runs the ops [begin, end),
-    applies the factor, stores the units.  The units live in registers of the
-    block's own, so nothing has to be moved at its boundary."""
+    """PTX of one phase: loads the thread's units, runs the ops from `begin` to the
+    end code, applies the factor, stores the units to the tile or (direct) to the
+    state.  The units live in registers of the block's own, so nothing has to
+    be moved at its boundary."""
     def L(name):
         return "%s_%s" % (prefix, name)
     body = cases(full)
     n = len(body)
     lines = ["{",
              ".reg .pred qp;",
-             ".reg .u32 qo, qc, qcn, qa, qh, a0, a1, b<%d>;" % RB,
-             ".reg .b64 qm, qt, qS, qn, qu, qM1, qP2;",
-             ".reg .f32 xr, xi, yr, yi, xx, pa, pb, na, nb;",
+             ".reg .u32 qo, qc, qn, qa, qh, a0, a1, b<%d>;" % RB,
+             ".reg .b64 qm, qt, qS, qv, qu, qM1, qP2, d<%d>;" % RB,
+             ".reg .f32 xr, xi, yr, yi, pa, pb, nb, nc;",
+             ".reg .f32 " + ", ".join(t + str(n) for n in range(TEMPS) for t in ("xr", "xi", "yr", "yi", "na", "xx")) + ";",
              ".reg .b64 u<%d>;" % NS,
              "add.u32 qh, %s, %s;" % (BASE, PHASE)]
     lines += slots(False)
+    lines += next_tile(L)
     lines += ["mov.b64 qM1, {%s, %s};" % (F_M1, F_M1),
               "mov.b64 qP2, {%s, %s};" % (F_2, F_2),
               "mov.u32 qo, %s;" % BEGIN,
               "add.u32 qa, %s, qo;" % BASE,
-              "ld.shared.u8 qcn, [qa+%s];" % O_CODES,
-              L("TBL") + ": .branchtargets " + ", ".join([L("C%d" % c) for c in range(n)] + [L("NEXT")]) + ";",
-              L("NEXT") + ":"]
-    lines += dispatch(L, n)
+              "ld.shared.u8 qc, [qa+%s];" % O_CODES,
+              "ld.shared.u8 qn, [qa+%s+1];" % O_CODES,
+              L("TBL") + ": .branchtargets " + ", ".join([L("C%d" % c) for c in range(n)] + [L("DONE")]) + ";",
+              "min.u32 qc, qc, %d;" % n]
+    lines += branch(L)
     for c, b in enumerate(body):
         lines.append(L("C%d" % c) + ":")
-        lines += b
-        lines += dispatch(L, n)
+        lines += head(n) + b + branch(L)
     lines.append(L("DONE") + ":")
     lines += factor(L)
     lines.append(L("STORE") + ":")
+    lines += direct_store(L)
     lines.append("add.u32 qh, %s, %s;" % (BASE, PHASE))
     lines += slots(True)
-    lines.append("}")
+    lines += [L("END") + ":", "}"]
     return lines
 
 
@@ -374,17 +452,19 @@ def emit():
            "template <bool FULL> struct OpLoop;"]
     for full, prefix in ((False, "QSWCT"), (True, "QSWFL")):
         out.append("template <> struct OpLoop<%s> {" % ("true" if full else "false"))
-        out.append("    template <int O_CODES, int O_RECS>")
+        out.append("    template <int O_CODES, int O_RECS, int O_UNIT, int O_DREG, int O_DST>")
         out.append("    static __device__ __forceinline__ void run(uint32_t addr, uint32_t tile, uint32_t base,")
-        out.append("                                               uint32_t phase, int ob, int ub,")
+        out.append("                                               uint32_t phase, int ob,")
         out.append("                                               unsigned long long idx, float fr, float fi,")
-        out.append("                                               uint32_t fmode)")
+        out.append("                                               uint32_t flags, uint32_t swt, const void *nsrc,")
+        out.append("                                               uint32_t barid, uint32_t nthr)")
         out.append("    {")
         out.append("        asm volatile(")
         for line in asm_text(prefix, full):
-            out.append('            "%s\\n"' % line)
-        out.append('            : : "r"(addr), "r"(tile), "r"(base), "r"(phase), "r"(ob), "r"(ub), "l"(idx), "f"(fr), "f"(fi), "r"(fmode),')
-        out.append('                "n"(O_CODES), "n"(O_RECS)')
+            out.append('            "%s\\n"' % line.replace("%tid", "%%tid"))
+        out.append('            : : "r"(addr), "r"(tile), "r"(base), "r"(phase), "r"(ob), "l"(idx), "f"(fr), "f"(fi),')
+        out.append('                "r"(flags), "r"(swt), "l"(nsrc), "r"(barid), "r"(nthr), "n"(O_CODES), "n"(O_RECS), "n"(O_UNIT),')
+        out.append('                "n"(O_DREG), "n"(O_DST)')
         out.append('            : "memory");')
         out.append("    }")
         out.append("};")

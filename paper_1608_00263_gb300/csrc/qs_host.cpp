@@ -580,6 +580,62 @@ static uint64_t choose_tile(const std::vector<PGate> &g, const std::vector<int> 
     return choose_local(g, cand, done, n, local, pool, want - added, allq);
 }
 
+// One phase of a wide pass: its register qubits and its gates in order.
+struct PhaseSet {
+    uint64_t reg;
+    std::vector<int> gates;
+};
+
+// Ops a gate becomes in a plan: 5 for RX, 3 for RY, else 1.
+static int gate_ops(const PGate &x) { return x.kind == QS_RX ? 5 : x.kind == QS_RY ? 3 : 1; }
+
+// Greedy phases for the gates of `cand` not yet done (marked done as they
+// are placed), qubit 0 always among the r register qubits.  Returns false
+// when they do not fit `max_phases`.
+static bool greedy_phases(const std::vector<PGate> &g, const std::vector<int> &cand, std::vector<char> *done, int n,
+                          uint64_t local, int r, int max_phases, std::vector<PhaseSet> *out)
+{
+    size_t left = 0;
+    for (int i : cand) left += !(*done)[i];
+    while (left) {
+        if ((int)out->size() >= max_phases) return false;
+        PhaseSet p;
+        int cnt;
+        p.reg = choose_local(g, cand, *done, n, 1, local, r - 1);
+        collect(g, cand, *done, p.reg, &p.gates, &cnt);
+        if (cnt == 0) return false;
+        for (int i : p.gates) (*done)[i] = 1;
+        left -= p.gates.size();
+        out->push_back(std::move(p));
+    }
+    return true;
+}
+
+// Phases of a wide pass whose last phase leaves qubits 1..4 out of its
+// register set, so that a warp's lanes can run along them and the phase's
+// stores to the state are whole 256-byte runs (see WidePass::direct).  The
+// last phase is chosen first: the greedy set for the gate list read
+// backwards, among the tile's other qubits; the gates it takes can follow
+// all others (the blocking rule of collect is symmetric in time).  The rest
+// is greedy as before.  False when that takes more phases than `limit`.
+static bool direct_phases(const std::vector<PGate> &g, const std::vector<int> &pass_gates, int n, uint64_t local,
+                          int r, int limit, std::vector<PhaseSet> *out)
+{
+    std::vector<char> done(g.size(), 1);
+    for (int i : pass_gates) done[i] = 0;
+    const std::vector<int> back(pass_gates.rbegin(), pass_gates.rend());
+    PhaseSet last;
+    int cnt;
+    last.reg = choose_local(g, back, done, n, 1, local & ~0x1Eull, r - 1);
+    collect(g, back, done, last.reg, &last.gates, &cnt);
+    std::reverse(last.gates.begin(), last.gates.end());
+    for (int i : last.gates) done[i] = 1;
+    out->clear();
+    if (!greedy_phases(g, pass_gates, &done, n, local, r, limit - 1, out)) return false;
+    out->push_back(std::move(last));
+    return true;
+}
+
 // Shared-memory wavefronts of one phase's slot loads (the stores mirror
 // them).  A warp's shared access is served per group of lanes -- 16 lanes
 // for 8-byte accesses, 8 for 16-byte ones -- and a group costs the largest
@@ -1003,6 +1059,8 @@ void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> 
             std::vector<WideOp> tail;
             std::vector<uint8_t> tail_codes;
             lower_phase(P, H, ops, out, &tail, &tail_codes, &full);
+            out->ops.push_back(WideOp{0, 0, 1.f, 0.f});
+            out->codes.push_back(W_END);
             V.tail_begin = (int16_t)(out->ops.size() - W.op_begin);
             out->ops.insert(out->ops.end(), tail.begin(), tail.end());
             out->codes.insert(out->codes.end(), tail_codes.begin(), tail_codes.end());
@@ -1013,6 +1071,10 @@ void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> 
         // them; the first reads and the last writes canonical order
         W.canon_in = &P == &passes.front();
         W.canon_out = &P == &passes.back();
+        const DevPhase &last = phases[P.phase_begin + P.nphases - 1];
+        W.direct = 1;
+        for (int k = 0; k < 4; ++k) W.direct &= last.T[k] == k + 1;
+        for (int j = 0; j < kWideRegBits; ++j) W.dreg[j] = 8ull << P.L[last.R[j]];
         W.full = full;
         out->passes.push_back(W);
     }
@@ -1282,11 +1344,41 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
         size_t prem = pass_gates.size();
         int pass_ops = 0;
         int tc_in_pass = 0;
-        while (prem && dp.nphases < kMaxPhasesPerPass && pass_ops < kMaxOpsPerPass) {
+        // (a lowered wide pass holds an end code per phase too)
+        const int max_ops = pp.pack0 ? kMaxOpsPerPass - kMaxPhasesPerPass : kMaxOpsPerPass;
+        // wide passes: all phases are chosen ahead, with a last phase that can
+        // store to the state where that takes no more phases (37 of 51 passes
+        // of five 30-qubit circuits; 13 would take one more)
+        std::vector<PhaseSet> ahead;
+        bool direct = false;
+        if (pp.pack0) {
+            int ops = 0;
+            for (int i : pass_gates) ops += gate_ops(g[i]);
+            std::vector<char> pd(pdone);
+            if (ops <= max_ops && greedy_phases(g, pass_gates, &pd, n, local, dp.r, kMaxPhasesPerPass, &ahead)) {
+                std::vector<PhaseSet> alt;
+                if (direct_phases(g, pass_gates, n, local, dp.r, (int)ahead.size(), &alt)) {
+                    ahead.swap(alt);
+                    direct = true;
+                }
+            } else {
+                ahead.clear();
+            }
+        }
+        while (prem && dp.nphases < kMaxPhasesPerPass && pass_ops < max_ops) {
             // (with pack0 qubit 0 is always a register qubit)
-            uint64_t reg = pp.pack0 ? choose_local(g, pass_gates, pdone, n, 1, local, dp.r - 1)
-                                    : choose_local(g, pass_gates, pdone, n, 0, local, dp.r);
-            collect(g, pass_gates, pdone, reg, &phase_gates, &cnt);
+            uint64_t reg;
+            bool direct_last = false;
+            if (!ahead.empty()) {
+                reg = ahead[dp.nphases].reg;
+                phase_gates = ahead[dp.nphases].gates;
+                cnt = (int)phase_gates.size();
+                direct_last = direct && dp.nphases + 1 == (int)ahead.size();
+            } else {
+                reg = pp.pack0 ? choose_local(g, pass_gates, pdone, n, 1, local, dp.r - 1)
+                               : choose_local(g, pass_gates, pdone, n, 0, local, dp.r);
+                collect(g, pass_gates, pdone, reg, &phase_gates, &cnt);
+            }
             if (cnt == 0) return set_error(QS_ERR_INVALID_ARG, "planner made no phase progress");
             if (pp.tc_ok && tc_in_pass < kMaxTcPerPass && dp.t == 13) {
                 // tensor-core block candidate: worth it when it absorbs many
@@ -1325,7 +1417,7 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
                 int ops_needed = 0;
                 for (int gi : phase_gates) {
                     const int k = g[gi].kind == QS_RX ? 5 : g[gi].kind == QS_RY ? 3 : 1;
-                    if (pass_ops + ops_needed + k > kMaxOpsPerPass) break;
+                    if (pass_ops + ops_needed + k > max_ops) break;
                     ops_needed += k;
                     ++keep;
                 }
@@ -1342,14 +1434,24 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
             for (int q = 0; q < n; ++q) reg_bit_of[q] = -1;
             for (int q = 0; q < n; ++q)
                 if ((reg >> q) & 1) { reg_bit_of[q] = j; ph.R[j++] = (uint8_t)tile_bit_of[q]; }
-            // pad with unused tile bits so the phase always has dp.r register bits
-            for (int b = 0; j < dp.r && b < dp.t; ++b) {
+            // pad with unused tile bits so the phase always has dp.r register
+            // bits (tile bits 1..4 of a direct last phase stay lane bits)
+            for (int b = direct_last ? 5 : 0; j < dp.r && b < dp.t; ++b) {
                 bool used = false;
                 for (int i2 = 0; i2 < j; ++i2) used |= ph.R[i2] == b;
                 if (!used) ph.R[j++] = (uint8_t)b;
             }
             std::sort(ph.R, ph.R + dp.r);
-            choose_thread_bits(ph.R, dp.r, dp.t, pp.esz, ph.T);
+            if (direct_last) {
+                int k = 0;
+                for (int b = 1; b < dp.t; ++b) {
+                    bool used = false;
+                    for (int i2 = 0; i2 < dp.r; ++i2) used |= ph.R[i2] == b;
+                    if (!used) ph.T[k++] = (uint8_t)b;
+                }
+            } else {
+                choose_thread_bits(ph.R, dp.r, dp.t, pp.esz, ph.T);
+            }
             for (int q = 0; q < n; ++q) reg_bit_of[q] = -1;
             for (int i2 = 0; i2 < dp.r; ++i2) reg_bit_of[dp.L[ph.R[i2]]] = i2;
             ph.op_begin = (int)P.ops.size();

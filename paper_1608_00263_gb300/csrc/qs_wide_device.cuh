@@ -26,7 +26,9 @@ constexpr int kWideThreads = 1 << (13 - kWideRegBits);   // threads of a 13-qubi
 constexpr int kWideSlots = 1 << kWideRegBits;
 constexpr int kWideUnits = kWideSlots / 2;               // 16-byte units per thread
 
-struct WideUnit {           // unit `it` of every thread
+constexpr uint32_t kWideDirect = 4, kWideMore = 8, kWideCanon = 16;   // phase flags (gen_op_loop.py)
+
+struct alignas(16) WideUnit {           // unit `it` of every thread
     uint64_t goff;          // byte offset in the state
     uint32_t soff;          // swizzled byte offset in the tile
     uint32_t pad;
@@ -36,12 +38,18 @@ struct WideSmem {
     WidePass P;
     WideOp ops[kMaxOpsPerPass];
     uint32_t codes[kMaxOpsPerPass / 4 + 4];
-    uint64_t toff[kWideThreads];                     // byte offset of the thread's unit 0 in the state
+    uint64_t toff[kWideThreads];                     // byte offset in the state of the thread's first copied unit
+    uint64_t doff[kWideThreads];                     // ... of its slot 0 in the last phase
+    uint64_t dst[kWideThreads];                      // direct pass: state address of the thread's slot 0
     uint64_t gmask;                                  // out-of-tile qubits
     uint16_t thr[kMaxPhasesPerPass][kWideThreads];   // tile element of the thread's slot 0
     WideUnit unit[kWideUnits];
     float2 w8[8];                                    // e^{i pi k / 4}
 };
+
+static_assert(sizeof(WidePass) % 16 == 0 && offsetof(WidePass, ph) % 16 == 0 && offsetof(WideSmem, ops) % 16 == 0 &&
+                  offsetof(WideSmem, unit) % 16 == 0 && sizeof(WideUnit) == 16,
+              "staged in 16-byte units");
 
 // Tables of the folded diagonal prefix (first pass of a circuit, see
 // FoldArgs): CZ partners as a qubit mask and as a mask of tile bits, T
@@ -143,7 +151,10 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             F->w[k] = k < 4 ? make_float2((float)re, (float)im) : make_float2((float)-re, (float)-im);
         }
     }
-    if (gi == 0) S.toff[tid] = deposit(2u * (uint32_t)tid, S.P.L, t) * 8u;
+    if (gi == 0) {
+        S.toff[tid] = deposit(2u * (uint32_t)tid, S.P.L, t) * 8u;
+        S.doff[tid] = deposit(S.thr[nph - 1][tid], S.P.L, t) * 8u;
+    }
     if (threadIdx.x == 0) {
         uint64_t m = 0;
         for (int i = 0; i < ng; ++i) m |= 1ULL << S.P.G[i];
@@ -221,6 +232,11 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             }
         }
         wide_sync<GROUPED>(nthr, gi);
+        // (the next tile's base is formed where it is used: registers are
+        // what the phases are short of)
+        auto next_base = [&]() {
+            return GROUPED && ngr > 1 ? deposit(tau + (uint32_t)ngr, S.P.G, ng) : (((base | ~S.gmask) + 1) & S.gmask);
+        };
         for (int ph = 0; ph < nph; ++ph) {
             const WidePhase &H = S.P.ph[ph];
             const uint32_t te = S.thr[ph][tid], to = tau;
@@ -234,6 +250,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             uint32_t mode = 0;
             if (ub < oe || last) {
                 uint32_t k = 0;
+#pragma unroll 2
                 for (int o = ub; o < oe; ++o) {
                     const WideOp op = S.ops[o];
                     if ((te & op.sel_tile) == op.sel_tile && (to & op.sel_out) == op.sel_out) {
@@ -257,32 +274,60 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
                 }
                 mode = __any_sync(0xffffffffu, fi != 0.f) ? 2u : 1u;
             }
-            OpLoop<FULL>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16>(
+            const bool direct = last && S.P.direct;
+            const char *nsrc = nullptr;
+            if (direct) {
+                S.dst[threadIdx.x] = reinterpret_cast<uint64_t>(amps) + base * 8u + S.doff[tid];
+                mode |= kWideDirect | (S.P.canon_out ? kWideCanon : 0u);
+                if (!FOLD && tau + (uint32_t)ngr < t_end && inside(next_base())) {
+                    mode |= kWideMore;
+                    nsrc = reinterpret_cast<const char *>(amps) + (next_base() * 8u + S.toff[tid]);
+                }
+            }
+            OpLoop<FULL>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16,
+                                       (int)offsetof(WideSmem, unit),
+                                       (int)(offsetof(WideSmem, P) + offsetof(WidePass, dreg)),
+                                       (int)offsetof(WideSmem, dst)>(
                 swz<2>(te) * 8u, tile_sa, smem_addr(&S),
                 (uint32_t)(offsetof(WideSmem, P) + offsetof(WidePass, ph)) + (uint32_t)ph * (uint32_t)sizeof(WidePhase),
-                H.op_begin, ub, ((uint64_t)to << 32) | te, fr, fi, mode);
-            wide_sync<GROUPED>(nthr, gi);
+                H.op_begin, ((uint64_t)to << 32) | te, fr, fi, mode, sw_tid,
+                nsrc, GROUPED ? (uint32_t)gi + 1u : 0u,
+                (uint32_t)nthr);
+            if (!direct) wide_sync<GROUPED>(nthr, gi);
         }
-        // ---- store the tile; each unit's place takes the same unit of the
-        // next tile as soon as this thread has read it (no other thread
-        // touches it before the next barrier) ----
-        const uint64_t toff = S.toff[tid];
-        const bool canon_out = S.P.canon_out != 0;
-        char *dst = reinterpret_cast<char *>(amps) + (base * 8u + toff);
-        tau += (uint32_t)ngr;
-        base = GROUPED && ngr > 1 ? deposit(tau, S.P.G, ng) : (((base | ~S.gmask) + 1) & S.gmask);
-        const bool more = !FOLD && tau < t_end && inside(base);
-        const char *src = reinterpret_cast<const char *>(amps) + (base * 8u + toff);
+        // ---- staged pass: store the tile; each unit's place takes the same
+        // unit of the next tile as soon as this thread has read it (no other
+        // thread touches it before the next barrier) ----
+        if (!S.P.direct) {
+            const uint64_t toff = S.toff[tid], nbase = next_base();
+            const bool more = !FOLD && tau + (uint32_t)ngr < t_end && inside(nbase), canon_out = S.P.canon_out != 0;
+            char *dst = reinterpret_cast<char *>(amps) + (base * 8u + toff);
+            const char *src = reinterpret_cast<const char *>(amps) + (nbase * 8u + toff);
 #pragma unroll 4
-        for (int it = 0; it < NU; ++it) {
-            const WideUnit u = S.unit[it];
-            const uint32_t so = sw_tid ^ u.soff;
-            const float4 v = *reinterpret_cast<const float4 *>(gsm + so);
-            *reinterpret_cast<float4 *>(dst + u.goff) = canon_out ? swap_unit(v) : v;
-            if (more)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tile_sa + so), "l"(src + u.goff)
-                             : "memory");
+            for (int i0 = 0; i0 < NU; i0 += 2) {
+                WideUnit u[2];
+                float4 v[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    u[i] = S.unit[i0 + i];
+                    u[i].soff ^= sw_tid;
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) v[i] = *reinterpret_cast<const float4 *>(gsm + u[i].soff);
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    *reinterpret_cast<float4 *>(dst + u[i].goff) = canon_out ? swap_unit(v[i]) : v[i];
+                if (more) {
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(tile_sa + u[i].soff),
+                                     "l"(src + u[i].goff)
+                                     : "memory");
+                }
+            }
         }
+        base = next_base();
+        tau += (uint32_t)ngr;
     }
     __syncthreads();
 }

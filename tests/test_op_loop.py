@@ -1,7 +1,8 @@
 """The wide pass's phase in inline PTX (csrc/gen_op_loop.py), run on the CPU by
 an interpreter of the instruction forms it uses: one thread loads its 64
 amplitudes from a tile in shared memory through swizzled addresses, runs a
-list of ops, applies its factor and stores them back.  Every access must fall
+list of ops, applies its factor and stores them back, to the tile or (direct)
+to the state while it copies the next tile in.  Every shared access must fall
 inside the tile or the staged pass and be aligned to its width; the tile
 starts at an address that is no multiple of its size.  Checked against the
 gates' definitions in FP64 for every byte code, with several register sets.
@@ -30,8 +31,9 @@ def _gen():
 
 
 G = _gen()
-SMEM_STATIC, TILE = 1024, 1024 + 8512        # staged pass; the tile follows it
-O_PHASE, O_OPS, O_CODES = 96, 480, 4576
+SMEM_STATIC, TILE = 1024, 1024 + 10608       # staged pass; the tile follows it
+O_PHASE, O_DREG, O_OPS, O_CODES, O_UNIT, O_DST = 144, 96, 528, 4624, 5008, 6000
+STATE, NEXT = 1 << 40, 3 << 40                # addresses in the state
 
 
 def swizzle(e):
@@ -43,6 +45,7 @@ class Thread:
     def __init__(self, lines, mem, lo, hi, operands):
         self.mem, self.lo, self.hi = mem, lo, hi
         self.r = dict(operands)
+        self.stores, self.copies = {}, []
         self.labels, self.code, self.table = {}, [], None
         for line in lines:
             line = line.strip().rstrip(";").strip()
@@ -78,6 +81,8 @@ class Thread:
                     continue
                 op, rest = rest.split(None, 1)
             a = [x.strip() for x in rest.replace("{", "").replace("}", "").split(",")]
+            if op == "bar.sync":
+                continue
             if op == "bra.uni":
                 pc = self.labels[a[0]]
             elif op == "brx.idx.uni":
@@ -108,7 +113,7 @@ class Thread:
                 r[a[0]] = f32(np.float64(self.val(a[1])) * np.float64(self.val(a[2])) + np.float64(self.val(a[3])))
             elif op == "neg.f32":
                 r[a[0]] = f32(-self.val(a[1]))
-            elif op == "add.u32":
+            elif op in ("add.u32", "add.u64", "add.s64"):
                 r[a[0]] = int(self.val(a[1])) + int(self.val(a[2]))
             elif op == "xor.b32":
                 r[a[0]] = int(self.val(a[1])) ^ int(self.val(a[2]))
@@ -120,6 +125,20 @@ class Thread:
                 r[a[0]] = self.val(a[1]) >= self.val(a[2])
             elif op in ("setp.eq.u32", "setp.eq.u64"):
                 r[a[0]] = self.val(a[1]) == self.val(a[2])
+            elif op == "sub.s64":
+                r[a[0]] = int(self.val(a[1])) - int(self.val(a[2]))
+            elif op == "cvt.u32.u64":
+                r[a[0]] = r[a[1]] & 0xFFFFFFFF
+            elif op == "and.b32":
+                r[a[0]] = int(self.val(a[1])) & int(a[2])
+            elif op == "cp.async.cg.shared.global":
+                self.copies.append((self.addr(a[0], 16), int(r[a[1].strip("[]")])))
+            elif op in ("st.global.v2.b64", "st.global.v4.f32"):
+                at = int(r[a[0].strip("[]")])
+                assert at % 16 == 0 and at not in self.stores
+                self.stores[at] = r[a[1]] + r[a[2]] if "b64" in op else [r[x] for x in a[1:5]]
+            elif op == "ld.shared.v2.u64":
+                r[a[0]], r[a[1]] = struct.unpack_from("<2Q", self.mem, self.addr(a[2], 16))
             elif op == "and.b64":
                 r[a[0]] = r[a[1]] & r[a[2]]
             elif op == "selp.f32":
@@ -223,22 +242,44 @@ def test_phase_on_one_thread(full, t, regs):
             struct.pack_into("<Q2f", mem, SMEM_STATIC + O_OPS + 16 * (first + k), want, *p)
             mem[SMEM_STATIC + O_CODES + first + k] = c
             ops.append((c, p[0], p[1], sel))
-        for mode, fac in ((0, 1.0), (1, -0.25), (2, 0.6 + 0.8j)):
+        mem[SMEM_STATIC + O_CODES + first + len(codes)] = 255      # the end code
+        # the state: tile bit b is qubit 2 b; the thread's copies and slot 0
+        qbit = [8 << (2 * b) for b in range(t)]
+        deposit = lambda e: sum(qbit[b] for b in range(t) if (e >> b) & 1)
+        units = [(deposit(2 * (1 << len(others)) * k), swizzle(2 * (1 << len(others)) * k) * 8) for k in range(32)]
+        for k, (goff, soff) in enumerate(units):
+            struct.pack_into("<2Q", mem, SMEM_STATIC + O_UNIT + 16 * k, goff, soff)
+        struct.pack_into("<6Q", mem, SMEM_STATIC + O_DREG, *[qbit[b] for b in regs])
+        struct.pack_into("<Q", mem, SMEM_STATIC + O_DST + 8 * tid, STATE + deposit(e0))
+        swt = swizzle(2 * tid) * 8
+        for mode, fac in ((0, 1.0), (1, -0.25), (2, 0.6 + 0.8j), (1 | G.F_DIRECT, 0.5), (2 | G.F_DIRECT | G.F_MORE, 1j),
+                          (1 | G.F_DIRECT | G.F_CANON, 2.0)):
             m2 = bytearray(mem)
             fac = complex(fac)
-            operands = dict(zip(["%%%d" % k for k in range(12)],
-                                [swizzle(e0) * 8, TILE, SMEM_STATIC, O_PHASE, first, first + len(codes), tau << 32 | e0,
-                                 f32(fac.real), f32(fac.imag), mode, O_CODES, O_OPS - 16]))
-            Thread(lines, m2, SMEM_STATIC, TILE + (8 << t), operands).run()
+            operands = dict(zip(["%%%d" % k for k in range(18)] + ["%tid.x"],
+                                [swizzle(e0) * 8, TILE, SMEM_STATIC, O_PHASE, first, tau << 32 | e0,
+                                 f32(fac.real), f32(fac.imag), mode, swt, NEXT, 0, 128, O_CODES, O_OPS - 16, O_UNIT,
+                                 O_DREG, O_DST, tid]))
+            th = Thread(lines, m2, SMEM_STATIC, TILE + (8 << t), operands)
+            th.run()
+            assert th.copies == ([(TILE + (soff ^ swt), NEXT + goff) for goff, soff in units] if mode & G.F_MORE else [])
             elems = [e0 | sum(((s >> j) & 1) << b for j, b in enumerate(regs)) for s in range(64)]
             v = expected(tile[elems, 0].astype(complex) + 1j * tile[elems, 1], t, ops, None) * fac
             got = np.empty(64, complex)
-            for s, e in enumerate(elems):
+            if mode & G.F_DIRECT:
+                for s, e in enumerate(elems):
+                    q = th.stores[STATE + deposit(e & ~1)]
+                    got[s] = complex(*(q[2 * (e & 1):][:2] if mode & G.F_CANON else (q[e & 1], q[2 + (e & 1)])))
+                assert len(th.stores) == 32 and m2 == mem
+            for s, e in enumerate(elems if not mode & G.F_DIRECT else []):
                 q = struct.unpack_from("<4f", m2, TILE + swizzle(e & ~1) * 8)
                 got[s] = complex(q[e & 1], q[2 + (e & 1)])
             scale = np.max(np.abs(v)) + 1.0     # butterflies grow by sqrt(2) each
             assert np.max(np.abs(got - v)) < 9e-6 * scale, (full, t, regs, codes, mode)
+            if mode & G.F_DIRECT:
+                continue
             # nothing else in the tile moved
+            assert not th.stores
             mine = {TILE + swizzle(e & ~1) * 8 for e in elems}
             for u in range(1 << (t - 1)):
                 a = TILE + swizzle(2 * u) * 8
