@@ -473,11 +473,11 @@ qs_status qs_batch_set_options(qs_batch *b, const qs_opts *opts);
 /* Engines of the batched ensemble (qs_batch_set_engine). */
 enum {
     QS_BATCH_PERSISTENT = 0,   /* one launch per run: a persistent kernel
-                                  (two CTAs of 256 threads per SM) takes
+                                  (as many CTAs as are resident) takes
                                   work items from a device queue: every
                                   instance's initial-state chunks (2^16
                                   amplitudes), then its fused passes in
-                                  items of 2^18 amplitudes, round-major
+                                  items of up to 2^18 amplitudes, round-major
                                   (pass r of every instance before pass
                                   r + 1 of any; larger instances first),
                                   then its statistics chunks; an item waits

@@ -105,6 +105,12 @@ static void batch_release_plan(qs_batch *b)
     b->ready = false;
 }
 
+static qs_status batch_setup()
+{
+    if (qs_status s0 = batch_kernel_setup()) return s0;
+    return batch_wide_setup();
+}
+
 // Tile sizes chosen by the autotuner, per (device, qubits, engine): a process-wide
 // cache, so later batches with instances of the same size skip the timing.
 static std::mutex g_tune_mu;
@@ -118,6 +124,10 @@ static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const u
                                 const std::vector<int> &tbits, std::vector<Plan> *plans)
 {
     plans->assign(b->count, Plan());
+    // one kernel runs every pass of a launch: wide passes when every listed
+    // instance's tile fills whole warps of them, else five register bits
+    bool wide = true;
+    for (int i : idx) wide = wide && std::min(tbits[i] ? tbits[i] : 13, b->n[i]) >= kWideMinTile;
     std::vector<qs_status> st(idx.size(), QS_OK);
     std::vector<std::string> msg(idx.size());
     const unsigned nth = std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
@@ -132,8 +142,10 @@ static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const u
                 o.mode = QS_MODE_FUSED;
                 o.tile_log2 = tbits[i];
                 PlanParams pp = default_plan_params(b->n[i], QS_C64, &o);
-                pp.r = std::min(5, pp.t);      // the batched passes hold five register bits
-                pp.pack0 = 0;
+                if (!wide) {
+                    pp.r = std::min(5, pp.t);
+                    pp.pack0 = 0;
+                }
                 st[k] = build_plan(pp, gates + offsets[i] + hl[i], ng, &(*plans)[i]);
                 if (st[k]) msg[k] = last_error_cstr();
             }
@@ -159,7 +171,25 @@ struct Rounds {
     std::vector<unsigned char> items;
     std::vector<RoundLaunch> launches;
     double bytes = 0;                // algorithmic bytes (16 per amplitude per pass)
+    WidePlan wide;                   // the passes lowered, when they are wide passes
 };
+
+// Lowers the listed instances' plans in list order (the order in which
+// their passes are concatenated) when all are wide passes; else empty.
+static void lower_instances(const std::vector<Plan> &plans, const std::vector<int> &idx, WidePlan *out)
+{
+    *out = WidePlan();
+    for (int i : idx)
+        if (!plans[i].passes.empty() && !wide_plan(plans[i].passes, plans[i].phases)) return;
+    for (int i : idx) lower_wide(plans[i].passes, plans[i].phases, plans[i].ops, out);
+}
+
+static bool any_full(const WidePlan &w)
+{
+    for (const WidePass &p : w.passes)
+        if (p.full) return true;
+    return false;
+}
 
 static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, const std::vector<int> &idx,
                          Rounds *R)
@@ -183,6 +213,7 @@ static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, cons
         max_passes = std::max(max_passes, (int)plans[i].passes.size());
         R->bytes += (double)plans[i].passes.size() * 16.0 * std::ldexp(1.0, b->n[i]);
     }
+    lower_instances(plans, idx, &R->wide);
     const size_t isz = batch_item_bytes();
     for (int r = 0; r < max_passes; ++r)
         for (int tb = 5; tb <= 13; ++tb) {
@@ -205,35 +236,59 @@ static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, cons
         }
 }
 
-// Section offsets of a Rounds layout in a device buffer: passes | phases |
-// ops | items, each 256-byte aligned.
+// Section offsets of a packed run in a device buffer: passes | phases | ops
+// (wide: passes | codes | records) | items, each 256-byte aligned.
 struct RoundOffsets {
     size_t pass, phase, op, item, total;
 };
-static RoundOffsets round_offsets(const Rounds &R)
+template <class T>
+static RoundOffsets pack_offsets(const T &R, const WidePlan &w, size_t item_bytes)
 {
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const bool wide = !w.passes.empty();
     RoundOffsets o;
     o.pass = 0;
-    o.phase = align(o.pass + R.passes.size() * sizeof(DevPass));
-    o.op = align(o.phase + R.phases.size() * sizeof(DevPhase));
-    o.item = align(o.op + R.ops.size() * sizeof(DevOp));
-    o.total = align(o.item + R.items.size());
+    o.phase = align(o.pass + (wide ? w.passes.size() * sizeof(WidePass) : R.passes.size() * sizeof(DevPass)));
+    o.op = align(o.phase + (wide ? w.codes.size() : R.phases.size() * sizeof(DevPhase)));
+    o.item = align(o.op + (wide ? w.ops.size() * sizeof(WideOp) : R.ops.size() * sizeof(DevOp)));
+    o.total = align(o.item + item_bytes);
     return o;
 }
-
+template <class T>
+static void pack_run(const T &R, const WidePlan &w, const RoundOffsets &o, const void *items, size_t item_bytes,
+                     unsigned char *host)
+{
+    if (!w.passes.empty()) {
+        std::memcpy(host + o.pass, w.passes.data(), w.passes.size() * sizeof(WidePass));
+        std::memcpy(host + o.phase, w.codes.data(), w.codes.size());
+        std::memcpy(host + o.op, w.ops.data(), w.ops.size() * sizeof(WideOp));
+    } else {
+        std::memcpy(host + o.pass, R.passes.data(), R.passes.size() * sizeof(DevPass));
+        std::memcpy(host + o.phase, R.phases.data(), R.phases.size() * sizeof(DevPhase));
+        std::memcpy(host + o.op, R.ops.data(), R.ops.size() * sizeof(DevOp));
+    }
+    if (item_bytes) std::memcpy(host + o.item, items, item_bytes);
+}
+static RoundOffsets round_offsets(const Rounds &R) { return pack_offsets(R, R.wide, R.items.size()); }
 static void round_pack(const Rounds &R, const RoundOffsets &o, unsigned char *host)
 {
-    std::memcpy(host + o.pass, R.passes.data(), R.passes.size() * sizeof(DevPass));
-    std::memcpy(host + o.phase, R.phases.data(), R.phases.size() * sizeof(DevPhase));
-    std::memcpy(host + o.op, R.ops.data(), R.ops.size() * sizeof(DevOp));
-    if (!R.items.empty()) std::memcpy(host + o.item, R.items.data(), R.items.size());
+    pack_run(R, R.wide, o, R.items.data(), R.items.size(), host);
 }
 
 static qs_status launch_rounds(const qs_batch *b, cudaStream_t st, const Rounds &R, const RoundOffsets &o,
                                const unsigned char *D)
 {
     const size_t isz = batch_item_bytes();
+    if (!R.wide.passes.empty()) {
+        // one interpreter for the whole run, as in the persistent engine
+        const bool full = any_full(R.wide);
+        for (const RoundLaunch &L : R.launches)
+            if (qs_status rs = launch_batch_round_wide(st, b->num_sms, b->amps, D + o.item + L.first * isz, (int)L.count,
+                                                       L.tbits, (const WidePass *)(D + o.pass),
+                                                       (const WideOp *)(D + o.op), D + o.phase, full))
+                return rs;
+        return QS_OK;
+    }
     for (const RoundLaunch &L : R.launches)
         if (qs_status rs = launch_batch_round(st, b->num_sms, b->amps, D + o.item + L.first * isz, (int)L.count,
                                               L.tbits, (const DevPass *)(D + o.pass),
@@ -252,41 +307,33 @@ static std::vector<std::vector<char>> full_flags(const std::vector<Plan> &plans)
     return f;
 }
 
-// Work layout in one device buffer: passes | phases | ops | items, each
-// 256-byte aligned.
-static RoundOffsets work_offsets(const Work &W)
+static RoundOffsets work_offsets(const Work &W, const WidePlan &w)
 {
-    auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    RoundOffsets o;
-    o.pass = 0;
-    o.phase = align(o.pass + W.passes.size() * sizeof(DevPass));
-    o.op = align(o.phase + W.phases.size() * sizeof(DevPhase));
-    o.item = align(o.op + W.ops.size() * sizeof(DevOp));
-    o.total = align(o.item + W.items.size() * sizeof(PersistItem));
-    return o;
+    return pack_offsets(W, w, W.items.size() * sizeof(PersistItem));
 }
-
-static void work_pack(const Work &W, const RoundOffsets &o, unsigned char *host)
+static void work_pack(const Work &W, const WidePlan &w, const RoundOffsets &o, unsigned char *host)
 {
-    std::memcpy(host + o.pass, W.passes.data(), W.passes.size() * sizeof(DevPass));
-    std::memcpy(host + o.phase, W.phases.data(), W.phases.size() * sizeof(DevPhase));
-    std::memcpy(host + o.op, W.ops.data(), W.ops.size() * sizeof(DevOp));
-    if (!W.items.empty()) std::memcpy(host + o.item, W.items.data(), W.items.size() * sizeof(PersistItem));
+    pack_run(W, w, o, W.items.data(), W.items.size() * sizeof(PersistItem), host);
 }
 
 // Zeroes the queue head, the abort / error words and the completion
 // counters, then launches the persistent kernel over the packed work.
-static qs_status launch_work(const qs_batch *b, cudaStream_t st, const Work &W, const RoundOffsets &o,
-                             const unsigned char *D, uint32_t *sync, double *part, double *sums)
+static qs_status launch_work(const qs_batch *b, cudaStream_t st, const Work &W, const WidePlan &wide,
+                             const RoundOffsets &o, const unsigned char *D, uint32_t *sync, double *part, double *sums)
 {
     const size_t words = sizeof(PersistCtl) / 4 + (size_t)b->count;
     QS_CUDA_TRY(cudaMemsetAsync(sync, 0, words * 4, st));
-    bool any_full = false;
-    for (const PersistItem &w : W.items) any_full = any_full || w.kind == kPersistPassFull;
+    if (!wide.passes.empty())
+        return launch_batch_persistent_wide(st, b->num_sms, b->amps, (const PersistItem *)(D + o.item),
+                                            (int)W.items.size(), (const WidePass *)(D + o.pass),
+                                            (const WideOp *)(D + o.op), D + o.phase, sync + sizeof(PersistCtl) / 4,
+                                            (PersistCtl *)sync, part, sums, any_full(wide));
+    bool full = false;
+    for (const PersistItem &w : W.items) full = full || w.kind == kPersistPassFull;
     return launch_batch_persistent(st, b->num_sms, b->amps, (const PersistItem *)(D + o.item), (int)W.items.size(),
                                    (const DevPass *)(D + o.pass), (const DevPhase *)(D + o.phase),
                                    (const DevOp *)(D + o.op), sync + sizeof(PersistCtl) / 4, (PersistCtl *)sync,
-                                   part, sums, any_full);
+                                   part, sums, full);
 }
 
 // Reads the persistent kernel's error word after its stream has finished.
@@ -306,6 +353,7 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
 {
     Rounds R;
     Work W;
+    WidePlan wide;
     RoundOffsets o;
     std::vector<unsigned char> host;
     if (b->engine == QS_BATCH_ROUNDS) {
@@ -317,9 +365,10 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
     } else {
         build_work(b->n, b->off, plans, full_flags(plans), idx, hl, false, &W);
         *empty = W.passes.empty();
-        o = work_offsets(W);
+        lower_instances(plans, idx, &wide);
+        o = work_offsets(W, wide);
         host.assign(o.total, 0);
-        work_pack(W, o, host.data());
+        work_pack(W, wide, o, host.data());
     }
     if (*empty) return QS_OK;
     void *dev = nullptr, *sync = nullptr;
@@ -334,7 +383,7 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
     e = cudaMemcpy(dev, host.data(), o.total, cudaMemcpyHostToDevice);
     auto run = [&]() -> qs_status {
         if (b->engine == QS_BATCH_ROUNDS) return launch_rounds(b, b->cap_stream, R, o, (const unsigned char *)dev);
-        return launch_work(b, b->cap_stream, W, o, (const unsigned char *)dev, (uint32_t *)sync, nullptr, nullptr);
+        return launch_work(b, b->cap_stream, W, wide, o, (const unsigned char *)dev, (uint32_t *)sync, nullptr, nullptr);
     };
     if (e == cudaSuccess) rc = run();
     if (e == cudaSuccess && !rc) {
@@ -364,7 +413,7 @@ static qs_status batch_autotune(qs_batch *b, const qs_gate *gates, const uint64_
 {
     std::map<int, std::vector<int>> by_n;
     for (int i = 0; i < b->count; ++i) by_n[b->n[i]].push_back(i);
-    if (qs_status s0 = batch_kernel_setup()) return s0;
+    if (qs_status s0 = batch_setup()) return s0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     QS_CUDA_TRY(cudaEventCreate(&e0));
     QS_CUDA_TRY(cudaEventCreate(&e1));
@@ -612,19 +661,21 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
         Work W;
         build_work(b->n, b->off, plans, full_flags(plans), all, hl, true, &W);
         b->round_bytes = W.bytes;
-        const RoundOffsets wo = work_offsets(W);
+        WidePlan wide;
+        lower_instances(plans, all, &wide);
+        const RoundOffsets wo = work_offsets(W, wide);
         std::vector<unsigned char> host(wo.total, 0);
-        work_pack(W, wo, host.data());
+        work_pack(W, wide, wo, host.data());
         batch_release_plan(b);
         QS_CUDA_TRY(cudaMalloc(&b->dev, wo.total));
         QS_CUDA_TRY(cudaMalloc((void **)&b->part, (size_t)std::max(1, W.nslots) * kStatSums * sizeof(double)));
         QS_CUDA_TRY(cudaMalloc((void **)&b->sums, (size_t)C * kStatSums * sizeof(double)));
         QS_CUDA_TRY(cudaMalloc((void **)&b->sync, sizeof(PersistCtl) + 4 * (size_t)C));
         QS_CUDA_TRY(cudaMemcpy(b->dev, host.data(), wo.total, cudaMemcpyHostToDevice));
-        if (qs_status s0 = batch_kernel_setup()) return s0;
+        if (qs_status s0 = batch_setup()) return s0;
         QS_CUDA_TRY(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
         const qs_status rs =
-            launch_work(b, b->cap_stream, W, wo, (const unsigned char *)b->dev, b->sync, b->part, b->sums);
+            launch_work(b, b->cap_stream, W, wide, wo, (const unsigned char *)b->dev, b->sync, b->part, b->sums);
         return batch_end_capture(b, rs);
     }
     Rounds R;
@@ -678,7 +729,7 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
     unsigned char *D = (unsigned char *)b->dev;
 
     // record: reset all states, rounds, statistics
-    if (qs_status s0 = batch_kernel_setup()) return s0;
+    if (qs_status s0 = batch_setup()) return s0;
     QS_CUDA_TRY(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
     qs_status rs = QS_OK;
     k_batch_init<<<std::min(nsi, 16 * b->num_sms), 256, 0, b->cap_stream>>>(
@@ -688,7 +739,8 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
     if (!rs)
         rs = launch_batch_stats(b->cap_stream, b->num_sms, b->amps, (const uint64_t *)(D + o_so),
                                 (const uint64_t *)(D + o_sc), (const float *)(D + o_ss), nsi,
-                                (const int *)(D + o_fi), C, b->part, b->sums);
+                                (const int *)(D + o_fi), C, b->part, b->sums,
+                                R.wide.passes.empty() ? 256 : 128);
     return batch_end_capture(b, rs);
 }
 

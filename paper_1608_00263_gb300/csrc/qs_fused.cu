@@ -1192,13 +1192,6 @@ static bool pass_needs_full(const Plan &plan, const DevPass &hp)
 // Batched form: work item = (instance amplitudes, pass, tile range); the
 // CTA restages the pass for every item.  All items of a launch share one
 // tile size (blockDim.x = 2^(t - RB)).
-struct BatchItem {
-    uint64_t amp_off;       // element offset of the instance's state
-    uint32_t pass;          // index into the batch's pass array
-    uint32_t tile_begin, tile_end;
-    uint32_t pad;
-};
-
 template <typename R, int RB, bool FULL>
 __global__ void __launch_bounds__(kThreadsMax, 2)
 k_batch_pass(typename V2T<R>::T *__restrict__ amps, const BatchItem *__restrict__ items, int nitems,

@@ -1033,7 +1033,6 @@ static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<D
 void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
                 const std::vector<DevOp> &ops, WidePlan *out)
 {
-    *out = WidePlan();
     for (const DevPass &P : passes) {
         WidePass W;
         std::memset(&W, 0, sizeof W);
@@ -1084,9 +1083,16 @@ void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> 
 
 // Persistent ensemble work list (declared with its order and dependency
 // rules in qs_internal.h).
-static uint64_t tiles_per_item(int t)
+static uint64_t tiles_per_item(int t, int item_bits) { return t >= item_bits ? 1 : (1ULL << (item_bits - t)); }
+
+// Amplitudes of a pass item, log2: kPassItemBits, less for a batch so small
+// that a round of its instances would be fewer than ~1000 items (the GPU
+// holds 456 CTAs).  64 instances of 20 qubits: 256 items a round before.
+static int pass_item_bits(uint64_t total)
 {
-    return t >= kPassItemBits ? 1 : (1ULL << (kPassItemBits - t));
+    int lg = 0;
+    while ((total >> lg) > 1) ++lg;
+    return std::min(kPassItemBits, std::max(14, lg - 10));
 }
 
 void build_work(const std::vector<int> &n, const std::vector<uint64_t> &off, const std::vector<Plan> &plans,
@@ -1098,6 +1104,9 @@ void build_work(const std::vector<int> &n, const std::vector<uint64_t> &off, con
     std::vector<int> first_pass(C, 0);
     std::vector<uint32_t> ninit(C, 0), npass(C, 0), nstat(C, 0), before(C, 0);
     int max_passes = 0;
+    uint64_t total = 0;
+    for (int i : idx) total += 1ULL << n[i];
+    const int item_bits = pass_item_bits(total);
     for (int i : idx) {
         first_pass[i] = (int)W->passes.size();
         const int pb = (int)W->phases.size(), ob = (int)W->ops.size();
@@ -1117,7 +1126,7 @@ void build_work(const std::vector<int> &n, const std::vector<uint64_t> &off, con
         ninit[i] = (uint32_t)((N + kWorkChunk - 1) / kWorkChunk);
         nstat[i] = stats ? ninit[i] : 0;
         for (const DevPass &p : plans[i].passes) {
-            const uint64_t nt = 1ULL << (n[i] - p.t), per = tiles_per_item(p.t);
+            const uint64_t nt = 1ULL << (n[i] - p.t), per = tiles_per_item(p.t, item_bits);
             npass[i] += (uint32_t)((nt + per - 1) / per);
         }
     }
@@ -1149,7 +1158,7 @@ void build_work(const std::vector<int> &n, const std::vector<uint64_t> &off, con
             if (r >= (int)plans[i].passes.size()) continue;
             const DevPass &p = plans[i].passes[r];
             const uint32_t kind = full[i][r] ? kPersistPassFull : kPersistPass;
-            const uint64_t nt = 1ULL << (n[i] - p.t), per = tiles_per_item(p.t);
+            const uint64_t nt = 1ULL << (n[i] - p.t), per = tiles_per_item(p.t, item_bits);
             uint32_t cnt = 0;
             for (uint64_t t0 = 0; t0 < nt; t0 += per, ++cnt) {
                 PersistItem w = item(kind, i);

@@ -282,7 +282,8 @@ struct WidePlan {
 // Whether a plan's passes can run the wide form: six register bits, register
 // phases only, tiles of at least 2^kWideMinTile.
 bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases);
-// Lowers a pass list (phase and op indices into the given arrays).
+// Lowers one plan's passes (phase and op indices into the given arrays) and
+// appends them to *out.
 void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
                 const std::vector<DevOp> &ops, WidePlan *out);
 
@@ -322,6 +323,13 @@ struct PersistItem {
     uint32_t nslots;       // stats: the instance's partial slots
     float f0, f1;          // init: fill value, first amplitude; stats: f0 = N
 };
+// Lockstep work item: tiles [tile_begin, tile_end) of one instance's pass.
+struct BatchItem {
+    uint64_t amp_off;       // element offset of the instance's state
+    uint32_t pass;          // index into the batch's pass array
+    uint32_t tile_begin, tile_end;
+    uint32_t pad;
+};
 struct PersistCtl {
     uint32_t next;         // queue head
     uint32_t abort;        // a wait ran out: the remaining items drain without work
@@ -337,7 +345,8 @@ struct PersistCtl {
 // instance's initial-state chunks (kWorkChunk amplitudes), then the passes
 // round-major (pass r of every instance, larger instances first, before
 // pass r + 1 of any; items of 2^kPassItemBits amplitudes = 2^(18 - t)
-// tiles, so a CTA restages a pass once per 32 tiles of 2^13), then, with
+// tiles, so a CTA restages a pass once per 32 tiles of 2^13; fewer in a small
+// batch, so that a round still has items for every CTA), then, with
 // `stats`, the statistics chunks (kWorkChunk amplitudes, as the lockstep
 // engine's; slot order = list order).  Item need = the number of the instance's items in
 // all earlier levels (initial chunks; pass 0; pass 1; ...; statistics), so
@@ -526,6 +535,15 @@ constexpr uint64_t kPersistWaitNs = 2000000000ull;   // per dependency wait
 qs_status launch_batch_persistent(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
                                   const DevPass *passes, const DevPhase *phases, const DevOp *ops,
                                   uint32_t *done, PersistCtl *ctl, double *part, double *sums, bool any_full);
+// The same engines on lowered plans (wide passes): 128-thread CTAs, three per
+// SM, every tile of at least 2^kWideMinTile amplitudes.
+qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, const void *items, int nitems,
+                                  int tile_bits, const WidePass *passes, const WideOp *ops, const uint8_t *codes,
+                                  bool full);
+qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
+                                       const WidePass *passes, const WideOp *ops, const uint8_t *codes,
+                                       uint32_t *done, PersistCtl *ctl, double *part, double *sums, bool any_full);
+qs_status batch_wide_setup();
 // Resident CTAs per SM of the persistent kernel (after batch_kernel_setup).
 int batch_persistent_ctas_per_sm(bool any_full);
 void batch_item_fill(void *dst, uint64_t amp_off, uint32_t pass, uint32_t tb, uint32_t te);
@@ -544,7 +562,7 @@ qs_status batch_mean_probs_run(cudaStream_t st, int num_sms, const void *amps, i
                                double *device_out);
 qs_status launch_batch_stats(cudaStream_t st, int num_sms, const void *amps, const uint64_t *item_off,
                              const uint64_t *item_cnt, const float *item_scale, int nitems,
-                             const int *first_item, int count, double *part, double *out);
+                             const int *first_item, int count, double *part, double *out, int threads);
 void stats_from_sums(const double *h, int n, int kmax, double *norm, double *entropy, double *uniform_ce,
                      double *moments);
 

@@ -259,13 +259,14 @@ qs_status stats_moments(const qs_state *s, int kmax, double *moments, double *en
 // batched statistics: item = (element offset, count) of one instance's state;
 // per-item partials are summed per instance in item order
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kStatThreads)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
 k_batch_stats(const float2 *__restrict__ amps, const uint64_t *__restrict__ item_off,
               const uint64_t *__restrict__ item_cnt, const float *__restrict__ item_scale, int nitems,
               double *__restrict__ part)
 {
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        batch_stats_chunk(amps + item_off[it], item_cnt[it], item_scale[it], part + (size_t)it * kStatAcc);
+        batch_stats_chunk<THREADS>(amps + item_off[it], item_cnt[it], item_scale[it], part + (size_t)it * kStatAcc);
         __syncthreads();
     }
 }
@@ -284,11 +285,12 @@ __global__ void k_batch_stats_sum(const double *__restrict__ part, const int *__
 
 qs_status launch_batch_stats(cudaStream_t st, int num_sms, const void *amps, const uint64_t *item_off,
                              const uint64_t *item_cnt, const float *item_scale, int nitems,
-                             const int *first_item, int count, double *part, double *out)
+                             const int *first_item, int count, double *part, double *out, int threads)
 {
     const int grid = nitems < num_sms * 8 ? nitems : num_sms * 8;
-    k_batch_stats<<<grid, kStatThreads, 0, st>>>((const float2 *)amps, item_off, item_cnt, item_scale, nitems,
-                                                 part);
+    auto kern = threads == 128 ? k_batch_stats<128> : k_batch_stats<kStatThreads>;
+    kern<<<grid, threads == 128 ? 128 : kStatThreads, 0, st>>>((const float2 *)amps, item_off, item_cnt, item_scale,
+                                                               nitems, part);
     QS_LAUNCH_CHECK();
     k_batch_stats_sum<<<(count + 127) / 128, 128, 0, st>>>(part, first_item, count, out);
     QS_LAUNCH_CHECK();

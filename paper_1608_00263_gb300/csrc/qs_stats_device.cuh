@@ -47,13 +47,13 @@ __device__ __forceinline__ double warp_sum_many(const double (&acc)[K])
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
-// Sums acc over the block's kStatThreads threads (recursive halving inside a
+// Sums acc over the block's THREADS threads (recursive halving inside a
 // warp, then the warps' sums in warp order) and stores the K sums at dst
 // (threads < K).
-template <int K>
+template <int K, int THREADS = kStatThreads>
 __device__ __forceinline__ void block_sum_store(double (&acc)[K], double *dst)
 {
-    __shared__ double red[kStatThreads / 32][16];
+    __shared__ double red[THREADS / 32][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if constexpr (K >= 4) {
         const double v = warp_sum_many<K>(acc);
@@ -68,7 +68,7 @@ __device__ __forceinline__ void block_sum_store(double (&acc)[K], double *dst)
     __syncthreads();
     if (threadIdx.x < K) {
         double s = 0;
-        for (int w = 0; w < kStatThreads / 32; ++w) s += red[w][threadIdx.x];
+        for (int w = 0; w < THREADS / 32; ++w) s += red[w][threadIdx.x];
         dst[threadIdx.x] = s;
     }
 }
@@ -95,9 +95,10 @@ __device__ __forceinline__ void stat_terms(T y, T (&c)[kStatAcc])
 // at a time, and sums the terms of 64 amplitudes in FP32 before adding them
 // into FP64 accumulators (terms of y = N p > 4096 formed in FP64); then the
 // block's fixed-order sum goes to dst[0 .. kStatAcc).  The whole block
-// (kStatThreads threads) calls it.  Amplitudes are read through L2
+// (THREADS threads) calls it.  Amplitudes are read through L2
 // (ld.global.cg), so the chunk may have been written earlier in the same
 // launch by another CTA (after an acquire of that CTA's release).
+template <int THREADS = kStatThreads>
 __device__ __forceinline__ void batch_stats_chunk(const float2 *a, uint64_t cnt, float scaleN, double *dst)
 {
     constexpr int kLoads = 8;                      // 16-byte loads in flight per thread
@@ -111,8 +112,6 @@ __device__ __forceinline__ void batch_stats_chunk(const float2 *a, uint64_t cnt,
         float c[kStatAcc];
 #pragma unroll
         for (int k = 0; k < kStatAcc; ++k) c[k] = 0.f;
-        double big[kStatAcc];
-        bool any_big = false;
         for (int j0 = 0; j0 < kGroup; j0 += kLoads) {
             float4 v[kLoads];
 #pragma unroll
@@ -127,27 +126,15 @@ __device__ __forceinline__ void batch_stats_chunk(const float2 *a, uint64_t cnt,
                 for (int h = 0; h < 2; ++h) {
                     const float re = h ? v[k].z : v[k].x, im = h ? v[k].w : v[k].y;
                     const float y = (re * re + im * im) * scaleN;
-                    if (y > 4096.f) {
-                        if (!any_big) {
-#pragma unroll
-                            for (int q = 0; q < kStatAcc; ++q) big[q] = 0;
-                            any_big = true;
-                        }
-                        stat_terms<double>(((double)re * re + (double)im * im) * (double)scaleN, big);
-                    } else {
-                        stat_terms<float>(y, c);
-                    }
+                    if (y > 4096.f) stat_terms<double>(((double)re * re + (double)im * im) * (double)scaleN, acc);
+                    else stat_terms<float>(y, c);
                 }
             }
         }
 #pragma unroll
         for (int k = 0; k < kStatAcc; ++k) acc[k] += (double)c[k];
-        if (any_big) {
-#pragma unroll
-            for (int k = 0; k < kStatAcc; ++k) acc[k] += big[k];
-        }
     }
-    block_sum_store<kStatAcc>(acc, dst);
+    block_sum_store<kStatAcc, THREADS>(acc, dst);
 }
 
 }  // namespace qs

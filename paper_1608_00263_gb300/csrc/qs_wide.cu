@@ -1,5 +1,7 @@
-// qs_wide.cu -- launches of the wide fused pass on one state (complex64, 64
-// amplitudes per thread; qs_wide_device.cuh holds the pass itself).
+// qs_wide.cu -- launches of the wide fused pass (complex64, 64 amplitudes per
+// thread; qs_wide_device.cuh holds the pass itself) on one state and in the
+// batch engines.
+#include "qs_stats_device.cuh"
 #include "qs_wide_device.cuh"
 
 namespace qs {
@@ -51,6 +53,136 @@ qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t
             (float2 *)s->amps, dpass + p, dops, dcodes, ntiles, first && fold ? *fold : none);
         QS_LAUNCH_CHECK();
     }
+    return QS_OK;
+}
+
+// ---- batch engines on wide passes ----
+// Lockstep round: blockDim.x = 2^(t - 6), the launch's tile size.
+template <bool FULL>
+__global__ void __launch_bounds__(kWideThreads, 3)
+k_batch_pass_wide(float2 *__restrict__ amps, const BatchItem *__restrict__ items, int nitems,
+                  const WidePass *__restrict__ passes, const WideOp *__restrict__ ops,
+                  const uint8_t *__restrict__ codes)
+{
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    __shared__ WideSmem S;
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const BatchItem w = items[it];
+        wide_pass_body<FULL, false, false>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
+                                           nullptr, smem_dyn);
+    }
+}
+
+// Persistent engine (PersistItem, see k_batch_persistent): the same queue,
+// dependency waits and completion counts with CTAs of kWideThreads threads,
+// three per SM.  FULL: some item's pass holds parameterised gates; the loop
+// that knows them then runs every pass.
+template <bool FULL>
+__global__ void __launch_bounds__(kWideThreads, 3)
+k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int nitems,
+                        const WidePass *__restrict__ passes, const WideOp *__restrict__ ops,
+                        const uint8_t *__restrict__ codes, uint32_t *done, PersistCtl *ctl, double *part, double *sums,
+                        uint64_t wait_ns)
+{
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    __shared__ WideSmem S;
+    __shared__ int s_item, s_go, s_last;
+    __shared__ PersistItem w;        // the item: no registers held across a pass
+    for (;;) {
+        if (threadIdx.x == 0) {
+            s_item = (int)atomicAdd(&ctl->next, 1u);
+            if (s_item < nitems) w = items[s_item];
+        }
+        __syncthreads();
+        if (s_item >= nitems) break;
+        if (threadIdx.x == 0) {
+            int go = *(volatile const uint32_t *)&ctl->abort == 0;
+            if (go && w.need) {
+                const int r = flag_wait_bounded(done + w.inst, w.need, &ctl->abort, wait_ns);
+                if (r == 1) {
+                    atomicExch(&ctl->err, 1u);
+                    atomicExch(&ctl->abort, 1u);
+                }
+                go = r == 0;
+            }
+            s_go = go;
+        }
+        __syncthreads();
+        if (s_go) {
+            if (w.kind == kPersistInit) {
+                float4 *a = reinterpret_cast<float4 *>(amps + w.amp_off);
+                const float4 u = make_float4(w.f0, 0.f, w.f0, 0.f);
+                for (uint32_t e = threadIdx.x; e < w.lo / 2; e += blockDim.x) a[e] = u;
+                if (threadIdx.x == 0) a[0] = make_float4(w.f1, 0.f, w.f0, 0.f);
+            } else if (w.kind == kPersistStats) {
+                batch_stats_chunk<kWideThreads>(amps + w.amp_off, w.lo, w.f0, part + (size_t)w.pass * kStatAcc);
+            } else {
+                wide_pass_body<FULL, false, true>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, nullptr,
+                                                  smem_dyn);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const uint32_t prev = atomicAdd(done + w.inst, 1u);
+            if (w.kind == kPersistStats) {
+                s_last = prev + 1 == w.total;
+                __threadfence();
+            }
+        }
+        if (w.kind == kPersistStats) {
+            __syncthreads();
+            if (s_last && threadIdx.x < kStatAcc) {
+                double acc = 0;
+                for (uint32_t j = 0; j < w.nslots; ++j) acc += __ldcg(part + (size_t)(w.hi + j) * kStatAcc + threadIdx.x);
+                sums[(size_t)w.inst * kStatAcc + threadIdx.x] = acc;
+            }
+        }
+    }
+}
+
+qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, const void *items, int nitems,
+                                  int tile_bits, const WidePass *passes, const WideOp *ops, const uint8_t *codes,
+                                  bool full)
+{
+    if (tile_bits < kWideMinTile || tile_bits > 13) return set_error(QS_ERR_INVALID_ARG, "batch tile bits %d", tile_bits);
+    auto kern = full ? k_batch_pass_wide<true> : k_batch_pass_wide<false>;
+    const int cap = num_sms * 3;
+    kern<<<nitems < cap ? nitems : cap, 1 << (tile_bits - kWideRegBits), (size_t(1) << tile_bits) * sizeof(float2), st>>>(
+        (float2 *)amps, (const BatchItem *)items, nitems, passes, ops, codes);
+    QS_LAUNCH_CHECK();
+    return QS_OK;
+}
+
+// Resident CTAs per SM of the two persistent variants (occupancy API, set by
+// batch_wide_setup before any launch or capture).
+static int g_wide_per_sm[2] = {3, 3};
+
+qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
+                                       const WidePass *passes, const WideOp *ops, const uint8_t *codes,
+                                       uint32_t *done, PersistCtl *ctl, double *part, double *sums, bool any_full)
+{
+    if (nitems <= 0) return QS_OK;
+    const int cap = num_sms * g_wide_per_sm[any_full ? 1 : 0];
+    auto kern = any_full ? k_batch_persistent_wide<true> : k_batch_persistent_wide<false>;
+    kern<<<nitems < cap ? nitems : cap, kWideThreads, 65536, st>>>((float2 *)amps, items, nitems, passes, ops, codes, done,
+                                                                   ctl, part, sums, kPersistWaitNs);
+    QS_LAUNCH_CHECK();
+    return QS_OK;
+}
+
+qs_status batch_wide_setup()
+{
+    const int dyn = 65536;
+    QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_persistent_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_persistent_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_pass_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_pass_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    QS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_wide_per_sm[0], k_batch_persistent_wide<false>,
+                                                              kWideThreads, dyn));
+    QS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_wide_per_sm[1], k_batch_persistent_wide<true>,
+                                                              kWideThreads, dyn));
+    for (int &v : g_wide_per_sm) v = v < 1 ? 1 : v;
     return QS_OK;
 }
 
