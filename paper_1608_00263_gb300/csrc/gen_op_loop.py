@@ -26,6 +26,19 @@ qs_host.cpp) and a 16-byte record: the selection outside the register set
     W_RX + j   R_X on register bit j: the same shears between x and i y
     W_PH + j   amplitudes with bit j set times a + i b where the selection holds
     W_PP + p   amplitudes with both bits of pair p set times a + i b
+  and, in the loop of the adjoint sweep (ADJ), where register bit 5 selects
+  psi (0) or lambda (1), so that every gate runs on both, the derivative terms
+  of a thread, sums over its amplitudes:
+    W_DX + j   Im <lambda| X_j |psi>          W_DY + j   Im <lambda| Y_j |psi>
+    W_DZ + j   Im <lambda| Z_j |psi>
+    W_DP + j   Im <lambda| psi> over the amplitudes with bit j set where the
+               selection holds, else 0
+    W_DPP + p  the same over the amplitudes with both bits of pair p set
+    W_DW       w = Im <lambda| psi> (kept for the next two)
+    W_DTZ      -w where the selection holds, else w
+    W_DTP      w where the selection holds, else 0
+    W_RED      the last (1 to 4) terms, widened to FP64 and summed over the
+               warp, are added to the warp's partials of their parameters
 
 Every case ends with its own indexed branch to the next op's case (threaded
 code); the code is known when the case starts, and the end of a phase is a
@@ -46,6 +59,11 @@ W_RX = W_RY + RB
 W_PH = W_RX + RB
 W_PP = W_PH + RB
 W_ALL = W_PP + NPAIR         # codes of the full loop
+AB = RB - 1                  # register bits of the adjoint sweep (the last selects the state)
+W_DX = W_ALL
+W_DY, W_DZ, W_DP, W_DPP = W_DX + AB, W_DX + 2 * AB, W_DX + 3 * AB, W_DX + 4 * AB
+W_DW = W_DPP + AB * (AB - 1) // 2
+W_DTZ, W_DTP, W_RED, W_ADJ = W_DW + 1, W_DW + 2, W_DW + 3, W_DW + 4
 
 F_C = "0f3F3504F3"       # 1/sqrt2 rounded to FP32
 F_2C = "0f3FB504F3"      # 2 * that (exact)
@@ -61,15 +79,21 @@ F_0 = "0f00000000"
 # mode, then the F_ bits below), swizzled offset of the thread's copies,
 # source of the next tile's copies, barrier and its threads, then immediate
 # offsets in the staged pass: codes, records (less one), unit table, state
-# offsets of the last phase's register bits, threads' state addresses
+# offsets of the last phase's register bits, threads' state addresses, the
+# partials' address and stride
 (ADDR, TILE, BASE, PHASE, BEGIN, IDX, FR, FI, FLAGS, SWT, NSRC, BARID, NTHR,
- O_CODES, O_RECS, O_UNIT, O_DREG, O_DST) = ("%%%d" % k for k in range(18))
+ O_CODES, O_RECS, O_UNIT, O_DREG, O_DST, O_PART) = ("%%%d" % k for k in range(19))
 F_DIRECT, F_MORE, F_CANON = 4, 8, 16    # store to the state; copy the next tile in; canonical order
 
 
 def pair_index(j, k):
     """Pairs (j, k), j < k < RB, numbered (0,1) (0,2) ... (1,2) (1,3) ..."""
     return j * (RB - 1) - (j * (j - 1)) // 2 + (k - j - 1)
+
+
+def adj_pair_index(j, k):
+    """Pairs of the adjoint sweep's register bits."""
+    return j * (AB - 1) - (j * (j - 1)) // 2 + (k - j - 1)
 
 
 def re(k):
@@ -259,6 +283,112 @@ def case_pp(j, k):
                   else phase_units((1 << (j - 1)) | (1 << (k - 1))))
 
 
+HALF = NU // 2     # adjoint: unit k of psi, unit k + HALF of lambda
+
+
+def push(value):
+    return ["mov.f32 da3, da2;", "mov.f32 da2, da1;", "mov.f32 da1, da0;"] + value
+
+
+def packed_sum(terms):
+    """Two packed sums each of the positive and the negative products (qS, qu
+    and qt, qm): terms (sign, a, b) -> +- a b."""
+    acc = {1: ["qS", "qu"], -1: ["qt", "qm"]}
+    seen, n, out = set(), {1: 0, -1: 0}, []
+    for sign, a, b in terms:
+        r = acc[sign][n[sign] & 1]
+        n[sign] += 1
+        out.append("mul.rn.f32x2 %s, %s, %s;" % (r, a, b) if r not in seen
+                   else "fma.rn.f32x2 %s, %s, %s, %s;" % (r, a, b, r))
+        seen.add(r)
+    for sign, r in ((1, "qS"), (-1, "qt")):
+        other = {"qS": "qu", "qt": "qm"}[r]
+        if other in seen:
+            out.append("add.rn.f32x2 %s, %s, %s;" % (r, r, other))
+    return out + ["mov.b64 {pa, nb}, qS;", "mov.b64 {pb, nc}, qt;", "sub.rn.f32 pa, pa, pb;", "sub.rn.f32 nb, nb, nc;"]
+
+
+def inner(k, sign=1):
+    """Im conj(lambda) psi of unit k."""
+    return [(sign, re(k + HALF), im(k)), (-sign, im(k + HALF), re(k))]
+
+
+def case_dx(j, which):
+    """X (which 0): (l0r p1i - l0i p1r) + (l1r p0i - l1i p0r);
+    Y (which 1): (l1r p0r + l1i p0i) - (l0r p1r + l0i p1i)."""
+    if j == 0:
+        out = []
+        for k in range(HALF):
+            regs = (re(k), im(k), re(k + HALF), im(k + HALF))
+            u = ["mov.b64 {xr0, yr0}, %s;" % regs[0], "mov.b64 {xi0, yi0}, %s;" % regs[1],
+                 "mov.b64 {xr1, yr1}, %s;" % regs[2], "mov.b64 {xi1, yi1}, %s;" % regs[3]]
+            terms = ([("pa", "xr1", "yi0"), ("pb", "xi1", "yr0"), ("nb", "yr1", "xi0"), ("nc", "yi1", "xr0")]
+                     if which == 0 else
+                     [("pa", "yr1", "xr0"), ("nb", "yi1", "xi0"), ("pb", "xr1", "yr0"), ("nc", "xi1", "yi0")])
+            out += u + [("mul.rn.f32 %s, %s, %s;" % t) if k == 0 else "fma.rn.f32 %s, %s, %s, %s;" % (t + (t[0],))
+                        for t in terms]
+        return out + ["add.rn.f32 pa, pa, nb;", "add.rn.f32 pb, pb, nc;"] + push(["sub.rn.f32 da0, pa, pb;"])
+    terms = []
+    b = 1 << (j - 1)
+    for x in range(HALF):
+        if x & b:
+            continue
+        y = x | b
+        if which == 0:
+            terms += [(1, re(x + HALF), im(y)), (-1, im(x + HALF), re(y)), (1, re(y + HALF), im(x)), (-1, im(y + HALF), re(x))]
+        else:
+            terms += [(1, re(y + HALF), re(x)), (-1, re(x + HALF), re(y)), (1, im(y + HALF), im(x)), (-1, im(x + HALF), im(y))]
+    return packed_sum(terms) + push(["add.rn.f32 da0, pa, nb;"])
+
+
+def case_dz(j):
+    if j == 0:
+        return packed_sum([t for k in range(HALF) for t in inner(k)]) + push(["sub.rn.f32 da0, pa, nb;"])
+    b = 1 << (j - 1)
+    return packed_sum([t for k in range(HALF) for t in inner(k, -1 if k & b else 1)]) + push(["add.rn.f32 da0, pa, nb;"])
+
+
+def subset_sum(mask, hi):
+    """w over the units whose bits include mask (hi: their element 1 only)."""
+    out = packed_sum([t for k in range(HALF) if (k & mask) == mask for t in inner(k)])
+    return out + (["mov.f32 pa, nb;"] if hi else ["add.rn.f32 pa, pa, nb;"])
+
+
+def case_dp(j):
+    return subset_sum(0 if j == 0 else 1 << (j - 1), j == 0) + RECORD + SELECTED + push(
+        ["selp.f32 da0, pa, %s, qp;" % F_0])
+
+
+def case_dpp(j, k):
+    return subset_sum((0 if j == 0 else 1 << (j - 1)) | 1 << (k - 1), j == 0) + push(["mov.f32 da0, pa;"])
+
+
+def case_red():
+    out = RECORD + ["add.u32 qa, qa, %s;" % O_RECS, "ld.shared.v2.u32 {a0, a1}, [qa+8];", "mov.u32 b0, %laneid;"]
+    out += ["cvt.f64.f32 e%d, da%d;" % (k, k) for k in range(4)]
+
+    def swap(dst, a, o):                       # dst = a of lane ^ o
+        return ["mov.b64 {b2, b3}, %s;" % a, "shfl.sync.bfly.b32 b2, b2, %d, 31, -1;" % o,
+                "shfl.sync.bfly.b32 b3, b3, %d, 31, -1;" % o, "mov.b64 %s, {b2, b3};" % dst]
+    # recursive halving: lane bit 1 keeps terms 2 and 3, lane bit 0 the odd one
+    out += ["and.b32 b1, b0, 2;", "setp.ne.u32 qp, b1, 0;"]
+    for k in (0, 1):
+        out += ["selp.f64 e4, e%d, e%d, qp;" % (k, k + 2), "selp.f64 e%d, e%d, e%d, qp;" % (k, k + 2, k)]
+        out += swap("e4", "e4", 2) + ["add.rn.f64 e%d, e%d, e4;" % (k, k)]
+    out += ["and.b32 b1, b0, 1;", "setp.ne.u32 qp, b1, 0;",
+            "selp.f64 e4, e0, e1, qp;", "selp.f64 e0, e1, e0, qp;"]
+    out += swap("e4", "e4", 1) + ["add.rn.f64 e0, e0, e4;"]
+    for o in (4, 8, 16):
+        out += swap("e4", "e0", o) + ["add.rn.f64 e0, e0, e4;"]
+    # lane i < count holds term i, the (count - 1 - i)-th parameter from a0
+    out += ["sub.u32 b1, a1, b0;", "add.u32 b1, b1, a0;", "sub.u32 b1, b1, 1;",
+            "ld.shared.v2.u64 {qt, qm}, [%s+%s];" % (BASE, O_PART),
+            "cvt.u64.u32 qS, b1;", "mul.lo.u64 qS, qS, qm;", "add.u64 qt, qt, qS;",
+            "mov.u32 b1, %tid.x;", "shr.u32 b1, b1, 5;", "mul.wide.u32 qS, b1, 8;", "add.u64 qt, qt, qS;",
+            "setp.lt.u32 qp, b0, a1;", "@qp red.global.add.f64 [qt], e0;"]
+    return out
+
+
 GROUP = 8     # independent chains interleaved
 
 
@@ -274,9 +404,10 @@ def interleave(chains):
     return out
 
 
-def cases(full):
-    body = [None] * (W_ALL if full else W_CT)
-    for j in range(RB):
+def cases(full, adj=False):
+    """Case bodies by code; None: a code this loop does not hold."""
+    body = [None] * (W_ADJ if adj else W_ALL if full else W_CT)
+    for j in range(AB if adj else RB):
         body[W_H + j] = case_h(j)
         body[W_XH + j] = case_xh(j)
         body[W_YH + j] = case_yh(j)
@@ -286,11 +417,23 @@ def cases(full):
             body[W_RY + j] = case_ry(j)
             body[W_RX + j] = case_rx(j)
             body[W_PH + j] = case_ph(j)
-        for k in range(j + 1, RB):
+        if adj:
+            body[W_DX + j] = case_dx(j, 0)
+            body[W_DY + j] = case_dx(j, 1)
+            body[W_DZ + j] = case_dz(j)
+            body[W_DP + j] = case_dp(j)
+            for k in range(j + 1, AB):
+                body[W_DPP + adj_pair_index(j, k)] = case_dpp(j, k)
+        for k in range(j + 1, AB if adj else RB):
             body[W_CZ + pair_index(j, k)] = case_cz(j, k)
             if full:
                 body[W_PP + pair_index(j, k)] = case_pp(j, k)
-    assert all(b is not None for b in body)
+    if adj:
+        body[W_DW] = subset_sum(0, False) + ["mov.f32 dw, pa;"]
+        body[W_DTZ] = RECORD + SELECTED + ["neg.f32 pb, dw;"] + push(["selp.f32 da0, pb, dw, qp;"])
+        body[W_DTP] = RECORD + SELECTED + push(["selp.f32 da0, dw, %s, qp;" % F_0])
+        body[W_RED] = case_red()
+    assert adj or all(b is not None for b in body)
     return body
 
 
@@ -400,14 +543,14 @@ def direct_store(L):
     return out
 
 
-def asm_text(prefix, full):
+def asm_text(prefix, full, adj=False):
     """PTX of one phase: loads the thread's units, runs the ops from `begin` to the
     end code, applies the factor, stores the units to the tile or (direct) to the
     state.  The units live in registers of the block's own, so nothing has to
     be moved at its boundary."""
     def L(name):
         return "%s_%s" % (prefix, name)
-    body = cases(full)
+    body = cases(full, adj)
     n = len(body)
     lines = ["{",
              ".reg .pred qp;",
@@ -415,7 +558,7 @@ def asm_text(prefix, full):
              ".reg .b64 qm, qt, qS, qv, qu, qM1, qP2, d<%d>;" % RB,
              ".reg .f32 xr, xi, yr, yi, pa, pb, nb, nc;",
              ".reg .f32 " + ", ".join(t + str(n) for n in range(TEMPS) for t in ("xr", "xi", "yr", "yi", "na", "xx")) + ";",
-             ".reg .b64 u<%d>;" % NS,
+             ".reg .b64 u<%d>;" % NS] + ([".reg .f32 da0, da1, da2, da3, dw;", ".reg .f64 e<5>;"] if adj else []) + [
              "add.u32 qh, %s, %s;" % (BASE, PHASE)]
     lines += slots(False)
     lines += next_tile(L)
@@ -425,12 +568,14 @@ def asm_text(prefix, full):
               "add.u32 qa, %s, qo;" % BASE,
               "ld.shared.u8 qc, [qa+%s];" % O_CODES,
               "ld.shared.u8 qn, [qa+%s+1];" % O_CODES,
-              L("TBL") + ": .branchtargets " + ", ".join([L("C%d" % c) for c in range(n)] + [L("DONE")]) + ";",
+              L("TBL") + ": .branchtargets " + ", ".join([L("C%d" % c if body[c] else "DONE") for c in range(n)]
+                                                              + [L("DONE")]) + ";",
               "min.u32 qc, qc, %d;" % n]
     lines += branch(L)
     for c, b in enumerate(body):
-        lines.append(L("C%d" % c) + ":")
-        lines += head(n) + b + branch(L)
+        if b:
+            lines.append(L("C%d" % c) + ":")
+            lines += head(n) + b + branch(L)
     lines.append(L("DONE") + ":")
     lines += factor(L)
     lines.append(L("STORE") + ":")
@@ -446,13 +591,13 @@ def emit():
            "//",
            "// The op loop of the wide fused pass (complex64, %d slots, %d register" % (NS, RB),
            "// bits) as inline PTX: one byte-code load and one indexed branch per op.",
-           "// OpLoop<false>: the Clifford+T gates; OpLoop<true>: also the",
-           "// parameterised gates.",
+           "// OpLoop<0>: the Clifford+T gates; OpLoop<1>: also the parameterised",
+           "// gates; OpLoop<2>: the adjoint sweep.",
            "",
-           "template <bool FULL> struct OpLoop;"]
-    for full, prefix in ((False, "QSWCT"), (True, "QSWFL")):
-        out.append("template <> struct OpLoop<%s> {" % ("true" if full else "false"))
-        out.append("    template <int O_CODES, int O_RECS, int O_UNIT, int O_DREG, int O_DST>")
+           "template <int KIND> struct OpLoop;"]
+    for kind, prefix in enumerate(("QSWCT", "QSWFL", "QSWAD")):
+        out.append("template <> struct OpLoop<%d> {" % kind)
+        out.append("    template <int O_CODES, int O_RECS, int O_UNIT, int O_DREG, int O_DST, int O_PART>")
         out.append("    static __device__ __forceinline__ void run(uint32_t addr, uint32_t tile, uint32_t base,")
         out.append("                                               uint32_t phase, int ob,")
         out.append("                                               unsigned long long idx, float fr, float fi,")
@@ -460,11 +605,11 @@ def emit():
         out.append("                                               uint32_t barid, uint32_t nthr)")
         out.append("    {")
         out.append("        asm volatile(")
-        for line in asm_text(prefix, full):
-            out.append('            "%s\\n"' % line.replace("%tid", "%%tid"))
+        for line in asm_text(prefix, kind > 0, kind == 2):
+            out.append('            "%s\\n"' % line.replace("%tid", "%%tid").replace("%laneid", "%%laneid"))
         out.append('            : : "r"(addr), "r"(tile), "r"(base), "r"(phase), "r"(ob), "l"(idx), "f"(fr), "f"(fi),')
         out.append('                "r"(flags), "r"(swt), "l"(nsrc), "r"(barid), "r"(nthr), "n"(O_CODES), "n"(O_RECS), "n"(O_UNIT),')
-        out.append('                "n"(O_DREG), "n"(O_DST)')
+        out.append('                "n"(O_DREG), "n"(O_DST), "n"(O_PART)')
         out.append('            : "memory");')
         out.append("    }")
         out.append("};")

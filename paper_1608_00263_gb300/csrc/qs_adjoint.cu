@@ -28,9 +28,6 @@ template <typename R> struct AdjMat {
     R m[8];   // G^dagger, u00 u01 u10 u11 as (re, im)
 };
 
-// derivative kinds
-enum { D_NONE = 0, D_X = 1, D_Y = 2, D_Z = 3, D_P11 = 4 };
-
 // lambda = -sum_j psi(x_j) / (m p(x_j)) |x_j>; lambda is zero on entry.
 template <typename R>
 __global__ void k_adj_seed(const typename V2T<R>::T *__restrict__ psi, typename V2T<R>::T *__restrict__ lam,
@@ -429,8 +426,93 @@ static qs_status adjoint_t(qs_state *s, const qs_gate *g, size_t ng, const uint6
     return st;
 }
 
+// complex64 states of at least kWideMinTile - 1 qubits: the sweep as wide
+// passes over psi and lambda (build_adjoint).  A pass undoes ~50 gates in
+// registers where a tile group undid ~7 in shared memory with a barrier
+// after each: 24 qubits, depth 30: 8 passes instead of 56 group launches.
+static qs_status adjoint_wide(qs_state *s, const qs_gate *g, size_t ng, const uint64_t *dev_x, uint64_t m, double *grad)
+{
+    AdjointSlot &A = s->adjoint;
+    const bool same = A.dev && A.gates.size() == ng && std::memcmp(A.gates.data(), g, ng * sizeof(qs_gate)) == 0;
+    if (!same) {
+        A.gates.clear();
+        if (qs_status st = build_adjoint(s->n, g, ng, &A.plan, &A.param_of_slot)) return st;
+        std::vector<size_t> gate_of_param;
+        for (size_t k = 0; k < ng; ++k)
+            if (is_param(g[k].kind)) gate_of_param.push_back(k);
+        std::vector<double> scale;
+        for (int p : A.param_of_slot) scale.push_back(g[gate_of_param[(size_t)p]].kind == QS_CPHASE ? -2.0 : 1.0);
+        const size_t b_pass = A.plan.passes.size() * sizeof(WidePass), b_ops = A.plan.ops.size() * sizeof(WideOp);
+        const size_t o_scale = (b_pass + b_ops + A.plan.codes.size() + 15) / 16 * 16;
+        const size_t total = o_scale + scale.size() * sizeof(double) + 16;
+        std::vector<unsigned char> host(total, 0);
+        std::memcpy(host.data(), A.plan.passes.data(), b_pass);
+        std::memcpy(host.data() + b_pass, A.plan.ops.data(), b_ops);
+        std::memcpy(host.data() + b_pass + b_ops, A.plan.codes.data(), A.plan.codes.size());
+        if (!scale.empty()) std::memcpy(host.data() + o_scale, scale.data(), scale.size() * sizeof(double));
+        if (A.bytes < total) {
+            if (A.dev) cudaFree(A.dev);
+            A.dev = nullptr;
+            A.bytes = 0;
+            if (cudaMalloc(&A.dev, total + total / 2) != cudaSuccess) {
+                cudaGetLastError();
+                A.dev = nullptr;
+                return set_error(QS_ERR_OOM, "adjoint plan of %zu bytes", total);
+            }
+            A.bytes = total + total / 2;
+        }
+        QS_CUDA_TRY(cudaMemcpyAsync(A.dev, host.data(), total, cudaMemcpyHostToDevice, s->stream));
+        QS_CUDA_TRY(cudaStreamSynchronize(s->stream));
+        A.gates.assign(g, g + ng);
+    }
+    const size_t nparam = A.param_of_slot.size(), parts = (size_t)adjoint_wide_partials(s);
+    const size_t o_scale = (A.plan.passes.size() * sizeof(WidePass) + A.plan.ops.size() * sizeof(WideOp) +
+                            A.plan.codes.size() + 15) / 16 * 16;
+    const uint64_t N = 1ULL << s->n;
+    const size_t b_part = nparam * parts * sizeof(double), b_out = (nparam ? nparam : 1) * sizeof(double);
+    float2 *lam = nullptr;
+    unsigned char *work = nullptr;
+    QS_CUDA_TRY(cudaMallocAsync((void **)&lam, N * sizeof(float2), s->stream));
+    qs_status st = QS_OK;
+    cudaError_t e = cudaMallocAsync((void **)&work, b_part + b_out, s->stream);
+    if (e != cudaSuccess) {
+        st = set_error(QS_ERR_OOM, "adjoint workspace: %s", cudaGetErrorString(e));
+    } else {
+        double *part = (double *)work, *out = (double *)(work + b_part);
+        e = cudaMemsetAsync(lam, 0, N * sizeof(float2), s->stream);
+        if (e == cudaSuccess && b_part) e = cudaMemsetAsync(part, 0, b_part, s->stream);
+        if (e == cudaSuccess) {
+            k_adj_seed<float><<<grid_for(m, 256, s->num_sms, 4), 256, 0, s->stream>>>((const float2 *)s->amps, lam, dev_x, m);
+            st = launch_adjoint_wide(s, lam, A.plan, A.dev, part);
+            if (!st && nparam)
+                k_adj_sums<<<grid_for(nparam * 32, 128, s->num_sms, 4), 128, 0, s->stream>>>(
+                    part, (int)parts, (int)nparam, (const double *)((const unsigned char *)A.dev + o_scale), out);
+            e = cudaGetLastError();
+            std::vector<double> h(nparam);
+            if (!st && e == cudaSuccess && nparam)
+                e = cudaMemcpyAsync(h.data(), out, nparam * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
+            if (!st && e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+            if (!st && e == cudaSuccess) {
+                std::vector<size_t> gate_of_param;
+                for (size_t k = 0; k < ng; ++k) {
+                    grad[k] = 0.0;
+                    if (is_param(g[k].kind)) gate_of_param.push_back(k);
+                }
+                for (size_t j = 0; j < nparam; ++j) grad[gate_of_param[(size_t)A.param_of_slot[j]]] = h[j];
+            }
+        }
+        if (!st && e != cudaSuccess) st = set_error(QS_ERR_CUDA, "adjoint sweep: %s", cudaGetErrorString(e));
+    }
+    if (lam) cudaFreeAsync(lam, s->stream);
+    if (work) cudaFreeAsync(work, s->stream);
+    cudaStreamSynchronize(s->stream);
+    return st;
+}
+
 qs_status adjoint_run(qs_state *s, const qs_gate *g, size_t ng, const uint64_t *dev_x, uint64_t m, double *grad)
 {
+    if (s->dt == QS_C64 && s->n + 1 >= kWideMinTile && s->n < kMaxQubits && ng)
+        return adjoint_wide(s, g, ng, dev_x, m, grad);
     return s->dt == QS_C64 ? adjoint_t<float>(s, g, ng, dev_x, m, grad)
                            : adjoint_t<double>(s, g, ng, dev_x, m, grad);
 }

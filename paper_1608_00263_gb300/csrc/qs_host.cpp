@@ -449,7 +449,11 @@ struct PGate {
     int q0, q1;
     bool two, diag;
     double theta;
+    int deriv = D_NONE;     // adjoint sweep: derivative term taken with the gate
+    int param = 0;          // ... of this parameter
 };
+constexpr int kPhase1 = 100;    // diag(1, e^{i theta}) on q0 (adjoint sweep: T undone)
+constexpr int kSign1 = 101;     // diag(1, -1) on q0
 
 // Returns the indices (in order) of gates applicable with the local set
 // `local` (bitmask over qubits), among gates not yet done.  A gate left
@@ -586,14 +590,15 @@ struct PhaseSet {
     std::vector<int> gates;
 };
 
-// Ops a gate becomes in a plan: 5 for RX, 3 for RY, else 1.
-static int gate_ops(const PGate &x) { return x.kind == QS_RX ? 5 : x.kind == QS_RY ? 3 : 1; }
+// Ops a gate becomes in a plan: 5 for RX, 3 for RY, else 1.  (With a
+// derivative term a lowered pass holds up to 2 1/4 ops per gate.)
+static int gate_ops(const PGate &x) { return x.kind == QS_RX ? 5 : x.kind == QS_RY || x.deriv ? 3 : 1; }
 
 // Greedy phases for the gates of `cand` not yet done (marked done as they
-// are placed), qubit 0 always among the r register qubits.  Returns false
+// are placed), the qubits `must` always among the r register qubits.  Returns false
 // when they do not fit `max_phases`.
 static bool greedy_phases(const std::vector<PGate> &g, const std::vector<int> &cand, std::vector<char> *done, int n,
-                          uint64_t local, int r, int max_phases, std::vector<PhaseSet> *out)
+                          uint64_t local, uint64_t must, int r, int max_phases, std::vector<PhaseSet> *out)
 {
     size_t left = 0;
     for (int i : cand) left += !(*done)[i];
@@ -601,7 +606,7 @@ static bool greedy_phases(const std::vector<PGate> &g, const std::vector<int> &c
         if ((int)out->size() >= max_phases) return false;
         PhaseSet p;
         int cnt;
-        p.reg = choose_local(g, cand, *done, n, 1, local, r - 1);
+        p.reg = choose_local(g, cand, *done, n, must, local, r - __builtin_popcountll(must));
         collect(g, cand, *done, p.reg, &p.gates, &cnt);
         if (cnt == 0) return false;
         for (int i : p.gates) (*done)[i] = 1;
@@ -619,19 +624,19 @@ static bool greedy_phases(const std::vector<PGate> &g, const std::vector<int> &c
 // all others (the blocking rule of collect is symmetric in time).  The rest
 // is greedy as before.  False when that takes more phases than `limit`.
 static bool direct_phases(const std::vector<PGate> &g, const std::vector<int> &pass_gates, int n, uint64_t local,
-                          int r, int limit, std::vector<PhaseSet> *out)
+                          uint64_t must, int r, int limit, std::vector<PhaseSet> *out)
 {
     std::vector<char> done(g.size(), 1);
     for (int i : pass_gates) done[i] = 0;
     const std::vector<int> back(pass_gates.rbegin(), pass_gates.rend());
     PhaseSet last;
     int cnt;
-    last.reg = choose_local(g, back, done, n, 1, local & ~0x1Eull, r - 1);
+    last.reg = choose_local(g, back, done, n, must, local & ~0x1Eull, r - __builtin_popcountll(must));
     collect(g, back, done, last.reg, &last.gates, &cnt);
     std::reverse(last.gates.begin(), last.gates.end());
     for (int i : last.gates) done[i] = 1;
     out->clear();
-    if (!greedy_phases(g, pass_gates, &done, n, local, r, limit - 1, out)) return false;
+    if (!greedy_phases(g, pass_gates, &done, n, local, must, r, limit - 1, out)) return false;
     out->push_back(std::move(last));
     return true;
 }
@@ -951,9 +956,13 @@ bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &
 // of R_Y and R_X back to one op each, diagonal ops without a register bit to
 // the tail.
 static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<DevOp> &ops, WidePlan *out,
-                        std::vector<WideOp> *tail, std::vector<uint8_t> *tail_codes, bool *full)
+                        std::vector<WideOp> *tail, std::vector<uint8_t> *tail_codes, bool *full,
+                        std::vector<int> *slots)
 {
     const size_t begin = out->codes.size();
+    // adjoint sweep: derivative terms not yet summed, and whether w is formed
+    int pending = 0;
+    bool have_w = false;
     auto selection = [&](uint64_t qmask, WideOp *w) {
         for (int b = 0; b < P.t; ++b)
             if ((qmask >> P.L[b]) & 1) w->sel_tile |= 1u << b;
@@ -963,6 +972,15 @@ static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<D
     auto put = [&](int code, const WideOp &w) {
         out->codes.push_back((uint8_t)code);
         out->ops.push_back(w);
+    };
+    auto reduce = [&]() {
+        if (!pending) return;
+        WideOp w{0, 0, 0.f, 0.f};
+        const uint32_t first = (uint32_t)slots->size() - (uint32_t)pending, count = (uint32_t)pending;
+        std::memcpy(&w.p0, &first, 4);
+        std::memcpy(&w.p1, &count, 4);
+        put(W_RED, w);
+        pending = 0;
     };
     for (int o = H.op_begin; o < H.op_end; ++o) {
         const DevOp &d = ops[o];
@@ -975,6 +993,22 @@ static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<D
                 ++bits;
             }
         switch (d.type) {
+        case OP_DERIV: {
+            selection(d.qmask, &w);
+            if (d.pad0 == D_X) put(W_DX + d.a, w);
+            else if (d.pad0 == D_Y) put(W_DY + d.a, w);
+            else if (bits == 0) {
+                if (!have_w) put(W_DW, WideOp{0, 0, 1.f, 0.f});
+                have_w = true;
+                put(d.pad0 == D_Z ? W_DTZ : W_DTP, w);
+            } else if (d.pad0 == D_Z) put(W_DZ + hi, w);
+            else if (bits == 1) put(W_DP + hi, w);
+            else put(W_DPP + wide_adj_pair_index(lo, hi), w);
+            slots->push_back((int)d.m[0]);
+            if (++pending == 4) reduce();
+            *full = true;
+            break;
+        }
         case OP_H: put(W_H + d.a, w); break;
         case OP_XH: put(W_XH + d.a, w); break;
         case OP_YH: put(W_YH + d.a, w); break;
@@ -1028,10 +1062,11 @@ static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<D
         default: break;
         }
     }
+    reduce();
 }
 
 void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
-                const std::vector<DevOp> &ops, WidePlan *out)
+                const std::vector<DevOp> &ops, WidePlan *out, std::vector<int> *slots)
 {
     for (const DevPass &P : passes) {
         WidePass W;
@@ -1057,7 +1092,7 @@ void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> 
             V.op_begin = (int16_t)(out->ops.size() - W.op_begin);
             std::vector<WideOp> tail;
             std::vector<uint8_t> tail_codes;
-            lower_phase(P, H, ops, out, &tail, &tail_codes, &full);
+            lower_phase(P, H, ops, out, &tail, &tail_codes, &full, slots);
             out->ops.push_back(WideOp{0, 0, 1.f, 0.f});
             out->codes.push_back(W_END);
             V.tail_begin = (int16_t)(out->ops.size() - W.op_begin);
@@ -1297,22 +1332,14 @@ static void hoist_diagonals_to_last_phase(Plan *P, const DevPass &dp)
     }
 }
 
-qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *out)
+static qs_status plan_gates(const PlanParams &pp, const std::vector<PGate> &g, Plan *out)
 {
     const int n = pp.n;
+    const size_t ng = g.size();
     if (pp.t < 1 || pp.t > kMaxTileBits || pp.t > n || pp.r < 1 || pp.r > kMaxRegBits ||
         pp.r > pp.t || pp.c < 0 || pp.c > pp.t)
         return set_error(QS_ERR_INVALID_ARG, "bad plan parameters t=%d r=%d c=%d n=%d",
                          pp.t, pp.r, pp.c, n);
-    std::vector<PGate> g(ng);
-    for (size_t i = 0; i < ng; ++i) {
-        g[i].kind = gin[i].kind;
-        g[i].q0 = gin[i].q0;
-        g[i].q1 = gin[i].q1;
-        g[i].two = gate_is_two_qubit(gin[i].kind);
-        g[i].diag = gate_is_diagonal(gin[i].kind);
-        g[i].theta = gin[i].theta;
-    }
     Plan &P = *out;
     P = Plan();
     P.n = n; P.t = pp.t; P.r = pp.r; P.c = pp.c; P.mode = pp.mode;
@@ -1323,11 +1350,15 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
     std::vector<int> all(ng);
     for (size_t i = 0; i < ng; ++i) all[i] = (int)i;
     size_t remaining = ng;
-    const uint64_t allq = (n == 64) ? ~0ULL : ((1ULL << n) - 1);
-    const uint64_t low = (pp.c >= 64) ? ~0ULL : ((1ULL << pp.c) - 1);
+    // qubits of every tile: the lowest, and those of pp.must (which no gate
+    // acts on); register qubits of every wide phase: qubit 0 and pp.must
+    const uint64_t allq = ((n == 64) ? ~0ULL : ((1ULL << n) - 1)) & ~pp.must;
+    const uint64_t low = ((pp.c >= 64) ? ~0ULL : ((1ULL << pp.c) - 1)) | pp.must;
+    const uint64_t must = 1 | pp.must;
     std::vector<int> pass_gates, phase_gates;
     while (remaining) {
-        uint64_t local = choose_tile(g, all, done, n, low & allq, allq & ~low, pp.t - pp.c, allq, pp.look_steps,
+        uint64_t local = choose_tile(g, all, done, n, low & (allq | pp.must), allq & ~low,
+                                     pp.t - pp.c - popcount64(pp.must), allq, pp.look_steps,
                                      pp.look_top);
         int cnt;
         collect(g, all, done, local, &pass_gates, &cnt, allq);
@@ -1364,9 +1395,9 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
             int ops = 0;
             for (int i : pass_gates) ops += gate_ops(g[i]);
             std::vector<char> pd(pdone);
-            if (ops <= max_ops && greedy_phases(g, pass_gates, &pd, n, local, dp.r, kMaxPhasesPerPass, &ahead)) {
+            if (ops <= max_ops && greedy_phases(g, pass_gates, &pd, n, local, must, dp.r, kMaxPhasesPerPass, &ahead)) {
                 std::vector<PhaseSet> alt;
-                if (direct_phases(g, pass_gates, n, local, dp.r, (int)ahead.size(), &alt)) {
+                if (direct_phases(g, pass_gates, n, local, must, dp.r, (int)ahead.size(), &alt)) {
                     ahead.swap(alt);
                     direct = true;
                 }
@@ -1384,7 +1415,7 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
                 cnt = (int)phase_gates.size();
                 direct_last = direct && dp.nphases + 1 == (int)ahead.size();
             } else {
-                reg = pp.pack0 ? choose_local(g, pass_gates, pdone, n, 1, local, dp.r - 1)
+                reg = pp.pack0 ? choose_local(g, pass_gates, pdone, n, must, local, dp.r - popcount64(must))
                                : choose_local(g, pass_gates, pdone, n, 0, local, dp.r);
                 collect(g, pass_gates, pdone, reg, &phase_gates, &cnt);
             }
@@ -1425,7 +1456,7 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
                 size_t keep = 0;
                 int ops_needed = 0;
                 for (int gi : phase_gates) {
-                    const int k = g[gi].kind == QS_RX ? 5 : g[gi].kind == QS_RY ? 3 : 1;
+                    const int k = gate_ops(g[gi]);
                     if (pass_ops + ops_needed + k > max_ops) break;
                     ops_needed += k;
                     ++keep;
@@ -1468,6 +1499,22 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
                 const PGate &x = g[gi];
                 DevOp op;
                 std::memset(&op, 0, sizeof op);
+                if (x.deriv) {
+                    // the derivative term commutes with its own gate
+                    DevOp d = op;
+                    d.type = OP_DERIV;
+                    d.pad0 = (uint8_t)x.deriv;
+                    d.m[0] = x.param;
+                    if (!x.diag) {
+                        d.a = (uint8_t)reg_bit_of[x.q0];
+                    } else {
+                        for (int q : {x.q0, x.two ? x.q1 : x.q0}) {
+                            if (reg_bit_of[q] >= 0) d.rmask |= (uint8_t)(1u << reg_bit_of[q]);
+                            else d.qmask |= 1ULL << q;
+                        }
+                    }
+                    P.ops.push_back(d);
+                }
                 if (!x.diag) {
                     op.a = (uint8_t)reg_bit_of[x.q0];
                     switch (x.kind) {
@@ -1507,7 +1554,7 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
                         if (reg_bit_of[q] >= 0) op.rmask |= (uint8_t)(1u << reg_bit_of[q]);
                         else op.qmask |= 1ULL << q;
                     }
-                    if (x.kind == QS_CZ) {
+                    if (x.kind == QS_CZ || x.kind == kSign1) {
                         op.type = OP_NEG;
                     } else {
                         op.type = OP_PHASE;
@@ -1536,7 +1583,7 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
             // set only scale a thread's slots by a constant: they commute
             // with every other op of the phase and go to its end
             std::stable_partition(P.ops.begin() + ph.op_begin, P.ops.end(), [](const DevOp &o) {
-                return !((o.type == OP_PHASE || o.type == OP_NEG) && o.rmask == 0);
+                return !((o.type == OP_PHASE || o.type == OP_NEG || (o.type == OP_DERIV && o.pad0 >= D_Z)) && o.rmask == 0);
             });
             ph.op_end = (int)P.ops.size();
             P.phases.push_back(ph);
@@ -1556,6 +1603,75 @@ qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *
         dp.gscale_im = gim * sc;
         P.passes.push_back(dp);
     }
+    return QS_OK;
+}
+
+qs_status build_plan(const PlanParams &pp, const qs_gate *gin, size_t ng, Plan *out)
+{
+    std::vector<PGate> g(ng);
+    for (size_t i = 0; i < ng; ++i) {
+        g[i].kind = gin[i].kind;
+        g[i].q0 = gin[i].q0;
+        g[i].q1 = gin[i].q1;
+        g[i].two = gate_is_two_qubit(gin[i].kind);
+        g[i].diag = gate_is_diagonal(gin[i].kind);
+        g[i].theta = gin[i].theta;
+    }
+    return plan_gates(pp, g, out);
+}
+
+// The reverse sweep as a plan (declared in qs_internal.h): every gate undone,
+// last first, on n + 1 qubits, qubit n selecting psi or lambda.
+qs_status build_adjoint(int n, const qs_gate *gin, size_t ng, WidePlan *out, std::vector<int> *param_of_slot)
+{
+    std::vector<PGate> g;
+    int params = 0;
+    for (size_t i = 0; i < ng; ++i)
+        params += gin[i].kind == QS_RX || gin[i].kind == QS_RY || gin[i].kind == QS_RZ || gin[i].kind == QS_CPHASE;
+    for (size_t i = ng; i-- > 0;) {
+        const qs_gate &x = gin[i];
+        PGate p;
+        p.kind = x.kind;
+        p.q0 = x.q0;
+        p.q1 = x.q1;
+        p.two = gate_is_two_qubit(x.kind);
+        p.diag = gate_is_diagonal(x.kind);
+        p.theta = -x.theta;
+        switch (x.kind) {
+        case QS_H: {
+            // R_Y(pi/2) diag(1, -1): no factor is deferred, which would
+            // scale the derivative terms of the gates after it
+            PGate z = p;
+            z.kind = kSign1;
+            z.diag = true;
+            g.push_back(z);
+            p.kind = QS_RY;
+            p.theta = M_PI / 2;
+            break;
+        }
+        case QS_X_HALF: p.kind = QS_RX; p.theta = -M_PI / 2; break;
+        case QS_Y_HALF: p.kind = QS_RY; p.theta = -M_PI / 2; break;
+        case QS_T: p.kind = kPhase1; p.theta = -M_PI / 4; break;
+        case QS_RX: p.deriv = D_X; break;
+        case QS_RY: p.deriv = D_Y; break;
+        case QS_RZ: p.deriv = D_Z; break;
+        case QS_CPHASE: p.deriv = D_P11; break;
+        default: break;
+        }
+        if (p.deriv) p.param = --params;
+        g.push_back(p);
+    }
+    PlanParams pp = default_plan_params(n + 1, QS_C64, nullptr);
+    pp.r = kWideRegBits;
+    pp.pack0 = 1;
+    pp.must = 1ULL << n;
+    pp.hoist_diagonals = 0;
+    Plan plan;
+    if (qs_status st = plan_gates(pp, g, &plan)) return st;
+    *out = WidePlan();
+    param_of_slot->clear();
+    if (!wide_plan(plan.passes, plan.phases)) return set_error(QS_ERR_INVALID_ARG, "adjoint plan is not wide");
+    lower_wide(plan.passes, plan.phases, plan.ops, out, param_of_slot);
     return QS_OK;
 }
 

@@ -88,7 +88,12 @@ enum OpType : uint8_t {
                     // block matrix in `a`
     OP_SHX = 7,     // shear x += m[0] * y on register bit `a` (x: bit 0, y: bit 1)
     OP_SHY = 8,     // shear y += m[0] * x on register bit `a`
+    OP_DERIV = 9,   // adjoint sweep: derivative term of kind pad0 (D_*) for
+                    // parameter m[0]; X, Y on register bit `a`, Z and P11
+                    // selected like a phase op
 };
+// Derivative terms of the adjoint sweep: Im <lambda| X, Y, Z, Pi_11 |psi>.
+enum { D_NONE = 0, D_X = 1, D_Y = 2, D_Z = 3, D_P11 = 4 };
 
 struct DevOp {          // 80 bytes
     uint8_t type;
@@ -193,6 +198,7 @@ struct PlanParams {
     int look_steps = 2;   // tile choice: additions scored by greedy completion
     int look_top = 6;     // ... among this many best-scoring candidates
     int pack0 = 0;        // qubit 0 in every register set (the wide pass)
+    uint64_t must = 0;    // qubits in every tile and register set; no gate acts on them
     int hoist_diagonals = 1;   // move late diagonal ops to the last phase's uniform tail
 };
 
@@ -266,11 +272,15 @@ constexpr int wide_pair_index(int j, int k)
 {
     return j * (kWideRegBits - 1) - (j * (j - 1)) / 2 + (k - j - 1);
 }
+constexpr int wide_adj_pair_index(int j, int k) { return j * 4 - (j * (j - 1)) / 2 + (k - j - 1); }
 enum : uint8_t {
     W_H = 0, W_XH = kWideRegBits, W_YH = 2 * kWideRegBits, W_T = 3 * kWideRegBits, W_CZ = 4 * kWideRegBits,
     W_CZO = W_CZ + kWideRegBits * (kWideRegBits - 1) / 2,
     W_CT = W_CZO + kWideRegBits,                 // codes of the Clifford+T loop
     W_RY = W_CT, W_RX = W_RY + kWideRegBits, W_PH = W_RX + kWideRegBits, W_PP = W_PH + kWideRegBits,
+    // adjoint sweep (register bits 0..4; bit 5 selects psi or lambda)
+    W_DX = W_PP + kWideRegBits * (kWideRegBits - 1) / 2, W_DY = W_DX + 5, W_DZ = W_DX + 10, W_DP = W_DX + 15,
+    W_DPP = W_DX + 20, W_DW = W_DPP + 10, W_DTZ, W_DTP, W_RED,
     W_END = 255                                  // any code past the table ends the phase
 };
 
@@ -285,7 +295,15 @@ bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &
 // Lowers one plan's passes (phase and op indices into the given arrays) and
 // appends them to *out.
 void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
-                const std::vector<DevOp> &ops, WidePlan *out);
+                const std::vector<DevOp> &ops, WidePlan *out, std::vector<int> *slots = nullptr);
+// The adjoint method's reverse sweep over `gates` on n >= kWideMinTile - 1
+// qubits as wide passes of n + 1 qubits, where qubit n -- in every tile, the
+// last register bit of every phase -- selects psi (0) or lambda (1): each gate
+// is undone on both at once, and each parameterised gate's derivative term is
+// taken where the gate is undone (it commutes with its own gate and with every
+// gate the planner may move across it).  param_of_slot: parameter (index among
+// the parameterised gates) of each partial slot.
+qs_status build_adjoint(int n, const qs_gate *gates, size_t ng, WidePlan *out, std::vector<int> *param_of_slot);
 
 qs_status build_plan(const PlanParams &pp, const qs_gate *g, size_t ng, Plan *out);
 uint16_t f64_to_f16_bits(double x);
@@ -386,6 +404,16 @@ struct DevicePlanSlot {
     size_t wide_ops = 0;          // records (and codes) uploaded
 };
 
+// Lowered reverse sweep of the last gradient (complex64), kept with the state
+// while the gate list stays the same.
+struct AdjointSlot {
+    std::vector<qs_gate> gates;
+    WidePlan plan;
+    std::vector<int> param_of_slot;
+    void *dev = nullptr;       // passes | records | codes | scales
+    size_t bytes = 0;
+};
+
 struct DevicePlanCache {
     DevicePlanSlot slot[2];
     uint64_t clock = 0;
@@ -406,6 +434,7 @@ struct qs_state {
     size_t ws_f64_count;
     uint64_t *ws_u64;        // small integer scratch (flags, counters)
     qs::DevicePlanCache plan_cache;
+    qs::AdjointSlot adjoint;
     // |0...0> bookkeeping, for applying a leading layer of Hadamards as one
     // uniform write: is_zero -- the state is |0...0> (written, or pending:
     // zero_pending defers the reset's write to the next use); escaped -- the
@@ -461,6 +490,11 @@ qs_status run_fused_plan(qs_state *s, const Plan &plan, const void *dev_plan, do
 // The same for a lowered plan; dev holds passes | records | codes.
 qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t nops, const void *dev,
                         double uniform, const FoldArgs *fold);
+// Reverse sweep of a lowered adjoint plan (dev: passes | records | codes) on
+// the state (psi) and lam; partials of slot j at part[j * stride ..),
+// stride = adjoint_wide_partials(s), zeroed beforehand.
+qs_status launch_adjoint_wide(const qs_state *s, void *lam, const WidePlan &plan, const void *dev, double *part);
+int adjoint_wide_partials(const qs_state *s);
 qs_status run_tc_plan(qs_state *s, const Plan &plan, const void *dev_plan,
                       int precision);
 qs_status launch_probabilities(const qs_state *s, void *out, int fp64,

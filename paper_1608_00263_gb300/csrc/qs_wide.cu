@@ -28,9 +28,9 @@ k_wide_pass(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g, cons
             F.m[1] = fold.m2;
             F.m[2] = fold.m4;
         }
-        wide_pass_body<FULL, true, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, true, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
     } else {
-        wide_pass_body<FULL, false, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, false, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
     }
 }
 
@@ -56,6 +56,46 @@ qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t
     return QS_OK;
 }
 
+// ---- adjoint sweep: one pass over psi and lambda ----
+// Partials: warp w of CTA b adds its sums of slot s at part[s * stride + b *
+// (warps per CTA) + w]; each address has one warp, so the order is fixed.
+__global__ void __launch_bounds__(kWideThreads, 3)
+k_adj_wide(float2 *__restrict__ psi, uint64_t lam_off, const WidePass *__restrict__ pass_g,
+           const WideOp *__restrict__ ops_g, const uint8_t *__restrict__ codes_g, uint32_t ntiles, double *part,
+           uint32_t stride)
+{
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    __shared__ WideSmem S;
+    if (threadIdx.x == 0) {
+        S.part = reinterpret_cast<uint64_t>(part + (size_t)blockIdx.x * (blockDim.x >> 5));
+        S.part_stride = (uint64_t)stride * 8u;
+    }
+    const uint32_t per = ntiles / gridDim.x, extra = ntiles % gridDim.x;
+    const uint32_t t_begin = blockIdx.x * per + (blockIdx.x < extra ? blockIdx.x : extra);
+    wide_pass_body<2, false, false>(psi, pass_g, ops_g, codes_g, t_begin,
+                                    t_begin + per + (blockIdx.x < extra ? 1 : 0), S, nullptr, smem_dyn, lam_off);
+}
+
+int adjoint_wide_partials(const qs_state *s) { return 3 * s->num_sms * (kWideThreads / 32); }
+
+qs_status launch_adjoint_wide(const qs_state *s, void *lam, const WidePlan &plan, const void *dev, double *part)
+{
+    const WidePass *dpass = static_cast<const WidePass *>(dev);
+    const WideOp *dops = reinterpret_cast<const WideOp *>(dpass + plan.passes.size());
+    const uint8_t *dcodes = reinterpret_cast<const uint8_t *>(dops + plan.ops.size());
+    const uint64_t lam_off = (uint64_t)((const char *)lam - (const char *)s->amps);
+    for (size_t p = 0; p < plan.passes.size(); ++p) {
+        const WidePass &P = plan.passes[p];
+        const size_t smem = (size_t(1) << P.t) * sizeof(float2);
+        if (p == 0) QS_CUDA_TRY(cudaFuncSetAttribute(k_adj_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        const uint32_t ntiles = 1u << (P.n - P.t), cap = (uint32_t)s->num_sms * 3;
+        k_adj_wide<<<(int)(ntiles < cap ? ntiles : cap), 1 << (P.t - kWideRegBits), smem, s->stream>>>(
+            (float2 *)s->amps, lam_off, dpass + p, dops, dcodes, ntiles, part, (uint32_t)adjoint_wide_partials(s));
+        QS_LAUNCH_CHECK();
+    }
+    return QS_OK;
+}
+
 // ---- batch engines on wide passes ----
 // Lockstep round: blockDim.x = 2^(t - 6), the launch's tile size.
 template <bool FULL>
@@ -68,7 +108,7 @@ k_batch_pass_wide(float2 *__restrict__ amps, const BatchItem *__restrict__ items
     __shared__ WideSmem S;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const BatchItem w = items[it];
-        wide_pass_body<FULL, false, false>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
+        wide_pass_body<FULL ? 1 : 0, false, false>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
                                            nullptr, smem_dyn);
     }
 }
@@ -117,7 +157,7 @@ k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int
             } else if (w.kind == kPersistStats) {
                 batch_stats_chunk<kWideThreads>(amps + w.amp_off, w.lo, w.f0, part + (size_t)w.pass * kStatAcc);
             } else {
-                wide_pass_body<FULL, false, true>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, nullptr,
+                wide_pass_body<FULL ? 1 : 0, false, true>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, nullptr,
                                                   smem_dyn);
             }
         }

@@ -41,6 +41,8 @@ struct WideSmem {
     uint64_t toff[kWideThreads];                     // byte offset in the state of the thread's first copied unit
     uint64_t doff[kWideThreads];                     // ... of its slot 0 in the last phase
     uint64_t dst[kWideThreads];                      // direct pass: state address of the thread's slot 0
+    alignas(16) uint64_t part;                       // adjoint sweep: partials of this CTA's warps,
+    uint64_t part_stride;                            // bytes per slot
     uint64_t gmask;                                  // out-of-tile qubits
     uint16_t thr[kMaxPhasesPerPass][kWideThreads];   // tile element of the thread's slot 0
     WideUnit unit[kWideUnits];
@@ -48,7 +50,7 @@ struct WideSmem {
 };
 
 static_assert(sizeof(WidePass) % 16 == 0 && offsetof(WidePass, ph) % 16 == 0 && offsetof(WideSmem, ops) % 16 == 0 &&
-                  offsetof(WideSmem, unit) % 16 == 0 && sizeof(WideUnit) == 16,
+                  offsetof(WideSmem, unit) % 16 == 0 && offsetof(WideSmem, part) % 16 == 0 && sizeof(WideUnit) == 16,
               "staged in 16-byte units");
 
 // Tables of the folded diagonal prefix (first pass of a circuit, see
@@ -80,11 +82,14 @@ __device__ __forceinline__ void wide_sync(int nthr, int gi)
 // (the uniform state times the folded prefix's phases) instead of loading
 // them; F's nb and m are set by the caller (published by the first barrier).
 // The caller's CTA is converged; ends with a CTA barrier.
-template <bool FULL, bool FOLD, bool GROUPED>
+// KIND: the op loop (0 Clifford+T, 1 all gates, 2 the adjoint sweep, whose
+// tile bit t - 1 selects psi or lambda, lam_off bytes away; S.part and
+// S.part_stride are set by the caller).
+template <int KIND, bool FOLD, bool GROUPED>
 __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g,
                                                const WideOp *__restrict__ ops_g, const uint8_t *__restrict__ codes_g,
                                                uint32_t t_begin, uint32_t t_end, WideSmem &S, WideFoldSmem *F,
-                                               unsigned char *smem_raw)
+                                               unsigned char *smem_raw, uint64_t lam_off = 0)
 {
     constexpr int RB = kWideRegBits, NS = kWideSlots, NU = kWideUnits;
     for (int i = threadIdx.x; i < (int)(sizeof(WidePass) / 4); i += blockDim.x)
@@ -95,6 +100,13 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
     const int tid = GROUPED ? (int)(threadIdx.x & (unsigned)(nthr - 1)) : (int)threadIdx.x;
     const int gi = GROUPED ? (int)(threadIdx.x >> (t - RB)) : 0;
     const int ngr = GROUPED ? (int)(blockDim.x >> (t - RB)) : 1;
+    // byte offset in the state of tile element e
+    auto state_off = [&](uint32_t e) -> uint64_t {
+        if constexpr (KIND == 2)
+            return deposit(e & ((1u << (t - 1)) - 1u), S.P.L, t - 1) * 8u + ((e >> (t - 1)) & 1u ? lam_off : 0ull);
+        else
+            return deposit(e, S.P.L, t) * 8u;
+    };
     // ---- stage the ops and the per-thread tables (once per CTA and pass) ----
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(ops_g + S.P.op_begin);
@@ -110,7 +122,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         }
     for (int i = threadIdx.x; i < NU; i += blockDim.x) {
         const uint32_t e = 2u * (uint32_t)nthr * (uint32_t)i;
-        S.unit[i].goff = deposit(e, S.P.L, t) * 8u;
+        S.unit[i].goff = state_off(e);
         S.unit[i].soff = swz<2>(e) * 8u;
     }
     if (threadIdx.x < 8) {
@@ -152,13 +164,14 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         }
     }
     if (gi == 0) {
-        S.toff[tid] = deposit(2u * (uint32_t)tid, S.P.L, t) * 8u;
-        S.doff[tid] = deposit(S.thr[nph - 1][tid], S.P.L, t) * 8u;
+        S.toff[tid] = state_off(2u * (uint32_t)tid);
+        S.doff[tid] = state_off(S.thr[nph - 1][tid]);
     }
     if (threadIdx.x == 0) {
         uint64_t m = 0;
         for (int i = 0; i < ng; ++i) m |= 1ULL << S.P.G[i];
         S.gmask = m;
+        if constexpr (KIND == 2) S.P.dreg[RB - 1] = lam_off;
     }
     __syncthreads();
     unsigned char *gsm = GROUPED ? smem_raw + (((size_t)gi << t) * sizeof(float2)) : smem_raw;
@@ -255,7 +268,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
                     const WideOp op = S.ops[o];
                     if ((te & op.sel_tile) == op.sel_tile && (to & op.sel_out) == op.sel_out) {
                         k += reinterpret_cast<const uint8_t *>(S.codes)[o];
-                        if constexpr (FULL) {
+                        if constexpr (KIND > 0) {
                             const float x = fr * op.p0 - fi * op.p1;
                             fi = fr * op.p1 + fi * op.p0;
                             fr = x;
@@ -284,10 +297,10 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
                     nsrc = reinterpret_cast<const char *>(amps) + (next_base() * 8u + S.toff[tid]);
                 }
             }
-            OpLoop<FULL>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16,
+            OpLoop<KIND>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16,
                                        (int)offsetof(WideSmem, unit),
                                        (int)(offsetof(WideSmem, P) + offsetof(WidePass, dreg)),
-                                       (int)offsetof(WideSmem, dst)>(
+                                       (int)offsetof(WideSmem, dst), (int)offsetof(WideSmem, part)>(
                 swz<2>(te) * 8u, tile_sa, smem_addr(&S),
                 (uint32_t)(offsetof(WideSmem, P) + offsetof(WidePass, ph)) + (uint32_t)ph * (uint32_t)sizeof(WidePhase),
                 H.op_begin, ((uint64_t)to << 32) | te, fr, fi, mode, sw_tid,

@@ -75,3 +75,31 @@ def test_generated_and_held_states_agree(n):
     finally:
         qs.qs_state_destroy(held)
         qs.qs_state_destroy(made)
+
+
+@pytest.mark.parametrize("n", [9, 10, 11, 13, 16])
+def test_adjoint_sweep(n):
+    """Gradient of every parameterised gate of a list with all gate kinds: the
+    complex64 sweep (wide passes from 10 qubits on, tile groups below) against
+    the complex128 one, which the adjoint tests pin to exact parameter shifts.
+    Tolerance: theirs for complex64, 1e-4 of the largest derivative."""
+    rng = np.random.default_rng(40 + n)
+    g = np.concatenate([O.generate_circuit(1, n, 0, 0)[:n], gate_list(rng, n, 220, ALL)]).astype(qs.GATE_DTYPE)
+    x = rng.integers(0, 1 << n, size=500).astype(np.uint64)
+    out = {}
+    for dt in (qs.QS_C128, qs.QS_C64):
+        h = qs.qs_state_create(n, dt)
+        try:
+            loss, grad = qs.qs_adjoint_gradient(h, g, x)
+            loss2, grad2 = qs.qs_adjoint_gradient(h, g, x)          # the kept plan
+            assert loss == loss2 and np.max(np.abs(grad - grad2)) <= 1e-5 * np.max(np.abs(grad))
+            g2 = g.copy()
+            g2["theta"] *= 1.01                                     # another list: a new plan
+            out[dt] = (grad, qs.qs_adjoint_gradient(h, g2, x)[1])
+            psi = qs.qs_state_copy_out(h, n, dt)                    # the sweep undoes the circuit
+            assert abs(psi[0] - 1) < (1e-4 if dt == qs.QS_C64 else 1e-10)
+        finally:
+            qs.qs_state_destroy(h)
+    for a, b in zip(out[qs.QS_C64], out[qs.QS_C128]):
+        assert np.max(np.abs(a - b)) < 1e-4 * np.max(np.abs(b))
+        assert np.all(a[g["kind"] < qs.QS_RX] == 0)

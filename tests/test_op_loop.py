@@ -101,6 +101,8 @@ class Thread:
                     r[a[0]], r[a[1]] = r[a[2]]
                 else:
                     r[a[0]] = [self.val(a[1]), self.val(a[2])]
+            elif op == "mov.f32":
+                r[a[0]] = self.val(a[1])
             elif op == "mov.u32":
                 r[a[0]] = int(self.val(a[1]))
             elif op == "add.rn.f32":
@@ -285,3 +287,50 @@ def test_phase_on_one_thread(full, t, regs):
                 a = TILE + swizzle(2 * u) * 8
                 if a not in mine:
                     assert m2[a:a + 16] == mem[a:a + 16]
+
+
+@pytest.mark.parametrize("code", [c for c in range(G.W_DX, G.W_RED) if c != G.W_DW])
+@pytest.mark.parametrize("sel", [False, True])
+def test_derivative_terms(code, sel):
+    """The adjoint loop's terms of one thread against their definitions; the
+    selector of psi and lambda is register bit 5.  64 products of values <= 1
+    in FP32: 64 * 2^-23 absolute at most."""
+    t, regs, e0 = 13, (0, 3, 4, 7, 9, 12), (1 << 5) | (1 << 8)
+    rng = np.random.default_rng(code)
+    mem = bytearray(TILE + (8 << t))
+    elems = [e0 | sum(((s >> j) & 1) << b for j, b in enumerate(regs)) for s in range(64)]
+    v = rng.uniform(-1, 1, 64).astype(f32) + 1j * rng.uniform(-1, 1, 64).astype(f32)
+    for s, e in enumerate(elems):
+        a = TILE + swizzle(e & ~1) * 8
+        struct.pack_into("<f", mem, a + 4 * (e & 1), v[s].real)
+        struct.pack_into("<f", mem, a + 8 + 4 * (e & 1), v[s].imag)
+    struct.pack_into("<6I", mem, SMEM_STATIC + O_PHASE, *[swizzle(1 << b) * 8 for b in regs])
+    for k, c in enumerate([G.W_DW, code, 255]):
+        struct.pack_into("<Q2f", mem, SMEM_STATIC + O_OPS + 16 * k, (1 << 5) if sel else (1 << 6), 1.0, 0.0)
+        mem[SMEM_STATIC + O_CODES + k] = c
+    operands = dict(zip(["%%%d" % k for k in range(19)] + ["%tid.x"],
+                        [swizzle(e0) * 8, TILE, SMEM_STATIC, O_PHASE, 0, e0, f32(1), f32(0), 0, 0, NEXT, 0, 128,
+                         O_CODES, O_OPS - 16, O_UNIT, O_DREG, O_DST, 0, 0]))
+    operands.update({"da0": f32(0), "da1": f32(0), "da2": f32(0)})
+    th = Thread(G.asm_text("A", True, True), mem, SMEM_STATIC, TILE + (8 << t), operands)
+    th.run()
+    psi, lam = v[:32].astype(complex), v[32:].astype(complex)
+    idx = np.arange(32)
+    if code < G.W_DZ:
+        j = (code - G.W_DX) % G.AB
+        p = psi[idx ^ (1 << j)] * (1 if code < G.W_DY else np.where((idx >> j) & 1, 1j, -1j))
+        want = np.vdot(lam, p).imag
+    else:
+        w = (np.conj(lam) * psi).imag
+        if code < G.W_DP:
+            want = np.sum(w * np.where((idx >> (code - G.W_DZ)) & 1, -1, 1))
+        elif code < G.W_DPP:
+            want = np.sum(w[(idx >> (code - G.W_DP)) & 1 == 1]) if sel else 0.0
+        elif code < G.W_DW:
+            j, k = [(j, k) for j in range(G.AB) for k in range(j + 1, G.AB)][code - G.W_DPP]
+            want = np.sum(w[((idx >> j) & (idx >> k) & 1) == 1])
+        elif code == G.W_DTZ:
+            want = np.sum(w) * (-1 if sel else 1)
+        else:
+            want = np.sum(w) if sel else 0.0
+    assert abs(float(th.r["da0"]) - want) < 64 * 2.0 ** -23 * 2
