@@ -168,12 +168,26 @@ __device__ __forceinline__ void reg_phase(V *a, R pr, R pi, bool tgate)
     }
 }
 
-template <int NS, int M, typename V, typename R>
-__device__ __forceinline__ void reg_sign(V *a, R sg)
+// Sign (sg = 1 or -1) on the slots whose register bits include all of M;
+// complex128 flips the sign bits: the FP64 pipe is what bounds its passes (a
+// fifth of their FP64 instructions were these multiplications).
+template <int NS, int M>
+__device__ __forceinline__ void reg_sign(float2 *a, float sg)
 {
 #pragma unroll
     for (int s = 0; s < NS; ++s)
         if ((s & M) == M) mul_sign(a[s], sg);
+}
+template <int NS, int M>
+__device__ __forceinline__ void reg_sign(double2 *a, double sg)
+{
+    const int flip = __double2hiint(sg) & (int)0x80000000;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+        if ((s & M) == M) {
+            a[s].x = __hiloint2double(__double2hiint(a[s].x) ^ flip, __double2loint(a[s].x));
+            a[s].y = __hiloint2double(__double2hiint(a[s].y) ^ flip, __double2loint(a[s].y));
+        }
 }
 
 
