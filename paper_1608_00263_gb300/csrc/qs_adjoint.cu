@@ -430,6 +430,7 @@ static qs_status adjoint_t(qs_state *s, const qs_gate *g, size_t ng, const uint6
 // passes over psi and lambda (build_adjoint).  A pass undoes ~50 gates in
 // registers where a tile group undid ~7 in shared memory with a barrier
 // after each: 24 qubits, depth 30: 8 passes instead of 56 group launches.
+constexpr size_t kAdjKeepBytes = size_t(1) << 30;
 static qs_status adjoint_wide(qs_state *s, const qs_gate *g, size_t ng, const uint64_t *dev_x, uint64_t m, double *grad)
 {
     AdjointSlot &A = s->adjoint;
@@ -470,15 +471,33 @@ static qs_status adjoint_wide(qs_state *s, const qs_gate *g, size_t ng, const ui
                             A.plan.codes.size() + 15) / 16 * 16;
     const uint64_t N = 1ULL << s->n;
     const size_t b_part = nparam * parts * sizeof(double), b_out = (nparam ? nparam : 1) * sizeof(double);
-    float2 *lam = nullptr;
+    // lambda and the partials in one workspace: kept with the state up to
+    // kAdjKeepBytes (allocating 134 MB anew cost ~0.5 ms a call), else
+    // allocated for the call
+    const size_t b_lam = N * sizeof(float2), b_work = b_lam + b_part + b_out;
+    const bool keep = b_work <= kAdjKeepBytes;
     unsigned char *work = nullptr;
-    QS_CUDA_TRY(cudaMallocAsync((void **)&lam, N * sizeof(float2), s->stream));
     qs_status st = QS_OK;
-    cudaError_t e = cudaMallocAsync((void **)&work, b_part + b_out, s->stream);
+    cudaError_t e = cudaSuccess;
+    if (keep) {
+        if (A.work_bytes < b_work) {
+            if (A.work) cudaFree(A.work);
+            A.work = nullptr;
+            A.work_bytes = 0;
+            e = cudaMalloc(&A.work, b_work);
+            if (e == cudaSuccess) A.work_bytes = b_work;
+            else A.work = nullptr;
+        }
+        work = (unsigned char *)A.work;
+    } else {
+        e = cudaMallocAsync((void **)&work, b_work, s->stream);
+    }
+    float2 *lam = (float2 *)work;
     if (e != cudaSuccess) {
+        cudaGetLastError();
         st = set_error(QS_ERR_OOM, "adjoint workspace: %s", cudaGetErrorString(e));
     } else {
-        double *part = (double *)work, *out = (double *)(work + b_part);
+        double *part = (double *)(work + b_lam), *out = (double *)(work + b_lam + b_part);
         e = cudaMemsetAsync(lam, 0, N * sizeof(float2), s->stream);
         if (e == cudaSuccess && b_part) e = cudaMemsetAsync(part, 0, b_part, s->stream);
         if (e == cudaSuccess) {
@@ -503,8 +522,7 @@ static qs_status adjoint_wide(qs_state *s, const qs_gate *g, size_t ng, const ui
         }
         if (!st && e != cudaSuccess) st = set_error(QS_ERR_CUDA, "adjoint sweep: %s", cudaGetErrorString(e));
     }
-    if (lam) cudaFreeAsync(lam, s->stream);
-    if (work) cudaFreeAsync(work, s->stream);
+    if (!keep && work) cudaFreeAsync(work, s->stream);
     cudaStreamSynchronize(s->stream);
     return st;
 }

@@ -123,6 +123,7 @@ void free_state(qs_state *s)
     if (s->hbox) cudaFreeHost(s->hbox);
     if (s->rc_buf) cudaFree(s->rc_buf);
     if (s->adjoint.dev) cudaFree(s->adjoint.dev);
+    if (s->adjoint.work) cudaFree(s->adjoint.work);
     if (s->stage) cudaFreeHost(s->stage);
     for (DevicePlanSlot &c : s->plan_cache.slot) {
         if (c.dev) cudaFree(c.dev);
@@ -780,15 +781,21 @@ extern "C" qs_status qs_cycle_statistics(qs_state *s, const qs_gate *gates, size
     s->zero_pending = false;
     if (qs_status st = launch_init_zero(s)) return st;
     s->is_zero = true;
+    // the cycles' statistics collect in the host box, so the host plans and
+    // launches ahead of the device and waits once per kStatRows cycles
     const int w = 4 + kmax;
-    std::vector<double> mom(kMaxMoments);
     for (size_t c = 0; c < starts.size(); ++c) {
         const size_t b = starts[c], e = c + 1 < starts.size() ? starts[c + 1] : ngates;
         if (qs_status st = qs_apply_circuit(s, gates + b, e - b, opts)) return st;
-        double *row = stats + c * w;
-        row[0] = (double)gates[b].cycle;
-        if (qs_status st = stats_moments(s, kmax, mom.data(), &row[2], &row[3], &row[1])) return st;
-        for (int k = 0; k < kmax; ++k) row[4 + k] = mom[k];
+        stats[c * w] = (double)gates[b].cycle;
+        const int row = (int)(c % kStatRows);
+        if (qs_status st = stats_enqueue(s, row)) return st;
+        if (row + 1 < kStatRows && c + 1 < starts.size()) continue;
+        QS_CUDA_TRY(cudaStreamSynchronize(s->stream));
+        for (int r = 0; r <= row; ++r) {
+            double *out = stats + (c - (size_t)row + (size_t)r) * w;
+            stats_from_sums((const double *)s->hbox + (size_t)r * kStatSums, s->n, kmax, &out[1], &out[2], &out[3], out + 4);
+        }
     }
     return QS_OK;
 }

@@ -412,6 +412,8 @@ struct AdjointSlot {
     std::vector<int> param_of_slot;
     void *dev = nullptr;       // passes | records | codes | scales
     size_t bytes = 0;
+    void *work = nullptr;      // lambda and partials, kept up to 1 GB
+    size_t work_bytes = 0;
 };
 
 struct DevicePlanCache {
@@ -499,6 +501,9 @@ qs_status run_tc_plan(qs_state *s, const Plan &plan, const void *dev_plan,
                       int precision);
 qs_status launch_probabilities(const qs_state *s, void *out, int fp64,
                                uint64_t first, uint64_t count);
+// Enqueues the current state's statistics: kStatSums sums into row `row` of
+// the state's host box (complete once the stream is; at most kStatRows rows).
+qs_status stats_enqueue(const qs_state *s, int row);
 qs_status stats_moments(const qs_state *s, int kmax, double *moments,
                         double *entropy, double *uniform_ce, double *norm);
 qs_status sampler_run(const qs_state *s, uint64_t k, uint64_t seed,
@@ -550,6 +555,7 @@ qs_status stage_view(const qs_state *s, size_t bytes, void **host, void **dev);
 
 // batched ensemble helpers
 constexpr int kStatSums = 12;
+constexpr int kStatRows = (int)(kHostBoxBytes / (kStatSums * sizeof(double)));
 // One lockstep round of the batched pass; `full` selects the interpreter
 // with the parameterised-gate cases (else the Clifford+T one, valid when
 // plan_pass_needs_full is false for every pass of the round's items).

@@ -132,16 +132,72 @@ __device__ __forceinline__ void stat_pair_p(float p0, float p1, bool two, float 
     }
 }
 
+// ---- complex128 statistics ----
+// Bound by the FP64 pipe (two lanes per clock and SM), so what counts is the
+// number of FP64 instructions per amplitude: 28 here against ~58 with log()
+// and a multiply and an add per power (2^20 amplitudes: 132 -> ~60 us).
+
+// ln y by the table method of Tang (ACM TOMS 16, 1990): y = 2^e m, c_i ~ 1 /
+// (1 + (i + 1/2) / 256) from the top eight bits i of m's fraction, r = m c_i -
+// 1 (|r| < 2^-8.9), ln y = e ln 2 - ln c_i + (r - r^2/2 + r^3/3 - r^4/4 +
+// r^5/5); the first term left out is below 2^-56.  Nine FP64 instructions.
+// Zero, subnormal and non-finite y take log().
+constexpr int kLogTable = 256;
+__device__ __forceinline__ void log_table_fill(double2 *tab)
+{
+    for (int i = threadIdx.x; i < kLogTable; i += blockDim.x) {
+        const double c = (double)(float)(1.0 / (1.0 + ((double)i + 0.5) / kLogTable));
+        tab[i] = make_double2(c, -log(c));
+    }
+}
+__device__ __forceinline__ double log_pos(double y, const double2 *tab)
+{
+    const long long b = __double_as_longlong(y);
+    const uint32_t e = (uint32_t)(b >> 52);          // (y >= 0)
+    if (e == 0 || e >= 0x7FFu) return log(y);
+    const double m = __longlong_as_double((b & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
+    const double2 t = tab[(b >> 44) & (kLogTable - 1)];
+    // e - 1023 as a double: 2^52 + 2^31 + (e - 1023) less 2^52 + 2^31
+    const double ed = __hiloint2double(0x43300000, (int)((e - 1023u) ^ 0x80000000u)) -
+                      __hiloint2double(0x43300000, (int)0x80000000);
+    const double r = fma(m, t.x, -1.0);
+    const double q = fma(r, fma(r, fma(r, 0.2, -0.25), 1.0 / 3.0), -0.5);
+    return fma(ed, 0.69314718055994530942, t.y) + fma(q, r * r, r);
+}
+
+// Accumulates one element's contributions (stat_terms), the powers as
+// products of y^2, y^3, y^4 and y^8.
+__device__ __forceinline__ void stat_terms_f64(double y, double (&c)[kStatAcc], const double2 *tab)
+{
+    const double ly = log_pos(y, tab);
+    c[0] += y;
+    c[1] = y > 0.0 ? fma(y, ly, c[1]) : c[1];
+    c[2] += ly;
+    const double y2 = y * y, y3 = y2 * y, y4 = y2 * y2, y8 = y4 * y4;
+    c[3] += y2;
+    c[4] += y3;
+    c[5] += y4;
+    c[6] = fma(y4, y, c[6]);
+    c[7] = fma(y4, y2, c[7]);
+    c[8] = fma(y4, y3, c[8]);
+    c[9] += y8;
+    c[10] = fma(y8, y, c[10]);
+    c[11] = fma(y8, y2, c[11]);
+}
+
 __global__ void __launch_bounds__(kStatThreads)
 k_stats_c128(const double2 *__restrict__ a, uint64_t N, double scaleN, double *__restrict__ part)
 {
+    __shared__ double2 tab[kLogTable];
+    log_table_fill(tab);
+    __syncthreads();
     double acc[kStatAcc];
 #pragma unroll
     for (int k = 0; k < kStatAcc; ++k) acc[k] = 0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
         double2 v = a[i];
-        stat_terms<double>((v.x * v.x + v.y * v.y) * scaleN, acc);
+        stat_terms_f64((v.x * v.x + v.y * v.y) * scaleN, acc, tab);
     }
     block_sum_store<kStatAcc>(acc, part + (size_t)blockIdx.x * kStatAcc);
 }
@@ -215,8 +271,7 @@ qs_status stage_view(const qs_state *s, size_t bytes, void **host, void **dev)
     return QS_OK;
 }
 
-qs_status stats_moments(const qs_state *s, int kmax, double *moments, double *entropy,
-                        double *uniform_ce, double *norm)
+qs_status stats_enqueue(const qs_state *s, int row)
 {
     const uint64_t N = 1ULL << s->n;
     int grid;
@@ -229,29 +284,26 @@ qs_status stats_moments(const qs_state *s, int kmax, double *moments, double *en
         part = readout_part(s);
         grid = readout_grid(s);
     } else {
-        grid = grid_for(N, kStatThreads, s->num_sms, 4);
+        // (one block per SM: eight warps keep the FP64 pipe busy, and the
+        // logarithm table is filled once per SM)
+        grid = grid_for(N, kStatThreads, s->num_sms, 1);
         k_stats_c128<<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, N,
                                                             std::ldexp(1.0, s->n), part);
         QS_LAUNCH_CHECK();
     }
+    k_sum_partials<<<1, kSumThreads, 0, s->stream>>>(part, grid, kStatAcc, (double *)s->hbox_dev + (size_t)row * kStatAcc);
+    QS_LAUNCH_CHECK();
+    return QS_OK;
+}
+
+qs_status stats_moments(const qs_state *s, int kmax, double *moments, double *entropy,
+                        double *uniform_ce, double *norm)
+{
+    if (qs_status st = stats_enqueue(s, 0)) return st;
+    QS_CUDA_TRY(cudaStreamSynchronize(s->stream));
     double h[kStatAcc];
-    if (qs_status st = sum_to_host(s, part, grid, kStatAcc, h)) return st;
-    // Statistics of the normalised distribution p / S, S = sum p: the
-    // arithmetic of the evolution leaves |S - 1| at the rounding level
-    // (systematic for FP32: rounded phase constants have modulus below 1),
-    // and dividing it out keeps that drift out of the entropy, moments and
-    // uniform cross entropy.  With y = N p and Y = sum y = N S:
-    //   H      = -sum (p/S) ln(p/S) = ln S + ln N - (sum y ln y) / Y
-    //   CE_u   = -(1/N) sum ln(p/S) = ln S + ln N - (sum ln y) / N
-    //   M_k    = N^{k-1} sum (p/S)^k = (sum y^k) / (N S^k)
-    const double Nd = (double)N, lnN = s->n * std::log(2.0);
-    const double S = h[0] / Nd;
-    if (norm) *norm = S;
-    const double lnS = S > 0 ? std::log(S) : -INFINITY;
-    if (entropy) *entropy = S > 0 ? lnS + lnN - h[1] / h[0] : 0.0;
-    if (uniform_ce) *uniform_ce = S > 0 ? lnS + lnN - h[2] / Nd : INFINITY;
-    for (int k = 1; k <= kmax; ++k)
-        moments[k - 1] = S > 0 ? (k == 1 ? 1.0 : h[k + 1] / (Nd * std::pow(S, k))) : 0.0;
+    std::memcpy(h, s->hbox, sizeof h);
+    stats_from_sums(h, s->n, kmax, norm, entropy, uniform_ce, moments);
     return QS_OK;
 }
 
@@ -297,6 +349,14 @@ qs_status launch_batch_stats(cudaStream_t st, int num_sms, const void *amps, con
     return QS_OK;
 }
 
+// Statistics of the normalised distribution p / S, S = sum p: the
+// arithmetic of the evolution leaves |S - 1| at the rounding level
+// (systematic for FP32: rounded phase constants have modulus below 1),
+// and dividing it out keeps that drift out of the entropy, moments and
+// uniform cross entropy.  With y = N p and Y = sum y = N S:
+//   H      = -sum (p/S) ln(p/S) = ln S + ln N - (sum y ln y) / Y
+//   CE_u   = -(1/N) sum ln(p/S) = ln S + ln N - (sum ln y) / N
+//   M_k    = N^{k-1} sum (p/S)^k = (sum y^k) / (N S^k)
 void stats_from_sums(const double *h, int n, int kmax, double *norm, double *entropy, double *uniform_ce,
                      double *moments)
 {
