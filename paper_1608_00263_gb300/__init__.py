@@ -300,7 +300,7 @@ def qs_batch_correlation(b, ref):
 
 def qs_batch_mean_probabilities(b, n):
     """Mean distribution over the batch's instances (all of n qubits)."""
-    out = np.zeros(1 << n, dtype=np.float64)
+    out = np.empty(1 << n, dtype=np.float64)
     N.check(N.lib().qs_batch_mean_probabilities(b, out.ctypes.data))
     return out
 
@@ -324,14 +324,21 @@ def qs_batch_create(nqubits, stream=None):
     return h.value
 
 
+def _concatenate(gl):
+    """The gate lists one after another and their offsets.  (As bytes: numpy
+    joins records field by field.)"""
+    offsets = np.zeros(len(gl) + 1, dtype=np.uint64)
+    offsets[1:] = np.cumsum([g.size for g in gl])
+    if not offsets[-1]:
+        return np.zeros(0, dtype=GATE_DTYPE), offsets
+    return np.concatenate([g.reshape(-1).view(np.uint8) for g in gl]).view(GATE_DTYPE), offsets
+
+
 def qs_batch_run(b, gate_lists, kmax=10):
     """Runs every instance's gate list; returns an array (count, 3 + kmax):
     norm, entropy, uniform cross entropy, moments 1..kmax."""
     gl = [_gates(g) for g in gate_lists]
-    offsets = np.zeros(len(gl) + 1, dtype=np.uint64)
-    offsets[1:] = np.cumsum([g.size for g in gl])
-    gates = np.concatenate(gl) if gl else np.zeros(0, dtype=GATE_DTYPE)
-    gates = np.ascontiguousarray(gates, dtype=GATE_DTYPE)
+    gates, offsets = _concatenate(gl)
     out = np.zeros((len(gl), 3 + kmax), dtype=np.float64)
     N.check(N.lib().qs_batch_run(b, gates.ctypes.data if gates.size else None, offsets.ctypes.data, kmax,
                                  out.ctypes.data))
@@ -340,10 +347,7 @@ def qs_batch_run(b, gate_lists, kmax=10):
 
 def qs_batch_apply(b, gate_lists):
     """Resets every instance and applies its gate list (no statistics)."""
-    gl = [_gates(g) for g in gate_lists]
-    offsets = np.zeros(len(gl) + 1, dtype=np.uint64)
-    offsets[1:] = np.cumsum([g.size for g in gl])
-    gates = np.ascontiguousarray(np.concatenate(gl) if gl else np.zeros(0, dtype=GATE_DTYPE), dtype=GATE_DTYPE)
+    gates, offsets = _concatenate([_gates(g) for g in gate_lists])
     N.check(N.lib().qs_batch_apply(b, gates.ctypes.data if gates.size else None, offsets.ctypes.data))
 
 

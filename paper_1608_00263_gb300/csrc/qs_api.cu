@@ -66,14 +66,11 @@ struct DeviceGuard {
     }
 };
 
-uint64_t fnv1a(const void *data, size_t n, uint64_t h = 1469598103934665603ULL)
+bool same_params(const PlanParams &a, const PlanParams &b)
 {
-    const unsigned char *p = (const unsigned char *)data;
-    for (size_t i = 0; i < n; ++i) {
-        h ^= p[i];
-        h *= 1099511628211ULL;
-    }
-    return h;
+    return a.n == b.n && a.t == b.t && a.r == b.r && a.c == b.c && a.mode == b.mode && a.k == b.k && a.tc_ok == b.tc_ok &&
+           a.esz == b.esz && a.precision == b.precision && a.look_steps == b.look_steps && a.look_top == b.look_top &&
+           a.pack0 == b.pack0 && a.must == b.must && a.hoist_diagonals == b.hoist_diagonals;
 }
 
 qs_status alloc_workspace(qs_state *s)
@@ -122,6 +119,7 @@ void free_state(qs_state *s)
     if (s->ws_u64) cudaFree(s->ws_u64);
     if (s->hbox) cudaFreeHost(s->hbox);
     if (s->rc_buf) cudaFree(s->rc_buf);
+    if (s->pt_buf) cudaFree(s->pt_buf);
     if (s->adjoint.dev) cudaFree(s->adjoint.dev);
     if (s->adjoint.work) cudaFree(s->adjoint.work);
     if (s->stage) cudaFreeHost(s->stage);
@@ -225,12 +223,12 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
         pp.r = 5;
         pp.pack0 = 0;
     }
-    uint64_t key = fnv1a(gates, ng * sizeof(qs_gate));
-    key = fnv1a(&pp, sizeof pp, key);
     DevicePlanCache &pc = s->plan_cache;
     DevicePlanSlot *c = nullptr;
     for (DevicePlanSlot &x : pc.slot)
-        if (x.valid && x.key == key && x.ngates == ng) c = &x;
+        if (x.valid && x.gates.size() == ng && same_params(x.params, pp) &&
+            std::memcmp(x.gates.data(), gates, ng * sizeof(qs_gate)) == 0)
+            c = &x;
     if (!c) {
         // least recently used slot; wait until the device is done with it
         c = pc.slot[0].last_use <= pc.slot[1].last_use ? &pc.slot[0] : &pc.slot[1];
@@ -279,8 +277,8 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
         QS_CUDA_TRY(cudaMemcpyAsync(c->dev, h, total, cudaMemcpyHostToDevice, s->stream));
         if (!c->done) QS_CUDA_TRY(cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming));
         QS_CUDA_TRY(cudaEventRecord(c->done, s->stream));
-        c->key = key;
-        c->ngates = ng;
+        c->params = pp;
+        c->gates.assign(gates, gates + ng);
         c->plan = std::move(p);
         c->wide_ops = wide.ops.size();
         c->wide = std::move(wide.passes);

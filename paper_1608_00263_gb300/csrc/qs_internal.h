@@ -392,8 +392,8 @@ void build_work(const std::vector<int> &n, const std::vector<uint64_t> &off, con
 // host planning of the next circuit overlaps the current evolution.
 struct DevicePlanSlot {
     bool valid = false;
-    uint64_t key = 0;          // hash of (gates, options)
-    size_t ngates = 0;
+    std::vector<qs_gate> gates;   // the planned list and parameters
+    PlanParams params{};
     void *dev = nullptr;       // passes | phases | ops | blocks on device
     void *staging = nullptr;   // pinned host source of the upload
     size_t bytes = 0;          // capacity of dev and staging
@@ -472,6 +472,9 @@ struct qs_state {
     mutable size_t rc_doubles = 0;
     mutable uint64_t rc_version = ~0ULL;
     mutable int rc_flags = 0;
+    // sampler: in-chunk prefix table (and complex128 chunk sums), see qs_stats.cu
+    mutable void *pt_buf = nullptr;
+    mutable size_t pt_bytes = 0;
 };
 
 namespace qs {
