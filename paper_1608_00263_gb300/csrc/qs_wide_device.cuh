@@ -40,7 +40,9 @@ struct WideSmem {
     uint32_t codes[kMaxOpsPerPass / 4 + 4];
     uint64_t toff[kWideThreads];                     // byte offset in the state of the thread's first copied unit
     uint64_t doff[kWideThreads];                     // ... of its slot 0 in the last phase
-    uint64_t dst[kWideThreads];                      // direct pass: state address of the thread's slot 0
+    uint64_t dst[kWideThreads];                      // state address of the thread's slot 0 of this tile
+    uint64_t amps;                                   // the state, and the end of the tile range: read
+    uint32_t t_end, pad;                             // again where used, registers are short
     alignas(16) uint64_t part;                       // adjoint sweep: partials of this CTA's warps,
     uint64_t part_stride;                            // bytes per slot
     uint64_t gmask;                                  // out-of-tile qubits
@@ -171,6 +173,8 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         uint64_t m = 0;
         for (int i = 0; i < ng; ++i) m |= 1ULL << S.P.G[i];
         S.gmask = m;
+        S.amps = reinterpret_cast<uint64_t>(amps);
+        S.t_end = t_end;
         if constexpr (KIND == 2) S.P.dreg[RB - 1] = lam_off;
     }
     __syncthreads();
@@ -190,7 +194,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         return QS_DCHECK(((b | lmask) >> S.P.n) == 0, 202);
     };
     if constexpr (!FOLD) {
-        if (tau < t_end && inside(base)) {
+        if (tau < S.t_end && inside(base)) {
             const char *src = reinterpret_cast<const char *>(amps) + (base * 8u + S.toff[tid]);
 #pragma unroll 4
             for (int it = 0; it < NU; ++it)
@@ -199,7 +203,8 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
                              : "memory");
         }
     }
-    while (tau < t_end && inside(base)) {
+    while (tau < S.t_end && inside(base)) {
+        S.dst[threadIdx.x] = S.amps + base * 8u + S.doff[tid];
         if constexpr (FOLD) {
             // element x gets 2^(-n/2) e^{i pi k(x) / 4}, k = 4 (CZ pairs within
             // x) + (T counts of x), mod 8, summed over the out-of-tile bits,
@@ -245,10 +250,12 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             }
         }
         wide_sync<GROUPED>(nthr, gi);
-        // (the next tile's base is formed where it is used: registers are
-        // what the phases are short of)
+        // (this tile's base is read back from the thread's address, and the
+        // next one formed, where they are used)
+        auto this_base = [&]() { return (S.dst[threadIdx.x] - S.amps - S.doff[tid]) >> 3; };
         auto next_base = [&]() {
-            return GROUPED && ngr > 1 ? deposit(tau + (uint32_t)ngr, S.P.G, ng) : (((base | ~S.gmask) + 1) & S.gmask);
+            return GROUPED && ngr > 1 ? deposit(tau + (uint32_t)ngr, S.P.G, ng)
+                                      : (((this_base() | ~S.gmask) + 1) & S.gmask);
         };
         for (int ph = 0; ph < nph; ++ph) {
             const WidePhase &H = S.P.ph[ph];
@@ -290,11 +297,11 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             const bool direct = last && S.P.direct;
             const char *nsrc = nullptr;
             if (direct) {
-                S.dst[threadIdx.x] = reinterpret_cast<uint64_t>(amps) + base * 8u + S.doff[tid];
                 mode |= kWideDirect | (S.P.canon_out ? kWideCanon : 0u);
-                if (!FOLD && tau + (uint32_t)ngr < t_end && inside(next_base())) {
+                const uint64_t nbase = next_base();
+                if (!FOLD && tau + (uint32_t)ngr < S.t_end && inside(nbase)) {
                     mode |= kWideMore;
-                    nsrc = reinterpret_cast<const char *>(amps) + (next_base() * 8u + S.toff[tid]);
+                    nsrc = reinterpret_cast<const char *>(S.amps + (nbase * 8u + S.toff[tid]));
                 }
             }
             OpLoop<KIND>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16,
@@ -313,9 +320,9 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         // thread touches it before the next barrier) ----
         if (!S.P.direct) {
             const uint64_t toff = S.toff[tid], nbase = next_base();
-            const bool more = !FOLD && tau + (uint32_t)ngr < t_end && inside(nbase), canon_out = S.P.canon_out != 0;
-            char *dst = reinterpret_cast<char *>(amps) + (base * 8u + toff);
-            const char *src = reinterpret_cast<const char *>(amps) + (nbase * 8u + toff);
+            const bool more = !FOLD && tau + (uint32_t)ngr < S.t_end && inside(nbase), canon_out = S.P.canon_out != 0;
+            char *dst = reinterpret_cast<char *>(S.amps + (this_base() * 8u + toff));
+            const char *src = reinterpret_cast<const char *>(S.amps + (nbase * 8u + toff));
 #pragma unroll 4
             for (int i0 = 0; i0 < NU; i0 += 2) {
                 WideUnit u[2];
