@@ -112,9 +112,11 @@ static std::map<std::tuple<int, int, int>, int> g_tuned_tile;
 // is only the Hadamard layer.
 static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const uint64_t *offsets,
                                 const std::vector<size_t> &hl, const std::vector<int> &idx,
-                                const std::vector<int> &tbits, std::vector<Plan> *plans)
+                                const std::vector<int> &tbits, std::vector<Plan> *plans,
+                                std::vector<FoldArgs> *folds)
 {
     plans->assign(b->count, Plan());
+    folds->assign(b->count, FoldArgs{});
     // one kernel runs every pass of a launch: wide passes when every listed
     // instance's tile fills whole warps of them, else five register bits
     bool wide = true;
@@ -136,6 +138,21 @@ static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const u
                 if (!wide) {
                     pp.r = std::min(5, pp.t);
                     pp.pack0 = 0;
+                }
+                // wide passes: the leading layer and the diagonal prefix after it
+                // are generated by the instance's first pass (nfold = -1: a
+                // generated uniform state)
+                std::vector<qs_gate> rest;
+                if (wide && hl[i]) {
+                    FoldArgs f;
+                    const size_t nf = fold_diagonal_prefix(gates + offsets[i] + hl[i], ng, &rest, &f);
+                    if (!rest.empty()) {
+                        (*folds)[i] = f;
+                        (*folds)[i].nfold = nf ? (int)nf : -1;
+                        st[k] = build_plan(pp, rest.data(), rest.size(), &(*plans)[i]);
+                        if (st[k]) msg[k] = last_error_cstr();
+                        continue;
+                    }
                 }
                 st[k] = build_plan(pp, gates + offsets[i] + hl[i], ng, &(*plans)[i]);
                 if (st[k]) msg[k] = last_error_cstr();
@@ -167,12 +184,27 @@ struct Rounds {
 
 // Lowers the listed instances' plans in list order (the order in which
 // their passes are concatenated) when all are wide passes; else empty.
-static void lower_instances(const std::vector<Plan> &plans, const std::vector<int> &idx, WidePlan *out)
+static void lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds,
+                            const std::vector<int> &idx, WidePlan *out)
 {
     *out = WidePlan();
     for (int i : idx)
         if (!plans[i].passes.empty() && !wide_plan(plans[i].passes, plans[i].phases)) return;
-    for (int i : idx) lower_wide(plans[i].passes, plans[i].phases, plans[i].ops, out);
+    for (int i : idx) {
+        const size_t first = out->passes.size();
+        lower_wide(plans[i].passes, plans[i].phases, plans[i].ops, out);
+        if (!folds[i].nfold || out->passes.size() == first) continue;
+        out->folds.push_back(folds[i]);
+        out->passes[first].fold = (int32_t)out->folds.size();
+        out->passes[first].canon_in = 0;
+    }
+}
+
+// Instances whose first pass generates their state need no initial chunks.
+static void drop_initial_chunks(const std::vector<FoldArgs> &folds, Work *W)
+{
+    for (PersistItem &w : W->items)
+        if (w.kind == kPersistInit && folds[w.inst].nfold) w.lo = 0;
 }
 
 static bool any_full(const WidePlan &w)
@@ -182,8 +214,8 @@ static bool any_full(const WidePlan &w)
     return false;
 }
 
-static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, const std::vector<int> &idx,
-                         Rounds *R)
+static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds,
+                         const std::vector<int> &idx, Rounds *R)
 {
     *R = Rounds();
     std::vector<int> first_pass(b->count, 0);
@@ -204,7 +236,7 @@ static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, cons
         max_passes = std::max(max_passes, (int)plans[i].passes.size());
         R->bytes += (double)plans[i].passes.size() * 16.0 * std::ldexp(1.0, b->n[i]);
     }
-    lower_instances(plans, idx, &R->wide);
+    lower_instances(plans, folds, idx, &R->wide);
     const size_t isz = batch_item_bytes();
     for (int r = 0; r < max_passes; ++r)
         for (int tb = 5; tb <= 13; ++tb) {
@@ -230,7 +262,7 @@ static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, cons
 // Section offsets of a packed run in a device buffer: passes | phases | ops
 // (wide: passes | codes | records) | items, each 256-byte aligned.
 struct RoundOffsets {
-    size_t pass, phase, op, item, total;
+    size_t pass, phase, op, fold, item, total;
 };
 template <class T>
 static RoundOffsets pack_offsets(const T &R, const WidePlan &w, size_t item_bytes)
@@ -241,7 +273,8 @@ static RoundOffsets pack_offsets(const T &R, const WidePlan &w, size_t item_byte
     o.pass = 0;
     o.phase = align(o.pass + (wide ? w.passes.size() * sizeof(WidePass) : R.passes.size() * sizeof(DevPass)));
     o.op = align(o.phase + (wide ? w.codes.size() : R.phases.size() * sizeof(DevPhase)));
-    o.item = align(o.op + (wide ? w.ops.size() * sizeof(WideOp) : R.ops.size() * sizeof(DevOp)));
+    o.fold = align(o.op + (wide ? w.ops.size() * sizeof(WideOp) : R.ops.size() * sizeof(DevOp)));
+    o.item = align(o.fold + w.folds.size() * sizeof(FoldArgs));
     o.total = align(o.item + item_bytes);
     return o;
 }
@@ -253,6 +286,7 @@ static void pack_run(const T &R, const WidePlan &w, const RoundOffsets &o, const
         std::memcpy(host + o.pass, w.passes.data(), w.passes.size() * sizeof(WidePass));
         std::memcpy(host + o.phase, w.codes.data(), w.codes.size());
         std::memcpy(host + o.op, w.ops.data(), w.ops.size() * sizeof(WideOp));
+        if (!w.folds.empty()) std::memcpy(host + o.fold, w.folds.data(), w.folds.size() * sizeof(FoldArgs));
     } else {
         std::memcpy(host + o.pass, R.passes.data(), R.passes.size() * sizeof(DevPass));
         std::memcpy(host + o.phase, R.phases.data(), R.phases.size() * sizeof(DevPhase));
@@ -276,7 +310,8 @@ static qs_status launch_rounds(const qs_batch *b, cudaStream_t st, const Rounds 
         for (const RoundLaunch &L : R.launches)
             if (qs_status rs = launch_batch_round_wide(st, b->num_sms, b->amps, D + o.item + L.first * isz, (int)L.count,
                                                        L.tbits, (const WidePass *)(D + o.pass),
-                                                       (const WideOp *)(D + o.op), D + o.phase, full))
+                                                       (const WideOp *)(D + o.op), D + o.phase,
+                                                       (const FoldArgs *)(D + o.fold), full))
                 return rs;
         return QS_OK;
     }
@@ -317,8 +352,8 @@ static qs_status launch_work(const qs_batch *b, cudaStream_t st, const Work &W, 
     if (!wide.passes.empty())
         return launch_batch_persistent_wide(st, b->num_sms, b->amps, (const PersistItem *)(D + o.item),
                                             (int)W.items.size(), (const WidePass *)(D + o.pass),
-                                            (const WideOp *)(D + o.op), D + o.phase, sync + sizeof(PersistCtl) / 4,
-                                            (PersistCtl *)sync, part, sums, any_full(wide));
+                                            (const WideOp *)(D + o.op), D + o.phase, (const FoldArgs *)(D + o.fold),
+                                            sync + sizeof(PersistCtl) / 4, (PersistCtl *)sync, part, sums, any_full(wide));
     bool full = false;
     for (const PersistItem &w : W.items) full = full || w.kind == kPersistPassFull;
     return launch_batch_persistent(st, b->num_sms, b->amps, (const PersistItem *)(D + o.item), (int)W.items.size(),
@@ -339,7 +374,8 @@ static qs_status work_error(const uint32_t *sync)
 // One untimed and one timed run (CUDA events) of the listed instances'
 // evolution with the given plans on the batch's engine; *ms = the timed
 // run.  The runs overwrite those instances' states.
-static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const std::vector<int> &idx,
+static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds,
+                            const std::vector<int> &idx,
                             const std::vector<size_t> &hl, cudaEvent_t e0, cudaEvent_t e1, float *ms, bool *empty)
 {
     Rounds R;
@@ -348,7 +384,7 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
     RoundOffsets o;
     std::vector<unsigned char> host;
     if (b->engine == QS_BATCH_ROUNDS) {
-        build_rounds(b, plans, idx, &R);
+        build_rounds(b, plans, folds, idx, &R);
         *empty = R.launches.empty();
         o = round_offsets(R);
         host.assign(o.total, 0);
@@ -356,7 +392,8 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
     } else {
         build_work(b->n, b->off, plans, full_flags(plans), idx, hl, false, &W);
         *empty = W.passes.empty();
-        lower_instances(plans, idx, &wide);
+        lower_instances(plans, folds, idx, &wide);
+        drop_initial_chunks(folds, &W);
         o = work_offsets(W, wide);
         host.assign(o.total, 0);
         work_pack(W, wide, o, host.data());
@@ -424,10 +461,11 @@ static qs_status batch_autotune(qs_batch *b, const qs_gate *gates, const uint64_
         for (int t = std::min(9, n); t <= std::min(13, n); ++t) {
             std::vector<int> tb(b->count, t);
             std::vector<Plan> plans;
-            if ((rc = plan_instances(b, gates, offsets, hl, kv.second, tb, &plans))) break;
+            std::vector<FoldArgs> folds;
+            if ((rc = plan_instances(b, gates, offsets, hl, kv.second, tb, &plans, &folds))) break;
             float ms = 0;
             bool empty = false;
-            if ((rc = time_plans(b, plans, kv.second, hl, e0, e1, &ms, &empty))) break;
+            if ((rc = time_plans(b, plans, folds, kv.second, hl, e0, e1, &ms, &empty))) break;
             if (empty) break;                       // only Hadamard layers: nothing to time
             if (ms < best_ms) {
                 best_ms = ms;
@@ -643,7 +681,8 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
         if (b->autotune && b->tile_for_n.count(b->n[i])) tbits[i] = b->tile_for_n[b->n[i]];
     }
     std::vector<Plan> plans;
-    if (qs_status s0 = plan_instances(b, gates, offsets, hl, all, tbits, &plans)) return s0;
+    std::vector<FoldArgs> folds;
+    if (qs_status s0 = plan_instances(b, gates, offsets, hl, all, tbits, &plans, &folds)) return s0;
     b->tile_used.assign(C, 0);
     for (int i = 0; i < C; ++i)
         if (!plans[i].passes.empty()) b->tile_used[i] = plans[i].passes[0].t;
@@ -653,7 +692,8 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
         build_work(b->n, b->off, plans, full_flags(plans), all, hl, true, &W);
         b->round_bytes = W.bytes;
         WidePlan wide;
-        lower_instances(plans, all, &wide);
+        lower_instances(plans, folds, all, &wide);
+        drop_initial_chunks(folds, &W);
         const RoundOffsets wo = work_offsets(W, wide);
         std::vector<unsigned char> host(wo.total, 0);
         work_pack(W, wide, wo, host.data());
@@ -670,7 +710,7 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
         return batch_end_capture(b, rs);
     }
     Rounds R;
-    build_rounds(b, plans, all, &R);
+    build_rounds(b, plans, folds, all, &R);
     b->round_bytes = R.bytes;
     // statistics items
     std::vector<uint64_t> s_off, s_cnt;

@@ -1385,7 +1385,7 @@ static qs_status plan_gates(const PlanParams &pp, const std::vector<PGate> &g, P
         int pass_ops = 0;
         int tc_in_pass = 0;
         // (a lowered wide pass holds an end code per phase too)
-        const int max_ops = pp.pack0 ? kMaxOpsPerPass - kMaxPhasesPerPass : kMaxOpsPerPass;
+        const int max_ops = pp.pack0 ? kMaxWideOps - kMaxPhasesPerPass : kMaxOpsPerPass;
         // wide passes: all phases are chosen ahead, with a last phase that can
         // store to the state where that takes no more phases (37 of 51 passes
         // of five 30-qubit circuits; 13 would take one more)

@@ -223,6 +223,7 @@ QS_HD inline uint32_t tile_swizzle(uint32_t e, uint32_t CE)
 // and 16-byte records, so the kernel's staging is a copy.
 // ---------------------------------------------------------------------------
 constexpr int kWideRegBits = 6;
+constexpr int kMaxWideOps = 216;        // ops of a pass, end codes included (shared memory)
 constexpr int kWideMinTile = 11;        // tiles of whole warps (2^(t - 6) threads)
 
 struct WideOp {             // 16 bytes
@@ -259,7 +260,7 @@ struct WidePass {
     int32_t canon_in, canon_out; // the pass reads / writes canonical units
                                  // (re, im, re, im), else (re, re, im, im)
     int32_t direct;              // the last phase stores to the state
-    int32_t pad;
+    int32_t fold;                // batches: the pass generates its tiles (prefix fold - 1)
     uint8_t L[kMaxTileBits];     // qubit of each tile bit (ascending)
     uint8_t G[32];               // qubits outside the tile (ascending)
     uint64_t dreg[kWideRegBits]; // byte offset in the state of the last phase's register bits
@@ -288,6 +289,7 @@ struct WidePlan {
     std::vector<WidePass> passes;
     std::vector<WideOp> ops;
     std::vector<uint8_t> codes;
+    std::vector<FoldArgs> folds;     // batches: folded prefixes (WidePass::fold)
 };
 // Whether a plan's passes can run the wide form: six register bits, register
 // phases only, tiles of at least 2^kWideMinTile.
@@ -582,10 +584,11 @@ qs_status launch_batch_persistent(cudaStream_t st, int num_sms, void *amps, cons
 // SM, every tile of at least 2^kWideMinTile amplitudes.
 qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, const void *items, int nitems,
                                   int tile_bits, const WidePass *passes, const WideOp *ops, const uint8_t *codes,
-                                  bool full);
+                                  const FoldArgs *folds, bool full);
 qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
                                        const WidePass *passes, const WideOp *ops, const uint8_t *codes,
-                                       uint32_t *done, PersistCtl *ctl, double *part, double *sums, bool any_full);
+                                       const FoldArgs *folds, uint32_t *done, PersistCtl *ctl, double *part,
+                                       double *sums, bool any_full);
 qs_status batch_wide_setup();
 // Resident CTAs per SM of the persistent kernel (after batch_kernel_setup).
 int batch_persistent_ctas_per_sm(bool any_full);

@@ -28,9 +28,9 @@ k_wide_pass(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g, cons
             F.m[1] = fold.m2;
             F.m[2] = fold.m4;
         }
-        wide_pass_body<FULL ? 1 : 0, true, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 1, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
     } else {
-        wide_pass_body<FULL ? 1 : 0, false, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 0, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
     }
 }
 
@@ -72,7 +72,7 @@ k_adj_wide(float2 *__restrict__ psi, uint64_t lam_off, const WidePass *__restric
     }
     const uint32_t per = ntiles / gridDim.x, extra = ntiles % gridDim.x;
     const uint32_t t_begin = blockIdx.x * per + (blockIdx.x < extra ? blockIdx.x : extra);
-    wide_pass_body<2, false, false>(psi, pass_g, ops_g, codes_g, t_begin,
+    wide_pass_body<2, 0, false>(psi, pass_g, ops_g, codes_g, t_begin,
                                     t_begin + per + (blockIdx.x < extra ? 1 : 0), S, nullptr, smem_dyn, lam_off);
 }
 
@@ -102,14 +102,15 @@ template <bool FULL>
 __global__ void __launch_bounds__(kWideThreads, 3)
 k_batch_pass_wide(float2 *__restrict__ amps, const BatchItem *__restrict__ items, int nitems,
                   const WidePass *__restrict__ passes, const WideOp *__restrict__ ops,
-                  const uint8_t *__restrict__ codes)
+                  const uint8_t *__restrict__ codes, const FoldArgs *__restrict__ folds)
 {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     __shared__ WideSmem S;
+    __shared__ WideFoldSmem F;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const BatchItem w = items[it];
-        wide_pass_body<FULL ? 1 : 0, false, false>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
-                                           nullptr, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 2, false>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
+                                               &F, smem_dyn, 0, folds);
     }
 }
 
@@ -121,11 +122,12 @@ template <bool FULL>
 __global__ void __launch_bounds__(kWideThreads, 3)
 k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int nitems,
                         const WidePass *__restrict__ passes, const WideOp *__restrict__ ops,
-                        const uint8_t *__restrict__ codes, uint32_t *done, PersistCtl *ctl, double *part, double *sums,
-                        uint64_t wait_ns)
+                        const uint8_t *__restrict__ codes, const FoldArgs *__restrict__ folds, uint32_t *done,
+                        PersistCtl *ctl, double *part, double *sums, uint64_t wait_ns)
 {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
     __shared__ WideSmem S;
+    __shared__ WideFoldSmem F;
     __shared__ int s_item, s_go, s_last;
     __shared__ PersistItem w;        // the item: no registers held across a pass
     for (;;) {
@@ -150,15 +152,16 @@ k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int
         __syncthreads();
         if (s_go) {
             if (w.kind == kPersistInit) {
+                // (lo = 0: the instance's first pass generates its state)
                 float4 *a = reinterpret_cast<float4 *>(amps + w.amp_off);
                 const float4 u = make_float4(w.f0, 0.f, w.f0, 0.f);
                 for (uint32_t e = threadIdx.x; e < w.lo / 2; e += blockDim.x) a[e] = u;
-                if (threadIdx.x == 0) a[0] = make_float4(w.f1, 0.f, w.f0, 0.f);
+                if (threadIdx.x == 0 && w.lo) a[0] = make_float4(w.f1, 0.f, w.f0, 0.f);
             } else if (w.kind == kPersistStats) {
                 batch_stats_chunk<kWideThreads>(amps + w.amp_off, w.lo, w.f0, part + (size_t)w.pass * kStatAcc);
             } else {
-                wide_pass_body<FULL ? 1 : 0, false, true>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, nullptr,
-                                                  smem_dyn);
+                wide_pass_body<FULL ? 1 : 0, 2, true>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, &F,
+                                                      smem_dyn, 0, folds);
             }
         }
         __syncthreads();
@@ -183,13 +186,13 @@ k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int
 
 qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, const void *items, int nitems,
                                   int tile_bits, const WidePass *passes, const WideOp *ops, const uint8_t *codes,
-                                  bool full)
+                                  const FoldArgs *folds, bool full)
 {
     if (tile_bits < kWideMinTile || tile_bits > 13) return set_error(QS_ERR_INVALID_ARG, "batch tile bits %d", tile_bits);
     auto kern = full ? k_batch_pass_wide<true> : k_batch_pass_wide<false>;
     const int cap = num_sms * 3;
     kern<<<nitems < cap ? nitems : cap, 1 << (tile_bits - kWideRegBits), (size_t(1) << tile_bits) * sizeof(float2), st>>>(
-        (float2 *)amps, (const BatchItem *)items, nitems, passes, ops, codes);
+        (float2 *)amps, (const BatchItem *)items, nitems, passes, ops, codes, folds);
     QS_LAUNCH_CHECK();
     return QS_OK;
 }
@@ -200,13 +203,14 @@ static int g_wide_per_sm[2] = {3, 3};
 
 qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
                                        const WidePass *passes, const WideOp *ops, const uint8_t *codes,
-                                       uint32_t *done, PersistCtl *ctl, double *part, double *sums, bool any_full)
+                                       const FoldArgs *folds, uint32_t *done, PersistCtl *ctl, double *part,
+                                       double *sums, bool any_full)
 {
     if (nitems <= 0) return QS_OK;
     const int cap = num_sms * g_wide_per_sm[any_full ? 1 : 0];
     auto kern = any_full ? k_batch_persistent_wide<true> : k_batch_persistent_wide<false>;
-    kern<<<nitems < cap ? nitems : cap, kWideThreads, 65536, st>>>((float2 *)amps, items, nitems, passes, ops, codes, done,
-                                                                   ctl, part, sums, kPersistWaitNs);
+    kern<<<nitems < cap ? nitems : cap, kWideThreads, 65536, st>>>((float2 *)amps, items, nitems, passes, ops, codes, folds,
+                                                                   done, ctl, part, sums, kPersistWaitNs);
     QS_LAUNCH_CHECK();
     return QS_OK;
 }

@@ -36,8 +36,8 @@ struct alignas(16) WideUnit {           // unit `it` of every thread
 
 struct WideSmem {
     WidePass P;
-    WideOp ops[kMaxOpsPerPass];
-    uint32_t codes[kMaxOpsPerPass / 4 + 4];
+    WideOp ops[kMaxWideOps];
+    uint32_t codes[kMaxWideOps / 4 + 4];
     uint64_t toff[kWideThreads];                     // byte offset in the state of the thread's first copied unit
     uint64_t doff[kWideThreads];                     // ... of its slot 0 in the last phase
     uint64_t dst[kWideThreads];                      // state address of the thread's slot 0 of this tile
@@ -80,24 +80,40 @@ __device__ __forceinline__ void wide_sync(int nthr, int gi)
 // Runs tiles [t_begin, t_end) of one pass on `amps`.  blockDim.x threads; a
 // tile takes 2^(t - 6) of them: all (GROUPED = false), or a group of whole
 // warps (t >= 11) with its own tile buffer, group g running tiles t_begin +
-// g, + groups, ...  FOLD: the circuit's first pass, which writes its tiles
+// g, + groups, ...  FOLD 1: a circuit's first pass, which writes its tiles
 // (the uniform state times the folded prefix's phases) instead of loading
 // them; F's nb and m are set by the caller (published by the first barrier).
+// FOLD 2: the same where the pass says so (its prefix in folds_g).
 // The caller's CTA is converged; ends with a CTA barrier.
 // KIND: the op loop (0 Clifford+T, 1 all gates, 2 the adjoint sweep, whose
 // tile bit t - 1 selects psi or lambda, lam_off bytes away; S.part and
 // S.part_stride are set by the caller).
-template <int KIND, bool FOLD, bool GROUPED>
+template <int KIND, int FOLD, bool GROUPED>
 __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g,
                                                const WideOp *__restrict__ ops_g, const uint8_t *__restrict__ codes_g,
                                                uint32_t t_begin, uint32_t t_end, WideSmem &S, WideFoldSmem *F,
-                                               unsigned char *smem_raw, uint64_t lam_off = 0)
+                                               unsigned char *smem_raw, uint64_t lam_off = 0,
+                                               const FoldArgs *__restrict__ folds_g = nullptr)
 {
     constexpr int RB = kWideRegBits, NS = kWideSlots, NU = kWideUnits;
     for (int i = threadIdx.x; i < (int)(sizeof(WidePass) / 4); i += blockDim.x)
         reinterpret_cast<uint32_t *>(&S.P)[i] = reinterpret_cast<const uint32_t *>(pass_g)[i];
     __syncthreads();
     const int t = S.P.t, ng = S.P.n - t, nph = S.P.nphases, nops = S.P.nops;
+    // whether the tiles are generated
+    auto gen = [&]() { return FOLD == 1 || (FOLD == 2 && S.P.fold != 0); };
+    if constexpr (FOLD == 2) {
+        if (S.P.fold) {
+            const FoldArgs &f = folds_g[S.P.fold - 1];
+            for (int i = threadIdx.x; i < kMaxQubits; i += blockDim.x) F->nb[i] = f.nb[i];
+            if (threadIdx.x == 0) {
+                F->m[0] = f.m1;
+                F->m[1] = f.m2;
+                F->m[2] = f.m4;
+            }
+            __syncthreads();
+        }
+    }
     const int nthr = GROUPED ? 1 << (t - RB) : (int)blockDim.x;
     const int tid = GROUPED ? (int)(threadIdx.x & (unsigned)(nthr - 1)) : (int)threadIdx.x;
     const int gi = GROUPED ? (int)(threadIdx.x >> (t - RB)) : 0;
@@ -137,7 +153,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
     auto fcount = [&](int q) -> uint32_t {
         return (uint32_t)((F->m[0] >> q) & 1) + 2u * (uint32_t)((F->m[1] >> q) & 1) + 4u * (uint32_t)((F->m[2] >> q) & 1);
     };
-    if constexpr (FOLD) {
+    if (FOLD && gen()) {
         // each qubit's CZ partners as tile bits
         for (int q = threadIdx.x; q < S.P.n; q += blockDim.x) {
             uint32_t m = 0;
@@ -193,7 +209,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         (void)b;
         return QS_DCHECK(((b | lmask) >> S.P.n) == 0, 202);
     };
-    if constexpr (!FOLD) {
+    if (!gen()) {
         if (tau < S.t_end && inside(base)) {
             const char *src = reinterpret_cast<const char *>(amps) + (base * 8u + S.toff[tid]);
 #pragma unroll 4
@@ -205,7 +221,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
     }
     while (tau < S.t_end && inside(base)) {
         S.dst[threadIdx.x] = S.amps + base * 8u + S.doff[tid];
-        if constexpr (FOLD) {
+        if (FOLD && gen()) {
             // element x gets 2^(-n/2) e^{i pi k(x) / 4}, k = 4 (CZ pairs within
             // x) + (T counts of x), mod 8, summed over the out-of-tile bits,
             // the thread's tile bits and the unit's, plus the pairs across
@@ -241,7 +257,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             }
         }
         asm volatile("cp.async.wait_all;\n" ::: "memory");
-        if (!FOLD && S.P.canon_in) {
+        if (FOLD != 1 && S.P.canon_in) {
             // the units this thread copied, to the order the phases work on
 #pragma unroll 4
             for (int it = 0; it < NU; ++it) {
@@ -299,7 +315,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             if (direct) {
                 mode |= kWideDirect | (S.P.canon_out ? kWideCanon : 0u);
                 const uint64_t nbase = next_base();
-                if (!FOLD && tau + (uint32_t)ngr < S.t_end && inside(nbase)) {
+                if (!gen() && tau + (uint32_t)ngr < S.t_end && inside(nbase)) {
                     mode |= kWideMore;
                     nsrc = reinterpret_cast<const char *>(S.amps + (nbase * 8u + S.toff[tid]));
                 }
@@ -320,7 +336,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         // thread touches it before the next barrier) ----
         if (!S.P.direct) {
             const uint64_t toff = S.toff[tid], nbase = next_base();
-            const bool more = !FOLD && tau + (uint32_t)ngr < S.t_end && inside(nbase), canon_out = S.P.canon_out != 0;
+            const bool more = !gen() && tau + (uint32_t)ngr < S.t_end && inside(nbase), canon_out = S.P.canon_out != 0;
             char *dst = reinterpret_cast<char *>(S.amps + (this_base() * 8u + toff));
             const char *src = reinterpret_cast<const char *>(S.amps + (nbase * 8u + toff));
 #pragma unroll 4
