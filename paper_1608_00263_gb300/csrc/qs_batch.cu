@@ -207,6 +207,14 @@ static void drop_initial_chunks(const std::vector<FoldArgs> &folds, Work *W)
         if (w.kind == kPersistInit && folds[w.inst].nfold) w.lo = 0;
 }
 
+// Whether some pass has several tiles smaller than a CTA's.
+static bool needs_groups(const WidePlan &w)
+{
+    for (const WidePass &p : w.passes)
+        if (p.t < 13 && p.n > p.t) return true;
+    return false;
+}
+
 static bool any_full(const WidePlan &w)
 {
     for (const WidePass &p : w.passes)
@@ -353,7 +361,7 @@ static qs_status launch_work(const qs_batch *b, cudaStream_t st, const Work &W, 
         return launch_batch_persistent_wide(st, b->num_sms, b->amps, (const PersistItem *)(D + o.item),
                                             (int)W.items.size(), (const WidePass *)(D + o.pass),
                                             (const WideOp *)(D + o.op), D + o.phase, (const FoldArgs *)(D + o.fold),
-                                            sync + sizeof(PersistCtl) / 4, (PersistCtl *)sync, part, sums, any_full(wide));
+                                            sync + sizeof(PersistCtl) / 4, (PersistCtl *)sync, part, sums, any_full(wide), needs_groups(wide));
     bool full = false;
     for (const PersistItem &w : W.items) full = full || w.kind == kPersistPassFull;
     return launch_batch_persistent(st, b->num_sms, b->amps, (const PersistItem *)(D + o.item), (int)W.items.size(),

@@ -581,14 +581,16 @@ qs_status launch_batch_persistent(cudaStream_t st, int num_sms, void *amps, cons
                                   const DevPass *passes, const DevPhase *phases, const DevOp *ops,
                                   uint32_t *done, PersistCtl *ctl, double *part, double *sums, bool any_full);
 // The same engines on lowered plans (wide passes): 128-thread CTAs, three per
-// SM, every tile of at least 2^kWideMinTile amplitudes.
+// SM, every tile of at least 2^kWideMinTile amplitudes.  grouped: some pass
+// has several tiles smaller than a CTA's (they run side by side in groups of
+// its threads; a single small tile takes part of the threads instead).
 qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, const void *items, int nitems,
                                   int tile_bits, const WidePass *passes, const WideOp *ops, const uint8_t *codes,
                                   const FoldArgs *folds, bool full);
 qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
                                        const WidePass *passes, const WideOp *ops, const uint8_t *codes,
                                        const FoldArgs *folds, uint32_t *done, PersistCtl *ctl, double *part,
-                                       double *sums, bool any_full);
+                                       double *sums, bool any_full, bool grouped);
 qs_status batch_wide_setup();
 // Resident CTAs per SM of the persistent kernel (after batch_kernel_setup).
 int batch_persistent_ctas_per_sm(bool any_full);

@@ -28,9 +28,9 @@ k_wide_pass(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g, cons
             F.m[1] = fold.m2;
             F.m[2] = fold.m4;
         }
-        wide_pass_body<FULL ? 1 : 0, 1, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 1, 0>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
     } else {
-        wide_pass_body<FULL ? 1 : 0, 0, false>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 0, 0>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
     }
 }
 
@@ -72,7 +72,7 @@ k_adj_wide(float2 *__restrict__ psi, uint64_t lam_off, const WidePass *__restric
     }
     const uint32_t per = ntiles / gridDim.x, extra = ntiles % gridDim.x;
     const uint32_t t_begin = blockIdx.x * per + (blockIdx.x < extra ? blockIdx.x : extra);
-    wide_pass_body<2, 0, false>(psi, pass_g, ops_g, codes_g, t_begin,
+    wide_pass_body<2, 0, 0>(psi, pass_g, ops_g, codes_g, t_begin,
                                     t_begin + per + (blockIdx.x < extra ? 1 : 0), S, nullptr, smem_dyn, lam_off);
 }
 
@@ -109,7 +109,7 @@ k_batch_pass_wide(float2 *__restrict__ amps, const BatchItem *__restrict__ items
     __shared__ WideFoldSmem F;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const BatchItem w = items[it];
-        wide_pass_body<FULL ? 1 : 0, 2, false>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
+        wide_pass_body<FULL ? 1 : 0, 2, 0>(amps + w.amp_off, passes + w.pass, ops, codes, w.tile_begin, w.tile_end, S,
                                                &F, smem_dyn, 0, folds);
     }
 }
@@ -117,8 +117,8 @@ k_batch_pass_wide(float2 *__restrict__ amps, const BatchItem *__restrict__ items
 // Persistent engine (PersistItem, see k_batch_persistent): the same queue,
 // dependency waits and completion counts with CTAs of kWideThreads threads,
 // three per SM.  FULL: some item's pass holds parameterised gates; the loop
-// that knows them then runs every pass.
-template <bool FULL>
+// that knows them then runs every pass.  GROUPED as in wide_pass_body.
+template <bool FULL, int GROUPED>
 __global__ void __launch_bounds__(kWideThreads, 3)
 k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int nitems,
                         const WidePass *__restrict__ passes, const WideOp *__restrict__ ops,
@@ -160,7 +160,7 @@ k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int
             } else if (w.kind == kPersistStats) {
                 batch_stats_chunk<kWideThreads>(amps + w.amp_off, w.lo, w.f0, part + (size_t)w.pass * kStatAcc);
             } else {
-                wide_pass_body<FULL ? 1 : 0, 2, true>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, &F,
+                wide_pass_body<FULL ? 1 : 0, 2, GROUPED>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, &F,
                                                       smem_dyn, 0, folds);
             }
         }
@@ -197,20 +197,27 @@ qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, cons
     return QS_OK;
 }
 
-// Resident CTAs per SM of the two persistent variants (occupancy API, set by
-// batch_wide_setup before any launch or capture).
-static int g_wide_per_sm[2] = {3, 3};
+// The persistent kernel by (parameterised gates, tiles in groups): with thread
+// groups the tile stride, the barrier id and the buffer address are per-thread
+// values and the kernel spills (512 bytes of reloads, 1004 with parameterised
+// gates); without, 308 and 404.  64 instances of 20 qubits 2.01 -> 1.87 ms,
+// eight of 23 2.16 -> 1.97 ms (lockstep rounds: 1.88 and 1.98).  Resident
+// CTAs per SM of each (occupancy API, set by batch_wide_setup before any
+// launch or capture).
+static decltype(&k_batch_persistent_wide<false, 2>) const g_wide_kern[2][2] = {
+    {k_batch_persistent_wide<false, 2>, k_batch_persistent_wide<false, 1>},
+    {k_batch_persistent_wide<true, 2>, k_batch_persistent_wide<true, 1>}};
+static int g_wide_per_sm[2][2] = {{3, 3}, {3, 3}};
 
 qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps, const PersistItem *items, int nitems,
                                        const WidePass *passes, const WideOp *ops, const uint8_t *codes,
                                        const FoldArgs *folds, uint32_t *done, PersistCtl *ctl, double *part,
-                                       double *sums, bool any_full)
+                                       double *sums, bool any_full, bool grouped)
 {
     if (nitems <= 0) return QS_OK;
-    const int cap = num_sms * g_wide_per_sm[any_full ? 1 : 0];
-    auto kern = any_full ? k_batch_persistent_wide<true> : k_batch_persistent_wide<false>;
-    kern<<<nitems < cap ? nitems : cap, kWideThreads, 65536, st>>>((float2 *)amps, items, nitems, passes, ops, codes, folds,
-                                                                   done, ctl, part, sums, kPersistWaitNs);
+    const int cap = num_sms * g_wide_per_sm[any_full][grouped];
+    g_wide_kern[any_full][grouped]<<<nitems < cap ? nitems : cap, kWideThreads, 65536, st>>>(
+        (float2 *)amps, items, nitems, passes, ops, codes, folds, done, ctl, part, sums, kPersistWaitNs);
     QS_LAUNCH_CHECK();
     return QS_OK;
 }
@@ -218,15 +225,15 @@ qs_status launch_batch_persistent_wide(cudaStream_t st, int num_sms, void *amps,
 qs_status batch_wide_setup()
 {
     const int dyn = 65536;
-    QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_persistent_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_persistent_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
     QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_pass_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
     QS_CUDA_TRY(cudaFuncSetAttribute(k_batch_pass_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    QS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_wide_per_sm[0], k_batch_persistent_wide<false>,
-                                                              kWideThreads, dyn));
-    QS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&g_wide_per_sm[1], k_batch_persistent_wide<true>,
-                                                              kWideThreads, dyn));
-    for (int &v : g_wide_per_sm) v = v < 1 ? 1 : v;
+    for (int f = 0; f < 2; ++f)
+        for (int g = 0; g < 2; ++g) {
+            QS_CUDA_TRY(cudaFuncSetAttribute(g_wide_kern[f][g], cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+            int &v = g_wide_per_sm[f][g];
+            QS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, g_wide_kern[f][g], kWideThreads, dyn));
+            v = v < 1 ? 1 : v;
+        }
     return QS_OK;
 }
 

@@ -70,17 +70,19 @@ struct WideFoldSmem {
 __device__ __forceinline__ float4 swap_unit(float4 v) { return make_float4(v.x, v.z, v.y, v.w); }
 
 // Barrier of a tile's threads: the CTA, or its group of whole warps.
-template <bool GROUPED>
+template <int GROUPED>
 __device__ __forceinline__ void wide_sync(int nthr, int gi)
 {
-    if constexpr (!GROUPED) __syncthreads();
+    if constexpr (GROUPED == 0) __syncthreads();
     else asm volatile("bar.sync %0, %1;" ::"r"(gi + 1), "r"(nthr) : "memory");
 }
 
 // Runs tiles [t_begin, t_end) of one pass on `amps`.  blockDim.x threads; a
-// tile takes 2^(t - 6) of them: all (GROUPED = false), or a group of whole
-// warps (t >= 11) with its own tile buffer, group g running tiles t_begin +
-// g, + groups, ...  FOLD 1: a circuit's first pass, which writes its tiles
+// tile takes 2^(t - 6) of them: all (GROUPED 0), a group of whole warps (t >=
+// 11) with its own tile buffer, group g running tiles t_begin + g, + groups,
+// ... (GROUPED 1), or the first ones, the others idle (GROUPED 2: fewer
+// registers than groups; for passes of one small tile).
+// FOLD 1: a circuit's first pass, which writes its tiles
 // (the uniform state times the folded prefix's phases) instead of loading
 // them; F's nb and m are set by the caller (published by the first barrier).
 // FOLD 2: the same where the pass says so (its prefix in folds_g).
@@ -88,7 +90,7 @@ __device__ __forceinline__ void wide_sync(int nthr, int gi)
 // KIND: the op loop (0 Clifford+T, 1 all gates, 2 the adjoint sweep, whose
 // tile bit t - 1 selects psi or lambda, lam_off bytes away; S.part and
 // S.part_stride are set by the caller).
-template <int KIND, int FOLD, bool GROUPED>
+template <int KIND, int FOLD, int GROUPED>
 __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g,
                                                const WideOp *__restrict__ ops_g, const uint8_t *__restrict__ codes_g,
                                                uint32_t t_begin, uint32_t t_end, WideSmem &S, WideFoldSmem *F,
@@ -115,9 +117,10 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         }
     }
     const int nthr = GROUPED ? 1 << (t - RB) : (int)blockDim.x;
-    const int tid = GROUPED ? (int)(threadIdx.x & (unsigned)(nthr - 1)) : (int)threadIdx.x;
-    const int gi = GROUPED ? (int)(threadIdx.x >> (t - RB)) : 0;
-    const int ngr = GROUPED ? (int)(blockDim.x >> (t - RB)) : 1;
+    const int tid = GROUPED == 1 ? (int)(threadIdx.x & (unsigned)(nthr - 1)) : (int)threadIdx.x;
+    const int gi = GROUPED == 1 ? (int)(threadIdx.x >> (t - RB)) : 0;
+    const int ngr = GROUPED == 1 ? (int)(blockDim.x >> (t - RB)) : 1;
+    const bool idle = GROUPED == 2 && (int)threadIdx.x >= nthr;
     // byte offset in the state of tile element e
     auto state_off = [&](uint32_t e) -> uint64_t {
         if constexpr (KIND == 2)
@@ -132,7 +135,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         const uint32_t *cw = reinterpret_cast<const uint32_t *>(codes_g + S.P.op_begin);
         for (int i = threadIdx.x; i < (nops + 7) / 4; i += blockDim.x) S.codes[i] = cw[i];
     }
-    if (gi == 0)
+    if (gi == 0 && !idle)
         for (int ph = 0; ph < nph; ++ph) {
             uint32_t e = 0;
             for (int k = 0; k < t - RB; ++k) e |= (((uint32_t)tid >> k) & 1u) << S.P.ph[ph].T[k];
@@ -181,7 +184,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
             F->w[k] = k < 4 ? make_float2((float)re, (float)im) : make_float2((float)-re, (float)-im);
         }
     }
-    if (gi == 0) {
+    if (gi == 0 && !idle) {
         S.toff[tid] = state_off(2u * (uint32_t)tid);
         S.doff[tid] = state_off(S.thr[nph - 1][tid]);
     }
@@ -194,10 +197,10 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         if constexpr (KIND == 2) S.P.dreg[RB - 1] = lam_off;
     }
     __syncthreads();
-    unsigned char *gsm = GROUPED ? smem_raw + (((size_t)gi << t) * sizeof(float2)) : smem_raw;
+    unsigned char *gsm = GROUPED == 1 ? smem_raw + (((size_t)gi << t) * sizeof(float2)) : smem_raw;
     const uint32_t tile_sa = smem_addr(gsm);
     const uint32_t sw_tid = swz<2>(2u * (uint32_t)tid) * 8u;
-    uint32_t tau = t_begin + (uint32_t)gi;
+    uint32_t tau = idle ? t_end : t_begin + (uint32_t)gi;
     uint64_t base = deposit(tau, S.P.G, ng);
     // the tile's highest element index must lie inside the state
     auto inside = [&](uint64_t b) {
@@ -270,7 +273,7 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
         // next one formed, where they are used)
         auto this_base = [&]() { return (S.dst[threadIdx.x] - S.amps - S.doff[tid]) >> 3; };
         auto next_base = [&]() {
-            return GROUPED && ngr > 1 ? deposit(tau + (uint32_t)ngr, S.P.G, ng)
+            return GROUPED == 1 && ngr > 1 ? deposit(tau + (uint32_t)ngr, S.P.G, ng)
                                       : (((this_base() | ~S.gmask) + 1) & S.gmask);
         };
         for (int ph = 0; ph < nph; ++ph) {

@@ -103,3 +103,27 @@ def test_adjoint_sweep(n):
     for a, b in zip(out[qs.QS_C64], out[qs.QS_C128]):
         assert np.max(np.abs(a - b)) < 1e-4 * np.max(np.abs(b))
         assert np.all(a[g["kind"] < qs.QS_RX] == 0)
+
+
+@pytest.mark.parametrize("kinds", [CT, ALL], ids=["clifford_t", "all"])
+@pytest.mark.parametrize("sizes,tile", [((11, 12, 13, 16, 11), 0), ((14, 11, 12), 11), ((19, 12, 12), 12)])
+def test_batch_engines(sizes, tile, kinds):
+    """Single tiles that take part of a CTA's threads (tile 0), tiles side by
+    side in groups (11, 12), both engines alike."""
+    rng = np.random.default_rng(7 * sum(sizes) + tile)
+    gl = [np.concatenate([O.generate_circuit(1, n, 0, 0)[:n], gate_list(rng, n, 150, kinds)]).astype(qs.GATE_DTYPE)
+          for n in sizes]
+    b = qs.qs_batch_create(sizes)
+    try:
+        qs.qs_batch_set_options(b, tile_log2=tile)
+        rows = {}
+        for engine in (qs.QS_BATCH_PERSISTENT, qs.QS_BATCH_ROUNDS):
+            qs.qs_batch_set_engine(b, engine)
+            rows[engine] = qs.qs_batch_run(b, gl, kmax=4)
+        assert np.array_equal(rows[qs.QS_BATCH_PERSISTENT], rows[qs.QS_BATCH_ROUNDS])
+        for i, n in enumerate(sizes):
+            p = O.probabilities(O.simulate(n, gl[i]))
+            assert rows[qs.QS_BATCH_ROUNDS][i, 1] == pytest.approx(O.entropy(p), rel=1e-6)
+            assert np.allclose(rows[qs.QS_BATCH_ROUNDS][i, 3:], O.moments(p, 4), rtol=1e-5)
+    finally:
+        qs.qs_batch_destroy(b)
