@@ -52,12 +52,14 @@ def _flags(checked=False):
 
 
 def _generate(build_dir):
-    """Writes the generated op loop of the wide pass into the build directory."""
-    spec = importlib.util.spec_from_file_location("gen_op_loop", os.path.join(CSRC, "gen_op_loop.py"))
-    gen = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(gen)
-    with open(os.path.join(build_dir, "qs_op_loop.inc"), "w") as f:
-        f.write(gen.emit())
+    """Writes the generated sources (the wide pass's op loop, the statistics'
+    logarithm table) into the build directory."""
+    for name in ("op_loop", "log_table"):
+        spec = importlib.util.spec_from_file_location("gen_" + name, os.path.join(CSRC, "gen_%s.py" % name))
+        gen = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(gen)
+        with open(os.path.join(build_dir, "qs_%s.inc" % name), "w") as f:
+            f.write(gen.emit())
 
 
 def _digest(paths, extra):

@@ -134,70 +134,84 @@ __device__ __forceinline__ void stat_pair_p(float p0, float p1, bool two, float 
 
 // ---- complex128 statistics ----
 // Bound by the FP64 pipe (two lanes per clock and SM), so what counts is the
-// number of FP64 instructions per amplitude: 28 here against ~58 with log()
-// and a multiply and an add per power (2^20 amplitudes: 132 -> ~60 us).
+// number of FP64 instructions per amplitude: 23 here.  58 with log() and a
+// multiply and an add per power took 132 us for 2^20 amplitudes; 29, with a
+// logarithm table of 256 entries filled by every block and scaling, exponent
+// and comparisons on the FP64 pipe, @STAT@.
+#include "qs_log_table.inc"
 
+// Exponents of y = N p that the table path takes: 2^-96 <= y < 2^32.
+constexpr int kLogExpMin = -96, kLogExps = 128;
+
+struct LogTables {
+    double2 c[1 << kLogBits];       // c_i, -ln c_i
+    double e[kLogExps];             // e ln 2
+};
+
+__device__ __forceinline__ void log_tables_fill(LogTables &t)
+{
+#pragma unroll 4
+    for (int i = threadIdx.x; i < (1 << kLogBits); i += blockDim.x) t.c[i] = kLogTable[i];
+    for (int i = threadIdx.x; i < kLogExps; i += blockDim.x) t.e[i] = (double)(i + kLogExpMin) * 0.69314718055994530942;
+}
+
+// Accumulates one amplitude's contributions (stat_terms) with y = 2^n p.
 // ln y by the table method of Tang (ACM TOMS 16, 1990): y = 2^e m, c_i ~ 1 /
-// (1 + (i + 1/2) / 256) from the top eight bits i of m's fraction, r = m c_i -
-// 1 (|r| < 2^-8.9), ln y = e ln 2 - ln c_i + (r - r^2/2 + r^3/3 - r^4/4 +
-// r^5/5); the first term left out is below 2^-56.  Nine FP64 instructions.
-// Zero, subnormal and non-finite y take log().
-constexpr int kLogTable = 256;
-__device__ __forceinline__ void log_table_fill(double2 *tab)
+// (1 + (i + 1/2) / 2048) from the top eleven bits i of m's fraction, r = m c_i
+// - 1 (|r| < 2^-11.9), ln y = e ln 2 - ln c_i + (r - r^2/2 + r^3/3 - r^4/4);
+// the first term left out is below 2^-61.  The factor 2^n and the exponent
+// are integer arithmetic on the high word; the powers are sums of 1, 2, 4 and
+// 5.  Other y (zero, tiny, large, non-finite) take log().
+__device__ __forceinline__ void stat_terms_f64(double p, int n, double scaleN, double (&c)[kStatAcc],
+                                               const LogTables &t)
 {
-    for (int i = threadIdx.x; i < kLogTable; i += blockDim.x) {
-        const double c = (double)(float)(1.0 / (1.0 + ((double)i + 0.5) / kLogTable));
-        tab[i] = make_double2(c, -log(c));
+    const uint32_t hi = (uint32_t)__double2hiint(p), lo = (uint32_t)__double2loint(p);
+    const uint32_t ei = (hi >> 20) + (uint32_t)n - (uint32_t)(1023 + kLogExpMin);   // (p = 0: out of range)
+    double y, ly;
+    if (ei < (uint32_t)kLogExps) {
+        y = __hiloint2double((int)(hi + ((uint32_t)n << 20)), (int)lo);
+        const double m = __hiloint2double((int)((hi & 0x000FFFFFu) | 0x3FF00000u), (int)lo);
+        const double2 k = t.c[(hi >> (20 - kLogBits)) & ((1u << kLogBits) - 1u)];
+        const double r = fma(m, k.x, -1.0);
+        ly = fma(r, fma(r, fma(r, fma(r, -0.25, 1.0 / 3.0), -0.5), 1.0), t.e[ei] + k.y);
+        c[1] = fma(y, ly, c[1]);
+    } else {
+        y = p * scaleN;
+        ly = log(y);
+        if (y > 0.0) c[1] = fma(y, ly, c[1]);
     }
-}
-__device__ __forceinline__ double log_pos(double y, const double2 *tab)
-{
-    const long long b = __double_as_longlong(y);
-    const uint32_t e = (uint32_t)(b >> 52);          // (y >= 0)
-    if (e == 0 || e >= 0x7FFu) return log(y);
-    const double m = __longlong_as_double((b & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-    const double2 t = tab[(b >> 44) & (kLogTable - 1)];
-    // e - 1023 as a double: 2^52 + 2^31 + (e - 1023) less 2^52 + 2^31
-    const double ed = __hiloint2double(0x43300000, (int)((e - 1023u) ^ 0x80000000u)) -
-                      __hiloint2double(0x43300000, (int)0x80000000);
-    const double r = fma(m, t.x, -1.0);
-    const double q = fma(r, fma(r, fma(r, 0.2, -0.25), 1.0 / 3.0), -0.5);
-    return fma(ed, 0.69314718055994530942, t.y) + fma(q, r * r, r);
-}
-
-// Accumulates one element's contributions (stat_terms), the powers as
-// products of y^2, y^3, y^4 and y^8.
-__device__ __forceinline__ void stat_terms_f64(double y, double (&c)[kStatAcc], const double2 *tab)
-{
-    const double ly = log_pos(y, tab);
     c[0] += y;
-    c[1] = y > 0.0 ? fma(y, ly, c[1]) : c[1];
     c[2] += ly;
-    const double y2 = y * y, y3 = y2 * y, y4 = y2 * y2, y8 = y4 * y4;
-    c[3] += y2;
-    c[4] += y3;
-    c[5] += y4;
+    const double y2 = y * y, y4 = y2 * y2, y5 = y4 * y;
+    c[3] = fma(y, y, c[3]);
+    c[4] = fma(y2, y, c[4]);
+    c[5] = fma(y2, y2, c[5]);
     c[6] = fma(y4, y, c[6]);
     c[7] = fma(y4, y2, c[7]);
-    c[8] = fma(y4, y3, c[8]);
-    c[9] += y8;
-    c[10] = fma(y8, y, c[10]);
-    c[11] = fma(y8, y2, c[11]);
+    c[8] = fma(y5, y2, c[8]);
+    c[9] = fma(y4, y4, c[9]);
+    c[10] = fma(y5, y4, c[10]);
+    c[11] = fma(y5, y5, c[11]);
 }
 
 __global__ void __launch_bounds__(kStatThreads)
-k_stats_c128(const double2 *__restrict__ a, uint64_t N, double scaleN, double *__restrict__ part)
+k_stats_c128(const double2 *__restrict__ a, int n, double *__restrict__ part)
 {
-    __shared__ double2 tab[kLogTable];
-    log_table_fill(tab);
+    __shared__ LogTables tab;
+    log_tables_fill(tab);
     __syncthreads();
     double acc[kStatAcc];
 #pragma unroll
     for (int k = 0; k < kStatAcc; ++k) acc[k] = 0;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += stride) {
-        double2 v = a[i];
-        stat_terms_f64((v.x * v.x + v.y * v.y) * scaleN, acc, tab);
+    const uint64_t N = 1ULL << n, stride = (uint64_t)gridDim.x * blockDim.x;
+    const double scaleN = __hiloint2double((1023 + n) << 20, 0);
+    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    double2 v = i < N ? a[i] : make_double2(0.0, 0.0);
+    while (i < N) {
+        const double p = v.x * v.x + v.y * v.y;
+        i += stride;
+        if (i < N) v = a[i];        // in flight under this one's arithmetic
+        stat_terms_f64(p, n, scaleN, acc, tab);
     }
     block_sum_store<kStatAcc>(acc, part + (size_t)blockIdx.x * kStatAcc);
 }
@@ -285,10 +299,9 @@ qs_status stats_enqueue(const qs_state *s, int row)
         grid = readout_grid(s);
     } else {
         // (one block per SM: eight warps keep the FP64 pipe busy, and the
-        // logarithm table is filled once per SM)
+        // logarithm table is copied once per SM)
         grid = grid_for(N, kStatThreads, s->num_sms, 1);
-        k_stats_c128<<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, N,
-                                                            std::ldexp(1.0, s->n), part);
+        k_stats_c128<<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, s->n, part);
         QS_LAUNCH_CHECK();
     }
     k_sum_partials<<<1, kSumThreads, 0, s->stream>>>(part, grid, kStatAcc, (double *)s->hbox_dev + (size_t)row * kStatAcc);
