@@ -477,6 +477,7 @@ struct qs_state {
     // sampler: in-chunk prefix table (and complex128 chunk sums), see qs_stats.cu
     mutable void *pt_buf = nullptr;
     mutable size_t pt_bytes = 0;
+    mutable bool rc_table_used = false;     // the sampler used a table since the last read-out
 };
 
 namespace qs {
@@ -543,7 +544,7 @@ qs_status read_back(const qs_state *s, void *host, const void *dev, size_t bytes
 // (out_kind 1: FP32, 2: FP64, 0: none; device-accessible, 16-byte aligned),
 // the statistics partials and the sampler's chunk sums into the read-out
 // cache, which it marks valid for the current state.
-constexpr int kReadoutStats = 1, kReadoutChunks = 2, kReadoutScanned = 4;
+constexpr int kReadoutStats = 1, kReadoutChunks = 2, kReadoutScanned = 4, kReadoutTable = 8;
 // Fused complex64 read-out (probabilities, statistics partials, sampler
 // chunk sums); with out_hi, chunks [csplit, nchunks) of the probabilities go
 // to out_hi (chunk csplit at its start) instead of out.  Chunks are

@@ -137,7 +137,7 @@ __device__ __forceinline__ void stat_pair_p(float p0, float p1, bool two, float 
 // number of FP64 instructions per amplitude: 23 here.  58 with log() and a
 // multiply and an add per power took 132 us for 2^20 amplitudes; 29, with a
 // logarithm table of 256 entries filled by every block and scaling, exponent
-// and comparisons on the FP64 pipe, @STAT@.
+// and comparisons on the FP64 pipe, 66 us; this 50 us.
 #include "qs_log_table.inc"
 
 // Exponents of y = N p that the table path takes: 2^-96 <= y < 2^32.
@@ -793,14 +793,16 @@ static void *sampler_work(const qs_state *s, size_t bytes)
 // 16-byte loads), one read of the state for three results: p = |psi|^2 (FP32,
 // or widened exactly to FP64; optional), the chunk sums of the sampler (the
 // lane totals and FP32 warp scan of lane_probs / chunk_scan, so the search
-// kernel's in-chunk prefixes agree with them) and the statistics partials of
-// each block (per-lane FP32 over eight chunks, then FP64, fixed order).  The
-// statistics and chunk sums are the same whether or not p is written.
+// kernel's in-chunk prefixes agree with them; all 32 lane prefixes of every
+// chunk too where `tab` is given) and the statistics partials of each block
+// (per-lane FP32 over eight chunks, then FP64, fixed order).  The statistics
+// and chunk sums are the same whether or not p is written.
 // ---------------------------------------------------------------------------
 template <int OUT>   // 0: no p, 1: FP32 p, 2: FP64 p
 __global__ void __launch_bounds__(kStatThreads, 3)
 k_readout_c64(const float2 *__restrict__ a, uint64_t N, uint64_t nchunks, float scaleN, void *__restrict__ out,
-              void *__restrict__ out_hi, uint64_t csplit, double *__restrict__ csum, double *__restrict__ part)
+              void *__restrict__ out_hi, uint64_t csplit, double *__restrict__ csum, float *__restrict__ tab,
+              double *__restrict__ part)
 {
     __shared__ __align__(16) float stage_all[kStatThreads / 32][kChunk];
     float *stage = stage_all[threadIdx.x >> 5];
@@ -863,9 +865,9 @@ k_readout_c64(const float2 *__restrict__ a, uint64_t N, uint64_t nchunks, float 
                     }
                 }
             }
-            double incl, excl;
-            chunk_scan(lane_total<float>(p), incl, excl);
-            if (lane == 31) csum[c] = incl;
+            const float incl = chunk_incl(lane_total<float>(p));
+            if (tab) tab[c * 32 + lane] = incl;
+            if (lane == 31) csum[c] = widen_f32(incl);
 #pragma unroll
             for (int i = 0; i < 8; i += 2) {
                 if (base + i < N)
@@ -923,18 +925,21 @@ qs_status readout_c64(const qs_state *s, void *out, int out_kind, void *out_hi, 
     const int grid = readout_grid(s);
     const float scaleN = (float)std::ldexp(1.0, s->n);
     const float2 *a = (const float2 *)s->amps;
-    if (out_kind == 2)
-        k_readout_c64<2><<<grid, kStatThreads, 0, s->stream>>>(a, N, nchunks, scaleN, out, out_hi, csplit,
-                                                                readout_csum(s), readout_part(s));
-    else if (out_kind == 1)
-        k_readout_c64<1><<<grid, kStatThreads, 0, s->stream>>>(a, N, nchunks, scaleN, out, out_hi, csplit,
-                                                                readout_csum(s), readout_part(s));
-    else
-        k_readout_c64<0><<<grid, kStatThreads, 0, s->stream>>>(a, N, nchunks, scaleN, nullptr, nullptr, nchunks,
-                                                                readout_csum(s), readout_part(s));
+    // The sampler's prefix table is written along (N / 2 bytes beside the 8 N
+    // read) where the sampler used one after the last read-out: 6 us instead
+    // of another read of the state, 89 us, at 26 qubits.
+    float *tab = s->rc_table_used ? (float *)s->pt_buf : nullptr;
+    s->rc_table_used = false;
+    auto kern = out_kind == 2 ? k_readout_c64<2> : out_kind == 1 ? k_readout_c64<1> : k_readout_c64<0>;
+    if (out_kind == 0) {
+        out = out_hi = nullptr;
+        csplit = nchunks;
+    }
+    kern<<<grid, kStatThreads, 0, s->stream>>>(a, N, nchunks, scaleN, out, out_hi, csplit, readout_csum(s), tab,
+                                               readout_part(s));
     QS_LAUNCH_CHECK();
     s->rc_version = s->version;
-    s->rc_flags = kReadoutStats | kReadoutChunks;
+    s->rc_flags = kReadoutStats | kReadoutChunks | (tab ? kReadoutTable : 0);
     return QS_OK;
 }
 
@@ -970,8 +975,11 @@ static qs_status sampler_run_c64(const qs_state *s, uint64_t k, uint64_t seed, u
         // (no room for the table: the rescans need none)
         float *tab = use_prefix_table(N, k, sizeof(float)) ? (float *)sampler_work(s, nchunks * 32 * sizeof(float)) : nullptr;
         if (tab) {
-            k_prefix_table<float><<<grid_for(nchunks * 32, th, s->num_sms, 8), th, 0, s->stream>>>(
-                (const float2 *)s->amps, N, nchunks, tab, nullptr);
+            if (!(s->rc_flags & kReadoutTable))
+                k_prefix_table<float><<<grid_for(nchunks * 32, th, s->num_sms, 8), th, 0, s->stream>>>(
+                    (const float2 *)s->amps, N, nchunks, tab, nullptr);
+            s->rc_flags |= kReadoutTable;
+            s->rc_table_used = true;
             k_sample_table<float><<<grid_for(k, th, s->num_sms, 8), th, 0, s->stream>>>(
                 (const float2 *)s->amps, N, nchunks, csum, tab, k, seed, dev_out);
         } else {
