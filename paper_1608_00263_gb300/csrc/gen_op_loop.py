@@ -2,7 +2,8 @@
 amplitudes, 6 register bits per thread) as inline PTX with one indexed branch
 per op.
 
-A thread's amplitudes are 32 units of two: the amplitudes that differ in
+A thread's amplitudes are 32 units of two (16 in the five-bit loops of small
+states, which know no code of register bit 5): the amplitudes that differ in
 register bit 0 (always tile bit 0, qubit 0).  A unit is two 64-bit registers,
 the two real parts and the two imaginary parts, so every gate on register
 bits 1..5 is packed FP32x2 arithmetic throughout -- with (re, im) in one
@@ -46,20 +47,21 @@ code like any other.
 
 The build writes the file into its object directory (build.py).
 """
-RB = 6           # register bits
+RB = 6           # register bits of the loop being written (see emit)
 NS = 1 << RB     # amplitudes per thread
 NU = NS // 2     # units: two amplitudes that differ in register bit 0
-NPAIR = RB * (RB - 1) // 2
-W_H, W_XH, W_YH, W_T = 0, RB, 2 * RB, 3 * RB
-W_CZ = 4 * RB
+CRB = 6          # register bits the codes are numbered for
+NPAIR = CRB * (CRB - 1) // 2
+W_H, W_XH, W_YH, W_T = 0, CRB, 2 * CRB, 3 * CRB
+W_CZ = 4 * CRB
 W_CZO = W_CZ + NPAIR
-W_CT = W_CZO + RB            # codes of the Clifford+T loop
+W_CT = W_CZO + CRB            # codes of the Clifford+T loop
 W_RY = W_CT
-W_RX = W_RY + RB
-W_PH = W_RX + RB
-W_PP = W_PH + RB
+W_RX = W_RY + CRB
+W_PH = W_RX + CRB
+W_PP = W_PH + CRB
 W_ALL = W_PP + NPAIR         # codes of the full loop
-AB = RB - 1                  # register bits of the adjoint sweep (the last selects the state)
+AB = CRB - 1                  # register bits of the adjoint sweep (the last selects the state)
 W_DX = W_ALL
 W_DY, W_DZ, W_DP, W_DPP = W_DX + AB, W_DX + 2 * AB, W_DX + 3 * AB, W_DX + 4 * AB
 W_DW = W_DPP + AB * (AB - 1) // 2
@@ -87,8 +89,8 @@ F_DIRECT, F_MORE, F_CANON = 4, 8, 16    # store to the state; copy the next tile
 
 
 def pair_index(j, k):
-    """Pairs (j, k), j < k < RB, numbered (0,1) (0,2) ... (1,2) (1,3) ..."""
-    return j * (RB - 1) - (j * (j - 1)) // 2 + (k - j - 1)
+    """Pairs (j, k), j < k < CRB, numbered (0,1) (0,2) ... (1,2) (1,3) ..."""
+    return j * (CRB - 1) - (j * (j - 1)) // 2 + (k - j - 1)
 
 
 def adj_pair_index(j, k):
@@ -433,7 +435,7 @@ def cases(full, adj=False):
         body[W_DTZ] = RECORD + SELECTED + ["neg.f32 pb, dw;"] + push(["selp.f32 da0, pb, dw, qp;"])
         body[W_DTP] = RECORD + SELECTED + push(["selp.f32 da0, dw, %s, qp;" % F_0])
         body[W_RED] = case_red()
-    assert adj or all(b is not None for b in body)
+    assert adj or RB < CRB or all(b is not None for b in body)
     return body
 
 
@@ -554,7 +556,7 @@ def asm_text(prefix, full, adj=False):
     n = len(body)
     lines = ["{",
              ".reg .pred qp;",
-             ".reg .u32 qo, qc, qn, qa, qh, a0, a1, b<%d>;" % RB,
+             ".reg .u32 qo, qc, qn, qa, qh, a0, a1, b<%d>;" % CRB,
              ".reg .b64 qm, qt, qS, qv, qu, qM1, qP2, d<%d>;" % RB,
              ".reg .f32 xr, xi, yr, yi, pa, pb, nb, nc;",
              ".reg .f32 " + ", ".join(t + str(n) for n in range(TEMPS) for t in ("xr", "xi", "yr", "yi", "na", "xx")) + ";",
@@ -586,17 +588,23 @@ def asm_text(prefix, full, adj=False):
     return lines
 
 
+def set_register_bits(rb):
+    global RB, NS, NU
+    RB, NS, NU = rb, 1 << rb, 1 << (rb - 1)
+
+
 def emit():
     out = ["// qs_op_loop.inc -- generated by gen_op_loop.py; do not edit.",
            "//",
-           "// The op loop of the wide fused pass (complex64, %d slots, %d register" % (NS, RB),
+           "// The op loop of the wide fused pass (complex64, 2^RB slots, RB register",
            "// bits) as inline PTX: one byte-code load and one indexed branch per op.",
-           "// OpLoop<0>: the Clifford+T gates; OpLoop<1>: also the parameterised",
-           "// gates; OpLoop<2>: the adjoint sweep.",
+           "// OpLoop<0, RB>: the Clifford+T gates; OpLoop<1, RB>: also the",
+           "// parameterised gates; OpLoop<2, 6>: the adjoint sweep.",
            "",
-           "template <int KIND> struct OpLoop;"]
-    for kind, prefix in enumerate(("QSWCT", "QSWFL", "QSWAD")):
-        out.append("template <> struct OpLoop<%d> {" % kind)
+           "template <int KIND, int RB> struct OpLoop;"]
+    for kind, rb, prefix in ((0, 6, "QSWCT"), (1, 6, "QSWFL"), (2, 6, "QSWAD"), (0, 5, "QSVCT"), (1, 5, "QSVFL")):
+        set_register_bits(rb)
+        out.append("template <> struct OpLoop<%d, %d> {" % (kind, rb))
         out.append("    template <int O_CODES, int O_RECS, int O_UNIT, int O_DREG, int O_DST, int O_PART>")
         out.append("    static __device__ __forceinline__ void run(uint32_t addr, uint32_t tile, uint32_t base,")
         out.append("                                               uint32_t phase, int ob,")
@@ -613,5 +621,6 @@ def emit():
         out.append('            : "memory");')
         out.append("    }")
         out.append("};")
+    set_register_bits(CRB)
     return "\n".join(out) + "\n"
 

@@ -135,7 +135,9 @@ static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const u
                 o.mode = QS_MODE_FUSED;
                 o.tile_log2 = tbits[i];
                 PlanParams pp = default_plan_params(b->n[i], QS_C64, &o);
-                if (!wide) {
+                if (wide) {
+                    pp.r = kWideRegBits;
+                } else {
                     pp.r = std::min(5, pp.t);
                     pp.pack0 = 0;
                 }

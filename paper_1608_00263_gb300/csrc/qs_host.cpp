@@ -946,7 +946,8 @@ bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &
 {
     if (passes.empty()) return false;
     for (const DevPass &p : passes)
-        if (p.r != kWideRegBits || p.t < kWideMinTile || p.t > 13) return false;
+        if (p.r != passes[0].r || (p.r != kWideRegBits && p.r != kWideFewRegBits) || p.t < kWideMinTile || p.t > 13)
+            return false;
     for (const DevPhase &h : phases)
         if (h.kind != 0 || h.R[0] != 0) return false;
     return true;
@@ -1087,7 +1088,7 @@ void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> 
         for (int ph = 0; ph < P.nphases; ++ph) {
             const DevPhase &H = phases[P.phase_begin + ph];
             WidePhase &V = W.ph[ph];
-            for (int j = 0; j < kWideRegBits; ++j) V.pb[j] = tile_swizzle(1u << H.R[j], 2) * 8u;
+            for (int j = 0; j < P.r; ++j) V.pb[j] = tile_swizzle(1u << H.R[j], 2) * 8u;
             std::memcpy(V.T, H.T, sizeof V.T);
             V.op_begin = (int16_t)(out->ops.size() - W.op_begin);
             std::vector<WideOp> tail;
@@ -1108,8 +1109,9 @@ void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> 
         const DevPhase &last = phases[P.phase_begin + P.nphases - 1];
         W.direct = 1;
         for (int k = 0; k < 4; ++k) W.direct &= last.T[k] == k + 1;
-        for (int j = 0; j < kWideRegBits; ++j) W.dreg[j] = 8ull << P.L[last.R[j]];
+        for (int j = 0; j < P.r; ++j) W.dreg[j] = 8ull << P.L[last.R[j]];
         W.full = full;
+        W.r = (int16_t)P.r;
         out->passes.push_back(W);
     }
     out->ops.resize((out->ops.size() + 31) / 16 * 16);
@@ -1252,7 +1254,7 @@ PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o)
     // register bits, evolve + read: 12 qubits 39.9 -> 37.2 us, 20 qubits 96.0
     // -> 88.1 us, 23 qubits 400 -> 331 us, 30 qubits 66.6 -> 51.8 ms
     if (dt == QS_C64 && pp.mode == QS_MODE_FUSED && pp.t >= kWideMinTile) {
-        pp.r = kWideRegBits;
+        pp.r = n - pp.t <= kWideFewTiles ? kWideFewRegBits : kWideRegBits;
         pp.pack0 = 1;
     }
     pp.r = std::min(pp.r, pp.t);

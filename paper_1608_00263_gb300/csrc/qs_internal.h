@@ -223,6 +223,8 @@ QS_HD inline uint32_t tile_swizzle(uint32_t e, uint32_t CE)
 // and 16-byte records, so the kernel's staging is a copy.
 // ---------------------------------------------------------------------------
 constexpr int kWideRegBits = 6;
+constexpr int kWideFewRegBits = 5;      // of states of few tiles (default_plan_params)
+constexpr int kWideFewTiles = 7;        // ... at most 2^7: fewer than the GPU has SMs
 constexpr int kMaxWideOps = 216;        // ops of a pass, end codes included (shared memory)
 constexpr int kWideMinTile = 11;        // tiles of whole warps (2^(t - 6) threads)
 
@@ -255,7 +257,8 @@ struct alignas(16) WidePhase {
 struct WidePass {
     int32_t t, n, nphases, nops;
     uint32_t op_begin;           // first record and code (a multiple of 16)
-    int32_t full;                // some op needs the loop with parameterised gates
+    int16_t full;                // some op needs the loop with parameterised gates
+    int16_t r;                   // register bits
     float gs_re, gs_im;          // pass-wide factor, applied in the last phase
     int32_t canon_in, canon_out; // the pass reads / writes canonical units
                                  // (re, im, re, im), else (re, re, im, im)

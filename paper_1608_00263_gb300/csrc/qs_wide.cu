@@ -8,13 +8,13 @@ namespace qs {
 
 // FOLD: the circuit's first pass (the uniform state with the folded
 // diagonal prefix is generated); the other passes carry none of that code.
-template <bool FULL, bool FOLD>
-__global__ void __launch_bounds__(kWideThreads, 3)
+template <bool FULL, bool FOLD, int RB>
+__global__ void __launch_bounds__(1 << (13 - RB), RB == kWideRegBits ? 3 : 2)
 k_wide_pass(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g, const WideOp *__restrict__ ops_g,
             const uint8_t *__restrict__ codes_g, uint32_t ntiles, FoldArgs fold)
 {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
-    __shared__ WideSmem S;
+    __shared__ WideSmemT<RB> S;
     // contiguous range of tiles per CTA
     const uint32_t per = ntiles / gridDim.x, extra = ntiles % gridDim.x;
     const uint32_t t_begin = blockIdx.x * per + (blockIdx.x < extra ? blockIdx.x : extra);
@@ -28,10 +28,17 @@ k_wide_pass(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g, cons
             F.m[1] = fold.m2;
             F.m[2] = fold.m4;
         }
-        wide_pass_body<FULL ? 1 : 0, 1, 0>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 1, 0, RB>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
     } else {
-        wide_pass_body<FULL ? 1 : 0, 0, 0>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
+        wide_pass_body<FULL ? 1 : 0, 0, 0, RB>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, nullptr, smem_dyn);
     }
+}
+
+template <int RB>
+static auto wide_pass_kernel(bool full, bool first)
+{
+    return full ? (first ? k_wide_pass<true, true, RB> : k_wide_pass<true, false, RB>)
+                : (first ? k_wide_pass<false, true, RB> : k_wide_pass<false, false, RB>);
 }
 
 qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t nops, const void *dev,
@@ -44,12 +51,12 @@ qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t
     for (size_t p = 0; p < passes.size(); ++p) {
         const WidePass &P = passes[p];
         const bool first = p == 0 && uniform != 0.0;
-        auto kern = P.full ? (first ? k_wide_pass<true, true> : k_wide_pass<true, false>)
-                           : (first ? k_wide_pass<false, true> : k_wide_pass<false, false>);
+        auto kern = P.r == kWideRegBits ? wide_pass_kernel<kWideRegBits>(P.full != 0, first)
+                                        : wide_pass_kernel<kWideFewRegBits>(P.full != 0, first);
         const size_t smem = (size_t(1) << P.t) * sizeof(float2);
         QS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        const uint32_t ntiles = 1u << (P.n - P.t), cap = (uint32_t)s->num_sms * 3;
-        kern<<<(int)(ntiles < cap ? ntiles : cap), 1 << (P.t - kWideRegBits), smem, s->stream>>>(
+        const uint32_t ntiles = 1u << (P.n - P.t), cap = (uint32_t)s->num_sms * (P.r == kWideRegBits ? 3 : 2);
+        kern<<<(int)(ntiles < cap ? ntiles : cap), 1 << (P.t - P.r), smem, s->stream>>>(
             (float2 *)s->amps, dpass + p, dops, dcodes, ntiles, first && fold ? *fold : none);
         QS_LAUNCH_CHECK();
     }

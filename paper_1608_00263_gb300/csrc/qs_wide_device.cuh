@@ -12,6 +12,12 @@
 // slot accesses are 16 bytes.  128 threads hold a 13-qubit tile at 168
 // registers and 75 KB of shared memory, so three CTAs share an SM: while one
 // waits for its tile, two compute.
+//
+// A state of at most as many tiles as SMs has one CTA per SM, one warp per
+// scheduler, and every latency shows (12 qubits: an instruction in 5 cycles,
+// waiting in turn for shared memory, fixed latencies and instruction fetch):
+// there 32 amplitudes (5 register bits) per thread and twice the warps are
+// the better split (RB = 5; rule and figures in default_plan_params).
 #pragma once
 
 #include <cstddef>
@@ -24,7 +30,6 @@ namespace qs {
 
 constexpr int kWideThreads = 1 << (13 - kWideRegBits);   // threads of a 13-qubit tile
 constexpr int kWideSlots = 1 << kWideRegBits;
-constexpr int kWideUnits = kWideSlots / 2;               // 16-byte units per thread
 
 constexpr uint32_t kWideDirect = 4, kWideMore = 8, kWideCanon = 16;   // phase flags (gen_op_loop.py)
 
@@ -34,22 +39,26 @@ struct alignas(16) WideUnit {           // unit `it` of every thread
     uint32_t pad;
 };
 
-struct WideSmem {
+template <int RB>
+struct WideSmemT {
+    static constexpr int kThreads = 1 << (13 - RB), kUnits = 1 << (RB - 1);   // 16-byte units per thread
     WidePass P;
     WideOp ops[kMaxWideOps];
     uint32_t codes[kMaxWideOps / 4 + 4];
-    uint64_t toff[kWideThreads];                     // byte offset in the state of the thread's first copied unit
-    uint64_t doff[kWideThreads];                     // ... of its slot 0 in the last phase
-    uint64_t dst[kWideThreads];                      // state address of the thread's slot 0 of this tile
+    uint64_t toff[kThreads];                     // byte offset in the state of the thread's first copied unit
+    uint64_t doff[kThreads];                     // ... of its slot 0 in the last phase
+    uint64_t dst[kThreads];                      // state address of the thread's slot 0 of this tile
     uint64_t amps;                                   // the state, and the end of the tile range: read
     uint32_t t_end, pad;                             // again where used, registers are short
     alignas(16) uint64_t part;                       // adjoint sweep: partials of this CTA's warps,
     uint64_t part_stride;                            // bytes per slot
     uint64_t gmask;                                  // out-of-tile qubits
-    uint16_t thr[kMaxPhasesPerPass][kWideThreads];   // tile element of the thread's slot 0
-    WideUnit unit[kWideUnits];
+    uint16_t thr[kMaxPhasesPerPass][kThreads];   // tile element of the thread's slot 0
+    WideUnit unit[kUnits];
     float2 w8[8];                                    // e^{i pi k / 4}
 };
+
+using WideSmem = WideSmemT<kWideRegBits>;
 
 static_assert(sizeof(WidePass) % 16 == 0 && offsetof(WidePass, ph) % 16 == 0 && offsetof(WideSmem, ops) % 16 == 0 &&
                   offsetof(WideSmem, unit) % 16 == 0 && offsetof(WideSmem, part) % 16 == 0 && sizeof(WideUnit) == 16,
@@ -90,14 +99,15 @@ __device__ __forceinline__ void wide_sync(int nthr, int gi)
 // KIND: the op loop (0 Clifford+T, 1 all gates, 2 the adjoint sweep, whose
 // tile bit t - 1 selects psi or lambda, lam_off bytes away; S.part and
 // S.part_stride are set by the caller).
-template <int KIND, int FOLD, int GROUPED>
+template <int KIND, int FOLD, int GROUPED, int RB = kWideRegBits>
 __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g,
                                                const WideOp *__restrict__ ops_g, const uint8_t *__restrict__ codes_g,
-                                               uint32_t t_begin, uint32_t t_end, WideSmem &S, WideFoldSmem *F,
+                                               uint32_t t_begin, uint32_t t_end, WideSmemT<RB> &S, WideFoldSmem *F,
                                                unsigned char *smem_raw, uint64_t lam_off = 0,
                                                const FoldArgs *__restrict__ folds_g = nullptr)
 {
-    constexpr int RB = kWideRegBits, NS = kWideSlots, NU = kWideUnits;
+    using Smem = WideSmemT<RB>;
+    constexpr int NS = 1 << RB, NU = NS / 2;
     for (int i = threadIdx.x; i < (int)(sizeof(WidePass) / 4); i += blockDim.x)
         reinterpret_cast<uint32_t *>(&S.P)[i] = reinterpret_cast<const uint32_t *>(pass_g)[i];
     __syncthreads();
@@ -323,12 +333,12 @@ __device__ __forceinline__ void wide_pass_body(float2 *__restrict__ amps, const 
                     nsrc = reinterpret_cast<const char *>(S.amps + (nbase * 8u + S.toff[tid]));
                 }
             }
-            OpLoop<KIND>::template run<(int)offsetof(WideSmem, codes), (int)offsetof(WideSmem, ops) - 16,
-                                       (int)offsetof(WideSmem, unit),
-                                       (int)(offsetof(WideSmem, P) + offsetof(WidePass, dreg)),
-                                       (int)offsetof(WideSmem, dst), (int)offsetof(WideSmem, part)>(
+            OpLoop<KIND, RB>::template run<(int)offsetof(Smem, codes), (int)offsetof(Smem, ops) - 16,
+                                           (int)offsetof(Smem, unit),
+                                           (int)(offsetof(Smem, P) + offsetof(WidePass, dreg)),
+                                           (int)offsetof(Smem, dst), (int)offsetof(Smem, part)>(
                 swz<2>(te) * 8u, tile_sa, smem_addr(&S),
-                (uint32_t)(offsetof(WideSmem, P) + offsetof(WidePass, ph)) + (uint32_t)ph * (uint32_t)sizeof(WidePhase),
+                (uint32_t)(offsetof(Smem, P) + offsetof(WidePass, ph)) + (uint32_t)ph * (uint32_t)sizeof(WidePhase),
                 H.op_begin, ((uint64_t)to << 32) | te, fr, fi, mode, sw_tid,
                 nsrc, GROUPED ? (uint32_t)gi + 1u : 0u,
                 (uint32_t)nthr);
