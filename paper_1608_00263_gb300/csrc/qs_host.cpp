@@ -1251,8 +1251,13 @@ PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o)
         pp.look_steps = pp.look_top = 8;
     // complex64 register passes run the wide form (six register bits, one of
     // them qubit 0) wherever a tile fills whole warps; measured against five
-    // register bits, evolve + read: 12 qubits 39.9 -> 37.2 us, 20 qubits 96.0
-    // -> 88.1 us, 23 qubits 400 -> 331 us, 30 qubits 66.6 -> 51.8 ms
+    // register bits of the (re, im) form, evolve + read: 23 qubits 400 -> 331
+    // us, 30 qubits 66.6 -> 51.8 ms.  Few tiles leave an SM one CTA and a
+    // scheduler one warp of it; with five register bits per thread it has two:
+    // at 11, 12, 16, 20, 21 qubits, depth 25, 35.8 -> 27.8, 35.7 -> 29.4, 61.3 ->
+    // 56.1, 85.8 -> 79.3, 97.5 -> 95.5 us (with rotations 56.6 -> 40.8, 57.8 ->
+    // 42.6, 75.5 -> 65.7, 104.0 -> 92.3, 123.7 -> 118.9); at 22 it loses, 155.7 ->
+    // 157.6 and 204.8 -> 214.3.
     if (dt == QS_C64 && pp.mode == QS_MODE_FUSED && pp.t >= kWideMinTile) {
         pp.r = n - pp.t <= kWideFewTiles ? kWideFewRegBits : kWideRegBits;
         pp.pack0 = 1;

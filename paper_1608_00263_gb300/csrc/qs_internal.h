@@ -224,7 +224,7 @@ QS_HD inline uint32_t tile_swizzle(uint32_t e, uint32_t CE)
 // ---------------------------------------------------------------------------
 constexpr int kWideRegBits = 6;
 constexpr int kWideFewRegBits = 5;      // of states of few tiles (default_plan_params)
-constexpr int kWideFewTiles = 7;        // ... at most 2^7: fewer than the GPU has SMs
+constexpr int kWideFewTiles = 8;        // ... at most 2^8 (the GPU holds 456 CTAs of the six-bit form)
 constexpr int kMaxWideOps = 216;        // ops of a pass, end codes included (shared memory)
 constexpr int kWideMinTile = 11;        // tiles of whole warps (2^(t - 6) threads)
 

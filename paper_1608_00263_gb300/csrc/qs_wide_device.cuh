@@ -13,7 +13,7 @@
 // registers and 75 KB of shared memory, so three CTAs share an SM: while one
 // waits for its tile, two compute.
 //
-// A state of at most as many tiles as SMs has one CTA per SM, one warp per
+// A state of few tiles has one or two CTAs per SM, one or two warps per
 // scheduler, and every latency shows (12 qubits: an instruction in 5 cycles,
 // waiting in turn for shared memory, fixed latencies and instruction fetch):
 // there 32 amplitudes (5 register bits) per thread and twice the warps are
