@@ -488,52 +488,76 @@ static void collect(const std::vector<PGate> &g, const std::vector<int> &cand,
     *count = cnt;
 }
 
-// First pending non-diagonal gate index per qubit (large if none).
-static void first_pending(const std::vector<PGate> &g, const std::vector<int> &cand,
-                          const std::vector<char> &done, int n, std::vector<int> *first)
-{
-    first->assign(n, 1 << 30);
-    for (int i : cand) {
-        if (done[i] || g[i].diag) continue;
-        int q = g[i].q0;
-        if ((*first)[q] > i) (*first)[q] = i;
-    }
-}
+// The gates of `cand` not yet done, for choosing a local set: planning spends
+// its time counting, for many sets, the gates that apply, so what that reads
+// is laid out once per choice: 16 bytes a gate and no test but the loop's
+// (host planning 20.5 -> @T30@ ms at 30 qubits, depth 40, 308 -> @T12@ us at 12).
+struct Pending {
+    struct Gate {
+        uint64_t qm, nd;            // qubits; the same if the gate is not diagonal, else 0
+    };
+    std::vector<Gate> gates;
+    std::vector<int> first;         // first non-diagonal gate per qubit (large if none)
+    std::vector<int> ndiag;         // diagonal gates per qubit
 
-// Pending diagonal gates per qubit.
-static void diag_pending(const std::vector<PGate> &g, const std::vector<int> &cand,
-                         const std::vector<char> &done, int n, std::vector<int> *cnt)
-{
-    cnt->assign(n, 0);
-    for (int i : cand) {
-        if (done[i] || !g[i].diag) continue;
-        ++(*cnt)[g[i].q0];
-        if (g[i].two) ++(*cnt)[g[i].q1];
+    Pending(const std::vector<PGate> &g, const std::vector<int> &cand, const std::vector<char> &done, int n)
+        : first(n, 1 << 30), ndiag(n, 0)
+    {
+        gates.reserve(cand.size());
+        for (int i : cand) {
+            if (done[i]) continue;
+            const PGate &x = g[i];
+            const uint64_t qm = (1ULL << x.q0) | (x.two ? (1ULL << x.q1) : 0);
+            gates.push_back({qm, x.diag ? 0 : qm});
+            if (x.diag) {
+                ++ndiag[x.q0];
+                if (x.two) ++ndiag[x.q1];
+            } else {
+                first[x.q0] = std::min(first[x.q0], i);
+            }
+        }
     }
-}
+
+    // Gates that apply with the local set (the rule of collect).
+    int count(uint64_t local, uint64_t allq) const
+    {
+        uint64_t blocked = 0, blocked_nd = 0;
+        int cnt = 0;
+        const uint64_t out = ~local;
+        for (const Gate &x : gates) {
+            if (x.nd) {
+                if (x.nd & (blocked | blocked_nd | out)) {
+                    blocked |= x.nd;
+                    if (blocked == allq) break;
+                } else {
+                    ++cnt;
+                }
+            } else if (x.qm & blocked) {
+                blocked_nd |= x.qm;
+            } else {
+                ++cnt;
+            }
+        }
+        return cnt;
+    }
+};
 
 // Greedy choice of `want` qubits added to `base` from `pool`, maximising the
 // number of applicable gates; ties go to the qubit whose next non-diagonal
 // gate is earliest, then to the qubit with the fewest pending diagonal gates
 // (a register phase applies those to whole threads when their qubits are
 // not register bits).
-static uint64_t choose_local(const std::vector<PGate> &g, const std::vector<int> &cand,
-                             const std::vector<char> &done, int n, uint64_t base,
-                             uint64_t pool, int want, uint64_t allq = ~0ULL)
+static uint64_t choose_local(const Pending &p, int n, uint64_t base, uint64_t pool, int want, uint64_t allq = ~0ULL)
 {
-    std::vector<int> first, ndiag;
-    first_pending(g, cand, done, n, &first);
-    diag_pending(g, cand, done, n, &ndiag);
     uint64_t local = base;
     for (int step = 0; step < want; ++step) {
         int best_q = -1, best_cnt = -1, best_first = 1 << 30, best_diag = 1 << 30;
         for (int q = 0; q < n; ++q) {
             if (!((pool >> q) & 1) || ((local >> q) & 1)) continue;
-            int cnt;
-            collect(g, cand, done, local | (1ULL << q), nullptr, &cnt, allq);
-            if (cnt > best_cnt || (cnt == best_cnt && (first[q] < best_first ||
-                                                       (first[q] == best_first && ndiag[q] < best_diag)))) {
-                best_q = q; best_cnt = cnt; best_first = first[q]; best_diag = ndiag[q];
+            const int cnt = p.count(local | (1ULL << q), allq);
+            if (cnt > best_cnt || (cnt == best_cnt && (p.first[q] < best_first ||
+                                                       (p.first[q] == best_first && p.ndiag[q] < best_diag)))) {
+                best_q = q; best_cnt = cnt; best_first = p.first[q]; best_diag = p.ndiag[q];
             }
         }
         if (best_q < 0) break;
@@ -542,29 +566,31 @@ static uint64_t choose_local(const std::vector<PGate> &g, const std::vector<int>
     return local;
 }
 
+static uint64_t choose_local(const std::vector<PGate> &g, const std::vector<int> &cand,
+                             const std::vector<char> &done, int n, uint64_t base, uint64_t pool, int want)
+{
+    return choose_local(Pending(g, cand, done, n), n, base, pool, want);
+}
+
 // Tile choice of a pass with a lookahead: for the first `look_steps`
 // additions, the `look_top` candidates with the most applicable gates are
 // each completed greedily to the full tile and scored by the gates the
 // completed tile applies; the remaining additions are greedy.  Fewer passes
 // than the plain greedy choice on the paper's circuits: 10 % at 30 qubits
-// (8 steps, 8 candidates, ~40 ms of host time against ~80 ms of evolution),
-// 14 % at 34 qubits (every step and candidate, ~0.2 s against ~1.4 s).
+// (8 steps, 8 candidates), 14 % at 34 qubits (every step and candidate).
 // Host planning of the next circuit overlaps the current evolution.
 static uint64_t choose_tile(const std::vector<PGate> &g, const std::vector<int> &cand,
                             const std::vector<char> &done, int n, uint64_t base, uint64_t pool,
                             int want, uint64_t allq, int look_steps, int look_top)
 {
+    const Pending p(g, cand, done, n);
     uint64_t local = base;
     for (int step = 0; step < want && step < look_steps; ++step) {
-        std::vector<int> first;
-        first_pending(g, cand, done, n, &first);
         struct C { int cnt, first, q; };
         std::vector<C> cs;
         for (int q = 0; q < n; ++q) {
             if (!((pool >> q) & 1) || ((local >> q) & 1)) continue;
-            int cnt;
-            collect(g, cand, done, local | (1ULL << q), nullptr, &cnt, allq);
-            cs.push_back({cnt, first[q], q});
+            cs.push_back({p.count(local | (1ULL << q), allq), p.first[q], q});
         }
         if (cs.empty()) return local;
         std::sort(cs.begin(), cs.end(), [](const C &a, const C &b) {
@@ -573,15 +599,14 @@ static uint64_t choose_tile(const std::vector<PGate> &g, const std::vector<int> 
         if ((int)cs.size() > look_top) cs.resize(look_top);
         int best_q = -1, best = -1;
         for (const C &c : cs) {
-            const uint64_t full = choose_local(g, cand, done, n, local | (1ULL << c.q), pool, want - step - 1, allq);
-            int cnt;
-            collect(g, cand, done, full, nullptr, &cnt, allq);
+            const uint64_t full = choose_local(p, n, local | (1ULL << c.q), pool, want - step - 1, allq);
+            const int cnt = p.count(full, allq);
             if (cnt > best) { best = cnt; best_q = c.q; }
         }
         local |= 1ULL << best_q;
     }
     const int added = __builtin_popcountll(local & ~base);
-    return choose_local(g, cand, done, n, local, pool, want - added, allq);
+    return choose_local(p, n, local, pool, want - added, allq);
 }
 
 // One phase of a wide pass: its register qubits and its gates in order.
@@ -733,8 +758,7 @@ static void collect_tc(const std::vector<PGate> &g, const std::vector<int> &cand
 static uint64_t choose_tc_block(const std::vector<PGate> &g, const std::vector<int> &cand,
                                 const std::vector<char> &done, int n, uint64_t pool, int want)
 {
-    std::vector<int> first;
-    first_pending(g, cand, done, n, &first);
+    const std::vector<int> first = Pending(g, cand, done, n).first;
     uint64_t block = 0;
     for (int step = 0; step < want; ++step) {
         int best_q = -1, best_cnt = -1, best_first = 1 << 30;
