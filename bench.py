@@ -483,7 +483,7 @@ def run_ours(args, rank, world, local):
         "config": workload_config(args, n, world),
         "apply_cycles_per_s": round(depth * args.steps / (passes_ms / 1000.0), 3),
         "passes_per_circuit": passes_total / args.steps,
-        "roofline": {"kernel": ("k_fused_pass<float,5,0,0>" if args.mode == "fused"
+        "roofline": {"kernel": ("k_wide_pass<0,0,6>" if args.mode == "fused"
                                 else "k_fused_pass<float,5,1,1>"),
                      "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak,
                      "peak_source": peak_src + " hbm_gbs", "unit": "GB/s",
@@ -781,8 +781,9 @@ def load_traffic(mode, n):
     except (OSError, ValueError):
         return None
     import hashlib
-    # both forms are compiled from qs_fused.cu; each has its own capture
-    src = os.path.join(ROOT, "paper_1608_00263_gb300", "csrc", "qs_fused.cu")
+    # each form has its own source and capture
+    src = os.path.join(ROOT, "paper_1608_00263_gb300", "csrc",
+                       "qs_wide_device.cuh" if mode == "fused" else "qs_fused.cu")
     try:
         digest = hashlib.sha1(open(src, "rb").read()).hexdigest()
     except OSError:
