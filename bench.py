@@ -781,15 +781,16 @@ def load_traffic(mode, n):
     except (OSError, ValueError):
         return None
     import hashlib
-    # each form has its own source and capture
-    src = os.path.join(ROOT, "paper_1608_00263_gb300", "csrc",
-                       "qs_wide_device.cuh" if mode == "fused" else "qs_fused.cu")
+    # the capture is of the current sources: qs_fused.cu (both forms share it
+    # for passes outside the wide form) and, for the fused form, the wide pass
+    r = rec.get(mode) or {}
+    csrc = os.path.join(ROOT, "paper_1608_00263_gb300", "csrc")
     try:
-        digest = hashlib.sha1(open(src, "rb").read()).hexdigest()
+        for key, name in (("source_sha1", "qs_fused.cu"),) + ((("wide_sha1", "qs_wide_device.cuh"),) if mode == "fused" else ()):
+            with open(os.path.join(csrc, name), "rb") as f:
+                if r.get(key) != hashlib.sha1(f.read()).hexdigest():
+                    return None
     except OSError:
-        return None
-    r = rec.get(mode)
-    if not r or r.get("source_sha1") != digest:
         return None
     # scale the captured launch's traffic to this state size
     return round(r["bytes_per_launch"] * (2.0 ** n) / (2.0 ** r["qubits"]), 1), r.get("launch")
