@@ -166,8 +166,9 @@ def kernel_launches_per_step(passes):
 
 
 # of those, the read-backs of the statistics and of the cross entropy (1 + 2)
-# no longer launch: the summing kernel writes the host's mapped memory
-UNLAUNCHED_READ_BACKS = 3
+# and the cross entropy's final sum no longer launch: the summing kernel
+# writes the host's mapped memory
+UNLAUNCHED_READ_BACKS = 4
 
 
 def leading_h_layer(qs, g, n):

@@ -78,6 +78,7 @@ qs_status alloc_workspace(qs_state *s)
     QS_CUDA_TRY(cudaMalloc((void **)&s->ws_f64, kWsDoubles * sizeof(double)));
     s->ws_f64_count = kWsDoubles;
     QS_CUDA_TRY(cudaMalloc((void **)&s->ws_u64, 64 * sizeof(uint64_t)));
+    QS_CUDA_TRY(cudaMemsetAsync(s->ws_u64, 0, 64 * sizeof(uint64_t), s->stream));
     QS_CUDA_TRY(cudaHostAlloc(&s->hbox, kHostBoxBytes, cudaHostAllocMapped));
     QS_CUDA_TRY(cudaHostGetDevicePointer(&s->hbox_dev, s->hbox, 0));
     return QS_OK;

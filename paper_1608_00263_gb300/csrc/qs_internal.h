@@ -547,6 +547,7 @@ qs_status read_back(const qs_state *s, void *host, const void *dev, size_t bytes
 // (out_kind 1: FP32, 2: FP64, 0: none; device-accessible, 16-byte aligned),
 // the statistics partials and the sampler's chunk sums into the read-out
 // cache, which it marks valid for the current state.
+constexpr int kDoneWord = 1;    // word of ws_u64: finished blocks of a summing launch, zero between launches
 constexpr int kReadoutStats = 1, kReadoutChunks = 2, kReadoutScanned = 4, kReadoutTable = 8;
 // Fused complex64 read-out (probabilities, statistics partials, sampler
 // chunk sums); with out_hi, chunks [csplit, nchunks) of the probabilities go

@@ -194,8 +194,34 @@ __device__ __forceinline__ void stat_terms_f64(double p, int n, double scaleN, d
     c[11] = fma(y5, y5, c[11]);
 }
 
+// Block partials to host sums in the launch that formed them: the block that
+// finishes last (`done` counts them, and is left at zero) sums them in block
+// order, lanes taking blocks lane, lane + 32, ..., and writes the host's mapped
+// memory.  A launch of its own cost ~4 us (k_sum_partials, which serves the
+// sums that are kept).
+template <int K>
+__device__ __forceinline__ void last_block_sums(const double *part, uint32_t *done, double *out)
+{
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < K; k += kStatThreads / 32) {
+        double s = 0;
+#pragma unroll 8
+        for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(part + (size_t)b * K + k);
+        s = warp_sum(s);
+        if (lane == 0) out[k] = s;
+    }
+    if (threadIdx.x == 0) *done = 0;
+}
+
 __global__ void __launch_bounds__(kStatThreads)
-k_stats_c128(const double2 *__restrict__ a, int n, double *__restrict__ part)
+k_stats_c128(const double2 *__restrict__ a, int n, double *part, uint32_t *done, double *out)
 {
     __shared__ LogTables tab;
     log_tables_fill(tab);
@@ -214,6 +240,7 @@ k_stats_c128(const double2 *__restrict__ a, int n, double *__restrict__ part)
         stat_terms_f64(p, n, scaleN, acc, tab);
     }
     block_sum_store<kStatAcc>(acc, part + (size_t)blockIdx.x * kStatAcc);
+    last_block_sums<kStatAcc>(part, done, out);
 }
 
 // Final fixed-order sum of block partials: warp k sums accumulator k (lanes
@@ -231,17 +258,6 @@ k_sum_partials(const double *__restrict__ part, int nblocks, int K, double *__re
     for (int b = lane; b < nblocks; b += 32) s += part[(size_t)b * K + k];
     s = warp_sum(s);
     if (lane == 0) out[k] = s;
-}
-
-// Sums `nblocks` partials of K accumulators into `host` (K doubles) through
-// the state's mapped host box: one launch and one synchronisation.
-static qs_status sum_to_host(const qs_state *s, const double *part, int nblocks, int K, double *host)
-{
-    k_sum_partials<<<1, 32 * K, 0, s->stream>>>(part, nblocks, K, (double *)s->hbox_dev);
-    QS_LAUNCH_CHECK();
-    QS_CUDA_TRY(cudaStreamSynchronize(s->stream));
-    std::memcpy(host, s->hbox, (size_t)K * sizeof(double));
-    return QS_OK;
 }
 
 __global__ void k_read_back(const unsigned long long *__restrict__ src, unsigned long long *__restrict__ dst, int n)
@@ -285,11 +301,14 @@ qs_status stage_view(const qs_state *s, size_t bytes, void **host, void **dev)
     return QS_OK;
 }
 
+// The state's counter of finished blocks (last_block_sums).
+static uint32_t *done_counter(const qs_state *s) { return (uint32_t *)(s->ws_u64 + kDoneWord); }
+
 qs_status stats_enqueue(const qs_state *s, int row)
 {
     const uint64_t N = 1ULL << s->n;
     int grid;
-    double *part = s->ws_f64;
+    double *part = s->ws_f64, *out = (double *)s->hbox_dev + (size_t)row * kStatAcc;
     if (s->dt == QS_C64) {
         // the read-out cache holds the partials of the current state, or a
         // fused read-out pass forms them (with the sampler's chunk sums)
@@ -301,10 +320,11 @@ qs_status stats_enqueue(const qs_state *s, int row)
         // (one block per SM: eight warps keep the FP64 pipe busy, and the
         // logarithm table is copied once per SM)
         grid = grid_for(N, kStatThreads, s->num_sms, 1);
-        k_stats_c128<<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, s->n, part);
+        k_stats_c128<<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, s->n, part, done_counter(s), out);
         QS_LAUNCH_CHECK();
+        return QS_OK;
     }
-    k_sum_partials<<<1, kSumThreads, 0, s->stream>>>(part, grid, kStatAcc, (double *)s->hbox_dev + (size_t)row * kStatAcc);
+    k_sum_partials<<<1, kSumThreads, 0, s->stream>>>(part, grid, kStatAcc, out);
     QS_LAUNCH_CHECK();
     return QS_OK;
 }
@@ -1322,7 +1342,7 @@ constexpr int kCeGroup = 8;
 template <typename R>
 __global__ void __launch_bounds__(kStatThreads)
 k_cross_entropy(const typename V2T<R>::T *__restrict__ a, uint64_t N, const uint64_t *__restrict__ x,
-                uint64_t m, double *__restrict__ part)
+                uint64_t m, double *part, uint32_t *done, double *out)
 {
     using V = typename V2T<R>::T;
     double acc[2] = {0.0, 0.0};
@@ -1360,6 +1380,7 @@ k_cross_entropy(const typename V2T<R>::T *__restrict__ a, uint64_t N, const uint
         acc[0] -= log(prod) + (double)esum * 0.69314718055994530942;
     }
     block_sum_store<2>(acc, part + 2 * blockIdx.x);
+    last_block_sums<2>(part, done, out);
 }
 
 qs_status cross_entropy_run(const qs_state *s, const uint64_t *dev_samples, uint64_t m, double *ce)
@@ -1368,12 +1389,15 @@ qs_status cross_entropy_run(const qs_state *s, const uint64_t *dev_samples, uint
     const int grid = grid_for((m + kCeGroup - 1) / kCeGroup, kStatThreads, s->num_sms, 4);
     double *part = s->ws_f64;
     if (s->dt == QS_C64)
-        k_cross_entropy<float><<<grid, kStatThreads, 0, s->stream>>>((const float2 *)s->amps, N, dev_samples, m, part);
+        k_cross_entropy<float><<<grid, kStatThreads, 0, s->stream>>>((const float2 *)s->amps, N, dev_samples, m, part,
+                                                                     done_counter(s), (double *)s->hbox_dev);
     else
-        k_cross_entropy<double><<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, N, dev_samples, m, part);
+        k_cross_entropy<double><<<grid, kStatThreads, 0, s->stream>>>((const double2 *)s->amps, N, dev_samples, m, part,
+                                                                      done_counter(s), (double *)s->hbox_dev);
     QS_LAUNCH_CHECK();
-    double sum[2] = {0, 0};
-    if (qs_status st = sum_to_host(s, part, grid, 2, sum)) return st;
+    QS_CUDA_TRY(cudaStreamSynchronize(s->stream));
+    double sum[2];
+    std::memcpy(sum, s->hbox, sizeof sum);
     if (sum[1] > 0) return set_error(QS_ERR_INVALID_ARG, "%llu sample indices >= 2^n", (unsigned long long)sum[1]);
     *ce = sum[0] / (double)m;
     return QS_OK;
