@@ -220,10 +220,7 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
                           bool narrow = false)
 {
     PlanParams pp = default_plan_params(s->n, s->dt, o);
-    if (narrow && pp.pack0) {
-        pp.r = 5;
-        pp.pack0 = 0;
-    }
+    if (narrow) pp = narrow_plan_params(pp);
     DevicePlanCache &pc = s->plan_cache;
     DevicePlanSlot *c = nullptr;
     for (DevicePlanSlot &x : pc.slot)
@@ -241,9 +238,9 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
         const size_t b_phase = p.phases.size() * sizeof(DevPhase);
         const size_t b_ops = p.ops.size() * sizeof(DevOp);
         const size_t b_blk = p.tc_words.size() * sizeof(uint32_t);
-        // complex64 plans of six register bits go up lowered
+        // plans made for the wide pass go up lowered
         WidePlan wide;
-        if (s->dt == QS_C64 && wide_plan(p.passes, p.phases)) lower_wide(p.passes, p.phases, p.ops, &wide);
+        lower_wide(p, &wide);
         const size_t w_pass = wide.passes.size() * sizeof(WidePass), w_ops = wide.ops.size() * sizeof(WideOp);
         const size_t total = (w_pass ? w_pass + w_ops + wide.codes.size() : b_pass + b_phase + b_ops + b_blk) + 16;
         if (c->bytes < total) {

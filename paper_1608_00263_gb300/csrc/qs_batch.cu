@@ -191,10 +191,10 @@ static void lower_instances(const std::vector<Plan> &plans, const std::vector<Fo
 {
     *out = WidePlan();
     for (int i : idx)
-        if (!plans[i].passes.empty() && !wide_plan(plans[i].passes, plans[i].phases)) return;
+        if (!plans[i].passes.empty() && !plans[i].wide) return;
     for (int i : idx) {
         const size_t first = out->passes.size();
-        lower_wide(plans[i].passes, plans[i].phases, plans[i].ops, out);
+        lower_wide(plans[i], out);
         if (!folds[i].nfold || out->passes.size() == first) continue;
         out->folds.push_back(folds[i]);
         out->passes[first].fold = (int32_t)out->folds.size();

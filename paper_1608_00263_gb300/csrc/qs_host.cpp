@@ -968,17 +968,6 @@ static void pack_block(const std::vector<Cplx> &U, int precision, std::vector<ui
 
 }  // namespace
 
-bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases)
-{
-    if (passes.empty()) return false;
-    for (const DevPass &p : passes)
-        if (p.r != passes[0].r || (p.r != kWideRegBits && p.r != kWideFewRegBits) || p.t < kWideMinTile || p.t > 13)
-            return false;
-    for (const DevPhase &h : phases)
-        if (h.kind != 0 || h.R[0] != 0) return false;
-    return true;
-}
-
 // Lowers one phase's ops: gates on register bits to byte codes, the shears
 // of R_Y and R_X back to one op each, diagonal ops without a register bit to
 // the tail.
@@ -1092,9 +1081,12 @@ static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<D
     reduce();
 }
 
-void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
-                const std::vector<DevOp> &ops, WidePlan *out, std::vector<int> *slots)
+void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots)
 {
+    if (!plan.wide) return;
+    const std::vector<DevPass> &passes = plan.passes;
+    const std::vector<DevPhase> &phases = plan.phases;
+    const std::vector<DevOp> &ops = plan.ops;
     for (const DevPass &P : passes) {
         WidePass W;
         std::memset(&W, 0, sizeof W);
@@ -1292,6 +1284,15 @@ PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o)
     return pp;
 }
 
+PlanParams narrow_plan_params(PlanParams pp)
+{
+    if (pp.pack0) {
+        pp.r = 5;
+        pp.pack0 = 0;
+    }
+    return pp;
+}
+
 double plan_bytes(const Plan &p, qs_dtype dt)
 {
     return (double)p.passes.size() * 2.0 * std::ldexp(1.0, p.n) * (double)dtype_bytes(dt);
@@ -1378,6 +1379,7 @@ static qs_status plan_gates(const PlanParams &pp, const std::vector<PGate> &g, P
     P.n = n; P.t = pp.t; P.r = pp.r; P.c = pp.c; P.mode = pp.mode;
     P.precision = pp.precision;
     P.gates = (int)ng;
+    P.wide = pp.pack0 && pp.t >= kWideMinTile && pp.t <= 13 ? pp.r : 0;
 
     std::vector<char> done(ng, 0);
     std::vector<int> all(ng);
@@ -1703,8 +1705,8 @@ qs_status build_adjoint(int n, const qs_gate *gin, size_t ng, WidePlan *out, std
     if (qs_status st = plan_gates(pp, g, &plan)) return st;
     *out = WidePlan();
     param_of_slot->clear();
-    if (!wide_plan(plan.passes, plan.phases)) return set_error(QS_ERR_INVALID_ARG, "adjoint plan is not wide");
-    lower_wide(plan.passes, plan.phases, plan.ops, out, param_of_slot);
+    if (plan.wide != kWideRegBits) return set_error(QS_ERR_INVALID_ARG, "adjoint plan is not wide");
+    lower_wide(plan, out, param_of_slot);
     return QS_OK;
 }
 

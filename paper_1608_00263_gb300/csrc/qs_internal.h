@@ -183,6 +183,7 @@ struct Plan {
     std::vector<uint32_t> tc_words;  // TC mode: packed block matrices (see tc_prec)
     int precision = QS_PREC_FP16X3;  // TC mode: operand precision of tc_words
     int gates = 0;
+    int wide = 0;                    // register bits of the wide pass the plan was made for (0: none)
 };
 
 struct PlanParams {
@@ -294,13 +295,12 @@ struct WidePlan {
     std::vector<uint8_t> codes;
     std::vector<FoldArgs> folds;     // batches: folded prefixes (WidePass::fold)
 };
-// Whether a plan's passes can run the wide form: six register bits, register
-// phases only, tiles of at least 2^kWideMinTile.
-bool wide_plan(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases);
-// Lowers one plan's passes (phase and op indices into the given arrays) and
-// appends them to *out.
-void lower_wide(const std::vector<DevPass> &passes, const std::vector<DevPhase> &phases,
-                const std::vector<DevOp> &ops, WidePlan *out, std::vector<int> *slots = nullptr);
+// Lowers a plan that was made for the wide form (Plan::wide: qubit 0 in every
+// register set, ops counted for a wide pass) and appends its passes to *out;
+// other plans leave *out as it is.  The planner records the form: a plan made
+// for the (re, im) form can have register sets of the same shape, and holds up
+// to kMaxOpsPerPass ops a pass where a wide pass holds kMaxWideOps.
+void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots = nullptr);
 // The adjoint method's reverse sweep over `gates` on n >= kWideMinTile - 1
 // qubits as wide passes of n + 1 qubits, where qubit n -- in every tile, the
 // last register bit of every phase -- selects psi (0) or lambda (1): each gate
@@ -321,6 +321,9 @@ double bf16_bits_to_f64(uint16_t h);
 uint32_t f64_to_tf32_bits(double x);
 double tf32_bits_to_f64(uint32_t w);
 PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o);
+// The same with the five register bits of the (re, im) form where they give the
+// wide form (the gradient's forward evolution).
+PlanParams narrow_plan_params(PlanParams pp);
 double plan_bytes(const Plan &p, qs_dtype dt);
 
 // Persistent ensemble kernel: one launch runs a batch's whole work list

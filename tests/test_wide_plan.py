@@ -1,0 +1,61 @@
+"""Which plans the wide pass runs: those the planner made for it, and no
+others, whatever register sets they happen to have.  Its shared memory holds
+216 records a pass (kMaxWideOps), end codes included; a plan made for the
+(re, im) form holds up to 256 ops."""
+import ctypes
+import os
+import subprocess
+import tempfile
+
+import numpy as np
+import pytest
+
+import paper_1608_00263_gb300 as qs
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+MAX_WIDE_OPS = 216
+
+
+@pytest.fixture(scope="module")
+def probe():
+    so = os.path.join(tempfile.mkdtemp(prefix="qs_wide_"), "libprobe.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I" + os.path.join(ROOT, "include"),
+                    os.path.join(ROOT, "tests", "wide_plan_probe.cpp"),
+                    os.path.join(ROOT, "paper_1608_00263_gb300", "csrc", "qs_host.cpp"), "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    lib.probe_state.argtypes = [ctypes.c_int] * 5 + [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
+    return lib
+
+
+def low_qubit_gates(count, kinds, seed=0, qubits=5):
+    """Gates on the lowest qubits only: one pass, every register set with
+    qubit 0."""
+    rng = np.random.default_rng(seed)
+    g = np.zeros(count, dtype=qs.GATE_DTYPE)
+    g["kind"] = rng.choice(kinds, size=count)
+    for x in g:
+        x["q0"], x["q1"] = rng.choice(qubits, size=2, replace=False)
+    g["theta"] = rng.uniform(-3, 3, size=count)
+    return g
+
+
+CT = [qs.QS_H, qs.QS_X_HALF, qs.QS_Y_HALF, qs.QS_T, qs.QS_CZ]
+DIAG = [qs.QS_T, qs.QS_CZ, qs.QS_RZ, qs.QS_CPHASE]
+
+
+@pytest.mark.parametrize("kinds", [CT, DIAG, CT + DIAG], ids=["clifford_t", "diagonal", "both"])
+@pytest.mark.parametrize("n", [11, 12, 13, 14, 20])
+def test_one_state(probe, n, kinds):
+    g = low_qubit_gates(250, kinds)
+    out = (ctypes.c_int * 5)()
+    for mode, tile, narrow in [(qs.QS_MODE_FUSED, 0, 0), (qs.QS_MODE_FUSED, 11, 0), (qs.QS_MODE_FUSED, 0, 1),
+                               (qs.QS_MODE_FUSED, 12 if n > 11 else 11, 1), (qs.QS_MODE_FUSED_TC, 0, 0)]:
+        assert probe.probe_state(n, qs.QS_C64, mode, tile, narrow, g.ctypes.data, g.size, out) == 0
+        regs, wide, passes, records, ops = out
+        if mode == qs.QS_MODE_FUSED and not narrow:
+            assert wide == regs and passes >= 1 and records <= MAX_WIDE_OPS
+        else:
+            # the list that must not be lowered: one pass of more ops than
+            # the wide pass holds (or tensor-core phases)
+            assert regs == 5 and wide == 0 and passes == 0
+            assert mode == qs.QS_MODE_FUSED_TC or ops > MAX_WIDE_OPS

@@ -1,0 +1,35 @@
+// Which plans go to the wide pass, and how many records their passes hold
+// (test support only): plans made by the library's own planner with the
+// parameters its entry points use.
+#include <algorithm>
+#include <vector>
+
+#include "../paper_1608_00263_gb300/csrc/qs_internal.h"
+
+using namespace qs;
+
+// One state's plan.  narrow: as the gradient's forward evolution.  out: the
+// register bits the plan was made for, its wide form's (0: none), passes of
+// the lowered plan, most records of one of them, most ops of a planned pass.
+extern "C" int probe_state(int n, int dtype, int mode, int tile, int narrow, const qs_gate *g, size_t ng, int *out)
+{
+    qs_opts o{};
+    o.mode = mode;
+    o.tile_log2 = tile;
+    PlanParams pp = default_plan_params(n, (qs_dtype)dtype, &o);
+    if (narrow) pp = narrow_plan_params(pp);
+    Plan plan;
+    if (build_plan(pp, g, ng, &plan) != QS_OK) return -1;
+    WidePlan w;
+    lower_wide(plan, &w);
+    out[0] = plan.r;
+    out[1] = plan.wide;
+    out[2] = (int)w.passes.size();
+    out[3] = out[4] = 0;
+    for (const WidePass &p : w.passes) out[3] = std::max(out[3], (int)p.nops);
+    for (const DevPass &p : plan.passes) {
+        const DevPhase *h = plan.phases.data() + p.phase_begin;
+        out[4] = std::max(out[4], h[p.nphases - 1].op_end - h[0].op_begin);
+    }
+    return 0;
+}
