@@ -131,16 +131,7 @@ static qs_status plan_instances(const qs_batch *b, const qs_gate *gates, const u
                 const int i = idx[k];
                 const size_t ng = (size_t)(offsets[i + 1] - offsets[i]) - hl[i];
                 if (ng == 0) continue;
-                qs_opts o{};
-                o.mode = QS_MODE_FUSED;
-                o.tile_log2 = tbits[i];
-                PlanParams pp = default_plan_params(b->n[i], QS_C64, &o);
-                if (wide) {
-                    pp.r = kWideRegBits;
-                } else {
-                    pp.r = std::min(5, pp.t);
-                    pp.pack0 = 0;
-                }
+                const PlanParams pp = batch_plan_params(b->n[i], tbits[i], wide);
                 // wide passes: the leading layer and the diagonal prefix after it
                 // are generated by the instance's first pass (nfold = -1: a
                 // generated uniform state)
@@ -183,24 +174,6 @@ struct Rounds {
     double bytes = 0;                // algorithmic bytes (16 per amplitude per pass)
     WidePlan wide;                   // the passes lowered, when they are wide passes
 };
-
-// Lowers the listed instances' plans in list order (the order in which
-// their passes are concatenated) when all are wide passes; else empty.
-static void lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds,
-                            const std::vector<int> &idx, WidePlan *out)
-{
-    *out = WidePlan();
-    for (int i : idx)
-        if (!plans[i].passes.empty() && !plans[i].wide) return;
-    for (int i : idx) {
-        const size_t first = out->passes.size();
-        lower_wide(plans[i], out);
-        if (!folds[i].nfold || out->passes.size() == first) continue;
-        out->folds.push_back(folds[i]);
-        out->passes[first].fold = (int32_t)out->folds.size();
-        out->passes[first].canon_in = 0;
-    }
-}
 
 // Instances whose first pass generates their state need no initial chunks.
 static void drop_initial_chunks(const std::vector<FoldArgs> &folds, Work *W)

@@ -1136,6 +1136,22 @@ void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots)
     out->codes.resize(out->ops.size(), 0);
 }
 
+void lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds, const std::vector<int> &idx,
+                     WidePlan *out)
+{
+    *out = WidePlan();
+    for (int i : idx)
+        if (!plans[i].passes.empty() && plans[i].wide != kWideRegBits) return;
+    for (int i : idx) {
+        const size_t first = out->passes.size();
+        lower_wide(plans[i], out);
+        if (!folds[i].nfold || out->passes.size() == first) continue;
+        out->folds.push_back(folds[i]);
+        out->passes[first].fold = (int32_t)out->folds.size();
+        out->passes[first].canon_in = 0;
+    }
+}
+
 // Persistent ensemble work list (declared with its order and dependency
 // rules in qs_internal.h).
 static uint64_t tiles_per_item(int t, int item_bits) { return t >= item_bits ? 1 : (1ULL << (item_bits - t)); }
@@ -1290,6 +1306,17 @@ PlanParams narrow_plan_params(PlanParams pp)
         pp.r = 5;
         pp.pack0 = 0;
     }
+    return pp;
+}
+
+PlanParams batch_plan_params(int n, int tile_log2, bool wide)
+{
+    qs_opts o{};
+    o.mode = QS_MODE_FUSED;
+    o.tile_log2 = tile_log2;
+    PlanParams pp = default_plan_params(n, QS_C64, &o);
+    pp.r = std::min(wide ? kWideRegBits : 5, pp.t);
+    pp.pack0 = wide;
     return pp;
 }
 

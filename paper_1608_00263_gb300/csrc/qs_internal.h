@@ -301,6 +301,12 @@ struct WidePlan {
 // for the (re, im) form can have register sets of the same shape, and holds up
 // to kMaxOpsPerPass ops a pass where a wide pass holds kMaxWideOps.
 void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots = nullptr);
+// Lowers the listed instances' plans in list order (the order in which their
+// passes are concatenated) when every one that has passes was made for the six
+// register bits of the batch kernels, and marks the first passes that generate
+// their instance's state (folds); else *out is left empty.
+void lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds, const std::vector<int> &idx,
+                     WidePlan *out);
 // The adjoint method's reverse sweep over `gates` on n >= kWideMinTile - 1
 // qubits as wide passes of n + 1 qubits, where qubit n -- in every tile, the
 // last register bit of every phase -- selects psi (0) or lambda (1): each gate
@@ -324,6 +330,9 @@ PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o);
 // The same with the five register bits of the (re, im) form where they give the
 // wide form (the gradient's forward evolution).
 PlanParams narrow_plan_params(PlanParams pp);
+// Of a batch instance, tile 2^tile_log2 (0: the default): for the batch
+// kernels' wide passes, or for five register bits of the (re, im) form.
+PlanParams batch_plan_params(int n, int tile_log2, bool wide);
 double plan_bytes(const Plan &p, qs_dtype dt);
 
 // Persistent ensemble kernel: one launch runs a batch's whole work list

@@ -59,3 +59,35 @@ def test_gradient(n):
     assert loss == pytest.approx(-np.mean(np.log(p[x])), abs=1e-9)
     assert loss32 == pytest.approx(loss, abs=1e-4)
     assert np.max(np.abs(grad32 - grad)) < 1e-4 * np.max(np.abs(grad))
+
+
+@pytest.mark.parametrize("first", ["empty", "layer"])
+@pytest.mark.parametrize("small", [8, 10])
+def test_batch_with_a_small_instance_without_passes(small, first):
+    """The others plan five register bits there; both engines against the
+    oracle.  Tolerance: the ensemble statistics', 1e-6 (entropy) and 1e-5
+    (moments) relative."""
+    sizes = (small, 12, 13)
+    rng = np.random.default_rng(small)
+    layer = lambda n: O.generate_circuit(1, n, 0, 0)[:n]
+    for count in (1, 3, 12, 60):
+        gl = [layer(small)[:0] if first == "empty" else layer(small)]
+        for n in sizes[1:]:
+            g = np.zeros(count, dtype=qs.GATE_DTYPE)
+            g["kind"] = rng.choice(CT + [qs.QS_RX, qs.QS_RY, qs.QS_RZ, qs.QS_CPHASE], size=count)
+            for x in g:
+                x["q0"], x["q1"] = rng.choice(n, size=2, replace=False)
+            g["kind"][0], g["q0"][0] = qs.QS_RY, 0
+            g["theta"] = rng.uniform(-3, 3, size=count)
+            gl.append(np.concatenate([layer(n), g]).astype(qs.GATE_DTYPE))
+        b = qs.qs_batch_create(sizes)
+        try:
+            for engine in (qs.QS_BATCH_PERSISTENT, qs.QS_BATCH_ROUNDS):
+                qs.qs_batch_set_engine(b, engine)
+                rows = qs.qs_batch_run(b, gl, kmax=4)
+                for i, n in enumerate(sizes[1:], 1):
+                    p = O.probabilities(O.simulate(n, gl[i]))
+                    assert rows[i, 1] == pytest.approx(O.entropy(p), rel=1e-6), (engine, count, i)
+                    assert np.allclose(rows[i, 3:], O.moments(p, 4), rtol=1e-5), (engine, count, i)
+        finally:
+            qs.qs_batch_destroy(b)

@@ -24,6 +24,7 @@ def probe():
                     os.path.join(ROOT, "paper_1608_00263_gb300", "csrc", "qs_host.cpp"), "-o", so], check=True)
     lib = ctypes.CDLL(so)
     lib.probe_state.argtypes = [ctypes.c_int] * 5 + [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
+    lib.probe_batch.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 3 + [ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
     return lib
 
 
@@ -59,3 +60,24 @@ def test_one_state(probe, n, kinds):
             # the wide pass holds (or tensor-core phases)
             assert regs == 5 and wide == 0 and passes == 0
             assert mode == qs.QS_MODE_FUSED_TC or ops > MAX_WIDE_OPS
+
+
+@pytest.mark.parametrize("count", [1, 5, 10, 20, 40])
+def test_batch(probe, count):
+    """An instance without passes (no gates) does not decide for the others:
+    plans of five register bits stay in their form, wide ones have six."""
+    rng = np.random.default_rng(count)
+    sizes = np.array([8, 12], dtype=np.int32)
+    regs = ctypes.c_int(0)
+    for _ in range(60):
+        g = np.zeros(count, dtype=qs.GATE_DTYPE)
+        g["kind"] = rng.choice(CT + DIAG + [qs.QS_RX, qs.QS_RY], size=count)
+        for x in g:
+            x["q0"], x["q1"] = rng.choice(12, size=2, replace=False)
+        g["theta"] = rng.uniform(-3, 3, size=count)
+        offsets = np.array([0, 0, count], dtype=np.uint64)
+        args = (2, sizes.ctypes.data, g.ctypes.data, offsets.ctypes.data)
+        assert probe.probe_batch(*args, 0, ctypes.byref(regs)) == 0
+    big = np.array([12, 12], dtype=np.int32)
+    assert probe.probe_batch(2, big.ctypes.data, g.ctypes.data, offsets.ctypes.data, 1, ctypes.byref(regs)) >= 1
+    assert regs.value == 6

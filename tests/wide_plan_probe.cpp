@@ -33,3 +33,23 @@ extern "C" int probe_state(int n, int dtype, int mode, int tile, int narrow, con
     }
     return 0;
 }
+
+// Instances of one batch, planned with five register bits of the (re, im)
+// form or for the wide pass, and lowered together.  Returns the number of
+// lowered passes (0: the batch runs the plans as they are); *regs: their
+// register bits.
+extern "C" int probe_batch(int count, const int *n, const qs_gate *g, const uint64_t *offsets, int wide, int *regs)
+{
+    std::vector<Plan> plans(count);
+    std::vector<int> idx(count);
+    for (int i = 0; i < count; ++i) {
+        idx[i] = i;
+        const size_t ng = (size_t)(offsets[i + 1] - offsets[i]);
+        if (ng && build_plan(batch_plan_params(n[i], 0, wide != 0), g + offsets[i], ng, &plans[i]) != QS_OK) return -1;
+    }
+    WidePlan w;
+    lower_instances(plans, std::vector<FoldArgs>(count), idx, &w);
+    *regs = 0;
+    for (const WidePass &p : w.passes) *regs |= p.r;
+    return (int)w.passes.size();
+}
