@@ -240,7 +240,7 @@ static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs
         const size_t b_blk = p.tc_words.size() * sizeof(uint32_t);
         // plans made for the wide pass go up lowered
         WidePlan wide;
-        lower_wide(p, &wide);
+        if (qs_status st = lower_wide(p, &wide)) return st;
         const size_t w_pass = wide.passes.size() * sizeof(WidePass), w_ops = wide.ops.size() * sizeof(WideOp);
         const size_t total = (w_pass ? w_pass + w_ops + wide.codes.size() : b_pass + b_phase + b_ops + b_blk) + 16;
         if (c->bytes < total) {

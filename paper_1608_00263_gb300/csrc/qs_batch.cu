@@ -197,8 +197,8 @@ static bool any_full(const WidePlan &w)
     return false;
 }
 
-static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds,
-                         const std::vector<int> &idx, Rounds *R)
+static qs_status build_rounds(const qs_batch *b, const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds,
+                              const std::vector<int> &idx, Rounds *R)
 {
     *R = Rounds();
     std::vector<int> first_pass(b->count, 0);
@@ -219,7 +219,7 @@ static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, cons
         max_passes = std::max(max_passes, (int)plans[i].passes.size());
         R->bytes += (double)plans[i].passes.size() * 16.0 * std::ldexp(1.0, b->n[i]);
     }
-    lower_instances(plans, folds, idx, &R->wide);
+    if (qs_status st = lower_instances(plans, folds, idx, &R->wide)) return st;
     const size_t isz = batch_item_bytes();
     for (int r = 0; r < max_passes; ++r)
         for (int tb = 5; tb <= 13; ++tb) {
@@ -240,6 +240,7 @@ static void build_rounds(const qs_batch *b, const std::vector<Plan> &plans, cons
             }
             if (L.count) R->launches.push_back(L);
         }
+    return QS_OK;
 }
 
 // Section offsets of a packed run in a device buffer: passes | phases | ops
@@ -367,7 +368,7 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
     RoundOffsets o;
     std::vector<unsigned char> host;
     if (b->engine == QS_BATCH_ROUNDS) {
-        build_rounds(b, plans, folds, idx, &R);
+        if (qs_status st = build_rounds(b, plans, folds, idx, &R)) return st;
         *empty = R.launches.empty();
         o = round_offsets(R);
         host.assign(o.total, 0);
@@ -375,7 +376,7 @@ static qs_status time_plans(qs_batch *b, const std::vector<Plan> &plans, const s
     } else {
         build_work(b->n, b->off, plans, full_flags(plans), idx, hl, false, &W);
         *empty = W.passes.empty();
-        lower_instances(plans, folds, idx, &wide);
+        if (qs_status st = lower_instances(plans, folds, idx, &wide)) return st;
         drop_initial_chunks(folds, &W);
         o = work_offsets(W, wide);
         host.assign(o.total, 0);
@@ -675,7 +676,7 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
         build_work(b->n, b->off, plans, full_flags(plans), all, hl, true, &W);
         b->round_bytes = W.bytes;
         WidePlan wide;
-        lower_instances(plans, folds, all, &wide);
+        if (qs_status s0 = lower_instances(plans, folds, all, &wide)) return s0;
         drop_initial_chunks(folds, &W);
         const RoundOffsets wo = work_offsets(W, wide);
         std::vector<unsigned char> host(wo.total, 0);
@@ -693,7 +694,7 @@ static qs_status batch_prepare(qs_batch *b, const qs_gate *gates, const uint64_t
         return batch_end_capture(b, rs);
     }
     Rounds R;
-    build_rounds(b, plans, folds, all, &R);
+    if (qs_status s0 = build_rounds(b, plans, folds, all, &R)) return s0;
     b->round_bytes = R.bytes;
     // statistics items
     std::vector<uint64_t> s_off, s_cnt;

@@ -1081,9 +1081,9 @@ static void lower_phase(const DevPass &P, const DevPhase &H, const std::vector<D
     reduce();
 }
 
-void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots)
+qs_status lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots)
 {
-    if (!plan.wide) return;
+    if (!plan.wide) return QS_OK;
     const std::vector<DevPass> &passes = plan.passes;
     const std::vector<DevPhase> &phases = plan.phases;
     const std::vector<DevOp> &ops = plan.ops;
@@ -1120,6 +1120,9 @@ void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots)
             V.op_end = (int16_t)(out->ops.size() - W.op_begin);
         }
         W.nops = (int)(out->ops.size() - W.op_begin);
+        if (W.nops > kMaxWideOps)
+            return set_error(QS_ERR_UNSUPPORTED, "pass %zu: %d records, a wide pass holds %d", out->passes.size(), W.nops,
+                             kMaxWideOps);
         // between the passes of a plan units are kept as the kernel works on
         // them; the first reads and the last writes canonical order
         W.canon_in = &P == &passes.front();
@@ -1134,22 +1137,25 @@ void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots)
     }
     out->ops.resize((out->ops.size() + 31) / 16 * 16);
     out->codes.resize(out->ops.size(), 0);
+    return QS_OK;
 }
 
-void lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds, const std::vector<int> &idx,
-                     WidePlan *out)
+qs_status lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds, const std::vector<int> &idx,
+                          WidePlan *out)
 {
     *out = WidePlan();
     for (int i : idx)
-        if (!plans[i].passes.empty() && plans[i].wide != kWideRegBits) return;
+        if (!plans[i].passes.empty() && plans[i].wide != kWideRegBits) return QS_OK;
     for (int i : idx) {
         const size_t first = out->passes.size();
-        lower_wide(plans[i], out);
+        if (qs_status st = lower_wide(plans[i], out))
+            return set_error(st, "instance %d: %s", i, last_error_cstr());
         if (!folds[i].nfold || out->passes.size() == first) continue;
         out->folds.push_back(folds[i]);
         out->passes[first].fold = (int32_t)out->folds.size();
         out->passes[first].canon_in = 0;
     }
+    return QS_OK;
 }
 
 // Persistent ensemble work list (declared with its order and dependency
@@ -1733,8 +1739,7 @@ qs_status build_adjoint(int n, const qs_gate *gin, size_t ng, WidePlan *out, std
     *out = WidePlan();
     param_of_slot->clear();
     if (plan.wide != kWideRegBits) return set_error(QS_ERR_INVALID_ARG, "adjoint plan is not wide");
-    lower_wide(plan, out, param_of_slot);
-    return QS_OK;
+    return lower_wide(plan, out, param_of_slot);
 }
 
 }  // namespace qs

@@ -300,13 +300,15 @@ struct WidePlan {
 // other plans leave *out as it is.  The planner records the form: a plan made
 // for the (re, im) form can have register sets of the same shape, and holds up
 // to kMaxOpsPerPass ops a pass where a wide pass holds kMaxWideOps.
-void lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots = nullptr);
+// QS_ERR_UNSUPPORTED where a pass would hold more records than a CTA has room
+// for (the planner's counts keep below that).
+qs_status lower_wide(const Plan &plan, WidePlan *out, std::vector<int> *slots = nullptr);
 // Lowers the listed instances' plans in list order (the order in which their
 // passes are concatenated) when every one that has passes was made for the six
 // register bits of the batch kernels, and marks the first passes that generate
 // their instance's state (folds); else *out is left empty.
-void lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds, const std::vector<int> &idx,
-                     WidePlan *out);
+qs_status lower_instances(const std::vector<Plan> &plans, const std::vector<FoldArgs> &folds, const std::vector<int> &idx,
+                          WidePlan *out);
 // The adjoint method's reverse sweep over `gates` on n >= kWideMinTile - 1
 // qubits as wide passes of n + 1 qubits, where qubit n -- in every tile, the
 // last register bit of every phase -- selects psi (0) or lambda (1): each gate

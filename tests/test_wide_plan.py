@@ -25,6 +25,8 @@ def probe():
     lib = ctypes.CDLL(so)
     lib.probe_state.argtypes = [ctypes.c_int] * 5 + [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
     lib.probe_batch.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 3 + [ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    lib.probe_oversize.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t]
+    lib.probe_sweep.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t]
     return lib
 
 
@@ -81,3 +83,26 @@ def test_batch(probe, count):
     big = np.array([12, 12], dtype=np.int32)
     assert probe.probe_batch(2, big.ctypes.data, g.ctypes.data, offsets.ctypes.data, 1, ctypes.byref(regs)) >= 1
     assert regs.value == 6
+
+
+@pytest.mark.parametrize("count,status", [(215, 0), (216, 5), (250, 5)])
+def test_a_pass_with_too_many_records_is_an_error(probe, count, status):
+    """215 ops and the end code are 216 records; more is QS_ERR_UNSUPPORTED
+    (status 5), not a write past the table."""
+    g = low_qubit_gates(count, [qs.QS_H, qs.QS_X_HALF, qs.QS_Y_HALF])
+    assert probe.probe_oversize(12, g.ctypes.data, g.size) == status
+
+
+ANY = CT + DIAG + [qs.QS_RX, qs.QS_RY]
+
+
+@pytest.mark.parametrize("kinds", [DIAG, [qs.QS_RZ, qs.QS_CPHASE], [qs.QS_RY, qs.QS_CZ], [qs.QS_RX, qs.QS_RZ], CT, ANY],
+                         ids=["diagonal", "phases", "ry_cz", "rx_rz", "clifford_t", "all"])
+@pytest.mark.parametrize("n", [10, 12, 13, 20])
+def test_records_of_a_reverse_sweep(probe, n, kinds):
+    """The planner's count bounds the records of the sweep's passes, which hold
+    derivative terms and their sums besides the gates."""
+    for count in (1, 60, 400, 900):
+        for qubits in (2, 5, n):
+            g = low_qubit_gates(count, kinds, seed=count + qubits, qubits=qubits)
+            assert 0 < probe.probe_sweep(n, g.ctypes.data, g.size) <= MAX_WIDE_OPS

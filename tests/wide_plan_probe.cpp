@@ -53,3 +53,27 @@ extern "C" int probe_batch(int count, const int *n, const qs_gate *g, const uint
     for (const WidePass &p : w.passes) *regs |= p.r;
     return (int)w.passes.size();
 }
+
+// A plan that says it was made for the wide pass and holds more ops than one
+// (the mistake is planted here): what lowering it returns.
+extern "C" int probe_oversize(int n, const qs_gate *g, size_t ng)
+{
+    Plan plan;
+    if (build_plan(batch_plan_params(n, 0, false), g, ng, &plan) != QS_OK) return -1;
+    plan.wide = kWideRegBits;
+    WidePlan w;
+    const qs_status st = lower_wide(plan, &w);
+    if (lower_instances({plan}, {FoldArgs{}}, {0}, &w) != st) return -1;
+    return (int)st;
+}
+
+// The reverse sweep's plan: most records of a pass, or -1.
+extern "C" int probe_sweep(int n, const qs_gate *g, size_t ng)
+{
+    WidePlan w;
+    std::vector<int> slots;
+    if (build_adjoint(n, g, ng, &w, &slots) != QS_OK) return -1;
+    int most = 0;
+    for (const WidePass &p : w.passes) most = std::max(most, (int)p.nops);
+    return most;
+}
