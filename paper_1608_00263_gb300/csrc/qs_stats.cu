@@ -1369,7 +1369,8 @@ k_cross_entropy(const typename V2T<R>::T *__restrict__ a, uint64_t N, const uint
             const double re = (double)v[g].x, im = (double)v[g].y;
             const double p = re * re + im * im;
             const long long b = __double_as_longlong(p);
-            const int e = (int)(b >> 52);             // p >= 0: no sign bit
+            // (with the sign bit: p >= 0, but a NaN may carry either sign)
+            const int e = (int)((unsigned long long)b >> 52);
             if (e == 0 || e >= 0x7FF) {
                 acc[0] -= log(p);
             } else {
