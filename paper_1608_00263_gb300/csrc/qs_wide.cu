@@ -171,22 +171,26 @@ k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int
                                                       smem_dyn, 0, folds);
             }
         }
+        // Thread 0 overwrites the item once it has taken the next one: the
+        // others have read what they need of it before the last barrier.
+        const bool stats = w.kind == kPersistStats;
         __syncthreads();
         if (threadIdx.x == 0) {
             __threadfence();
             const uint32_t prev = atomicAdd(done + w.inst, 1u);
-            if (w.kind == kPersistStats) {
+            if (stats) {
                 s_last = prev + 1 == w.total;
                 __threadfence();
             }
         }
-        if (w.kind == kPersistStats) {
+        if (stats) {
             __syncthreads();
             if (s_last && threadIdx.x < kStatAcc) {
                 double acc = 0;
                 for (uint32_t j = 0; j < w.nslots; ++j) acc += __ldcg(part + (size_t)(w.hi + j) * kStatAcc + threadIdx.x);
                 sums[(size_t)w.inst * kStatAcc + threadIdx.x] = acc;
             }
+            __syncthreads();
         }
     }
 }
