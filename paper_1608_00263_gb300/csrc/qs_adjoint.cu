@@ -363,7 +363,7 @@ static qs_status adjoint_t(qs_state *s, const qs_gate *g, size_t ng, const uint6
     V *psi = (V *)s->amps, *lam = nullptr;
     const int ctas = 3 * s->num_sms;          // three CTAs per SM (64 KB of tiles each)
     const size_t smem = 2 * ((size_t)1 << t) * sizeof(V);
-    QS_CUDA_TRY(cudaFuncSetAttribute(k_adj_group<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QS_CUDA_TRY(cudaFuncSetAttribute(k_adj_group<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes));
     // device tables: groups | gates | scale (in sweep-slot order) | partials | sums
     const size_t b_grp = groups.size() * sizeof(AdjGroup), b_gate = gates.size() * sizeof(AdjGate);
     const size_t b_scale = (nparam ? nparam : 1) * sizeof(double);

@@ -1362,7 +1362,7 @@ static qs_status run_fused_t(qs_state *s, const Plan &plan, const void *dev_plan
                             ? (fold_here ? k_fused_pass<R, RB, 0, true, true> : k_fused_pass<R, RB, 0, true>)
                             : (fold_here ? k_fused_pass<R, RB, 0, false, true> : k_fused_pass<R, RB, 0, false>);
             const size_t smem = (size_t(1) << hp.t) * sizeof(V);
-            QS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            QS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes));
             const uint64_t cap = (uint64_t)s->num_sms * 2;
             const int grid = (int)(ntiles < cap ? ntiles : cap);
             kern<<<grid, threads, smem, s->stream>>>((V *)s->amps, dpass + p, dphase, dops, ntiles, nullptr, nullptr,

@@ -107,6 +107,11 @@ struct DevOp {          // 80 bytes
 };
 
 constexpr int kMaxTileBits = 16;
+// Largest tile of a register pass (2^13 complex64 or 2^12 complex128
+// amplitudes).  Kernels are allowed this much dynamic shared memory whatever
+// tile a launch has: the allowance belongs to the kernel, and another host
+// thread's smaller tile would lower it between this thread's call and launch.
+constexpr int kTileBytes = 65536;
 constexpr int kMaxRegBits = 8;
 constexpr int kMaxPhasesPerPass = 8;    // per-thread phase tables live in shared memory
 constexpr int kMaxOpsPerPass = 256;     // op descriptors live in shared memory

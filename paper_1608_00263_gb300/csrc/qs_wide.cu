@@ -54,7 +54,7 @@ qs_status run_wide_plan(qs_state *s, const std::vector<WidePass> &passes, size_t
         auto kern = P.r == kWideRegBits ? wide_pass_kernel<kWideRegBits>(P.full != 0, first)
                                         : wide_pass_kernel<kWideFewRegBits>(P.full != 0, first);
         const size_t smem = (size_t(1) << P.t) * sizeof(float2);
-        QS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        QS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes));
         const uint32_t ntiles = 1u << (P.n - P.t), cap = (uint32_t)s->num_sms * (P.r == kWideRegBits ? 3 : 2);
         kern<<<(int)(ntiles < cap ? ntiles : cap), 1 << (P.t - P.r), smem, s->stream>>>(
             (float2 *)s->amps, dpass + p, dops, dcodes, ntiles, first && fold ? *fold : none);
@@ -94,7 +94,7 @@ qs_status launch_adjoint_wide(const qs_state *s, void *lam, const WidePlan &plan
     for (size_t p = 0; p < plan.passes.size(); ++p) {
         const WidePass &P = plan.passes[p];
         const size_t smem = (size_t(1) << P.t) * sizeof(float2);
-        if (p == 0) QS_CUDA_TRY(cudaFuncSetAttribute(k_adj_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (p == 0) QS_CUDA_TRY(cudaFuncSetAttribute(k_adj_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes));
         const uint32_t ntiles = 1u << (P.n - P.t), cap = (uint32_t)s->num_sms * 3;
         k_adj_wide<<<(int)(ntiles < cap ? ntiles : cap), 1 << (P.t - kWideRegBits), smem, s->stream>>>(
             (float2 *)s->amps, lam_off, dpass + p, dops, dcodes, ntiles, part, (uint32_t)adjoint_wide_partials(s));
