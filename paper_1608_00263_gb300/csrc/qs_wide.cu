@@ -27,6 +27,7 @@ k_wide_pass(float2 *__restrict__ amps, const WidePass *__restrict__ pass_g, cons
             F.m[0] = fold.m1;
             F.m[1] = fold.m2;
             F.m[2] = fold.m4;
+            F.plain = fold.nfold == 0;
         }
         wide_pass_body<FULL ? 1 : 0, 1, 0, RB>(amps, pass_g, ops_g, codes_g, t_begin, t_end, S, &F, smem_dyn);
     } else {
