@@ -215,12 +215,14 @@ extern "C" qs_status qs_state_reset(qs_state *s)
     return QS_OK;
 }
 
-static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs_opts *o,
+// generated: the first pass generates the state (else it reads it).
+static qs_status get_plan(qs_state *s, const qs_gate *gates, size_t ng, const qs_opts *o, bool generated,
                           const Plan **plan, const void **dev, DevicePlanSlot **slot_out = nullptr,
                           bool narrow = false)
 {
     PlanParams pp = default_plan_params(s->n, s->dt, o);
     if (narrow) pp = narrow_plan_params(pp);
+    if (!generated) pp = held_plan_params(pp, gates, ng);
     DevicePlanCache &pc = s->plan_cache;
     DevicePlanSlot *c = nullptr;
     for (DevicePlanSlot &x : pc.slot)
@@ -449,7 +451,7 @@ static qs_status qs_apply_circuit_impl(qs_state *s, const qs_gate *gates, size_t
     const Plan *plan;
     const void *dev;
     DevicePlanSlot *slot;
-    if (qs_status st = get_plan(s, gates, ngates, opts, &plan, &dev, &slot, narrow)) {
+    if (qs_status st = get_plan(s, gates, ngates, opts, uniform != 0.0, &plan, &dev, &slot, narrow)) {
         // the leading layer is still applied, as when it is written first
         if (uniform != 0.0) launch_init_uniform(s);
         return st;
@@ -478,6 +480,7 @@ extern "C" qs_status qs_prepare_circuit(qs_state *s, const qs_gate *gates, size_
     // a leading Hadamard layer is written as the uniform state when the
     // circuit starts from |0...0> (the usual reset + apply): plan the rest
     std::vector<qs_gate> rest;
+    bool generated = false;
     if (!s->escaped) {
         const size_t h = leading_h_layer(gates, ngates, s->n);
         if (h && ngates > h && s->n >= rb && mode == QS_MODE_FUSED) {
@@ -486,16 +489,17 @@ extern "C" qs_status qs_prepare_circuit(qs_state *s, const qs_gate *gates, size_
             if (fold_diagonal_prefix(gates + h, ngates - h, &rest, &fold) > 0 && !rest.empty()) {
                 const Plan *plan;
                 const void *dev;
-                return get_plan(s, rest.data(), rest.size(), opts, &plan, &dev);
+                return get_plan(s, rest.data(), rest.size(), opts, true, &plan, &dev);
             }
         }
         gates += h;
         ngates -= h;
         if (ngates == 0) return QS_OK;
+        generated = h != 0;
     }
     const Plan *plan;
     const void *dev;
-    return get_plan(s, gates, ngates, opts, &plan, &dev);
+    return get_plan(s, gates, ngates, opts, generated, &plan, &dev);
 }
 
 static qs_status qs_probabilities_impl(const qs_state *s, void *out, int out_is_fp64)

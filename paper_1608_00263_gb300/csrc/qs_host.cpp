@@ -1315,6 +1315,35 @@ PlanParams narrow_plan_params(PlanParams pp)
     return pp;
 }
 
+// A few gates that one pass applies to a state in memory: the pass moves the
+// state and does little else, and there two CTAs of 256 threads of the (re, im)
+// form beat three of 128 that reorder the units they read.  Microseconds of a
+// call, wide : (re, im), where the state or a good part of it stays in L2:
+//   qubits        22           23           24           25
+//   1 gate    32.6 : 27.6  41.7 : 34.2  71.8 : 66.3  113.8 : 109.4
+//   12 gates  33.1 : 32.8  42.4 : 41.5  73.5 : 73.0  120.0 : 121.0
+//   16 gates  32.6 : 32.5  44.0 : 41.9  76.2 : 76.7  119.0 : 121.4
+//   24 gates  33.7 : 36.8  44.0 : 46.0  75.4 : 82.4  124.2 : 131.7
+// so the line is at 16 gates up to 64 MB, at 12 above; at 21 qubits (five
+// register bits, 256 CTAs) at 5: 24.9 : 23.0 there, 1.0 at eight.  Larger states:
+// for the loop with parameterised gates only, 26 and 27 qubits, one gate 209.6 :
+// 203.1 and 392.0 : 386.6, eight 216.3 : 211.1 and 409.7 : 394.3, twelve 218.2 :
+// 227.9 and 408.3 : 425.4.  Elsewhere one gate takes the same within 1.5 %.
+PlanParams held_plan_params(PlanParams pp, const qs_gate *g, size_t ng)
+{
+    if (!pp.pack0 || pp.t != 13 || pp.n < 21 || pp.n > 27) return pp;
+    const size_t most = pp.n == 21 ? 5 : pp.n <= 23 ? 16 : pp.n <= 25 ? 12 : 8;
+    if (ng > most) return pp;
+    uint64_t tile = (1ULL << pp.c) - 1;
+    bool param = false;
+    for (size_t i = 0; i < ng; ++i) {
+        if (!gate_is_diagonal(g[i].kind)) tile |= 1ULL << g[i].q0;
+        param = param || g[i].kind >= QS_RX;
+    }
+    if (popcount64(tile) > pp.t || (pp.n > 25 && !param)) return pp;
+    return narrow_plan_params(pp);
+}
+
 PlanParams batch_plan_params(int n, int tile_log2, bool wide)
 {
     qs_opts o{};

@@ -337,6 +337,8 @@ PlanParams default_plan_params(int n, qs_dtype dt, const qs_opts *o);
 // The same with the five register bits of the (re, im) form where they give the
 // wide form (the gradient's forward evolution).
 PlanParams narrow_plan_params(PlanParams pp);
+// The same for a list of a few gates on a state that its first pass reads.
+PlanParams held_plan_params(PlanParams pp, const qs_gate *g, size_t ng);
 // Of a batch instance, tile 2^tile_log2 (0: the default): for the batch
 // kernels' wide passes, or for five register bits of the (re, im) form.
 PlanParams batch_plan_params(int n, int tile_log2, bool wide);

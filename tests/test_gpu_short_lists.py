@@ -1,6 +1,7 @@
-"""Lists of a few gates on one state against the FP64 oracle: on the uniform
-state that the first pass generates with nothing folded into it.  Tolerance:
-the state bound of complex64, 1e-5 relative L2."""
+"""Lists of a few gates on one state against the FP64 oracle: on a state in
+memory on both sides of the line between the (re, im) form and the wide pass
+(5 gates at 21 qubits, 16 at 22), and on the uniform state that the first pass generates with nothing folded into
+it.  Tolerance: the state bound of complex64, 1e-5 relative L2."""
 import numpy as np
 import pytest
 
@@ -27,6 +28,29 @@ def gate_list(rng, n, count, kinds):
         x["q0"], x["q1"] = rng.choice(n, size=2, replace=False)
     g["theta"] = rng.uniform(-7, 7, size=count)
     return g
+
+
+@pytest.mark.parametrize("kinds", [CT, ALL], ids=["clifford_t", "all"])
+@pytest.mark.parametrize("n", [21, 22])
+def test_state_in_memory(n, kinds):
+    rng = np.random.default_rng(n)
+    start = (rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)) * 2.0 ** (-0.5 * (n + 1))
+    start = start.astype(np.complex64)
+    h = qs.qs_state_create(n)
+    try:
+        for count in (1, 5, 6, 16, 17):
+            g = gate_list(rng, n, count, kinds)
+            for prepare in (False, True):
+                qs.qs_state_copy_in(h, start)
+                if prepare:
+                    qs.qs_prepare_circuit(h, g)
+                qs.qs_apply_circuit(h, g)
+                ref = start.astype(np.complex128)
+                O.apply_circuit(ref, g)
+                got = qs.qs_state_copy_out(h, n)
+                assert np.linalg.norm(got - ref) < 1e-5 * np.linalg.norm(ref), (count, prepare)
+    finally:
+        qs.qs_state_destroy(h)
 
 
 @pytest.mark.parametrize("n", [5, 10, 11, 12, 13, 14, 19, 21, 22])

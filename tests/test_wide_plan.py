@@ -25,6 +25,7 @@ def probe():
     lib = ctypes.CDLL(so)
     lib.probe_state.argtypes = [ctypes.c_int] * 5 + [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p]
     lib.probe_batch.argtypes = [ctypes.c_int] + [ctypes.c_void_p] * 3 + [ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    lib.probe_held.argtypes = [ctypes.c_int] * 4 + [ctypes.c_void_p, ctypes.c_size_t, ctypes.POINTER(ctypes.c_int)]
     lib.probe_oversize.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t]
     lib.probe_sweep.argtypes = [ctypes.c_int, ctypes.c_void_p, ctypes.c_size_t]
     return lib
@@ -106,3 +107,32 @@ def test_records_of_a_reverse_sweep(probe, n, kinds):
         for qubits in (2, 5, n):
             g = low_qubit_gates(count, kinds, seed=count + qubits, qubits=qubits)
             assert 0 < probe.probe_sweep(n, g.ctypes.data, g.size) <= MAX_WIDE_OPS
+
+
+@pytest.mark.parametrize("n", [12, 20, 21, 22, 23, 24, 25, 26, 27, 28, 30])
+def test_short_lists_on_a_state_in_memory(probe, n):
+    """A few gates that one pass applies run the (re, im) form at 21 to 25
+    qubits, with a parameterised one among them at 26 and 27; everything else is
+    planned as before."""
+    most = {21: 5, 22: 16, 23: 16, 24: 12, 25: 12, 26: 8, 27: 8}.get(n, 0)
+    passes = ctypes.c_int(0)
+    wide = 5 if n <= 21 else 6
+
+    def form(g, mode=qs.QS_MODE_FUSED, tile=0, dt=qs.QS_C64):
+        return probe.probe_held(n, dt, mode, tile, g.ctypes.data, g.size, ctypes.byref(passes))
+
+    for count in (1, 5, 6, 8, 9, 12, 13, 16, 17, 40):
+        for kinds in (CT, DIAG, [qs.QS_RX, qs.QS_RY], [qs.QS_T, qs.QS_CZ]):
+            for qubits in (2, n):
+                g = low_qubit_gates(count, kinds, seed=count, qubits=qubits)
+                low = {0, 1, 2, 3, 4} | {int(x["q0"]) for x in g if x["kind"] not in DIAG}
+                param = bool(np.any(g["kind"] >= qs.QS_RX))
+                short = len(low) <= 13 and count <= most and (n <= 25 or param)
+                assert form(g) == (0 if short else wide), (count, kinds, qubits)
+                assert not short or passes.value == 1
+                assert form(g, qs.QS_MODE_FUSED_TC) == 0 and form(g, dt=qs.QS_C128) == 0
+                assert form(g, tile=12) == (wide if n <= 12 else 5 if n <= 20 else 6)
+    # non-diagonal gates on more qubits than a tile: two passes, the wide form
+    g = np.zeros(12, dtype=qs.GATE_DTYPE)
+    g["kind"], g["q0"] = qs.QS_X_HALF, n - 1 - np.arange(12)
+    assert form(g) == wide

@@ -77,3 +77,16 @@ extern "C" int probe_sweep(int n, const qs_gate *g, size_t ng)
     for (const WidePass &p : w.passes) most = std::max(most, (int)p.nops);
     return most;
 }
+
+// Register bits of the wide form a list is planned for on a state that its
+// first pass reads (0: the (re, im) form), and the plan's passes.
+extern "C" int probe_held(int n, int dtype, int mode, int tile, const qs_gate *g, size_t ng, int *passes)
+{
+    qs_opts o{};
+    o.mode = mode;
+    o.tile_log2 = tile;
+    Plan plan;
+    if (build_plan(held_plan_params(default_plan_params(n, (qs_dtype)dtype, &o), g, ng), g, ng, &plan) != QS_OK) return -1;
+    *passes = (int)plan.passes.size();
+    return plan.wide;
+}
