@@ -252,7 +252,7 @@ def applied_plan(qs, n, g, md, prec=0):
         return {"passes": st["passes"], "launches": st["passes"] + (1 if k else 0),
                 "bytes": st["bytes"] + (N8 if k else 0.0), "fill": k}
     return {"passes": st["passes"], "launches": st["passes"],
-            "bytes": st["bytes"] - (N8 if k else 0.0), "fill": k}
+            "bytes": st["bytes"] - (N8 if k else 0.0), "fill": k, "reg_log2": st["reg_log2"]}
 
 
 def run_ours(args, rank, world, local):
@@ -484,7 +484,7 @@ def run_ours(args, rank, world, local):
         "config": workload_config(args, n, world),
         "apply_cycles_per_s": round(depth * args.steps / (passes_ms / 1000.0), 3),
         "passes_per_circuit": passes_total / args.steps,
-        "roofline": {"kernel": ("k_wide_pass<0,0,6>" if args.mode == "fused"
+        "roofline": {"kernel": ("k_wide_pass<0,0,%d>" % plans_seen[0]["reg_log2"] if args.mode == "fused"
                                 else "k_fused_pass<float,5,1,1>"),
                      "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak,
                      "peak_source": peak_src + " hbm_gbs", "unit": "GB/s",
@@ -783,14 +783,22 @@ def load_traffic(mode, n):
         return None
     import hashlib
     # the capture is of the current sources: qs_fused.cu (both forms share it
-    # for passes outside the wide form) and, for the fused form, the wide pass
+    # for passes outside the wide form) and, for the fused form, the wide pass:
+    # its body, its launches, and the generator of its op loop (which stores to
+    # the state and copies the next tile in)
     r = rec.get(mode) or {}
     csrc = os.path.join(ROOT, "paper_1608_00263_gb300", "csrc")
+    sources = [("source_sha1", ("qs_fused.cu",))]
+    if mode == "fused":
+        sources.append(("wide_sha1", ("qs_wide_device.cuh", "qs_wide.cu", "gen_op_loop.py")))
     try:
-        for key, name in (("source_sha1", "qs_fused.cu"),) + ((("wide_sha1", "qs_wide_device.cuh"),) if mode == "fused" else ()):
-            with open(os.path.join(csrc, name), "rb") as f:
-                if r.get(key) != hashlib.sha1(f.read()).hexdigest():
-                    return None
+        for key, names in sources:
+            h = hashlib.sha1()
+            for name in names:
+                with open(os.path.join(csrc, name), "rb") as f:
+                    h.update(f.read())
+            if r.get(key) != h.hexdigest():
+                return None
     except OSError:
         return None
     # scale the captured launch's traffic to this state size
