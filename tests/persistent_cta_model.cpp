@@ -89,6 +89,8 @@ static void wide_pass_body(float2 *, const WidePass *pass, const WideOp *, const
 }
 
 #define __global__ static
+#define __device__ static
+#define __forceinline__ inline
 #define __restrict__
 #define __launch_bounds__(...)
 #define __shared__ static
@@ -117,7 +119,7 @@ int main()
     };
     for (int i = 0; i < kInst; ++i) {
         const size_t first = items.size();
-        const uint32_t slot0 = slots, npass = 1 + (uint32_t)i % 3, nstat = 1 + (uint32_t)i % 2;
+        const uint32_t slot0 = slots, npass = 1 + (uint32_t)i % 3, nstat = i == 4 ? 35 : 1 + (uint32_t)i % 2;
         add(kPersistInit, i);
         ++before[i];
         for (uint32_t p = 0; p < npass; ++p) {

@@ -13,7 +13,8 @@ def kernel_text():
     with open(os.path.join(ROOT, "paper_1608_00263_gb300", "csrc", "qs_wide.cu")) as f:
         s = f.read()
     at = s.index("k_batch_persistent_wide(float2")
-    text = s[s.rindex("template <", 0, at):s.index("\n}\n", at) + 3]
+    sum_at = s.index("__device__ __forceinline__ double sum_slots")
+    text = s[sum_at:s.index("\n}\n", sum_at) + 3] + s[s.rindex("template <", 0, at):s.index("\n}\n", at) + 3]
     dyn = "extern __shared__ __align__(16) unsigned char smem_dyn[];"
     assert text.count(dyn) == 1
     return text.replace(dyn, "static unsigned char smem_dyn[16];")
