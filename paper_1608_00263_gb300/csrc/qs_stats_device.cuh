@@ -98,7 +98,12 @@ __device__ __forceinline__ void stat_terms(T y, T (&c)[kStatAcc])
 // (THREADS threads) calls it.  Amplitudes are read through L2
 // (ld.global.cg), so the chunk may have been written earlier in the same
 // launch by another CTA (after an acquire of that CTA's release).
-template <int THREADS = kStatThreads>
+// BATCHED: one test per sixteen amplitudes, so that their logarithms and powers
+// overlap (with a branch at each, one chain runs after the other): for few warps
+// per SM, where nothing else hides the chains.  It takes 158 registers instead
+// of 122; with many CTAs per SM to hide them the plain form wins.  The same sums
+// either way.
+template <int THREADS = kStatThreads, bool BATCHED = false>
 __device__ __forceinline__ void batch_stats_chunk(const float2 *a, uint64_t cnt, float scaleN, double *dst)
 {
     constexpr int kLoads = 8;                      // 16-byte loads in flight per thread
@@ -118,6 +123,20 @@ __device__ __forceinline__ void batch_stats_chunk(const float2 *a, uint64_t cnt,
             for (int k = 0; k < kLoads; ++k) {
                 const uint64_t u = u0 + (uint64_t)(j0 + k) * bd;
                 v[k] = u < units ? __ldcg(a4 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if constexpr (BATCHED) {
+                float y[2 * kLoads], top = 0.f;
+#pragma unroll
+                for (int k = 0; k < kLoads; ++k) {
+                    y[2 * k] = (v[k].x * v[k].x + v[k].y * v[k].y) * scaleN;
+                    y[2 * k + 1] = (v[k].z * v[k].z + v[k].w * v[k].w) * scaleN;
+                    top = fmaxf(top, fmaxf(y[2 * k], y[2 * k + 1]));
+                }
+                if (top <= 4096.f && u0 + (uint64_t)(j0 + kLoads - 1) * bd < units) {
+#pragma unroll
+                    for (int k = 0; k < 2 * kLoads; ++k) stat_terms<float>(y[k], c);
+                    continue;
+                }
             }
 #pragma unroll
             for (int k = 0; k < kLoads; ++k) {

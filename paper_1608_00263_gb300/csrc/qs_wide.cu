@@ -183,7 +183,7 @@ k_batch_persistent_wide(float2 *amps, const PersistItem *__restrict__ items, int
                 for (uint32_t e = threadIdx.x; e < w.lo / 2; e += blockDim.x) a[e] = u;
                 if (threadIdx.x == 0 && w.lo) a[0] = make_float4(w.f1, 0.f, w.f0, 0.f);
             } else if (w.kind == kPersistStats) {
-                batch_stats_chunk<kWideThreads>(amps + w.amp_off, w.lo, w.f0, part + (size_t)w.pass * kStatAcc);
+                batch_stats_chunk<kWideThreads, true>(amps + w.amp_off, w.lo, w.f0, part + (size_t)w.pass * kStatAcc);
             } else {
                 wide_pass_body<FULL ? 1 : 0, 2, GROUPED>(amps + w.amp_off, passes + w.pass, ops, codes, w.lo, w.hi, S, &F,
                                                       smem_dyn, 0, folds);

@@ -73,7 +73,7 @@ static int flag_wait_bounded(const uint32_t *count, uint32_t target, const uint3
 }
 
 static const WidePass *pass_base;
-template <int THREADS>
+template <int THREADS, bool BATCHED>
 static void batch_stats_chunk(const float2 *, uint64_t cnt, float, double *dst)
 {
     ran[threadIdx.x].push_back({kPersistStats, (uint32_t)cnt, 0});
