@@ -257,7 +257,9 @@ qs_status qs_state_sync(const qs_state *s);
  * u_j = (SplitMix64 output j of a stream seeded with `seed`) >> 11, times
  * 2^-53, and returns the smallest x with C_x > u_j * C_{N-1}, where C is the
  * cumulative sum of p in index order.  The total C_{N-1} normalises away any
- * norm drift; x with p(x) = 0 is never returned.  `out` (host or device,
+ * norm drift; x with p(x) = 0 is never returned.  Where k samples would read
+ * about as much as the whole state (2^n <= 100 k), the state keeps a table of
+ * at most 64 MB for them until it is destroyed.  `out` (host or device,
  * caller-owned) receives k uint64 indices in sample order.  Synchronous for
  * host `out`.  Returns QS_ERR_INVALID_ARG if the state has zero norm. */
 qs_status qs_sample(const qs_state *s, uint64_t k, uint64_t seed, uint64_t *out);
@@ -305,10 +307,12 @@ qs_status qs_cross_entropy(const qs_state *s, const uint64_t *samples,
  *   dL/dtheta = Im <lambda|P|psi>            for R_P(theta) = exp(-i theta/2 P),
  *   dL/dphi   = -2 Im <lambda|Pi_11|psi>     for CPHASE(phi).
  * grad[k] receives the derivative for gate k (0 for fixed gates).  Uses one
- * extra state vector (lambda), allocated stream-ordered for the call.  On
- * return the state holds the uncomputed vector (|0...0> up to rounding).
- * The paper has no gradients; this serves circuit-parameter studies around
- * the paper's cross-entropy benchmark.  Synchronous. */
+ * extra state vector (lambda).  complex64 states of 10 to 26 qubits keep it
+ * and the partial sums (at most 1 GB together), and the plan of the last gate
+ * list, until the state is destroyed; all others allocate it stream-ordered
+ * for the call.  On return the state holds the uncomputed vector (|0...0> up
+ * to rounding).  The paper has no gradients; this serves circuit-parameter
+ * studies around the paper's cross-entropy benchmark.  Synchronous. */
 qs_status qs_adjoint_gradient(qs_state *s, const qs_gate *gates, size_t ngates,
                               const uint64_t *samples, uint64_t m, const qs_opts *opts,
                               double *loss, double *grad);

@@ -1,5 +1,5 @@
 """Writes qs_log_table.inc: the table of the complex128 statistics' logarithm
-(log_pos in qs_stats.cu), pairs (c_i, -ln c_i) with c_i the FP32 value nearest
+(stat_terms_f64 in qs_stats.cu), pairs (c_i, -ln c_i) with c_i the FP32 value nearest
 1 / (1 + (i + 1/2) / SIZE).
 
 The logarithms are formed in 40 decimal digits and rounded once.  The build

@@ -14,10 +14,13 @@
 // complex128 path is FP64 throughout.  Block partials are combined in a
 // fixed order, so results are deterministic.
 //
-// The sampler never materialises a 2^n array: it keeps one FP64 sum per
-// 256-amplitude chunk (N/32 bytes), scans those, and for each sample
-// rescans one chunk with exactly the arithmetic that produced the chunk's
-// sum.
+// The sampler keeps one FP64 sum per 256-amplitude chunk (N/32 bytes) and scans
+// those; a sample's chunk is found among them.  Within the chunk, one of two
+// searches, both with exactly the arithmetic that produced the chunk's sum: the
+// chunk is rescanned for each sample, or, where that would read more than the
+// state (use_prefix_table), a table of every chunk's 32 in-chunk prefixes (N/8
+// values of the state's precision, at most 64 MB, kept with the state) is
+// looked up.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

@@ -227,8 +227,8 @@ qs_status launch_batch_round_wide(cudaStream_t st, int num_sms, void *amps, cons
 
 // The persistent kernel by (parameterised gates, tiles in groups): with thread
 // groups the tile stride, the barrier id and the buffer address are per-thread
-// values and the kernel spills (512 bytes of reloads, 1004 with parameterised
-// gates); without, 308 and 404.  64 instances of 20 qubits 2.01 -> 1.87 ms,
+// values and the kernel spills (540 bytes of reloads, 1032 with parameterised
+// gates); without, 340 and 436.  64 instances of 20 qubits 2.01 -> 1.87 ms,
 // eight of 23 2.16 -> 1.97 ms (lockstep rounds: 1.88 and 1.98).  Resident
 // CTAs per SM of each (occupancy API, set by batch_wide_setup before any
 // launch or capture).
