@@ -903,9 +903,9 @@ __device__ __forceinline__ void fused_pass_body(typename V2T<R>::T *__restrict__
             S.fu[u] = (uint8_t)((4u * (pairs & 1u) + tcnt) & 7u);
         }
         // uniform * e^{i pi k / 4}: 2^(-n/2) and 2^(-n/2) / sqrt2 formed in
-        // FP64 from n (the latter a power of two for odd n)
-        if (threadIdx.x < 8) {
-            const int k = (int)threadIdx.x;
+        // FP64 from n (the latter a power of two for odd n); a small tile's
+        // CTA has fewer than eight threads
+        for (int k = (int)threadIdx.x; k < 8; k += (int)blockDim.x) {
             const double a = std::exp2(-0.5 * S.P.n), c = a * 0.70710678118654752440;
             const double re[8] = {a, c, 0.0, -c, -a, -c, 0.0, c};
             const double im[8] = {0.0, c, a, c, 0.0, -c, -a, -c};
